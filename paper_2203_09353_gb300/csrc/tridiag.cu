@@ -1,0 +1,837 @@
+// Householder reduction of each walker's Hermitian positive semidefinite
+// n x n Gram matrix to a real tridiagonal matrix (d, e), for the entanglement
+// entropy (Alg. 1, "Calculate Entropy"): the steps of LAPACK's zlatrd/zhetrd
+// for the lower triangle, in 57-bit fixed point (fixed57.cuh) on the integer
+// pipe, one kernel for the whole reduction.
+//
+// Why fixed point. The reduction is (16/3) n^3 FP64 flops, half of them in
+// products A v that read the whole trailing matrix for each column. The FP64
+// pipe (2 DFMA per clock per SM) bounded it; three 32 x 32 + 64 bit integer
+// multiply-adds per real product are five times faster than a DFMA. Every quantity of the reduction is bounded by the matrix norm, so a
+// single power of two B scales it: entries, W and y carry an absolute
+// resolution of 2^-57 B .. 2^-55 B, which is the size of the FP64 reduction's
+// own normwise backward error.
+//
+// Per panel of kNb columns (c = column, u = reflector vector, H = I - tau u u^H):
+//   1. column c minus the panel's earlier rank-2 updates; d[c], and the exact
+//      integer sum of squares below the diagonal;
+//   2. norm N, e[c] = beta = -+N, u = (alpha - beta, x...): the column itself,
+//      shifted to full scale, not divided by alpha - beta, so that only the
+//      square root is on the critical path; tau = -u0 / (beta |u0|^2) is formed
+//      while the product runs;
+//   3. y = A u over the full (mirrored) trailing matrix, and W^H u, V^H u;
+//   4. y -= V (W^H u) + W (V^H u), p = tau y, rho = u^H y;
+//   5. w = p - (|tau|^2 rho / 2) u. (u, w) are column i of the panel's [V W].
+// After a panel, A -= V W^H + W V^H on the lower triangle, mirrored.
+//
+// A walker runs on one CTA, or on a cluster of up to 8 when there are fewer
+// walkers than SMs: rows are dealt to the CTAs in groups of 32 (group g to
+// rank g mod CL), every CTA holds u, and partial sums and the u rows go
+// through distributed shared memory, four cluster barriers a column. The
+// last kTail columns (or a whole matrix up to that order) are reduced by one
+// CTA with the matrix in shared memory.
+//
+// Bounds used by the formats (B = 2^57 units "uA" of the entries), with
+// |u|^2 in [0.5, 4) after scaling (unit 2^-56) and lambda = ||A|| <= B (the
+// limbs leave room for lambda <= kScaleRoom B):
+//   |y| <= 2 B, |W^H u| <= 4 B, |V^H u| <= 4, |tau| <= 4, rho <= 4 B,
+//   |w| <= 1.25 lambda / |u| < 1.8 B (unit 2 uA).
+// Row and column norms of A are at most lambda, so sums of products stay in
+// 64 bits by the Cauchy-Schwarz inequality.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <mutex>
+
+#include "bgemm_internal.h"
+#include "fixed57.cuh"
+
+namespace bg {
+namespace {
+
+using fx::Sum;
+
+constexpr int kThreads = 512;
+constexpr int kWarps = kThreads / 32;
+constexpr int kNb = 16;       // panel width
+constexpr int kTail = 96;     // columns reduced with the matrix in shared memory
+constexpr int kTailLd = kTail + 1;
+constexpr int kStrip = 4;     // columns per update work item
+constexpr int kMaxCl = 8;
+constexpr float kScaleRoom = 1.4f;
+constexpr size_t kSmemMax = 227 * 1024;
+constexpr int kAttrDevices = 64;
+
+struct TriArgs {
+  double2* G;   // walkers x n x n, lower triangle; overwritten
+  int4* P;      // walkers x 2 kNb x n: the panel's [V W] (clusters, or when it exceeds shared memory)
+  double* d;
+  double* e;
+  int n;
+  int own;      // rows a CTA owns at most (a multiple of 32)
+};
+
+// An exact integer sum of squares, s2 2^54 + s1 2^28 + s0.
+struct alignas(16) SquareSum {
+  long long s2, s1, s0, pad;
+};
+
+struct Scalars2 {  // a column's scalars, written by one thread
+  int z;           // u = column 2^z
+  int skip;
+  long long u0r, u0i, nint;
+};
+
+struct Shared {
+  longlong2 alpha[2];
+  SquareSum norm[2][kMaxCl * kWarps];  // of every warp of the cluster
+  longlong2 spart[2 * kNb][kMaxCl];    // V^H u and W^H u, a partial per CTA
+  long long rho[kMaxCl * kWarps];
+  longlong2 pnext;                     // p of row c + 1
+  int4 rowV[kNb], rowW[kNb];           // row c + 1 of V and W
+  int4 scoef[kWarps][2 * kNb];
+  int4 tau;                            // limbs, unit 2^-55
+  int2 t2;                             // |tau|^2 / 2, unit 2^-54
+  Scalars2 sc;
+  double dred[kWarps];
+  float2 fsum[kMaxCl * kWarps];        // (sum of squares, trace) of every warp
+};
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+
+// Writes v to the same shared-memory variable of every CTA of the cluster.
+template <bool MULTI>
+__device__ __forceinline__ void publish(int4* dst, const int4& v, int cl) {
+  if constexpr (!MULTI) {
+    *dst = v;
+  } else {
+    const uint32_t a = smem_addr(dst);
+    for (int r = 0; r < cl; ++r)
+      asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(mapa(a, r)), "r"(v.x),
+                   "r"(v.y), "r"(v.z), "r"(v.w)
+                   : "memory");
+  }
+}
+template <bool MULTI>
+__device__ __forceinline__ void publish(longlong2* dst, long long x, long long y, int cl) {
+  if constexpr (!MULTI) {
+    *dst = make_longlong2(x, y);
+  } else {
+    const uint32_t a = smem_addr(dst);
+    for (int r = 0; r < cl; ++r)
+      asm volatile("st.shared::cluster.v2.b64 [%0], {%1, %2};" ::"r"(mapa(a, r)), "l"(x), "l"(y)
+                   : "memory");
+  }
+}
+template <bool MULTI>
+__device__ __forceinline__ void publish(long long* dst, long long x, int cl) {
+  if constexpr (!MULTI) {
+    *dst = x;
+  } else {
+    const uint32_t a = smem_addr(dst);
+    for (int r = 0; r < cl; ++r)
+      asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(mapa(a, r)), "l"(x) : "memory");
+  }
+}
+
+// Barrier over the walker's threads: the CTA, or the cluster (release / acquire).
+template <bool MULTI>
+__device__ __forceinline__ void walker_sync() {
+  if constexpr (MULTI) {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  } else {
+    __syncthreads();
+  }
+}
+
+// One walker's (or its tail's) reduction state.
+struct Red {
+  int4* A;       // full matrix (both triangles), column-major
+  int ld, n;     // leading dimension, order
+  int4* P;       // [V W] in global memory, column q at P + q n (or null)
+  int4* vw;      // [V W] of the own rows in shared memory, column q at vw + q own
+  int own;
+  int4* us;      // u
+  longlong2* part;  // partial products; also x and p of the own rows
+  int4* stage;   // per-warp copies of [V W] rows for the update
+  double* d;
+  double* e;
+  int eunit;     // uA = 2^eunit
+  int rank, cl;
+  Shared* S;
+};
+
+template <bool ASM>
+__device__ __forceinline__ int4 ldA(const int4* p) {
+  if constexpr (ASM) return *p;
+  else return __ldcg(p);
+}
+
+// Reduces columns 0 .. cend - 1 (cend <= n - 1). MULTI: a cluster shares the
+// walker. VWS: the panel's own rows of V and W are in shared memory. ASM: so
+// is A.
+template <bool MULTI, bool VWS, bool ASM>
+__device__ __forceinline__ void reduce(const Red& R, int cend) {
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int n = R.n, ld = R.ld, own = R.own;
+  const int cl = MULTI ? R.cl : 1, rank = MULTI ? R.rank : 0;
+  const int ngroups = (n + 31) >> 5;
+  const int kmax = (ngroups - rank + cl - 1) / cl;  // own groups
+  Shared& S = *R.S;
+  longlong2* xs = R.part;  // x of the own rows (between steps 1 and 2)
+  auto vptr = [&](int q, int lr, int r) -> int4* {
+    return VWS ? R.vw + q * own + lr : R.P + (size_t)q * n + r;
+  };
+  auto vload = [&](int q, int lr, int r) -> int4 {
+    return VWS ? *vptr(q, lr, r) : __ldcg(vptr(q, lr, r));
+  };
+  for (int p0 = 0; p0 < cend; p0 += kNb) {
+    const int nbp = min(kNb, cend - p0);
+    for (int i = 0; i < nbp; ++i) {
+      const int c = p0 + i, par = c & 1;
+      // ---- 1. column c with the panel's earlier updates; sums of squares
+      long long s2 = 0, s1 = 0, s0 = 0;
+      for (int k = warp; k < kmax; k += kWarps) {
+        const int r = 32 * (rank + cl * k) + lane, lr = 32 * k + lane;
+        if (32 * (rank + cl * k) + 31 < c) continue;
+        long long xr = 0, xi = 0;
+        if (r >= c && r < n) {
+          const int4 a = ldA<ASM>(R.A + r + (size_t)c * ld);
+          Sum s;
+          for (int q = 0; q < i; ++q) {
+            cmac_conj(s, vload(q, lr, r), S.rowW[q]);
+            cmac_conj(s, vload(kNb + q, lr, r), S.rowV[q]);
+          }
+          xr = fx::join(a.x, a.y) - ((s.re() + 1) >> 1);
+          xi = fx::join(a.z, a.w) - ((s.im() + 1) >> 1);
+          if (r == c) R.d[c] = scalbn((double)xr, R.eunit);
+          if (r == c + 1) publish<MULTI>(&S.alpha[par], xr, xi, cl);
+          if (r >= c + 2) {
+            const fx::Limb lr_ = fx::split(xr), li_ = fx::split(xi);
+            fx::mac(s2, lr_.h, lr_.h);
+            fx::mac(s2, li_.h, li_.h);
+            fx::mac(s1, lr_.h, lr_.l);
+            fx::mac(s1, li_.h, li_.l);
+            fx::mac(s0, lr_.l, lr_.l);
+            fx::mac(s0, li_.l, li_.l);
+          }
+        }
+        xs[lr] = make_longlong2(xr, xi);
+      }
+      s2 = fx::warp_sum(s2);
+      s1 = fx::warp_sum(s1);
+      s0 = fx::warp_sum(s0);
+      if (lane == 0) {
+        longlong2* dst = reinterpret_cast<longlong2*>(&S.norm[par][rank * kWarps + warp]);
+        publish<MULTI>(dst, s2, s1, cl);
+        publish<MULTI>(dst + 1, s0, 0, cl);
+      }
+      walker_sync<MULTI>();
+      // ---- 2. norm, beta, u0: one warp of every CTA, from the same numbers
+      if (warp == 0) {
+        long long a2 = 0, a1 = 0, a0 = 0;
+        for (int x = lane; x < cl * kWarps; x += 32) {
+          const SquareSum v = S.norm[par][x];
+          a2 += v.s2;
+          a1 += v.s1;
+          a0 += v.s0;
+        }
+        a2 = fx::warp_sum(a2);
+        a1 = fx::warp_sum(a1);
+        a0 = fx::warp_sum(a0);
+        if (lane == 0) {
+          const longlong2 al = S.alpha[par];
+          Scalars2 sc{0, 0, 0, 0, 0};
+          double beta;
+          if (a2 == 0 && a1 == 0 && a0 == 0 && al.y == 0) {
+            sc.skip = 1;  // already reduced: H = I
+            beta = (double)al.x;
+          } else {
+            const double ar = (double)al.x, ai = (double)al.y;
+            double n2 = fma((double)a2, 0x1p54,
+                            fma((double)a1, 0x1p28, (double)(unsigned long long)a0));
+            n2 = fma(ar, ar, fma(ai, ai, n2));
+            const double N = sqrt(n2);
+            const int eN = (int)((__double2hiint(N) >> 20) & 0x7FF) - 1022;  // N in [2^(eN-1), 2^eN)
+            sc.z = 56 - eN;
+            sc.nint = __double2ll_rn(N * __hiloint2double((1023 + sc.z) << 20, 0));
+            const long long xr = fx::shift(al.x, sc.z);
+            sc.u0r = al.x < 0 ? xr - sc.nint : xr + sc.nint;
+            sc.u0i = fx::shift(al.y, sc.z);
+            beta = al.x < 0 ? N : -N;
+          }
+          if (rank == 0) R.e[c] = scalbn(beta, R.eunit);
+          S.sc = sc;
+        }
+      }
+      __syncthreads();
+      const Scalars2 sc = S.sc;
+      // u to every CTA; V's column i
+      for (int k = warp; k < kmax; k += kWarps) {
+        const int r = 32 * (rank + cl * k) + lane, lr = 32 * k + lane;
+        if (32 * (rank + cl * k) + 31 <= c) continue;
+        if (r > c && r < n) {
+          int4 u = make_int4(0, 0, 0, 0);
+          if (!sc.skip) {
+            const longlong2 x = xs[lr];
+            u = r == c + 1 ? fx::pack(sc.u0r, sc.u0i)
+                           : fx::pack(fx::shift(x.x, sc.z), fx::shift(x.y, sc.z));
+            publish<MULTI>(R.us + r, u, cl);
+          }
+          if constexpr (VWS) *vptr(i, lr, r) = u;
+          if (MULTI || !VWS) R.P[(size_t)i * n + r] = u;
+          if (sc.skip) {
+            if constexpr (VWS) *vptr(kNb + i, lr, r) = u;
+            if (MULTI || !VWS) R.P[(size_t)(kNb + i) * n + r] = u;
+          }
+        }
+      }
+      const int gnext = (c + 1) >> 5;  // the group holding row c + 1
+      const bool owns_next = gnext % cl == rank && (gnext / cl) % kWarps == warp;
+      // row c + 1 of V and W for the next column's step 1 (columns below i;
+      // its owner publishes them, column i follows from u and p)
+      auto publish_row = [&]() {
+        if (!owns_next) return;
+        const int r = c + 1, lr = 32 * (gnext / cl) + (r & 31);
+        const int q = lane & 15;
+        if (q < i) {
+          const int4 v = vload((lane & 16) + q, lr, r);
+          publish<MULTI>((lane & 16) ? &S.rowW[q] : &S.rowV[q], v, cl);
+        }
+      };
+      if (sc.skip) {
+        publish_row();
+        if (t == 0) S.rowV[i] = S.rowW[i] = make_int4(0, 0, 0, 0);
+        walker_sync<MULTI>();
+        continue;
+      }
+      walker_sync<MULTI>();
+      // ---- 3. tau, by one thread beside the products
+      if (t == kThreads - 32) {
+        const double br = (sc.u0r < 0 ? 1.0 : -1.0) * (double)sc.nint * 0x1p-56;  // beta, scaled
+        const double ur = (double)sc.u0r * 0x1p-56, ui = (double)sc.u0i * 0x1p-56;
+        const double rden = -1.0 / (br * fma(ur, ur, ui * ui));
+        const double tr = ur * rden, ti = ui * rden;
+        S.tau = fx::pack(__double2ll_rn(tr * 0x1p55), __double2ll_rn(ti * 0x1p55));
+        const fx::Limb l = fx::split(__double2ll_rn(fma(tr, tr, ti * ti) * 0x1p53));
+        S.t2 = make_int2(l.h, l.l);
+      }
+      // V^H u and W^H u over the own rows, a warp per column
+      for (int it = warp; it < 2 * i; it += kWarps) {
+        const int q = it >> 1, vq = (it & 1) ? kNb + q : q;
+        Sum s;
+        for (int k = max(0, (c + 1) / 32 / cl - 1); k < kmax; ++k) {
+          const int r = 32 * (rank + cl * k) + lane, lr = 32 * k + lane;
+          if (r > c && r < n) {
+            const int4 v = vload(vq, lr, r);
+            cmac(s, make_int4(v.x, v.y, -v.z, -v.w), R.us[r]);
+          }
+        }
+        const long long sr = fx::warp_sum(s.re()), si = fx::warp_sum(s.im());
+        if (lane == 0) publish<MULTI>(&S.spart[vq][rank], sr, si, cl);
+      }
+      // y = A u: items of one own group of rows x a run of columns
+      int kfirst = (c + 1) / 32;  // first own group with a row > c
+      kfirst = kfirst > rank ? (kfirst - rank + cl - 1) / cl : 0;
+      const int cnt = kmax - kfirst;
+      const int nch = cnt > 0 ? max(1, kWarps / cnt) : 1;
+      for (int it = warp; it < cnt * nch; it += kWarps) {
+        const int gi = it % cnt, ch = it / cnt;
+        const int r = 32 * (rank + cl * (kfirst + gi)) + lane;
+        const int m = n - c - 1;
+        int j = c + 1 + m * ch / nch;
+        const int j1 = c + 1 + m * (ch + 1) / nch;
+        const int4* a = R.A + min(r, n - 1) + (size_t)j * ld;
+        Sum s;
+        constexpr int U = 8;
+        int4 nx[U];
+        if (j + U <= j1) {
+#pragma unroll
+          for (int x = 0; x < U; ++x) nx[x] = ldA<ASM>(a + (size_t)x * ld);
+        }
+        for (; j + U <= j1; j += U) {
+          int4 cur[U];
+#pragma unroll
+          for (int x = 0; x < U; ++x) cur[x] = nx[x];
+          a += (size_t)U * ld;
+          if (j + 2 * U <= j1) {
+#pragma unroll
+            for (int x = 0; x < U; ++x) nx[x] = ldA<ASM>(a + (size_t)x * ld);
+          }
+#pragma unroll
+          for (int x = 0; x < U; ++x) cmac(s, cur[x], R.us[j + x]);
+        }
+        for (; j < j1; ++j, a += ld) cmac(s, ldA<ASM>(a), R.us[j]);
+        R.part[it * 32 + lane] = make_longlong2(s.re(), s.im());  // unit uA / 4
+      }
+      walker_sync<MULTI>();
+      // ---- 4. corrections, p = tau y, rho
+      long long rho = 0;
+      {
+        // lane x: coefficient column x (V^H u below 16, W^H u above), in limbs
+        long long cr = 0, ci = 0;
+        if ((lane & 15) < i) {
+          for (int x = 0; x < cl; ++x) {
+            const longlong2 v = S.spart[lane][x];
+            cr += v.x;
+            ci += v.y;
+          }
+        }
+        S.scoef[warp][lane] = fx::pack((cr + 4) >> 3, (ci + 4) >> 3);
+        __syncwarp();
+      }
+      const int4 tau = S.tau;
+      // (the own groups from kfirst on, each by the warp that owns it in steps 1 and 5)
+      for (int k = warp; k < kmax; k += kWarps) {
+        if (k < kfirst) continue;
+        const int r = 32 * (rank + cl * k) + lane, lr = 32 * k + lane, gi = k - kfirst;
+        long long yr = 0, yi = 0;
+        for (int ch = 0; ch < nch; ++ch) {
+          const longlong2 v = R.part[(ch * cnt + gi) * 32 + lane];
+          yr += v.x;
+          yi += v.y;
+        }
+        long long pr = 0, pi = 0;
+        if (r > c && r < n) {
+          Sum s;
+          for (int q = 0; q < i; ++q) {
+            cmac(s, vload(q, lr, r), S.scoef[warp][kNb + q]);       // V (W^H u)
+            cmac(s, vload(kNb + q, lr, r), S.scoef[warp][q]);       // W (V^H u)
+          }
+          yr -= (s.rh << 2) + ((s.rx + (1ll << 24)) >> 25);
+          yi -= (s.ih << 2) + ((s.ix + (1ll << 24)) >> 25);
+          const int4 yq = fx::pack((yr + 4) >> 3, (yi + 4) >> 3);  // unit 2 uA
+          Sum ps;
+          cmac(ps, tau, yq);
+          pr = ps.re();
+          pi = ps.im();
+          const int4 u = R.us[r];
+          long long h = 0, x = 0;
+          fx::mac(h, u.x, yq.x);
+          fx::mac(h, u.z, yq.z);
+          fx::mac(x, u.x, yq.y);
+          fx::mac(x, u.y, yq.x);
+          fx::mac(x, u.z, yq.w);
+          fx::mac(x, u.w, yq.z);
+          rho += fx::val(h, x);  // unit uA / 2
+          if (r == c + 1) publish<MULTI>(&S.pnext, pr, pi, cl);
+        }
+        R.part[gi * 32 + lane] = make_longlong2(pr, pi);
+      }
+      rho = fx::warp_sum(rho);
+      if (lane == 0) publish<MULTI>(&S.rho[rank * kWarps + warp], rho, cl);
+      publish_row();
+      walker_sync<MULTI>();
+      // ---- 5. w = p - (|tau|^2 rho / 2) u
+      rho = 0;
+      for (int x = lane; x < cl * kWarps; x += 32) rho += S.rho[x];
+      rho = fx::warp_sum(rho);
+      const fx::Limb rq = fx::split((rho + 4) >> 3);  // unit 4 uA
+      const int2 t2 = S.t2;
+      long long ch_ = 0, cx_ = 0;
+      fx::mac(ch_, t2.x, rq.h);
+      fx::mac(cx_, t2.x, rq.l);
+      fx::mac(cx_, t2.y, rq.h);
+      const fx::Limb cc = fx::split(fx::val(ch_, cx_));  // unit 4 uA
+      auto make_w = [&](long long pr, long long pi, const int4& u) -> int4 {
+        long long rh = 0, rx = 0, ih = 0, ix = 0;
+        fx::mac(rh, cc.h, u.x);
+        fx::mac(rx, cc.h, u.y);
+        fx::mac(rx, cc.l, u.x);
+        fx::mac(ih, cc.h, u.z);
+        fx::mac(ix, cc.h, u.w);
+        fx::mac(ix, cc.l, u.z);
+        return fx::pack((pr - fx::val(rh, rx) + 1) >> 1, (pi - fx::val(ih, ix) + 1) >> 1);
+      };
+      for (int k = warp; k < kmax; k += kWarps) {
+        if (k < kfirst) continue;
+        const int r = 32 * (rank + cl * k) + lane, lr = 32 * k + lane;
+        if (r > c && r < n) {
+          const longlong2 p = R.part[(k - kfirst) * 32 + lane];
+          const int4 w = make_w(p.x, p.y, R.us[r]);
+          if constexpr (VWS) *vptr(kNb + i, lr, r) = w;
+          if (MULTI || !VWS) R.P[(size_t)(kNb + i) * n + r] = w;
+        }
+      }
+      if (t == kThreads - 1) {
+        S.rowV[i] = R.us[c + 1];
+        S.rowW[i] = make_w(S.pnext.x, S.pnext.y, R.us[c + 1]);
+      }
+      __syncthreads();
+    }
+    walker_sync<MULTI>();
+    // ---- trailing update on rows and columns q0 ..: a warp per 32 rows x
+    // kStrip columns of the lower triangle, written to both triangles
+    const int q0 = p0 + nbp;
+    {
+      const int nw = cl * kWarps, gw = rank * kWarps + warp;
+      const int c00 = q0 / kStrip * kStrip;
+      int base = 0;
+      for (int I = q0 >> 5; I < ngroups; ++I) {
+        const int cntI = (min(32 * I + 32, n) - c00 + kStrip - 1) / kStrip;
+        int s = (gw - base) % nw;
+        if (s < 0) s += nw;
+        base += cntI;
+        for (; s < cntI; s += nw) {
+          const int cs = c00 + s * kStrip;
+          const int r = 32 * I + lane, rc = min(r, n - 1);
+          const int4* st = nullptr;
+          if constexpr (MULTI || !VWS) {
+            int4* sg = R.stage + warp * (2 * kNb * kStrip);
+            __syncwarp();
+#pragma unroll
+            for (int x = 0; x < kStrip; ++x) {
+              const int q = x * (32 / kStrip) + lane / kStrip, cc = cs + lane % kStrip;
+              sg[q * kStrip + lane % kStrip] = (q & 15) < nbp && cc < n
+                                                   ? __ldcg(R.P + (size_t)q * n + cc)
+                                                   : make_int4(0, 0, 0, 0);
+            }
+            __syncwarp();
+            st = sg;
+          }
+          int4 a[kStrip];
+#pragma unroll
+          for (int x = 0; x < kStrip; ++x)
+            a[x] = ldA<ASM>(R.A + rc + (size_t)min(cs + x, n - 1) * ld);
+          Sum sum[kStrip];
+#pragma unroll 2
+          for (int q = 0; q < nbp; ++q) {
+            int4 v, w;
+            if constexpr (MULTI || !VWS) {
+              v = __ldcg(R.P + (size_t)q * n + rc);
+              w = __ldcg(R.P + (size_t)(kNb + q) * n + rc);
+            } else {
+              v = R.vw[q * own + rc];
+              w = R.vw[(kNb + q) * own + rc];
+            }
+#pragma unroll
+            for (int x = 0; x < kStrip; ++x) {
+              int4 cv, cw;
+              if constexpr (MULTI || !VWS) {
+                cv = st[q * kStrip + x];
+                cw = st[(kNb + q) * kStrip + x];
+              } else {
+                cv = R.vw[q * own + min(cs + x, n - 1)];
+                cw = R.vw[(kNb + q) * own + min(cs + x, n - 1)];
+              }
+              cmac_conj(sum[x], v, cw);
+              cmac_conj(sum[x], w, cv);
+            }
+          }
+#pragma unroll
+          for (int x = 0; x < kStrip; ++x) {
+            const int cc = cs + x;
+            if (r >= n || cc > r || cc < q0) continue;
+            const long long re = fx::join(a[x].x, a[x].y) - ((sum[x].re() + 1) >> 1);
+            const long long im = r == cc ? 0 : fx::join(a[x].z, a[x].w) - ((sum[x].im() + 1) >> 1);
+            const int4 v = fx::pack(re, im);
+            R.A[r + (size_t)cc * ld] = v;
+            if (r != cc) R.A[cc + (size_t)r * ld] = fx::pack(re, -im);
+          }
+        }
+      }
+    }
+    walker_sync<MULTI>();
+  }
+}
+
+// |x| 2^-e as a float rounded down by at most 2^-20 of itself (inf for a
+// non-finite x, 0 below 2^-126).
+__device__ __forceinline__ float scaled_abs(double x, int e) {
+  const uint32_t h = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
+  const int eb = (int)(h >> 20);
+  const int ef = eb - 1023 - e + 127;
+  if (eb == 0x7FF || ef >= 255) return __int_as_float(0x7F800000);
+  if (ef <= 0 || eb == 0) return 0.0f;
+  return __int_as_float((ef << 23) | (int)((h & 0xFFFFFu) << 3));
+}
+
+// The whole reduction of walker blockIdx.x / cl. SMALL: n <= kTail, the
+// matrix goes straight to shared memory.
+template <bool MULTI, bool VWS, bool SMALL>
+__global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g) {
+  extern __shared__ __align__(16) int4 sm4[];
+  __shared__ Shared S;
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  int cl = 1, rank = 0;
+  if constexpr (MULTI) {
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(cl));
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  }
+  const int n = g.n;
+  const size_t w = blockIdx.x / cl;
+  double2* G = g.G + w * n * n;
+  double* dw = g.d + w * n;
+  double* ew = g.e + w * n;
+  // ---- the scale: with t the mean eigenvalue (trace / n), the largest one is
+  // at most t + sqrt((n - 1) (||G||_F^2 / n - t^2))
+  double dm = 0.0;
+  for (int i = t; i < n; i += kThreads) dm = fmax(dm, fabs(__ldcg(&G[i + (size_t)i * n].x)));
+  for (int o = 16; o > 0; o >>= 1) dm = fmax(dm, __shfl_xor_sync(0xFFFFFFFFu, dm, o));
+  if (lane == 0) S.dred[warp] = dm;
+  walker_sync<MULTI>();  // also: every CTA of the cluster runs before its memory is written
+  dm = 0.0;
+  for (int i = 0; i < kWarps; ++i) dm = fmax(dm, S.dred[i]);
+  const int e0 = dm > 0.0 ? (int)((__double2hiint(dm) >> 20) & 0x7FF) - 1022 : 0;
+  const int ngroups = (n + 31) >> 5;
+  float f2 = 0.0f, tr = 0.0f;
+  for (int idx = rank * kWarps + warp; idx < n; idx += cl * kWarps) {
+    // a warp per column, its lower part
+    for (int r = idx + lane; r < n; r += 32) {
+      const double2 z = __ldcg(&G[r + (size_t)idx * n]);
+      const float a = scaled_abs(z.x, e0), b = r == idx ? 0.0f : scaled_abs(z.y, e0);
+      const float q = fmaf(a, a, b * b);
+      f2 += r == idx ? q : 2.0f * q;
+      tr += r == idx ? a : 0.0f;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    f2 += __shfl_xor_sync(0xFFFFFFFFu, f2, o);
+    tr += __shfl_xor_sync(0xFFFFFFFFu, tr, o);
+  }
+  if (lane == 0) {
+    if constexpr (MULTI) {
+      for (int x = 0; x < cl; ++x)
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(
+                         mapa(smem_addr(&S.fsum[rank * kWarps + warp]), x)),
+                     "f"(f2), "f"(tr)
+                     : "memory");
+    } else {
+      S.fsum[warp] = make_float2(f2, tr);
+    }
+  }
+  walker_sync<MULTI>();
+  float F2 = 0.0f, mean = 0.0f;
+  for (int x = 0; x < cl * kWarps; ++x) {
+    F2 += S.fsum[x].x;
+    mean += S.fsum[x].y;
+  }
+  mean /= (float)n;
+  if (!(F2 < __int_as_float(0x7F800000))) {  // a NaN or infinity in G
+    const double nan = __longlong_as_double(0x7FF8000000000000ll);
+    if (rank == 0)
+      for (int i = t; i < n; i += kThreads) {
+        dw[i] = nan;
+        ew[i] = i + 1 < n ? nan : 0.0;
+      }
+    return;
+  }
+  // the bound, with 4e-5 of the sum of squares for the float sums' rounding
+  const float var = fmaxf(F2 / (float)n - mean * mean, 0.0f) + 4e-5f * F2 / (float)n;
+  const float lam = (mean + sqrtf((float)(n - 1) * var)) * 1.0001f;
+  // B = 2^eB >= bound / kScaleRoom; a zero matrix takes any scale
+  const float B = lam * (1.0f / kScaleRoom);
+  const int eB = e0 + (B > 0.0f ? (int)((__float_as_uint(B) >> 23) & 0xFF) - 126 : 0);
+  const int eunit = eB - fx::kLow - 30;  // uA = 2^(eB - 57)
+  Red R;
+  R.S = &S;
+  R.eunit = eunit;
+  R.rank = rank;
+  R.cl = cl;
+  R.d = dw;
+  R.e = ew;
+  int4* sm = sm4;
+  const int nt = SMALL ? n : kTail;
+  // ---- fixed point, both triangles (in place, or into shared memory)
+  Red T = R;  // the shared-memory reduction
+  T.n = nt;
+  T.ld = kTailLd;
+  T.own = kTail;
+  T.us = sm;
+  T.part = reinterpret_cast<longlong2*>(T.us + kTail);
+  T.vw = reinterpret_cast<int4*>(T.part + kWarps * 32);
+  T.A = T.vw + 2 * kNb * kTail;
+  T.P = nullptr;
+  T.stage = nullptr;
+  T.rank = 0;
+  T.cl = 1;
+  T.d = dw + (n - nt);
+  T.e = ew + (n - nt);
+  {
+    int4* A = SMALL ? T.A : reinterpret_cast<int4*>(G);
+    const int ld = SMALL ? T.ld : n;
+    const int nw = cl * kWarps, gw = rank * kWarps + warp;
+    int base = 0;
+    for (int I = 0; I < ngroups; ++I) {
+      const int cntI = (min(32 * I + 32, n) + kStrip - 1) / kStrip;
+      int s = (gw - base) % nw;
+      if (s < 0) s += nw;
+      base += cntI;
+      for (; s < cntI; s += nw) {
+        const int r = 32 * I + lane;
+        double2 z[kStrip];
+#pragma unroll
+        for (int x = 0; x < kStrip; ++x) {
+          const int cc = s * kStrip + x;
+          z[x] = r < n && cc <= r ? __ldcg(&G[r + (size_t)cc * n]) : make_double2(0.0, 0.0);
+        }
+#pragma unroll
+        for (int x = 0; x < kStrip; ++x) {
+          const int cc = s * kStrip + x;
+          if (r >= n || cc > r) continue;
+          const long long re = fx::from_double(z[x].x, -eunit);
+          const long long im = r == cc ? 0 : fx::from_double(z[x].y, -eunit);
+          A[r + (size_t)cc * ld] = fx::pack(re, im);
+          if (r != cc) A[cc + (size_t)r * ld] = fx::pack(re, -im);
+        }
+      }
+    }
+  }
+  walker_sync<MULTI>();
+  if constexpr (!SMALL) {
+    R.A = reinterpret_cast<int4*>(G);
+    R.ld = n;
+    R.n = n;
+    R.own = g.own;
+    R.P = g.P ? g.P + w * (size_t)(2 * kNb) * n : nullptr;
+    R.us = sm;
+    R.part = reinterpret_cast<longlong2*>(R.us + n);
+    const int nparts = max(kWarps, g.own / 32) * 32;
+    R.vw = reinterpret_cast<int4*>(R.part + nparts);
+    R.stage = reinterpret_cast<int4*>(R.part + nparts) + (VWS ? 2 * kNb * g.own : 0);
+    reduce<MULTI, VWS, false>(R, n - kTail);  // ends with a barrier of the walker
+    if (rank != 0) return;
+    const int4* A0 = R.A + (n - kTail) + (size_t)(n - kTail) * n;
+    for (int x = t; x < kTail * kTail; x += kThreads) {
+      const int r = x % kTail, c = x / kTail;
+      T.A[r + c * kTailLd] = __ldcg(A0 + r + (size_t)c * n);
+    }
+    __syncthreads();
+  }
+  reduce<false, true, true>(T, nt - 1);
+  if (t == 0) {
+    const int4 v = T.A[(nt - 1) + (size_t)(nt - 1) * T.ld];
+    dw[n - 1] = scalbn((double)fx::join(v.x, v.y), eunit);
+    ew[n - 1] = 0.0;
+  }
+}
+
+constexpr size_t tail_smem() {
+  return (size_t)kTail * 16 + (size_t)kWarps * 32 * 16 + (size_t)2 * kNb * kTail * 16 +
+         (size_t)kTail * kTailLd * 16;
+}
+
+struct TriShape {
+  int cl = 1, own = 0;
+  bool vws = false;
+  size_t smem = 0;
+};
+
+TriShape shape_for(int n, int cl) {
+  TriShape s;
+  s.cl = cl;
+  const int groups = (n + 31) / 32;
+  s.own = (groups + cl - 1) / cl * 32;
+  const size_t fixed = (size_t)n * 16 + (size_t)std::max(kWarps, s.own / 32) * 32 * 16;
+  const size_t vw = (size_t)2 * kNb * s.own * 16;
+  const size_t stage = (size_t)kWarps * 2 * kNb * kStrip * 16;
+  const size_t budget = kSmemMax - sizeof(Shared) - 512;
+  s.vws = fixed + vw + (cl > 1 ? stage : 0) <= budget;
+  s.smem = std::max(tail_smem(), fixed + (s.vws ? vw : 0) + (cl > 1 || !s.vws ? stage : 0));
+  return s;
+}
+
+void launch_config(const TriShape& s, int64_t walkers, cudaStream_t st, cudaLaunchConfig_t* cfg,
+                   cudaLaunchAttribute* at) {
+  cfg->gridDim = dim3((unsigned)(walkers * s.cl));
+  cfg->blockDim = dim3(kThreads);
+  cfg->dynamicSmemBytes = s.smem;
+  cfg->stream = st;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = (unsigned)s.cl;
+  at->val.clusterDim.y = 1;
+  at->val.clusterDim.z = 1;
+  cfg->attrs = at;
+  cfg->numAttrs = s.cl > 1 ? 1 : 0;
+}
+
+template <bool MULTI, bool VWS, bool SMALL>
+cudaError_t launch_reduce(const TriArgs& a, int64_t walkers, const TriShape& s, cudaStream_t st) {
+  auto kernel = tri_reduce_kernel<MULTI, VWS, SMALL>;
+  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)s.smem);
+  if (err != cudaSuccess) return err;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  launch_config(s, walkers, st, &cfg, at);
+  err = cudaLaunchKernelEx(&cfg, kernel, a);
+  if (err != cudaSuccess) return err;
+  count_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+// CTAs per walker: the most (up to 8, and a group of 32 rows each before the
+// tail) for which the device holds every walker's cluster at once. Clusters
+// of 8 fit 15 times on a GB300 (GPCs of 18 to 20 SMs, one CTA per SM), of 4
+// 36 times, so 16 walkers run on clusters of 7 at most; a second wave would
+// double the time.
+int tri_cluster(int64_t walkers, int n) {
+  if (n <= kTail || walkers <= 0) return 1;
+  static std::mutex mu;
+  static int active[kAttrDevices][kMaxCl + 1];  // clusters the device holds, 0 = not asked yet
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kAttrDevices) return 1;
+  std::lock_guard<std::mutex> lk(mu);
+  for (int cl = std::min(kMaxCl, (n - kTail) / 32); cl > 1; --cl) {
+    int& a = active[dev][cl];
+    if (a == 0) {
+      // the largest request any order makes: one CTA per SM
+      auto kernel = tri_reduce_kernel<true, true, false>;
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute at[1];
+      TriShape s;
+      s.cl = cl;
+      s.smem = kSmemMax - sizeof(Shared) - 512;
+      int c = 0;
+      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)s.smem) != cudaSuccess)
+        return 1;
+      launch_config(s, 1, nullptr, &cfg, at);
+      if (cudaOccupancyMaxActiveClusters(&c, kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+      }
+      a = std::max(c, 1);
+    }
+    if (a >= walkers) return cl;
+  }
+  return 1;
+}
+
+size_t tri_workspace(int64_t walkers, int n) {
+  if (n <= kTail) return 0;
+  const TriShape s = shape_for(n, tri_cluster(walkers, n));
+  return s.cl > 1 || !s.vws ? (size_t)walkers * 2 * kNb * n * sizeof(int4) : 0;
+}
+
+cudaError_t launch_tridiag(double2* gram, int64_t walkers, int n, void* panel, double* d,
+                           double* e, cudaStream_t st) {
+  if (walkers <= 0) return cudaSuccess;
+  TriArgs a{gram, static_cast<int4*>(panel), d, e, n, 0};
+  if (n <= kTail) {
+    TriShape s;
+    s.smem = tail_smem();
+    return launch_reduce<false, true, true>(a, walkers, s, st);
+  }
+  const TriShape s = shape_for(n, tri_cluster(walkers, n));
+  a.own = s.own;
+  if (s.cl > 1)
+    return s.vws ? launch_reduce<true, true, false>(a, walkers, s, st)
+                 : launch_reduce<true, false, false>(a, walkers, s, st);
+  return s.vws ? launch_reduce<false, true, false>(a, walkers, s, st)
+               : launch_reduce<false, false, false>(a, walkers, s, st);
+}
+
+}  // namespace bg
