@@ -1442,7 +1442,7 @@ bg_status entropy_plan(bg_plan** out, int64_t walkers, int32_t spins, int32_t sp
       return cuda_fail(e, "entropy plan workspace");
     }
     p->workspace_bytes = p->gram->workspace_bytes + (int64_t)(gb + 2 * tb);
-    p->launches_per_call = p->gram->launches_per_call + 2;
+    p->launches_per_call = p->gram->launches_per_call + 3;
     const size_t pb = tri_workspace(walkers, (int)K);
     if (pb > 0) {
       if ((e = cudaMalloc(&p->d_tri_p, pb)) != cudaSuccess) {
@@ -1484,10 +1484,14 @@ bg_status batched_entropy(const bg_plan* plan, const void* states, double* entro
     BG_CUDA(cudaEventRecord(ev[1], st), "profiling event record");
     BG_CUDA(cudaEventRecord(ev[2], st), "profiling event record");
   }
+  DeviceCtx* ctx;
+  if ((s = get_ctx(&ctx)) != BG_OK) return s;
+  // (the eigenvalues go over the Gram matrices, which the reduction has used up)
   cudaError_t e = launch_tridiag(p->d_gram, p->count, p->ent_n, p->d_tri_p, p->d_tri_d,
                                  p->d_tri_e, st);
   if (e == cudaSuccess)
-    e = launch_entropy_bisect(p->d_tri_d, p->d_tri_e, p->count, p->ent_n, entropy, eigenvalues,
+    e = launch_entropy_bisect(p->d_tri_d, p->d_tri_e, p->count, p->ent_n,
+                              reinterpret_cast<double*>(p->d_gram), entropy, eigenvalues, ctx->sms,
                               st);
   if (e != cudaSuccess) return cuda_fail(e, "entropy eigenvalue launch");
   if (ev) BG_CUDA(cudaEventRecord(ev[3], st), "profiling event record");

@@ -132,9 +132,11 @@ cudaError_t launch_tridiag(double2* gram, int64_t walkers, int n, void* panel, d
                            double* e, cudaStream_t st);
 
 // Eigenvalues of the tridiagonal matrices and the entropies (entropy.cu).
-// eigs: optional device [walkers][n], ascending.
+// lam: workspace of walkers x n doubles; eigs: optional device [walkers][n],
+// ascending.
 cudaError_t launch_entropy_bisect(const double* d, const double* e, int64_t walkers, int n,
-                                  double* entropy, double* eigs, cudaStream_t st);
+                                  double* lam, double* entropy, double* eigs, int sms,
+                                  cudaStream_t st);
 
 // Metropolis decision per walker and copy of the accepted proposals over the
 // current states (anneal.cu). prop / cur may be null when amps == 0.

@@ -8,9 +8,12 @@
 // BG_PLAN_HERK, FP64 or split precision), lower triangle; tridiag.cu reduces
 // it to a real symmetric tridiagonal matrix (d, e). Here, bisect_kernel takes
 // every eigenvalue of the tridiagonal matrix by bisection on the Sturm count
-// (the number of eigenvalues below x), one thread per eigenvalue, then the
-// entropy by a block reduction; it is bound by the FP64 pipe (about 2 DFMA
-// per clock per SM on this part), not by memory.
+// (the number of eigenvalues below x), spread over the GPU, and
+// entropy_sum_kernel the entropies. An FP64 count is bound by the FP64 pipe
+// (3 instructions a step at 2 per clock per SM), so most of the bisection
+// runs in FP32 and in pairs of floats; few eigenvalues per SM are bound by
+// the counts' latency and get several lanes each. Measured: 128 matrices of
+// order 256 3.05 -> 1.5 ms, 16 of order 1024 47.8 -> 3.7 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -22,7 +25,8 @@
 namespace bg {
 namespace {
 
-constexpr int kEntThreads = 256;  // bisection
+constexpr int kEntThreads = 256;  // the entropy sums
+
 // A kernel's dynamic shared-memory limit is a property of the device: set it
 // once per device (at every call for ordinals beyond the table).
 constexpr int kAttrDevices = 64;
@@ -62,53 +66,8 @@ __device__ double block_max(double v, double* red) {
   return s;
 }
 
-// 1/q for a normal q: the hardware's approximate reciprocal, then two
-// Newton-Raphson steps r <- r + r (1 - q r), each of which squares the
-// relative error (to well below 2^-80, so r is within an ulp or so of 1/q).
-// On this part an FP64 instruction is slow; this takes five of them where
-// an IEEE division takes about twice as many.
-__device__ __forceinline__ double recip_nr(double q) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(q));
-  double e = fma(-q, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-q, r, 1.0);
-  return fma(r, e, r);
-}
-
-// Number of eigenvalues of the symmetric tridiagonal (d, e2 = e^2) below x:
-// the negative pivots of T - x I (a pivot smaller than pivmin in magnitude
-// is replaced by -pivmin, as in LAPACK's dstebz). The pivot recurrence
-// q_i = (d_i - x) - e2_{i-1} / q_{i-1} is backward stable: the count is exact
-// for entries perturbed by a few ulps, which also covers a quotient formed
-// with a reciprocal that is not correctly rounded. The sign and the pivmin
-// test read the bit pattern (integer compares of |q|'s bits order like the
-// magnitudes), so that they stay off the FP64 pipe.
-__device__ __forceinline__ int sturm_count(const double* d, const double* e2, int n, double x,
-                                           double pivmin) {
-  const long long pmin_bits = __double_as_longlong(pivmin);
-  const double neg_pmin = -pivmin;
-  double q = d[0] - x;
-  long long qb = __double_as_longlong(q);
-  if ((qb & 0x7FFFFFFFFFFFFFFFll) < pmin_bits) {
-    q = neg_pmin;
-    qb = __double_as_longlong(q);
-  }
-  int cnt = (int)((unsigned long long)qb >> 63);
-  for (int i = 1; i < n; ++i) {
-    q = fma(-e2[i - 1], recip_nr(q), d[i] - x);
-    qb = __double_as_longlong(q);
-    if ((qb & 0x7FFFFFFFFFFFFFFFll) < pmin_bits) {
-      q = neg_pmin;
-      qb = __double_as_longlong(q);
-    }
-    cnt += (int)((unsigned long long)qb >> 63);
-  }
-  return cnt;
-}
-
-// The same count by the three-term recurrence of the leading principal
-// minors, p_0 = 1, p_1 = d_0 - x, p_i = (d_{i-1} - x) p_{i-1} - e_{i-2}^2
+// Number of eigenvalues of the symmetric tridiagonal (d, e2 = e^2) below x, by
+// the three-term recurrence of the leading principal minors, p_0 = 1, p_1 = d_0 - x, p_i = (d_{i-1} - x) p_{i-1} - e_{i-2}^2
 // p_{i-2}: the number of sign changes along p_0 .. p_n is the number of
 // negative pivots q_i = p_i / p_{i-1}, that is, of eigenvalues below x. No
 // division: a DADD, a DMUL and a DFMA a step, with the sign and zero tests
@@ -136,13 +95,20 @@ __device__ __forceinline__ void sturm3_step(double dx, double e2, double& p, dou
   p = __longlong_as_double(nb);
 }
 
-__device__ __forceinline__ int sturm_count3(const double* d, const double* e2, int n, double x) {
+// Also returns det(T - x I) as value 2^(500 shifts).
+struct SturmValue {
+  int cnt, shifts;
+  double value;
+};
+
+__device__ __forceinline__ SturmValue sturm_count3(const double* d, const double* e2, int n,
+                                                   double x) {
   double pm = 1.0, p = d[0] - x;
   long long pb = __double_as_longlong(p);
   if ((pb << 1) == 0) pb = __double_as_longlong(-0x1p-60);
   p = __longlong_as_double(pb);
   int neg = (int)((unsigned long long)pb >> 63);
-  int cnt = neg;
+  int cnt = neg, shifts = 0;
   int i = 1;
   for (; i + 8 <= n; i += 8) {
 #pragma unroll 1
@@ -152,14 +118,16 @@ __device__ __forceinline__ int sturm_count3(const double* d, const double* e2, i
       p *= 0x1p-500;
       pm *= 0x1p-500;
       pb = __double_as_longlong(p);
+      ++shifts;
     } else if (ex < -500) {
       p *= 0x1p500;
       pm *= 0x1p500;
       pb = __double_as_longlong(p);
+      --shifts;
     }
   }
   for (; i < n; ++i) sturm3_step(d[i] - x, e2[i - 1], p, pm, pb, neg, cnt);
-  return cnt;
+  return {cnt, shifts, p};
 }
 
 // The same recurrence in FP32 on the float copy of the scaled matrix, the
@@ -167,13 +135,14 @@ __device__ __forceinline__ int sturm_count3(const double* d, const double* e2, i
 // by -2^-24 p_{i-1}. Its backward error, a few FP32 ulps of the scaled
 // entries, stays below the 32 x 2^-24 by which the FP32 brackets are
 // widened.
-__device__ __forceinline__ int sturm_count3f(const float* d, const float* e2, int n, float x) {
-  float pm = 1.0f, p = d[0] - x;
+__device__ __forceinline__ int sturm_count3f(const float4* de, int n, float x) {
+  float pm = 1.0f, p = de[0].x - x;
   if (p == 0.0f) p = -0x1p-24f;
   bool neg = p < 0.0f;
   int cnt = neg;
   for (int i = 1; i < n; ++i) {
-    float pn = fmaf(-e2[i - 1], pm, (d[i] - x) * p);
+    const float4 v = de[i];  // (d_i, -, e_{i-1}^2, -)
+    float pn = fmaf(-v.z, pm, (v.x - x) * p);
     if (pn == 0.0f) pn = -0x1p-24f * p;
     const bool s = pn < 0.0f;
     cnt += s != neg;
@@ -192,142 +161,304 @@ __device__ __forceinline__ int sturm_count3f(const float* d, const float* e2, in
   return cnt;
 }
 
-// Eigenvalues of each walker's tridiagonal matrix by bisection, then
-// S = -sum p ln p with p = lambda / sum(lambda) over p > 0. The matrix is
-// scaled by a power of two into [-1, 1] and counted by the three-term
-// recurrence; the brackets are first narrowed in FP32: from there a bracket
-// [a, b] with count32(a) <= k < count32(b) holds lambda_k within
-// [a - del, b + del] (del = 32 x 2^-24, above the FP32 count's error
-// bound), and FP64 bisection takes it on to the tolerance. That saves about
-// 10 of the 45 FP64 Sturm counts per eigenvalue, and the recurrence halves
-// the FP64 instructions of a count. Matrices whose scale lies outside
-// [2^-1000, 2^1000] take the pivot form unscaled, in FP64 only. Dynamic
-// shared memory: d, e^2 and the eigenvalues (3 n doubles), T + 1 int
-// counts, then d and e^2 as scaled floats (2 n).
-__global__ void __launch_bounds__(kEntThreads) bisect_kernel(const double* d, const double* e,
-                                                             int n, double* entropy,
-                                                             double* eigs) {
-  extern __shared__ double sb[];
-  double* sd = sb;
-  double* se2 = sb + n;
-  double* lam = sb + 2 * n;
-  __shared__ double red[kEntThreads / 32];
-  const int t = threadIdx.x, T = blockDim.x;
-  const double* dw = d + (size_t)blockIdx.x * n;
-  const double* ew = e + (size_t)blockIdx.x * n;
-  double lo = DBL_MAX, hi = -DBL_MAX, e2max = 0.0;
-  for (int i = t; i < n; i += T) {
-    sd[i] = dw[i];
-    const double ei = i + 1 < n ? ew[i] : 0.0;
-    se2[i] = ei * ei;
-    e2max = fmax(e2max, ei * ei);
-    // Gershgorin interval of row i
-    const double r = fabs(ei) + (i > 0 ? fabs(ew[i - 1]) : 0.0);
-    lo = fmin(lo, dw[i] - r);
-    hi = fmax(hi, dw[i] + r);
+// The same recurrence on pairs of floats (the value hi + lo, 48 bits):
+// products by Dekker's error-free transformation with FMA, their difference
+// by Knuth's two-sum of the high parts and one addition of the low ones. The
+// rounding of a step is at most about 10 x 2^-48 of each of its two products
+// (the dropped low x low term of the product with d - x is below 2^-48 of p),
+// which perturbs d - x (at most 3) and e^2 (at most 1) by that much, so the
+// count is exact for a matrix within 2^-42 of the scaled one. A step takes
+// about 30 FP32 instructions at 128 per clock per SM, against three FP64 ones
+// at 2: six times faster. p is kept within 2^-40 .. 2^40 by powers of 2^60.
+__device__ __forceinline__ int sturm_count3ff(const float4* de, int n, float xh, float xl) {
+  // de[i] = (d_i hi, d_i lo, e_{i-1}^2 hi, e_{i-1}^2 lo)
+  float ph = 1.0f, pl = 0.0f, mh = 0.0f, ml = 0.0f;
+  bool neg = false;
+  int cnt = 0;
+#pragma unroll 4
+  for (int i = 0; i < n; ++i) {
+    const float4 v = de[i];
+    // d - x
+    const float th = __fsub_rn(v.x, xh), tb = __fsub_rn(th, v.x);
+    const float tl = __fadd_rn(__fsub_rn(__fsub_rn(v.x, __fsub_rn(th, tb)), __fadd_rn(xh, tb)),
+                               __fsub_rn(v.y, xl));
+    // (d - x) p and e^2 p_{i-2}
+    const float ah = __fmul_rn(th, ph);
+    const float al = __fmaf_rn(th, pl, __fmaf_rn(tl, ph, __fmaf_rn(th, ph, -ah)));
+    const float bh = __fmul_rn(v.z, mh);
+    const float bl = __fmaf_rn(v.z, ml, __fmaf_rn(v.w, mh, __fmaf_rn(v.z, mh, -bh)));
+    const float sh = __fsub_rn(ah, bh), sb = __fsub_rn(sh, ah);
+    const float sl = __fsub_rn(__fsub_rn(ah, __fsub_rn(sh, sb)), __fadd_rn(bh, sb));
+    const float lo = __fadd_rn(sl, __fsub_rn(al, bl));
+    mh = ph;
+    ml = pl;
+    ph = __fadd_rn(sh, lo);
+    pl = __fsub_rn(lo, __fsub_rn(ph, sh));
+    if (ph == 0.0f) {  // a zero minor: the pivot -2^-48
+      ph = -0x1p-48f * mh;
+      pl = 0.0f;
+    }
+    const bool s = ph < 0.0f;
+    cnt += s != neg;
+    neg = s;
+    const uint32_t ex = (__float_as_uint(ph) >> 23) & 0xFF;
+    if (ex - 87u > 80u) {
+      const float f = ex > 127u ? 0x1p-60f : 0x1p60f;
+      ph *= f;
+      pl *= f;
+      mh *= f;
+      ml *= f;
+    }
   }
+  return cnt;
+}
+
+// One narrowing of the bracket [a, b] of eigenvalue k by P lanes, one point
+// each: `below` says whether this lane's point j (at a + w (j + 1) / (P + 1))
+// has at most k eigenvalues below it. Returns how many points, from the
+// first on, do.
+template <int P>
+__device__ __forceinline__ int points_below(bool below) {
+  if constexpr (P == 1) {
+    return below ? 1 : 0;
+  } else {
+    const uint32_t all = __ballot_sync(0xFFFFFFFFu, below);
+    const uint32_t mask = P == 32 ? all : (all >> (threadIdx.x & 31 & ~(P - 1))) & ((1u << (P & 31)) - 1u);
+    return P == 32 && mask == 0xFFFFFFFFu ? 32 : __ffs(~mask) - 1;
+  }
+}
+
+// Eigenvalues of each walker's tridiagonal matrix (blockIdx.y) by bisection,
+// kBisThreads / P of them per CTA, P lanes to each. The matrix is scaled by a
+// power of two into [-1, 1] and counted by the three-term recurrence, in
+// three precisions, each narrowing the bracket down to its own error bound:
+// in FP32 to 32 x 2^-24, in float pairs to 2^-40, then FP64. A bracket [a, b]
+// with count(a) <= k < count(b) in one precision holds lambda_k within
+// [a - del, b + del]. In FP64, a bracket that holds one eigenvalue is closed
+// around the secant of det(T - x I) over it, two counts either side of that
+// point proving the result; otherwise (a cluster, or a secant that missed)
+// the bisection goes on. That leaves about 5 FP64 counts per eigenvalue of
+// the 35 that bisecting from the FP32 bracket took.
+// P: batches with few eigenvalues per SM give each one several lanes, which
+// cut the bracket into P + 1 parts per count, so that fewer counts follow
+// one another.
+// Dynamic shared memory: d and e^2 (2 n doubles), the same as float pairs
+// (n float4).
+constexpr int kBisThreads = 128;
+template <int P>
+__global__ void __launch_bounds__(kBisThreads) bisect_kernel(const double* d, const double* e,
+                                                             int n, double* lam) {
+  extern __shared__ float4 sde[];
+  double* sd = reinterpret_cast<double*>(sde + n);
+  double* se2 = sd + n;
+  __shared__ double red[kBisThreads / 32];
+  __shared__ int cnt[kBisThreads + 1];
+  const int t = threadIdx.x;
+  constexpr int T = kBisThreads;
+  const double* dw = d + (size_t)blockIdx.y * n;
+  const double* ew = e + (size_t)blockIdx.y * n;
+  double lo = DBL_MAX, hi = -DBL_MAX;
+  bool finite = true;
+  for (int i = t; i < n; i += T) {
+    // Gershgorin interval of row i
+    const double di = dw[i];
+    const double r = (i + 1 < n ? fabs(ew[i]) : 0.0) + (i > 0 ? fabs(ew[i - 1]) : 0.0);
+    lo = fmin(lo, di - r);
+    hi = fmax(hi, di + r);
+    finite = finite && fabs(di) <= DBL_MAX && r <= DBL_MAX;
+  }
+  finite = __syncthreads_and(finite);
   lo = -block_max(-lo, red);
   hi = block_max(hi, red);
-  e2max = block_max(e2max, red);
-  const double pivmin = DBL_MIN * fmax(1.0, e2max);
   const double scale = fmax(fabs(lo), fabs(hi));
-  const double tol = 2.0 * DBL_EPSILON * scale + 2.0 * pivmin;
-  lo -= tol;
-  hi += tol;
-  int* cnt = reinterpret_cast<int*>(lam + n);  // T + 1 counts
-  float* d32 = reinterpret_cast<float*>(cnt + T + 1);
-  float* e32 = d32 + n;
-  int ex = 0;
-  frexp(scale, &ex);
-  const bool use32 = scale > 0x1p-1000 && scale < 0x1p1000;
-  const double sc = ldexp(1.0, -ex);  // scale x sc in [0.5, 1)
-  if (use32) {  // the scaled matrix, in place of d and e^2, and as floats
-    for (int i = t; i < n; i += T) {
-      sd[i] *= sc;
-      const double es = (i + 1 < n ? ew[i] : 0.0) * sc;
-      se2[i] = es * es;
-      d32[i] = (float)sd[i];
-      e32[i] = (float)se2[i];
-    }
+  const int kt = blockIdx.x * (T / P) + t / P, k = min(kt, n - 1), j = t % P;
+  const bool store = j == 0 && kt < n;
+  const size_t at = (size_t)blockIdx.y * n + k;
+  if (!finite || scale == 0.0 || scale > DBL_MAX) {  // uniform over the CTA
+    const double v = finite && scale == 0.0 ? 0.0 : __longlong_as_double(0x7FF8000000000000ll);
+    if (store) lam[at] = v;
+    return;
   }
+  int ex = 0;
+  frexp(scale, &ex);  // scale 2^-ex in [0.5, 1)
+  for (int i = t; i < n; i += T) {
+    const double di = scalbn(dw[i], -ex);
+    const double es = i > 0 ? scalbn(ew[i - 1], -ex) : 0.0;
+    const double e2 = es * es;
+    sd[i] = di;
+    if (i > 0) se2[i - 1] = e2;
+    const float dh = (float)di, eh = (float)e2;
+    sde[i] = make_float4(dh, (float)(di - (double)dh), eh, (float)(e2 - (double)eh));
+  }
+  lo = scalbn(lo, -ex);
+  hi = scalbn(hi, -ex);
+  const double tol = 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi));
   __syncthreads();
-  // multisection: one Sturm count per thread on an even grid gives every
+  // multisection: one FP32 count per thread on an even grid gives every
   // eigenvalue a bracket T times narrower to start from (the ends widened
   // by twice the FP32 bound, so that the counts there are 0 and n)
-  const float del32 = 32.0f * 0x1p-24f;
-  const float lo32 = (float)(lo * sc) - 2.0f * del32, hi32 = (float)(hi * sc) + 2.0f * del32;
+  constexpr float del32 = 32.0f * 0x1p-24f;
+  const float lo32 = (float)lo - 2.0f * del32, hi32 = (float)hi + 2.0f * del32;
   const float h32 = (hi32 - lo32) / (float)T;
-  const double hstep = (hi - lo) / T;
-  auto grid32 = [&](int j) { return __fmaf_rn((float)j, h32, lo32); };
-  auto grid64 = [&](int j) { return fma((double)j, hstep, lo); };
-  if (use32) cnt[t + 1] = t + 1 < T ? sturm_count3f(d32, e32, n, grid32(t + 1)) : n;
-  else cnt[t + 1] = t + 1 < T ? sturm_count(sd, se2, n, grid64(t + 1), pivmin) : n;
+  auto grid32 = [&](int i) { return __fmaf_rn((float)i, h32, lo32); };
+  cnt[t + 1] = t + 1 < T ? sturm_count3f(sde, n, grid32(t + 1)) : n;
   if (t == 0) cnt[0] = 0;
   __syncthreads();
-  for (int k = t; k < n; k += T) {
-    // the k-th smallest eigenvalue: count(a) <= k < count(b)
-    int g = 0;  // a grid cell with cnt[g] <= k < cnt[g + 1]
-    int lo_i = 0, hi_i = T;
-    while (hi_i - lo_i > 1) {
-      const int mid = (lo_i + hi_i) >> 1;
-      if (cnt[mid] <= k) lo_i = mid;
-      else hi_i = mid;
-    }
-    g = lo_i;
-    double a, b;
-    if (use32) {
-      float a32 = grid32(g), b32 = g + 1 < T ? grid32(g + 1) : hi32;
-      for (int it = 0; it < 40 && b32 - a32 > del32; ++it) {
-        const float mid = 0.5f * (a32 + b32);
-        if (sturm_count3f(d32, e32, n, mid) <= k) a32 = mid;
-        else b32 = mid;
-      }
-      // in scaled units from here
-      a = (double)a32 - (double)del32;
-      b = (double)b32 + (double)del32;
-      const double tol_s = tol * sc;
-      for (int it = 0; it < 200 && b - a > tol_s; ++it) {
-        const double mid = 0.5 * (a + b);
-        if (sturm_count3(sd, se2, n, mid) <= k) a = mid;
-        else b = mid;
-      }
-      lam[k] = 0.5 * (a + b) / sc;  // dividing by a power of two: exact
-    } else {
-      a = grid64(g);
-      b = g + 1 < T ? grid64(g + 1) : hi;
-      for (int it = 0; it < 200 && b - a > tol; ++it) {
-        const double mid = 0.5 * (a + b);
-        if (sturm_count(sd, se2, n, mid, pivmin) <= k) a = mid;
-        else b = mid;
-      }
-      lam[k] = 0.5 * (a + b);
+  // the k-th smallest eigenvalue: count(a) <= k < count(b)
+  int lo_i = 0, hi_i = T;
+  while (hi_i - lo_i > 1) {
+    const int mid = (lo_i + hi_i) >> 1;
+    if (cnt[mid] <= k) lo_i = mid;
+    else hi_i = mid;
+  }
+  constexpr float kPart = 1.0f / (float)(P + 1);
+  float a32 = grid32(lo_i), b32 = lo_i + 1 < T ? grid32(lo_i + 1) : hi32;
+  for (int it = 0; it < 40 && __any_sync(0xFFFFFFFFu, b32 - a32 > del32); ++it) {
+    const float w = (b32 - a32) * kPart;
+    const int m = points_below<P>(sturm_count3f(sde, n, __fmaf_rn((float)(j + 1), w, a32)) <= k);
+    if (b32 - a32 > del32) {
+      const float a0 = a32;
+      if (m > 0) a32 = __fmaf_rn((float)m, w, a0);
+      if (m < P) b32 = __fmaf_rn((float)(m + 1), w, a0);
     }
   }
-  __syncthreads();
+  double a = (double)a32 - (double)del32, b = (double)b32 + (double)del32;
+  constexpr double delff = 0x1p-40;
+  for (int it = 0; it < 60 && __any_sync(0xFFFFFFFFu, b - a > delff); ++it) {
+    const double w = (b - a) * (1.0 / (P + 1));
+    // (the points are pairs of floats: rounding x to 48 bits moves it by less than the bound)
+    const double x = fma((double)(j + 1), w, a);
+    const float xh = (float)x, xl = (float)(x - (double)xh);
+    const int m = points_below<P>(sturm_count3ff(sde, n, xh, xl) <= k);
+    if (b - a > delff) {
+      const double a0 = a;
+      if (m > 0) a = fma((double)m, w, a0);
+      if (m < P) b = fma((double)(m + 1), w, a0);
+    }
+  }
+  a -= delff;
+  b += delff;
+  // two points at once: by two lanes, or one after the other
+  auto two = [&](double x0, double x1, SturmValue& v0, SturmValue& v1) {
+    if constexpr (P == 1) {
+      v0 = sturm_count3(sd, se2, n, x0);
+      v1 = sturm_count3(sd, se2, n, x1);
+    } else {
+      const SturmValue v = sturm_count3(sd, se2, n, (j & 1) ? x1 : x0);
+      const int l0 = t & 31 & ~(P - 1);
+      v0.cnt = __shfl_sync(0xFFFFFFFFu, v.cnt, l0);
+      v0.shifts = __shfl_sync(0xFFFFFFFFu, v.shifts, l0);
+      v0.value = __shfl_sync(0xFFFFFFFFu, v.value, l0);
+      v1.cnt = __shfl_sync(0xFFFFFFFFu, v.cnt, l0 + 1);
+      v1.shifts = __shfl_sync(0xFFFFFFFFu, v.shifts, l0 + 1);
+      v1.value = __shfl_sync(0xFFFFFFFFu, v.value, l0 + 1);
+    }
+  };
+  SturmValue va, vb;
+  two(a, b, va, vb);
+  double x0 = a, x1 = b;
+  if (va.cnt > k) {  // outside the bracket after all: take the whole interval below
+    b = a;
+    a = lo - 4.0 * tol;
+  } else if (vb.cnt <= k) {
+    a = b;
+    b = hi + 4.0 * tol;
+  } else if (vb.cnt - va.cnt == 1 && va.shifts == vb.shifts) {
+    const double fa = fabs(va.value), fb = fabs(vb.value);
+    const double x = fma(b - a, fa / (fa + fb), a);
+    x0 = fmax(a, x - tol);
+    x1 = fmin(b, x + tol);
+  }
+  // (a lane with no secant asks again for the ends of its bracket, or stays at x0 = x1)
+  SturmValue w0, w1;
+  two(x0, x1, w0, w1);
+  if (x0 >= a && x1 <= b) {
+    if (w0.cnt <= k) a = fmax(a, x0);
+    else b = fmin(b, x0);
+    if (w1.cnt > k) b = fmin(b, x1);
+    else a = fmax(a, x1);
+  }
+  for (int it = 0; it < 200 && __any_sync(0xFFFFFFFFu, b - a > tol); ++it) {
+    const double w = (b - a) * (1.0 / (P + 1));
+    const int m =
+        points_below<P>(sturm_count3(sd, se2, n, fma((double)(j + 1), w, a)).cnt <= k);
+    if (b - a > tol) {
+      const double a0 = a;
+      if (m > 0) a = fma((double)m, w, a0);
+      if (m < P) b = fma((double)(m + 1), w, a0);
+    }
+  }
+  if (store) lam[at] = scalbn(0.5 * (a + b), ex);
+}
+
+// S = -sum p ln p over p = lambda / sum(lambda) > 0, a CTA per walker; eigs
+// (optional) receives the eigenvalues in ascending order: two that lie within
+// the bisection's tolerance of each other may come in either order, so each
+// takes the largest value up to it.
+__global__ void __launch_bounds__(kEntThreads) entropy_sum_kernel(const double* lam, int n,
+                                                                  double* entropy, double* eigs) {
+  __shared__ double red[kEntThreads / 32];
+  __shared__ double top[2][kEntThreads];
+  const int t = threadIdx.x, T = kEntThreads;
+  const double* l = lam + (size_t)blockIdx.x * n;
   double tot = 0.0;
-  for (int k = t; k < n; k += T) tot += lam[k];
+  for (int k = t; k < n; k += T) tot += l[k];
   tot = block_sum(tot, red);
-  double s = 0.0;
+  double s = tot != tot ? tot : 0.0;
   for (int k = t; k < n; k += T) {
-    if (eigs) eigs[(size_t)blockIdx.x * n + k] = lam[k];
-    const double p = tot > 0.0 ? lam[k] / tot : 0.0;
+    const double p = tot > 0.0 ? l[k] / tot : 0.0;
     if (p > 0.0) s -= p * log(p);
   }
   s = block_sum(s, red);
   if (t == 0) entropy[blockIdx.x] = s;
+  if (!eigs) return;
+  const int per = (n + T - 1) / T, k0 = t * per, k1 = min(n, k0 + per);
+  double m = -DBL_MAX;
+  for (int k = k0; k < k1; ++k) m = fmax(m, l[k]);
+  top[0][t] = m;
+  __syncthreads();
+  int cur = 0;
+  for (int o = 1; o < T; o <<= 1, cur ^= 1) {  // inclusive running maximum over the threads
+    top[cur ^ 1][t] = t >= o ? fmax(top[cur][t], top[cur][t - o]) : top[cur][t];
+    __syncthreads();
+  }
+  m = t > 0 ? top[cur][t - 1] : -DBL_MAX;
+  for (int k = k0; k < k1; ++k) {
+    const double v = l[k];
+    m = fmax(m, v);
+    eigs[(size_t)blockIdx.x * n + k] = v != v ? v : m;
+  }
+}
+
+template <int P>
+cudaError_t bisect_launch(const double* d, const double* e, int64_t walkers, int n, double* lam,
+                          cudaStream_t st) {
+  static bool attr[kAttrDevices] = {};
+  const cudaError_t err = smem_limit(bisect_kernel<P>, 96 * 1024, attr);
+  if (err != cudaSuccess) return err;
+  constexpr int per = kBisThreads / P;
+  bisect_kernel<P><<<dim3((unsigned)((n + per - 1) / per), (unsigned)walkers), kBisThreads,
+                     (size_t)n * 32, st>>>(d, e, n, lam);
+  count_launch();
+  return cudaGetLastError();
 }
 
 }  // namespace
 
+// Lanes per eigenvalue: as many as keep the eigenvalues' lanes within 256 per
+// SM (8 warps of dependent FP32 and FP64 chains fill the pipes; more lanes
+// than that cost more counts than the shorter chain saves).
 cudaError_t launch_entropy_bisect(const double* d, const double* e, int64_t walkers, int n,
-                                  double* entropy, double* eigs, cudaStream_t st) {
+                                  double* lam, double* entropy, double* eigs, int sms,
+                                  cudaStream_t st) {
   if (walkers <= 0) return cudaSuccess;
-  static bool attr[kAttrDevices] = {};
-  const cudaError_t err = smem_limit(bisect_kernel, 96 * 1024, attr);
+  const int64_t lanes = (int64_t)sms * 256 / (walkers * n);
+  cudaError_t err = lanes >= 32  ? bisect_launch<32>(d, e, walkers, n, lam, st)
+                    : lanes >= 8 ? bisect_launch<8>(d, e, walkers, n, lam, st)
+                    : lanes >= 2 ? bisect_launch<2>(d, e, walkers, n, lam, st)
+                                 : bisect_launch<1>(d, e, walkers, n, lam, st);
   if (err != cudaSuccess) return err;
-  const size_t sm2 = 3 * (size_t)n * sizeof(double) + (kEntThreads + 1) * sizeof(int) +
-                     2 * (size_t)n * sizeof(float);
-  bisect_kernel<<<(unsigned)walkers, kEntThreads, sm2, st>>>(d, e, n, entropy, eigs);
+  entropy_sum_kernel<<<(unsigned)walkers, kEntThreads, 0, st>>>(lam, n, entropy, eigs);
   count_launch();
   return cudaGetLastError();
 }

@@ -212,8 +212,8 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
             cmac_conj(s, vload(q, lr, r), S.rowW[q]);
             cmac_conj(s, vload(kNb + q, lr, r), S.rowV[q]);
           }
-          xr = fx::join(a.x, a.y) - ((s.re() + 1) >> 1);
-          xi = fx::join(a.z, a.w) - ((s.im() + 1) >> 1);
+          xr = fx::join(a.x, a.y) - fx::rne(s.re(), 1);
+          xi = fx::join(a.z, a.w) - fx::rne(s.im(), 1);
           if (r == c) R.d[c] = scalbn((double)xr, R.eunit);
           if (r == c + 1) publish<MULTI>(&S.alpha[par], xr, xi, cl);
           if (r >= c + 2) {
@@ -387,7 +387,7 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
             ci += v.y;
           }
         }
-        S.scoef[warp][lane] = fx::pack((cr + 4) >> 3, (ci + 4) >> 3);
+        S.scoef[warp][lane] = fx::pack(fx::rne(cr, 3), fx::rne(ci, 3));
         __syncwarp();
       }
       const int4 tau = S.tau;
@@ -410,7 +410,7 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
           }
           yr -= (s.rh << 2) + ((s.rx + (1ll << 24)) >> 25);
           yi -= (s.ih << 2) + ((s.ix + (1ll << 24)) >> 25);
-          const int4 yq = fx::pack((yr + 4) >> 3, (yi + 4) >> 3);  // unit 2 uA
+          const int4 yq = fx::pack(fx::rne(yr, 3), fx::rne(yi, 3));  // unit 2 uA
           Sum ps;
           cmac(ps, tau, yq);
           pr = ps.re();
@@ -436,7 +436,7 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
       rho = 0;
       for (int x = lane; x < cl * kWarps; x += 32) rho += S.rho[x];
       rho = fx::warp_sum(rho);
-      const fx::Limb rq = fx::split((rho + 4) >> 3);  // unit 4 uA
+      const fx::Limb rq = fx::split(fx::rne(rho, 3));  // unit 4 uA
       const int2 t2 = S.t2;
       long long ch_ = 0, cx_ = 0;
       fx::mac(ch_, t2.x, rq.h);
@@ -451,7 +451,7 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
         fx::mac(ih, cc.h, u.z);
         fx::mac(ix, cc.h, u.w);
         fx::mac(ix, cc.l, u.z);
-        return fx::pack((pr - fx::val(rh, rx) + 1) >> 1, (pi - fx::val(ih, ix) + 1) >> 1);
+        return fx::pack(fx::rne(pr - fx::val(rh, rx), 1), fx::rne(pi - fx::val(ih, ix), 1));
       };
       for (int k = warp; k < kmax; k += kWarps) {
         if (k < kfirst) continue;
@@ -532,8 +532,8 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
           for (int x = 0; x < kStrip; ++x) {
             const int cc = cs + x;
             if (r >= n || cc > r || cc < q0) continue;
-            const long long re = fx::join(a[x].x, a[x].y) - ((sum[x].re() + 1) >> 1);
-            const long long im = r == cc ? 0 : fx::join(a[x].z, a[x].w) - ((sum[x].im() + 1) >> 1);
+            const long long re = fx::join(a[x].x, a[x].y) - fx::rne(sum[x].re(), 1);
+            const long long im = r == cc ? 0 : fx::join(a[x].z, a[x].w) - fx::rne(sum[x].im(), 1);
             const int4 v = fx::pack(re, im);
             R.A[r + (size_t)cc * ld] = v;
             if (r != cc) R.A[cc + (size_t)r * ld] = fx::pack(re, -im);
