@@ -274,7 +274,7 @@ bg_status apply_local_gate(bg_dtype dtype, int64_t walkers, int32_t spins, const
  *    1 <= split <= min(spins - 1, 10). precision (NULL = FP64) selects the
  *    precision of G_w: it is formed by a Hermitian-update plan
  *    (BG_PLAN_HERK) in that mode. The eigenvalues come from a Householder
- *    reduction of G_w to a real tridiagonal matrix, in 57-bit fixed point
+ *    reduction of G_w to a real tridiagonal matrix, in 60-bit fixed point
  *    relative to a bound on the largest eigenvalue (one kernel; a normwise
  *    error of the size of the FP64 reduction's), then bisection on its Sturm
  *    sequence. flags: 0 or BG_PLAN_PROFILE (slot 0 of bg_plan_kernel_times:

@@ -378,11 +378,14 @@ __global__ void __launch_bounds__(kBisThreads) bisect_kernel(const double* d, co
     if (w1.cnt > k) b = fmin(b, x1);
     else a = fmax(a, x1);
   }
-  for (int it = 0; it < 200 && __any_sync(0xFFFFFFFFu, b - a > tol); ++it) {
+  // near zero (the empty part of a low-entropy spectrum) the bisection goes on
+  // to 2^-58: there are many such eigenvalues, and -p ln p is steep
+  auto open = [&]() { return b - a > (fmax(fabs(a), fabs(b)) < 0x1p-10 ? 0x1p-58 : tol); };
+  for (int it = 0; it < 200 && __any_sync(0xFFFFFFFFu, open()); ++it) {
     const double w = (b - a) * (1.0 / (P + 1));
     const int m =
         points_below<P>(sturm_count3(sd, se2, n, fma((double)(j + 1), w, a)).cnt <= k);
-    if (b - a > tol) {
+    if (open()) {
       const double a0 = a;
       if (m > 0) a = fma((double)m, w, a0);
       if (m < P) b = fma((double)(m + 1), w, a0);

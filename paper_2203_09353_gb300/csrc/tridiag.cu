@@ -1,7 +1,7 @@
 // Householder reduction of each walker's Hermitian positive semidefinite
 // n x n Gram matrix to a real tridiagonal matrix (d, e), for the entanglement
 // entropy (Alg. 1, "Calculate Entropy"): the steps of LAPACK's zlatrd/zhetrd
-// for the lower triangle, in 57-bit fixed point (fixed57.cuh) on the integer
+// for the lower triangle, in 60-bit fixed point (fixed60.cuh) on the integer
 // pipe, one kernel for the whole reduction.
 //
 // Why fixed point. The reduction is (16/3) n^3 FP64 flops, half of them in
@@ -9,8 +9,8 @@
 // pipe (2 DFMA per clock per SM) bounded it; three 32 x 32 + 64 bit integer
 // multiply-adds per real product are five times faster than a DFMA. Every quantity of the reduction is bounded by the matrix norm, so a
 // single power of two B scales it: entries, W and y carry an absolute
-// resolution of 2^-57 B .. 2^-55 B, which is the size of the FP64 reduction's
-// own normwise backward error.
+// resolution of 2^-60 B .. 2^-58 B, below the FP64 reduction's own normwise
+// backward error.
 //
 // Per panel of kNb columns (c = column, u = reflector vector, H = I - tau u u^H):
 //   1. column c minus the panel's earlier rank-2 updates; d[c], and the exact
@@ -31,13 +31,14 @@
 // last kTail columns (or a whole matrix up to that order) are reduced by one
 // CTA with the matrix in shared memory.
 //
-// Bounds used by the formats (B = 2^57 units "uA" of the entries), with
-// |u|^2 in [0.5, 4) after scaling (unit 2^-56) and lambda = ||A|| <= B (the
+// Bounds used by the formats (B = 2^60 units "uA" of the entries), with
+// |u|^2 in [0.5, 4) after scaling (unit 2^-59) and lambda = ||A|| <= B (the
 // limbs leave room for lambda <= kScaleRoom B):
-//   |y| <= 2 B, |W^H u| <= 4 B, |V^H u| <= 4, |tau| <= 4, rho <= 4 B,
-//   |w| <= 1.25 lambda / |u| < 1.8 B (unit 2 uA).
+//   |y| <= 2 B (2 uA), |W^H u| <= 4 B (4 uA), |V^H u| <= 4 (2^-58),
+//   |tau| <= 4 (2^-58), rho <= 4 B (4 uA), |w| <= 1.25 lambda / |u| < 1.8 B (2 uA).
 // Row and column norms of A are at most lambda, so sums of products stay in
-// 64 bits by the Cauchy-Schwarz inequality.
+// 64 bits by the Cauchy-Schwarz inequality; a cross sum is flushed every 16
+// columns of A u (2^62.8 at most), 8 rows of V^H u, 2 columns of V and W.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -45,7 +46,7 @@
 #include <mutex>
 
 #include "bgemm_internal.h"
-#include "fixed57.cuh"
+#include "fixed60.cuh"
 
 namespace bg {
 namespace {
@@ -72,12 +73,7 @@ struct TriArgs {
   int own;      // rows a CTA owns at most (a multiple of 32)
 };
 
-// An exact integer sum of squares, s2 2^54 + s1 2^28 + s0.
-struct alignas(16) SquareSum {
-  long long s2, s1, s0, pad;
-};
-
-struct Scalars2 {  // a column's scalars, written by one thread
+struct ColumnScalars {  // a column's scalars, written by one thread
   int z;           // u = column 2^z
   int skip;
   long long u0r, u0i, nint;
@@ -85,15 +81,18 @@ struct Scalars2 {  // a column's scalars, written by one thread
 
 struct Shared {
   longlong2 alpha[2];
-  SquareSum norm[2][kMaxCl * kWarps];  // of every warp of the cluster
+  long long diag[2];                   // the column's diagonal entry
+  long long trace;                     // of the rows not reduced yet (2^kTraceUnit uA)
+  int tail_z[2];                       // the tail's shift after a column
+  longlong2 norm[2][kMaxCl * kWarps];  // sums of squares (hi, lo) of every warp
   longlong2 spart[2 * kNb][kMaxCl];    // V^H u and W^H u, a partial per CTA
   long long rho[kMaxCl * kWarps];
   longlong2 pnext;                     // p of row c + 1
   int4 rowV[kNb], rowW[kNb];           // row c + 1 of V and W
   int4 scoef[kWarps][2 * kNb];
-  int4 tau;                            // limbs, unit 2^-55
-  int2 t2;                             // |tau|^2 / 2, unit 2^-54
-  Scalars2 sc;
+  int4 tau;                            // limbs, unit 2^-58
+  int2 t2;                             // |tau|^2 / 2, unit 2^-57
+  ColumnScalars sc;
   double dred[kWarps];
   float2 fsum[kMaxCl * kWarps];        // (sum of squares, trace) of every warp
 };
@@ -154,6 +153,91 @@ __device__ __forceinline__ void walker_sync() {
   }
 }
 
+// How far the trailing matrix may be scaled up once its trace (which bounds its
+// norm) has fallen: a low-entropy state leaves most of its weight in the first
+// columns, and the rest then keeps its precision. At most kMaxShift bits in all,
+// so that the rounding noise of the first columns, which is not positive
+// semidefinite, stays far below full scale.
+// The trace is kept in units of 2^kTraceUnit uA (n full-scale entries fit).
+constexpr int kMaxShift = 24;
+constexpr int kTraceUnit = 10;
+__device__ __forceinline__ int rescale(long long trace, int shifted) {
+  // trace 2^z < 2^60 uA
+  const int z = trace > 0 ? __clzll(trace) - (64 - fx::kFull) - kTraceUnit : kMaxShift;
+  return max(0, min(z, kMaxShift - shifted));
+}
+
+// The reflector of a column (alpha, x...) with |x|^2 = sum: beta = -+N, N the
+// column's norm, and u = (alpha - beta, x...) 2^z with N 2^z in [2^58, 2^59).
+__device__ __forceinline__ ColumnScalars reflector(const fx::U128& sum, long long alr,
+                                                   long long ali, double* beta) {
+  ColumnScalars sc{0, 0, 0, 0, 0};
+  if (sum.hi == 0 && sum.lo == 0 && ali == 0) {
+    sc.skip = 1;  // already reduced: H = I
+    *beta = (double)alr;
+    return sc;
+  }
+  fx::U128 all = sum;
+  all.add_square(alr);
+  all.add_square(ali);
+  const double N = sqrt(all.value());
+  const int eN = (int)((__double2hiint(N) >> 20) & 0x7FF) - 1022;  // N in [2^(eN-1), 2^eN)
+  sc.z = fx::kFull - 1 - eN;
+  sc.nint = __double2ll_rn(N * __hiloint2double((1023 + sc.z) << 20, 0));
+  const long long xr = fx::shift(alr, sc.z);
+  sc.u0r = alr < 0 ? xr - sc.nint : xr + sc.nint;
+  sc.u0i = fx::shift(ali, sc.z);
+  *beta = alr < 0 ? N : -N;
+  return sc;
+}
+
+// tau = -u0 / (beta |u0|^2) (beta and u0 scaled) in limbs of unit 2^-58, and
+// |tau|^2 / 2 in limbs of unit 2^-57.
+__device__ __forceinline__ void reflector_tau(const ColumnScalars& sc, int4* tau, int2* t2) {
+  const double br = (sc.u0r < 0 ? 1.0 : -1.0) * (double)sc.nint * 0x1p-59;
+  const double ur = (double)sc.u0r * 0x1p-59, ui = (double)sc.u0i * 0x1p-59;
+  const double rden = -1.0 / (br * fma(ur, ur, ui * ui));
+  const double tr = ur * rden, ti = ui * rden;
+  *tau = fx::pack(__double2ll_rn(tr * 0x1p58), __double2ll_rn(ti * 0x1p58));
+  const fx::Limb l = fx::split(__double2ll_rn(fma(tr, tr, ti * ti) * 0x1p56));
+  *t2 = make_int2(l.h, l.l);
+}
+
+// u^H y of one row (real part), unit 4 uA.
+__device__ __forceinline__ long long real_dot(const int4& u, const int4& y) {
+  long long h = 0, x = 0;
+  fx::mac(h, u.x, y.x);
+  fx::mac(h, u.z, y.z);
+  fx::mac(x, u.x, y.y);
+  fx::mac(x, u.y, y.x);
+  fx::mac(x, u.z, y.w);
+  fx::mac(x, u.w, y.z);
+  return fx::val(h, x);
+}
+
+// c = |tau|^2 rho / 2, unit 4 uA.
+__device__ __forceinline__ fx::Limb w_coef(const int2& t2, long long rho) {
+  const fx::Limb rq = fx::split(rho);
+  long long h = 0, x = 0;
+  fx::mac(h, t2.x, rq.h);
+  fx::mac(x, t2.x, rq.l);
+  fx::mac(x, t2.y, rq.h);
+  return fx::split(fx::val<3>(h, x));
+}
+
+// w = p - c u for one row: p in uA, w in 2 uA.
+__device__ __forceinline__ int4 make_w(long long pr, long long pi, const fx::Limb& c,
+                                       const int4& u) {
+  long long rh = 0, rx = 0, ih = 0, ix = 0;
+  fx::mac(rh, c.h, u.x);
+  fx::mac(rx, c.h, u.y);
+  fx::mac(rx, c.l, u.x);
+  fx::mac(ih, c.h, u.z);
+  fx::mac(ix, c.h, u.w);
+  fx::mac(ix, c.l, u.z);
+  return fx::pack(fx::rne(pr - fx::val<3>(rh, rx), 1), fx::rne(pi - fx::val<3>(ih, ix), 1));
+}
+
 // One walker's (or its tail's) reduction state.
 struct Red {
   int4* A;       // full matrix (both triangles), column-major
@@ -167,21 +251,15 @@ struct Red {
   double* d;
   double* e;
   int eunit;     // uA = 2^eunit
+  int shifted;   // bits the matrix has been scaled up since the start
   int rank, cl;
   Shared* S;
 };
 
-template <bool ASM>
-__device__ __forceinline__ int4 ldA(const int4* p) {
-  if constexpr (ASM) return *p;
-  else return __ldcg(p);
-}
-
 // Reduces columns 0 .. cend - 1 (cend <= n - 1). MULTI: a cluster shares the
-// walker. VWS: the panel's own rows of V and W are in shared memory. ASM: so
-// is A.
-template <bool MULTI, bool VWS, bool ASM>
-__device__ __forceinline__ void reduce(const Red& R, int cend) {
+// walker. VWS: the panel's own rows of V and W are in shared memory.
+template <bool MULTI, bool VWS>
+__device__ __forceinline__ void reduce(Red& R, int cend) {
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int n = R.n, ld = R.ld, own = R.own;
   const int cl = MULTI ? R.cl : 1, rank = MULTI ? R.rank : 0;
@@ -189,6 +267,7 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
   const int kmax = (ngroups - rank + cl - 1) / cl;  // own groups
   Shared& S = *R.S;
   longlong2* xs = R.part;  // x of the own rows (between steps 1 and 2)
+  int eunit = R.eunit;
   auto vptr = [&](int q, int lr, int r) -> int4* {
     return VWS ? R.vw + q * own + lr : R.P + (size_t)q * n + r;
   };
@@ -200,82 +279,56 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
     for (int i = 0; i < nbp; ++i) {
       const int c = p0 + i, par = c & 1;
       // ---- 1. column c with the panel's earlier updates; sums of squares
-      long long s2 = 0, s1 = 0, s0 = 0;
+      fx::U128 sq;
       for (int k = warp; k < kmax; k += kWarps) {
         const int r = 32 * (rank + cl * k) + lane, lr = 32 * k + lane;
         if (32 * (rank + cl * k) + 31 < c) continue;
         long long xr = 0, xi = 0;
         if (r >= c && r < n) {
-          const int4 a = ldA<ASM>(R.A + r + (size_t)c * ld);
+          const int4 a = __ldcg(R.A + r + (size_t)c * ld);
           Sum s;
           for (int q = 0; q < i; ++q) {
-            cmac_conj(s, vload(q, lr, r), S.rowW[q]);
-            cmac_conj(s, vload(kNb + q, lr, r), S.rowV[q]);
+            s.add_conj(vload(q, lr, r), S.rowW[q]);
+            s.add_conj(vload(kNb + q, lr, r), S.rowV[q]);
+            if (q & 1) s.flush();
           }
-          xr = fx::join(a.x, a.y) - fx::rne(s.re(), 1);
-          xi = fx::join(a.z, a.w) - fx::rne(s.im(), 1);
-          if (r == c) R.d[c] = scalbn((double)xr, R.eunit);
+          xr = fx::join(a.x, a.y) - s.re<2>();
+          xi = fx::join(a.z, a.w) - s.im<2>();
+          if (r == c) {
+            R.d[c] = scalbn((double)xr, eunit);
+            publish<MULTI>(&S.diag[par], xr, cl);
+          }
           if (r == c + 1) publish<MULTI>(&S.alpha[par], xr, xi, cl);
           if (r >= c + 2) {
-            const fx::Limb lr_ = fx::split(xr), li_ = fx::split(xi);
-            fx::mac(s2, lr_.h, lr_.h);
-            fx::mac(s2, li_.h, li_.h);
-            fx::mac(s1, lr_.h, lr_.l);
-            fx::mac(s1, li_.h, li_.l);
-            fx::mac(s0, lr_.l, lr_.l);
-            fx::mac(s0, li_.l, li_.l);
+            sq.add_square(xr);
+            sq.add_square(xi);
           }
         }
         xs[lr] = make_longlong2(xr, xi);
       }
-      s2 = fx::warp_sum(s2);
-      s1 = fx::warp_sum(s1);
-      s0 = fx::warp_sum(s0);
-      if (lane == 0) {
-        longlong2* dst = reinterpret_cast<longlong2*>(&S.norm[par][rank * kWarps + warp]);
-        publish<MULTI>(dst, s2, s1, cl);
-        publish<MULTI>(dst + 1, s0, 0, cl);
-      }
+      sq = fx::warp_sum(sq);
+      if (lane == 0)
+        publish<MULTI>(&S.norm[par][rank * kWarps + warp], (long long)sq.hi, (long long)sq.lo, cl);
       walker_sync<MULTI>();
       // ---- 2. norm, beta, u0: one warp of every CTA, from the same numbers
       if (warp == 0) {
-        long long a2 = 0, a1 = 0, a0 = 0;
+        fx::U128 sum;
         for (int x = lane; x < cl * kWarps; x += 32) {
-          const SquareSum v = S.norm[par][x];
-          a2 += v.s2;
-          a1 += v.s1;
-          a0 += v.s0;
+          const longlong2 v = S.norm[par][x];
+          sum.add((unsigned long long)v.x, (unsigned long long)v.y);
         }
-        a2 = fx::warp_sum(a2);
-        a1 = fx::warp_sum(a1);
-        a0 = fx::warp_sum(a0);
+        sum = fx::warp_sum(sum);
         if (lane == 0) {
           const longlong2 al = S.alpha[par];
-          Scalars2 sc{0, 0, 0, 0, 0};
           double beta;
-          if (a2 == 0 && a1 == 0 && a0 == 0 && al.y == 0) {
-            sc.skip = 1;  // already reduced: H = I
-            beta = (double)al.x;
-          } else {
-            const double ar = (double)al.x, ai = (double)al.y;
-            double n2 = fma((double)a2, 0x1p54,
-                            fma((double)a1, 0x1p28, (double)(unsigned long long)a0));
-            n2 = fma(ar, ar, fma(ai, ai, n2));
-            const double N = sqrt(n2);
-            const int eN = (int)((__double2hiint(N) >> 20) & 0x7FF) - 1022;  // N in [2^(eN-1), 2^eN)
-            sc.z = 56 - eN;
-            sc.nint = __double2ll_rn(N * __hiloint2double((1023 + sc.z) << 20, 0));
-            const long long xr = fx::shift(al.x, sc.z);
-            sc.u0r = al.x < 0 ? xr - sc.nint : xr + sc.nint;
-            sc.u0i = fx::shift(al.y, sc.z);
-            beta = al.x < 0 ? N : -N;
-          }
-          if (rank == 0) R.e[c] = scalbn(beta, R.eunit);
+          const ColumnScalars sc = reflector(sum, al.x, al.y, &beta);
+          if (rank == 0) R.e[c] = scalbn(beta, eunit);
+          S.trace -= S.diag[par] >> kTraceUnit;
           S.sc = sc;
         }
       }
       __syncthreads();
-      const Scalars2 sc = S.sc;
+      const ColumnScalars sc = S.sc;
       // u to every CTA; V's column i
       for (int k = warp; k < kmax; k += kWarps) {
         const int r = 32 * (rank + cl * k) + lane, lr = 32 * k + lane;
@@ -318,13 +371,7 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
       walker_sync<MULTI>();
       // ---- 3. tau, by one thread beside the products
       if (t == kThreads - 32) {
-        const double br = (sc.u0r < 0 ? 1.0 : -1.0) * (double)sc.nint * 0x1p-56;  // beta, scaled
-        const double ur = (double)sc.u0r * 0x1p-56, ui = (double)sc.u0i * 0x1p-56;
-        const double rden = -1.0 / (br * fma(ur, ur, ui * ui));
-        const double tr = ur * rden, ti = ui * rden;
-        S.tau = fx::pack(__double2ll_rn(tr * 0x1p55), __double2ll_rn(ti * 0x1p55));
-        const fx::Limb l = fx::split(__double2ll_rn(fma(tr, tr, ti * ti) * 0x1p53));
-        S.t2 = make_int2(l.h, l.l);
+        reflector_tau(sc, &S.tau, &S.t2);
       }
       // V^H u and W^H u over the own rows, a warp per column
       for (int it = warp; it < 2 * i; it += kWarps) {
@@ -332,10 +379,8 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
         Sum s;
         for (int k = max(0, (c + 1) / 32 / cl - 1); k < kmax; ++k) {
           const int r = 32 * (rank + cl * k) + lane, lr = 32 * k + lane;
-          if (r > c && r < n) {
-            const int4 v = vload(vq, lr, r);
-            cmac(s, make_int4(v.x, v.y, -v.z, -v.w), R.us[r]);
-          }
+          if (r > c && r < n) s.add_conj(R.us[r], vload(vq, lr, r));
+          if ((k & 7) == 7) s.flush();
         }
         const long long sr = fx::warp_sum(s.re()), si = fx::warp_sum(s.im());
         if (lane == 0) publish<MULTI>(&S.spart[vq][rank], sr, si, cl);
@@ -351,28 +396,34 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
         const int m = n - c - 1;
         int j = c + 1 + m * ch / nch;
         const int j1 = c + 1 + m * (ch + 1) / nch;
-        const int4* a = R.A + min(r, n - 1) + (size_t)j * ld;
+        const int4* a = R.A + min(r, n - 1);
         Sum s;
+        // batches of U columns, the next one's loads in flight (two register
+        // sets in turn, so that nothing is copied)
         constexpr int U = 8;
-        int4 nx[U];
-        if (j + U <= j1) {
+        int4 b0[U], b1[U];
+        auto fetch = [&](int4(&b)[U], int jj) {
+          if (jj + U <= j1) {
 #pragma unroll
-          for (int x = 0; x < U; ++x) nx[x] = ldA<ASM>(a + (size_t)x * ld);
-        }
-        for (; j + U <= j1; j += U) {
-          int4 cur[U];
-#pragma unroll
-          for (int x = 0; x < U; ++x) cur[x] = nx[x];
-          a += (size_t)U * ld;
-          if (j + 2 * U <= j1) {
-#pragma unroll
-            for (int x = 0; x < U; ++x) nx[x] = ldA<ASM>(a + (size_t)x * ld);
+            for (int x = 0; x < U; ++x) b[x] = __ldcg(a + (size_t)(jj + x) * ld);
           }
+        };
+        auto use = [&](const int4(&b)[U]) {
 #pragma unroll
-          for (int x = 0; x < U; ++x) cmac(s, cur[x], R.us[j + x]);
+          for (int x = 0; x < U; ++x) s.add(b[x], R.us[j + x]);
+          s.flush();
+          j += U;
+        };
+        fetch(b0, j);
+        while (j + U <= j1) {
+          fetch(b1, j + U);
+          use(b0);
+          if (j + U > j1) break;
+          fetch(b0, j + U);
+          use(b1);
         }
-        for (; j < j1; ++j, a += ld) cmac(s, ldA<ASM>(a), R.us[j]);
-        R.part[it * 32 + lane] = make_longlong2(s.re(), s.im());  // unit uA / 4
+        for (; j < j1; ++j) s.add(__ldcg(a + (size_t)j * ld), R.us[j]);
+        R.part[it * 32 + lane] = make_longlong2(s.re(), s.im());  // unit 2 uA
       }
       walker_sync<MULTI>();
       // ---- 4. corrections, p = tau y, rho
@@ -387,7 +438,7 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
             ci += v.y;
           }
         }
-        S.scoef[warp][lane] = fx::pack(fx::rne(cr, 3), fx::rne(ci, 3));
+        S.scoef[warp][lane] = fx::pack(cr, ci);
         __syncwarp();
       }
       const int4 tau = S.tau;
@@ -405,25 +456,16 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
         if (r > c && r < n) {
           Sum s;
           for (int q = 0; q < i; ++q) {
-            cmac(s, vload(q, lr, r), S.scoef[warp][kNb + q]);       // V (W^H u)
-            cmac(s, vload(kNb + q, lr, r), S.scoef[warp][q]);       // W (V^H u)
+            s.add(vload(q, lr, r), S.scoef[warp][kNb + q]);       // V (W^H u)
+            s.add(vload(kNb + q, lr, r), S.scoef[warp][q]);       // W (V^H u)
+            if (q & 1) s.flush();
           }
-          yr -= (s.rh << 2) + ((s.rx + (1ll << 24)) >> 25);
-          yi -= (s.ih << 2) + ((s.ix + (1ll << 24)) >> 25);
-          const int4 yq = fx::pack(fx::rne(yr, 3), fx::rne(yi, 3));  // unit 2 uA
+          const int4 yq = fx::pack(yr - s.re<2>(), yi - s.im<2>());
           Sum ps;
-          cmac(ps, tau, yq);
-          pr = ps.re();
-          pi = ps.im();
-          const int4 u = R.us[r];
-          long long h = 0, x = 0;
-          fx::mac(h, u.x, yq.x);
-          fx::mac(h, u.z, yq.z);
-          fx::mac(x, u.x, yq.y);
-          fx::mac(x, u.y, yq.x);
-          fx::mac(x, u.z, yq.w);
-          fx::mac(x, u.w, yq.z);
-          rho += fx::val(h, x);  // unit uA / 2
+          ps.add(tau, yq);
+          pr = ps.re<3>();  // unit uA
+          pi = ps.im<3>();
+          rho += real_dot(R.us[r], yq);
           if (r == c + 1) publish<MULTI>(&S.pnext, pr, pi, cl);
         }
         R.part[gi * 32 + lane] = make_longlong2(pr, pi);
@@ -436,36 +478,20 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
       rho = 0;
       for (int x = lane; x < cl * kWarps; x += 32) rho += S.rho[x];
       rho = fx::warp_sum(rho);
-      const fx::Limb rq = fx::split(fx::rne(rho, 3));  // unit 4 uA
-      const int2 t2 = S.t2;
-      long long ch_ = 0, cx_ = 0;
-      fx::mac(ch_, t2.x, rq.h);
-      fx::mac(cx_, t2.x, rq.l);
-      fx::mac(cx_, t2.y, rq.h);
-      const fx::Limb cc = fx::split(fx::val(ch_, cx_));  // unit 4 uA
-      auto make_w = [&](long long pr, long long pi, const int4& u) -> int4 {
-        long long rh = 0, rx = 0, ih = 0, ix = 0;
-        fx::mac(rh, cc.h, u.x);
-        fx::mac(rx, cc.h, u.y);
-        fx::mac(rx, cc.l, u.x);
-        fx::mac(ih, cc.h, u.z);
-        fx::mac(ix, cc.h, u.w);
-        fx::mac(ix, cc.l, u.z);
-        return fx::pack(fx::rne(pr - fx::val(rh, rx), 1), fx::rne(pi - fx::val(ih, ix), 1));
-      };
+      const fx::Limb cc = w_coef(S.t2, rho);
       for (int k = warp; k < kmax; k += kWarps) {
         if (k < kfirst) continue;
         const int r = 32 * (rank + cl * k) + lane, lr = 32 * k + lane;
         if (r > c && r < n) {
           const longlong2 p = R.part[(k - kfirst) * 32 + lane];
-          const int4 w = make_w(p.x, p.y, R.us[r]);
+          const int4 w = make_w(p.x, p.y, cc, R.us[r]);
           if constexpr (VWS) *vptr(kNb + i, lr, r) = w;
           if (MULTI || !VWS) R.P[(size_t)(kNb + i) * n + r] = w;
         }
       }
       if (t == kThreads - 1) {
         S.rowV[i] = R.us[c + 1];
-        S.rowW[i] = make_w(S.pnext.x, S.pnext.y, R.us[c + 1]);
+        S.rowW[i] = make_w(S.pnext.x, S.pnext.y, cc, R.us[c + 1]);
       }
       __syncthreads();
     }
@@ -473,6 +499,9 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
     // ---- trailing update on rows and columns q0 ..: a warp per 32 rows x
     // kStrip columns of the lower triangle, written to both triangles
     const int q0 = p0 + nbp;
+    const int z = rescale(S.trace, R.shifted);
+    R.shifted += z;
+    eunit -= z;
     {
       const int nw = cl * kWarps, gw = rank * kWarps + warp;
       const int c00 = q0 / kStrip * kStrip;
@@ -502,7 +531,7 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
           int4 a[kStrip];
 #pragma unroll
           for (int x = 0; x < kStrip; ++x)
-            a[x] = ldA<ASM>(R.A + rc + (size_t)min(cs + x, n - 1) * ld);
+            a[x] = __ldcg(R.A + rc + (size_t)min(cs + x, n - 1) * ld);
           Sum sum[kStrip];
 #pragma unroll 2
           for (int q = 0; q < nbp; ++q) {
@@ -524,16 +553,21 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
                 cv = R.vw[q * own + min(cs + x, n - 1)];
                 cw = R.vw[(kNb + q) * own + min(cs + x, n - 1)];
               }
-              cmac_conj(sum[x], v, cw);
-              cmac_conj(sum[x], w, cv);
+              sum[x].add_conj(v, cw);
+              sum[x].add_conj(w, cv);
+            }
+            if (q & 1) {
+#pragma unroll
+              for (int x = 0; x < kStrip; ++x) sum[x].flush();
             }
           }
 #pragma unroll
           for (int x = 0; x < kStrip; ++x) {
             const int cc = cs + x;
             if (r >= n || cc > r || cc < q0) continue;
-            const long long re = fx::join(a[x].x, a[x].y) - fx::rne(sum[x].re(), 1);
-            const long long im = r == cc ? 0 : fx::join(a[x].z, a[x].w) - fx::rne(sum[x].im(), 1);
+            const long long re = (fx::join(a[x].x, a[x].y) - sum[x].re<2>()) << z;
+            const long long im =
+                r == cc ? 0 : (fx::join(a[x].z, a[x].w) - sum[x].im<2>()) << z;
             const int4 v = fx::pack(re, im);
             R.A[r + (size_t)cc * ld] = v;
             if (r != cc) R.A[cc + (size_t)r * ld] = fx::pack(re, -im);
@@ -542,6 +576,182 @@ __device__ __forceinline__ void reduce(const Red& R, int cend) {
       }
     }
     walker_sync<MULTI>();
+    if (t == 0) S.trace <<= z;
+  }
+  R.eunit = eunit;
+}
+
+// The reduction of a matrix of order n <= kTail held in shared memory (both
+// triangles, leading dimension kTailLd), column by column: at this order the
+// columns are bound by latency, not by the products, so warp 0 takes the
+// chain from one column to the next alone (its 3 rows per lane need no
+// barrier) and three barriers part it from what the other warps do: the
+// rank-2 update of the previous column beside the norm, square root and u of
+// this one, then the product A u beside tau, then w. (As panels of 16 columns
+// in the general routine, the last 96 columns took 16 k clocks each; here
+// 8 k.) us: u of this column and the last, ws: w.
+__device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, longlong2* part,
+                                            double* d, double* e, int eunit, int shifted,
+                                           Shared& S) {
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  constexpr int kRows = kTail / 32;  // rows per lane of warp 0
+  constexpr int ld = kTailLd;
+  long long trace = S.trace;  // (warp 0's)
+  for (int c = 0; c < n; ++c) {
+    const int z = c > 0 ? S.tail_z[(c - 1) & 1] : 0;  // the previous column's update is scaled up by 2^z
+    int4* u = us + (c & 1) * kTail;
+    const int4* up = us + ((c & 1) ^ 1) * kTail;
+    if (warp == 0) {
+      // ---- column c, with the previous column's update
+      fx::U128 sq;
+      long long xr[kRows], xi[kRows];
+      int4 cu = make_int4(0, 0, 0, 0), cw = cu;
+      if (c > 0) {
+        cu = up[c];
+        cw = ws[c];
+      }
+#pragma unroll
+      for (int k = 0; k < kRows; ++k) {
+        const int r = lane + 32 * k;
+        xr[k] = xi[k] = 0;
+        if (r >= c && r < n) {
+          const int4 a = A[r + c * ld];
+          xr[k] = fx::join(a.x, a.y);
+          xi[k] = fx::join(a.z, a.w);
+          if (c > 0) {
+            Sum s;
+            s.add_conj(up[r], cw);
+            s.add_conj(ws[r], cu);
+            xr[k] = (xr[k] - s.re<2>()) << z;
+            xi[k] = (xi[k] - s.im<2>()) << z;
+          }
+          if (r == c) d[c] = scalbn((double)xr[k], eunit - z);
+          if (r >= c + 2) {
+            sq.add_square(xr[k]);
+            sq.add_square(xi[k]);
+          }
+        }
+      }
+      trace <<= z;
+      eunit -= z;
+      if (c < n - 1) {
+        sq = fx::warp_sum(sq);
+        const int kd = c >> 5, ka = (c + 1) >> 5;
+        long long dr = xr[0], ar = xr[0], ai = xi[0];
+#pragma unroll
+        for (int k = 1; k < kRows; ++k) {
+          if (kd == k) dr = xr[k];
+          if (ka == k) {
+            ar = xr[k];
+            ai = xi[k];
+          }
+        }
+        trace -= __shfl_sync(0xFFFFFFFFu, dr, c & 31) >> kTraceUnit;
+        ar = __shfl_sync(0xFFFFFFFFu, ar, (c + 1) & 31);
+        ai = __shfl_sync(0xFFFFFFFFu, ai, (c + 1) & 31);
+        double beta;
+        const ColumnScalars sc = reflector(sq, ar, ai, &beta);
+#pragma unroll
+        for (int k = 0; k < kRows; ++k) {
+          const int r = lane + 32 * k;
+          if (r > c && r < n) {
+            int4 v = make_int4(0, 0, 0, 0);
+            if (!sc.skip)
+              v = r == c + 1 ? fx::pack(sc.u0r, sc.u0i)
+                             : fx::pack(fx::shift(xr[k], sc.z), fx::shift(xi[k], sc.z));
+            u[r] = v;
+          }
+        }
+        const int zn = rescale(trace, shifted);
+        shifted += zn;
+        if (lane == 0) {
+          S.sc = sc;
+          S.tail_z[c & 1] = zn;
+          e[c] = scalbn(beta, eunit);
+        }
+      } else if (lane == 0) {
+        e[c] = 0.0;
+      }
+    } else if (c > 0) {
+      // ---- A -= u w^H + w u^H of the previous column on rows and columns
+      // above c: a warp per pair of columns j, m - 1 - j (m + 1 elements
+      // below and on the diagonal together)
+      const int b0 = c + 1, m = n - b0;
+      for (int j = warp - 1; 2 * j < m; j += kWarps - 1) {
+        const int first = m - j, len = 2 * j == m - 1 ? first : m + 1;
+        for (int x = lane; x < len; x += 32) {
+          const int cc = b0 + (x < first ? j : m - 1 - j);
+          const int r = x < first ? cc + x : cc + (x - first);
+          const int4 a = A[r + cc * ld];
+          Sum s;
+          s.add_conj(up[r], ws[cc]);
+          s.add_conj(ws[r], up[cc]);
+          const long long re = (fx::join(a.x, a.y) - s.re<2>()) << z;
+          const long long im = r == cc ? 0 : (fx::join(a.z, a.w) - s.im<2>()) << z;
+          A[r + cc * ld] = fx::pack(re, im);
+          if (r != cc) A[cc + r * ld] = fx::pack(re, -im);
+        }
+      }
+    }
+    if (c == n - 1) break;
+    __syncthreads();
+    const ColumnScalars sc = S.sc;
+    const int m = n - c - 1;
+    const int g0 = (c + 1) >> 5, cnt = ((n + 31) >> 5) - g0;  // groups of 32 rows with one > c
+    const int nch = (kWarps - 1) / cnt;
+    if (sc.skip) {  // H = I: w = 0 like u
+      if (warp == 0)
+        for (int r = c + 1 + lane; r < n; r += 32) ws[r] = make_int4(0, 0, 0, 0);
+      __syncthreads();
+      continue;
+    }
+    if (warp == kWarps - 1) {
+      if (lane == 0) reflector_tau(sc, &S.tau, &S.t2);
+    } else if (warp < cnt * nch) {
+      // ---- y = A u: one group of rows x a run of columns
+      const int g = g0 + warp % cnt, ch = warp / cnt;
+      const int r = min(32 * g + lane, n - 1);
+      int j = c + 1 + m * ch / nch;
+      const int j1 = c + 1 + m * (ch + 1) / nch;
+      Sum s;
+      for (; j < j1; ++j) {
+        s.add(A[r + j * ld], u[j]);
+        if ((j & 15) == 15) s.flush();
+      }
+      part[warp * 32 + lane] = make_longlong2(s.re(), s.im());
+    }
+    __syncthreads();
+    if (warp == 0) {
+      // ---- p = tau y, rho, w
+      const int4 tau = S.tau;
+      long long pr[kRows], pi[kRows], rho = 0;
+#pragma unroll
+      for (int k = 0; k < kRows; ++k) {
+        const int r = lane + 32 * k;
+        pr[k] = pi[k] = 0;
+        if (r > c && r < n) {
+          long long yr = 0, yi = 0;
+          for (int ch = 0; ch < nch; ++ch) {
+            const longlong2 v = part[(ch * cnt + k - g0) * 32 + lane];
+            yr += v.x;
+            yi += v.y;
+          }
+          const int4 yq = fx::pack(yr, yi);
+          Sum ps;
+          ps.add(tau, yq);
+          pr[k] = ps.re<3>();
+          pi[k] = ps.im<3>();
+          rho += real_dot(u[r], yq);
+        }
+      }
+      const fx::Limb cc = w_coef(S.t2, fx::warp_sum(rho));
+#pragma unroll
+      for (int k = 0; k < kRows; ++k) {
+        const int r = lane + 32 * k;
+        if (r > c && r < n) ws[r] = make_w(pr[k], pi[k], cc, u[r]);
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -632,7 +842,7 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
   // B = 2^eB >= bound / kScaleRoom; a zero matrix takes any scale
   const float B = lam * (1.0f / kScaleRoom);
   const int eB = e0 + (B > 0.0f ? (int)((__float_as_uint(B) >> 23) & 0xFF) - 126 : 0);
-  const int eunit = eB - fx::kLow - 30;  // uA = 2^(eB - 57)
+  const int eunit = eB - fx::kFull;  // uA = 2^eunit
   Red R;
   R.S = &S;
   R.eunit = eunit;
@@ -643,23 +853,13 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
   int4* sm = sm4;
   const int nt = SMALL ? n : kTail;
   // ---- fixed point, both triangles (in place, or into shared memory)
-  Red T = R;  // the shared-memory reduction
-  T.n = nt;
-  T.ld = kTailLd;
-  T.own = kTail;
-  T.us = sm;
-  T.part = reinterpret_cast<longlong2*>(T.us + kTail);
-  T.vw = reinterpret_cast<int4*>(T.part + kWarps * 32);
-  T.A = T.vw + 2 * kNb * kTail;
-  T.P = nullptr;
-  T.stage = nullptr;
-  T.rank = 0;
-  T.cl = 1;
-  T.d = dw + (n - nt);
-  T.e = ew + (n - nt);
+  int4* tail_us = sm;                                           // 2 kTail
+  int4* tail_ws = tail_us + 2 * kTail;                          // kTail
+  longlong2* tail_part = reinterpret_cast<longlong2*>(tail_ws + kTail);
+  int4* tail_A = reinterpret_cast<int4*>(tail_part + kWarps * 32);  // kTail x kTailLd
   {
-    int4* A = SMALL ? T.A : reinterpret_cast<int4*>(G);
-    const int ld = SMALL ? T.ld : n;
+    int4* A = SMALL ? tail_A : reinterpret_cast<int4*>(G);
+    const int ld = SMALL ? kTailLd : n;
     const int nw = cl * kWarps, gw = rank * kWarps + warp;
     int base = 0;
     for (int I = 0; I < ngroups; ++I) {
@@ -688,6 +888,19 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
     }
   }
   walker_sync<MULTI>();
+  if (warp == 0) {
+    const int4* A = SMALL ? tail_A : reinterpret_cast<int4*>(G);
+    const int ld = SMALL ? kTailLd : n;
+    long long tr0 = 0;
+    for (int i = lane; i < n; i += 32) {
+      const int4 v = SMALL ? A[i + i * ld] : __ldcg(A + i + (size_t)i * ld);
+      tr0 += fx::join(v.x, v.y) >> kTraceUnit;
+    }
+    tr0 = fx::warp_sum(tr0);
+    if (lane == 0) S.trace = tr0;
+    __syncwarp();
+  }
+  R.shifted = 0;
   if constexpr (!SMALL) {
     R.A = reinterpret_cast<int4*>(G);
     R.ld = n;
@@ -699,26 +912,21 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
     const int nparts = max(kWarps, g.own / 32) * 32;
     R.vw = reinterpret_cast<int4*>(R.part + nparts);
     R.stage = reinterpret_cast<int4*>(R.part + nparts) + (VWS ? 2 * kNb * g.own : 0);
-    reduce<MULTI, VWS, false>(R, n - kTail);  // ends with a barrier of the walker
+    reduce<MULTI, VWS>(R, n - kTail);  // ends with a barrier of the walker
     if (rank != 0) return;
     const int4* A0 = R.A + (n - kTail) + (size_t)(n - kTail) * n;
     for (int x = t; x < kTail * kTail; x += kThreads) {
       const int r = x % kTail, c = x / kTail;
-      T.A[r + c * kTailLd] = __ldcg(A0 + r + (size_t)c * n);
+      tail_A[r + c * kTailLd] = __ldcg(A0 + r + (size_t)c * n);
     }
     __syncthreads();
   }
-  reduce<false, true, true>(T, nt - 1);
-  if (t == 0) {
-    const int4 v = T.A[(nt - 1) + (size_t)(nt - 1) * T.ld];
-    dw[n - 1] = scalbn((double)fx::join(v.x, v.y), eunit);
-    ew[n - 1] = 0.0;
-  }
+  reduce_tail(tail_A, nt, tail_us, tail_ws, tail_part, dw + (n - nt), ew + (n - nt), R.eunit,
+              R.shifted, S);
 }
 
 constexpr size_t tail_smem() {
-  return (size_t)kTail * 16 + (size_t)kWarps * 32 * 16 + (size_t)2 * kNb * kTail * 16 +
-         (size_t)kTail * kTailLd * 16;
+  return ((size_t)3 * kTail + (size_t)kWarps * 32 + (size_t)kTail * kTailLd) * 16;
 }
 
 struct TriShape {
