@@ -1328,8 +1328,8 @@ bg_status apply_local_gate(bg_dtype dtype, int64_t walkers, int32_t spins, const
   DeviceCtx* ctx;
   s = get_ctx(&ctx);
   if (s != BG_OK) return s;
-  cudaError_t e = launch_local_gate(walkers, spins, sites, gates, states, stride, ctx->d_err,
-                                    ctx->sms, reinterpret_cast<cudaStream_t>(stream));
+  cudaError_t e = launch_local_gate(walkers, spins, sites, gates, states, stride, states, stride,
+                                    ctx->d_err, ctx->sms, reinterpret_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "local gate launch");
   return BG_OK;
 }
@@ -1587,18 +1587,14 @@ bg_status anneal_step(const bg_plan* plan, void* states, double* energy, const i
   DeviceCtx* ctx;
   bg_status s = get_ctx(&ctx);
   if (s != BG_OK) return s;
-  // 1. the proposal: a copy of every current state ...
-  BG_CUDA(cudaMemcpy2DAsync(p->d_prop, amps * sizeof(double2), states,
-                            p->state_stride * sizeof(double2), amps * sizeof(double2), p->count,
-                            cudaMemcpyDeviceToDevice, st),
-          "proposal copy");
-  // 2. ... with the walker's local gate applied ("Apply Local Gate")
-  cudaError_t e = launch_local_gate(p->count, p->spins, sites, gates, p->d_prop, amps, ctx->d_err,
-                                    ctx->sms, st);
+  // 1. the proposal: every current state with the walker's local gate applied
+  // ("Apply Local Gate"), from the states to the proposal buffer
+  cudaError_t e = launch_local_gate(p->count, p->spins, sites, gates, states, p->state_stride,
+                                    p->d_prop, amps, ctx->d_err, ctx->sms, st);
   if (e != cudaSuccess) return cuda_fail(e, "local gate launch");
-  // 3. its entanglement entropy ("Calculate Entropy")
+  // 2. its entanglement entropy ("Calculate Entropy")
   if ((s = batched_entropy(p->ent, p->d_prop, p->d_enew, nullptr, stream)) != BG_OK) return s;
-  // 4. the Metropolis decision ("M.A"): accepted proposals replace the states
+  // 3. the Metropolis decision ("M.A"): accepted proposals replace the states
   e = launch_metropolis(p->count, temperature, direction, uniforms, p->d_enew, energy, accepted,
                         p->d_prop, amps, states, p->state_stride, amps, ctx->sms, st);
   if (e != cudaSuccess) return cuda_fail(e, "Metropolis launch");

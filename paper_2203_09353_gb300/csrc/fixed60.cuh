@@ -70,18 +70,21 @@ __device__ __forceinline__ int4 conj(const int4& a) { return make_int4(a.x, a.y,
 struct Sum {
   long long rh = 0, rx = 0, ih = 0, ix = 0;
   __device__ __forceinline__ void add(const int4& a, const int4& b) {  // += a b
-    const int nh = -b.z, nl = -b.w;
+    add(a, b, make_int2(-b.z, -b.w));
+  }
+  // (nb: -im b, where the caller has it)
+  __device__ __forceinline__ void add(const int4& a, const int4& b, const int2& nb) {
     mac(rh, a.x, b.x);
     mac(rx, a.x, b.y);
     mac(ih, a.x, b.z);
     mac(ix, a.x, b.w);
     mac(rx, a.y, b.x);
     mac(ix, a.y, b.z);
-    mac(rh, a.z, nh);
-    mac(rx, a.z, nl);
+    mac(rh, a.z, nb.x);
+    mac(rx, a.z, nb.y);
     mac(ih, a.z, b.x);
     mac(ix, a.z, b.y);
-    mac(rx, a.w, nh);
+    mac(rx, a.w, nb.x);
     mac(ix, a.w, b.x);
   }
   __device__ __forceinline__ void add_conj(const int4& a, const int4& b) { add(a, conj(b)); }
