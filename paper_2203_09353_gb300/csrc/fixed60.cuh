@@ -27,8 +27,9 @@ struct Limb {
 };
 
 __device__ __forceinline__ Limb split(long long x) {
-  const int l = (int)((uint32_t)x << (32 - kLow)) >> (32 - kLow);  // low bits, sign-extended
-  return {(int)((x - l) >> kLow), l};
+  const unsigned long long v = (unsigned long long)x + (1u << (kLow - 1));
+  return {(int)(uint32_t)(v >> kLow),
+          (int)((uint32_t)v & ((1u << kLow) - 1)) - (1 << (kLow - 1))};
 }
 __device__ __forceinline__ long long join(int h, int l) { return ((long long)h << kLow) + l; }
 
@@ -143,6 +144,74 @@ __device__ __forceinline__ U128 warp_sum(U128 v) {
   for (int o = 16; o > 0; o >>= 1)
     v.add(__shfl_xor_sync(0xFFFFFFFFu, v.hi, o), __shfl_xor_sync(0xFFFFFFFFu, v.lo, o));
   return v;
+}
+
+// ---- scalars of full precision without the FP64 pipe, whose instructions
+// follow one another at 70 clocks (a square root or a division takes 580).
+// Each starts from the 22 bits of the approximate FP32 instruction and takes
+// two Newton steps, x <- x + r / f'(x) with the exact integer residual r.
+
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// sqrt(v) 2^z, to the nearest few units, in [2^58, 2^59); 0 < v < 2^122.
+__device__ __forceinline__ long long sqrt_scaled(const U128& v, int* z) {
+  const int lz = v.hi ? __clzll((long long)v.hi) : 64 + __clzll((long long)v.lo);
+  const int sh = (lz & ~1) - 2;  // t = v 2^sh in [2^124, 2^126)
+  unsigned long long th, tl;
+  if (sh >= 64) {
+    th = v.lo << (sh - 64);
+    tl = 0;
+  } else {
+    th = v.hi << sh | v.lo >> (64 - sh);
+    tl = v.lo << sh;
+  }
+  const float f = (float)(uint32_t)(th >> 38), r = rsqrt_approx(f);
+  const uint32_t g = __float2uint_rn(f * r * 0x1p19f);  // sqrt(t) 2^-32, in [2^30, 2^31]
+  const long long rho = (long long)(th - (unsigned long long)g * g);
+  // (|rho| < 2^43: the start is within 2^-21)
+  const float d = (float)(int)(rho >> 13) * r * 0x1p13f;  // rho / (2 g) 2^20
+  unsigned long long s = ((unsigned long long)g << 32) + ((long long)__float2int_rn(d) << 12);
+  const unsigned long long pl = s * s, ph = __umul64hi(s, s);
+  const unsigned long long dl = tl - pl, dh = th - ph - (tl < pl ? 1ull : 0ull);
+  const int e = (int)(uint32_t)(dh << 7 | dl >> 57);  // (t - s^2) 2^-57
+  s += (long long)__float2int_rn((float)e * r * 0x1p5f);  // e 2^57 / (2 s)
+  *z = sh / 2 - 4;
+  return (long long)((s + 8) >> 4);
+}
+
+// 2^126 / q for q in [2^63, 2^64), to the nearest few units: in (2^62, 2^63].
+__device__ __forceinline__ unsigned long long recip126(unsigned long long q) {
+  const float r = rcp_approx((float)(uint32_t)(q >> 40));
+  const uint32_t g = __float2uint_rn(r * 0x1p54f);  // 2^94 / q
+  unsigned long long pl = q * g, ph = __umul64hi(q, g);
+  unsigned long long dl = 0 - pl, dh = (1ull << 30) - ph - (pl ? 1ull : 0ull);
+  const int e = (int)(uint32_t)(dh << 19 | dl >> 45);  // (2^94 - q g) 2^-45
+  unsigned long long x =
+      ((unsigned long long)g << 32) + ((long long)__float2int_rn((float)e * r * 0x1p25f) << 12);
+  pl = q * x;
+  ph = __umul64hi(q, x);
+  dl = 0 - pl;
+  dh = (1ull << 62) - ph - (pl ? 1ull : 0ull);
+  const int e2 = (int)(uint32_t)(dh << 7 | dl >> 57);  // (2^126 - q x) 2^-57
+  x += (long long)__float2int_rn((float)e2 * r * 0x1p17f);
+  return x;
+}
+
+// x 2^e as a double.
+__device__ __forceinline__ double to_double(long long x, int e) {
+  const double d = __ll2double_rn(x);
+  if (x != 0 && e > -900 && e < 900)
+    return __hiloint2double(__double2hiint(d) + (e << 20), __double2loint(d));
+  return scalbn(d, e);
 }
 
 }  // namespace fx

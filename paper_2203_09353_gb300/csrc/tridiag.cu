@@ -83,7 +83,7 @@ struct Shared {
   longlong2 alpha[2];
   long long diag[2];                   // the column's diagonal entry
   long long trace;                     // of the rows not reduced yet (2^kTraceUnit uA)
-  int tail_z[2];                       // the tail's shift after a column
+  int tail_z[2], unit[2];              // the tail's shift after a column, the column's unit
   longlong2 norm[2][kMaxCl * kWarps];  // sums of squares (hi, lo) of every warp
   longlong2 spart[2 * kNb][kMaxCl];    // V^H u and W^H u, a partial per CTA
   long long rho[kMaxCl * kWarps];
@@ -168,38 +168,51 @@ __device__ __forceinline__ int rescale(long long trace, int shifted) {
 }
 
 // The reflector of a column (alpha, x...) with |x|^2 = sum: beta = -+N, N the
-// column's norm, and u = (alpha - beta, x...) 2^z with N 2^z in [2^58, 2^59).
+// column's norm, and u = (alpha - beta, x...) 2^z with nint = N 2^z in
+// [2^58, 2^59).
 __device__ __forceinline__ ColumnScalars reflector(const fx::U128& sum, long long alr,
-                                                   long long ali, double* beta) {
+                                                   long long ali) {
   ColumnScalars sc{0, 0, 0, 0, 0};
   if (sum.hi == 0 && sum.lo == 0 && ali == 0) {
     sc.skip = 1;  // already reduced: H = I
-    *beta = (double)alr;
     return sc;
   }
   fx::U128 all = sum;
   all.add_square(alr);
   all.add_square(ali);
-  const double N = sqrt(all.value());
-  const int eN = (int)((__double2hiint(N) >> 20) & 0x7FF) - 1022;  // N in [2^(eN-1), 2^eN)
-  sc.z = fx::kFull - 1 - eN;
-  sc.nint = __double2ll_rn(N * __hiloint2double((1023 + sc.z) << 20, 0));
+  sc.nint = fx::sqrt_scaled(all, &sc.z);
   const long long xr = fx::shift(alr, sc.z);
   sc.u0r = alr < 0 ? xr - sc.nint : xr + sc.nint;
   sc.u0i = fx::shift(ali, sc.z);
-  *beta = alr < 0 ? N : -N;
   return sc;
 }
 
-// tau = -u0 / (beta |u0|^2) (beta and u0 scaled) in limbs of unit 2^-58, and
-// |tau|^2 / 2 in limbs of unit 2^-57.
+// The sub-diagonal entry beta of a column with first entry alr.
+__device__ __forceinline__ double column_beta(const ColumnScalars& sc, long long alr, int eunit) {
+  return sc.skip ? fx::to_double(alr, eunit)
+                 : fx::to_double(alr < 0 ? sc.nint : -sc.nint, eunit - sc.z);
+}
+
+// tau = -u0 / (beta |u0|^2) in limbs of unit 2^-58, and |tau|^2 / 2 in limbs of
+// unit 2^-57. With N = nint 2^-59 in [0.5, 1) and |u0|^2 in [0.25, 4), tau is
+// +-u0 times 1 / (N |u0|^2).
 __device__ __forceinline__ void reflector_tau(const ColumnScalars& sc, int4* tau, int2* t2) {
-  const double br = (sc.u0r < 0 ? 1.0 : -1.0) * (double)sc.nint * 0x1p-59;
-  const double ur = (double)sc.u0r * 0x1p-59, ui = (double)sc.u0i * 0x1p-59;
-  const double rden = -1.0 / (br * fma(ur, ur, ui * ui));
-  const double tr = ur * rden, ti = ui * rden;
-  *tau = fx::pack(__double2ll_rn(tr * 0x1p58), __double2ll_rn(ti * 0x1p58));
-  const fx::Limb l = fx::split(__double2ll_rn(fma(tr, tr, ti * ti) * 0x1p56));
+  fx::U128 M;
+  M.add_square(sc.u0r);
+  M.add_square(sc.u0i);
+  const unsigned long long a = (unsigned long long)sc.nint << 4, b = M.hi << 7 | M.lo >> 57;
+  const unsigned long long hi = __umul64hi(a, b), lo = a * b;
+  const int lz = __clzll((long long)hi);  // 2 .. 6
+  const unsigned long long R = fx::recip126(hi << lz | lo >> (64 - lz));
+  const long long r = (long long)(R >> 1), sr = sc.u0r < 0 ? -r : r;  // beta's sign is -u0r's
+  // u0 R 2^(lz - 67)
+  const long long tr = fx::shift(__mul64hi(sc.u0r << 2, sr), lz - 4);
+  const long long ti = fx::shift(__mul64hi(sc.u0i << 2, sr), lz - 4);
+  *tau = fx::pack(tr, ti);
+  fx::U128 T;
+  T.add_square(tr);
+  T.add_square(ti);
+  const fx::Limb l = fx::split((long long)(T.hi << 4 | T.lo >> 60));
   *t2 = make_int2(l.h, l.l);
 }
 
@@ -294,10 +307,7 @@ __device__ __forceinline__ void reduce(Red& R, int cend) {
           }
           xr = fx::join(a.x, a.y) - s.re<2>();
           xi = fx::join(a.z, a.w) - s.im<2>();
-          if (r == c) {
-            R.d[c] = scalbn((double)xr, eunit);
-            publish<MULTI>(&S.diag[par], xr, cl);
-          }
+          if (r == c) publish<MULTI>(&S.diag[par], xr, cl);
           if (r == c + 1) publish<MULTI>(&S.alpha[par], xr, xi, cl);
           if (r >= c + 2) {
             sq.add_square(xr);
@@ -320,15 +330,16 @@ __device__ __forceinline__ void reduce(Red& R, int cend) {
         sum = fx::warp_sum(sum);
         if (lane == 0) {
           const longlong2 al = S.alpha[par];
-          double beta;
-          const ColumnScalars sc = reflector(sum, al.x, al.y, &beta);
-          if (rank == 0) R.e[c] = scalbn(beta, eunit);
+          S.sc = reflector(sum, al.x, al.y);
           S.trace -= S.diag[par] >> kTraceUnit;
-          S.sc = sc;
         }
       }
       __syncthreads();
       const ColumnScalars sc = S.sc;
+      if (rank == 0 && t == kThreads - 32) {
+        R.d[c] = fx::to_double(S.diag[par], eunit);
+        R.e[c] = column_beta(sc, S.alpha[par].x, eunit);
+      }
       // u to every CTA; V's column i
       for (int k = warp; k < kmax; k += kWarps) {
         const int r = 32 * (rank + cl * k) + lane, lr = 32 * k + lane;
@@ -625,7 +636,6 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
             xr[k] = (xr[k] - s.re<2>()) << z;
             xi[k] = (xi[k] - s.im<2>()) << z;
           }
-          if (r == c) d[c] = scalbn((double)xr[k], eunit - z);
           if (r >= c + 2) {
             sq.add_square(xr[k]);
             sq.add_square(xi[k]);
@@ -646,11 +656,11 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
             ai = xi[k];
           }
         }
-        trace -= __shfl_sync(0xFFFFFFFFu, dr, c & 31) >> kTraceUnit;
+        dr = __shfl_sync(0xFFFFFFFFu, dr, c & 31);
+        trace -= dr >> kTraceUnit;
         ar = __shfl_sync(0xFFFFFFFFu, ar, (c + 1) & 31);
         ai = __shfl_sync(0xFFFFFFFFu, ai, (c + 1) & 31);
-        double beta;
-        const ColumnScalars sc = reflector(sq, ar, ai, &beta);
+        const ColumnScalars sc = reflector(sq, ar, ai);
 #pragma unroll
         for (int k = 0; k < kRows; ++k) {
           const int r = lane + 32 * k;
@@ -667,10 +677,18 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
         if (lane == 0) {
           S.sc = sc;
           S.tail_z[c & 1] = zn;
-          e[c] = scalbn(beta, eunit);
+          S.alpha[c & 1] = make_longlong2(ar, dr);
+          S.unit[c & 1] = eunit;
         }
-      } else if (lane == 0) {
-        e[c] = 0.0;
+      } else {
+        long long dr = xr[0];
+#pragma unroll
+        for (int k = 1; k < kRows; ++k)
+          if ((c >> 5) == k) dr = xr[k];
+        if (lane == (c & 31)) {
+          d[c] = fx::to_double(dr, eunit);
+          e[c] = 0.0;
+        }
       }
     } else if (c > 0) {
       // ---- A -= u w^H + w u^H of the previous column on rows and columns
@@ -699,6 +717,10 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
     const int m = n - c - 1;
     const int g0 = (c + 1) >> 5, cnt = ((n + 31) >> 5) - g0;  // groups of 32 rows with one > c
     const int nch = (kWarps - 1) / cnt;
+    if (t == kThreads - 64) {  // (a warp that seldom has a share of the product)
+      d[c] = fx::to_double(S.alpha[c & 1].y, S.unit[c & 1]);
+      e[c] = column_beta(sc, S.alpha[c & 1].x, S.unit[c & 1]);
+    }
     if (sc.skip) {  // H = I: w = 0 like u
       if (warp == 0)
         for (int r = c + 1 + lane; r < n; r += 32) ws[r] = make_int4(0, 0, 0, 0);
@@ -731,6 +753,7 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
         pr[k] = pi[k] = 0;
         if (r > c && r < n) {
           long long yr = 0, yi = 0;
+#pragma unroll 5
           for (int ch = 0; ch < nch; ++ch) {
             const longlong2 v = part[(ch * cnt + k - g0) * 32 + lane];
             yr += v.x;
