@@ -217,7 +217,8 @@ struct bg_plan {
   int32_t* d_order = nullptr;
   WorkItem* d_items = nullptr;
   int64_t n_items = 0;
-  int grid = 0;
+  int grid = 0;     // CTAs the FP64 work list is cut for
+  int ctas = 2;     // CTAs per SM of the FP64 kernel
   // chain
   int32_t walkers = 0, pool_count = 0;
   std::vector<int64_t> wn, woff, pool_n, pool_off;
@@ -281,25 +282,29 @@ bg_status upload(T** dptr, const std::vector<T>& v, int64_t* ws_bytes) {
 double item_cost(const WorkItem& w, const std::vector<int64_t>& mnk_k,
                  const std::vector<int64_t>& mnk_mn, const std::vector<int32_t>& order) {
   if (prog_is_small(w.prog)) {
-    const double lanes = 32.0 * (w.r0 > 0 ? w.r0 : 1);  // threads per instance
     double c = 0;
     for (int i = 0; i < w.count; ++i) {
       const int64_t id = order[w.inst + i];
-      c = std::max(c, std::ceil(mnk_mn[id] / lanes) * (double)mnk_k[id]);
+      c = std::max(c, std::ceil(mnk_mn[id] / 32.0) * (double)mnk_k[id]);
     }
     return c;
   }
   int tm, tn;
   prog_tile(w.prog, &tm, &tn);
+  tile_extent_of(w.count, tm, &tm, &tn);
   return (double)tm * tn / kFp64Threads * (double)mnk_k[w.inst];
 }
 
 // Build the FP64 work list for instances with the given program per instance.
 // `ids` are instance (or walker) ids, `sizes` their (m, n, k), `prog_of` the
-// chosen program. Small-program instances are grouped in `order`, 8 to a CTA,
-// or fewer (with several warps each) when there are too few of them to give
-// each of the `grid` CTAs an item; items are sorted longest first.
-void build_items(const std::vector<int64_t>& ids, const std::vector<std::array<int64_t, 3>>& mnk,
+// chosen program. Small-program instances are grouped in `order`, 8 to a CTA;
+// where there are too few of them to give each of the `grid` CTAs such a
+// group they run as tiles instead. Tiles split an instance evenly, further
+// while a tile holds more than a CTA's share of the whole work (a batch of few
+// instances would leave SMs idle). Items are sorted longest first. Returns the
+// CTAs per SM to run them with: one where full tiles hold most of the work,
+// three where every tile is small.
+int build_items(const std::vector<int64_t>& ids, const std::vector<std::array<int64_t, 3>>& mnk,
                  const std::vector<int>& prog_of, std::vector<WorkItem>* items,
                  std::vector<int32_t>* order, bool herk, int64_t grid) {
   items->clear();
@@ -312,39 +317,61 @@ void build_items(const std::vector<int64_t>& ids, const std::vector<std::array<i
   }
   // small programs: group by program, sort each group by cost descending
   std::map<int, std::vector<int64_t>> small;
+  double work = 0;
   for (int64_t id : ids) {
-    const int p = prog_of[id];
-    if (prog_is_small(p)) {
-      small[p].push_back(id);
-    } else {
-      int tm, tn;
-      prog_tile(p, &tm, &tn);
-      const int64_t m = mnk[id][0], n = mnk[id][1];
-      for (int64_t c0 = 0; c0 < n; c0 += tn)
-        for (int64_t r0 = 0; r0 < m; r0 += tm) {
-          if (herk && r0 + tm - 1 < c0) continue;  // wholly above the diagonal
-          WorkItem w;
-          w.inst = (int32_t)id;
-          w.prog = (int16_t)p;
-          w.count = 1;
-          w.r0 = (int32_t)r0;
-          w.c0 = (int32_t)c0;
-          items->push_back(w);
-        }
-    }
+    if (prog_is_small(prog_of[id])) small[prog_of[id]].push_back(id);
+    work += (double)mn[id] * (double)kk[id];
   }
+  const double share = work / (double)std::max<int64_t>(grid, 1);
+  double full = 0;  // work in full tiles
+  auto add_tiles = [&](int64_t id, int p) {
+    int T, tn0;
+    prog_tile(p, &T, &tn0);
+    const int64_t m = mnk[id][0], n = mnk[id][1];
+    int64_t tm = T, tn = tn0;
+    if (p != PROG_R64_DMMA) {
+      int64_t pm = (m + T - 1) / T, pn = (n + T - 1) / T;
+      tm = (m + pm - 1) / pm;
+      tn = (n + pn - 1) / pn;
+      const bg_dtype dt = p == PROG_C128_TILE ? BG_C128 : BG_R64;
+      while (!fp64_tile_ok(dt, tm, tn) ||
+             (tm * tn > kFp64Threads && (double)tm * tn * (double)kk[id] > share)) {
+        if (tm > tn) tm = (m + pm) / (pm + 1), ++pm;
+        else tn = (n + pn) / (pn + 1), ++pn;
+      }
+    }
+    for (int64_t c0 = 0; c0 < n; c0 += tn)
+      for (int64_t r0 = 0; r0 < m; r0 += tm) {
+        if (herk && r0 + tm - 1 < c0) continue;  // wholly above the diagonal
+        WorkItem w;
+        w.inst = (int32_t)id;
+        w.prog = (int16_t)p;
+        w.count = p == PROG_R64_DMMA ? 1 : tile_extent((int)tm, (int)tn);
+        w.r0 = (int32_t)r0;
+        w.c0 = (int32_t)c0;
+        items->push_back(w);
+        if (tm == T && tn == tn0 && r0 + tm <= m && c0 + tn <= n)
+          full += (double)tm * tn * (double)kk[id];
+      }
+  };
+  for (int64_t id : ids)
+    if (!prog_is_small(prog_of[id])) add_tiles(id, prog_of[id]);
   for (auto& kv : small) {
     auto& v = kv.second;
+    if (!small_fills((int64_t)v.size(), grid)) {
+      for (int64_t id : v)
+        add_tiles(id, kv.first == PROG_R64_SMALL ? PROG_R64_TILE : PROG_C128_TILE);
+      continue;
+    }
     std::stable_sort(v.begin(), v.end(), [&](int64_t a, int64_t b) {
       return std::ceil(mn[a] / 32.0) * kk[a] > std::ceil(mn[b] / 32.0) * kk[b];
     });
-    const int g = kv.first == PROG_R64_SMALL ? small_group((int64_t)v.size(), grid) : kSmallPerCta;
-    for (size_t s = 0; s < v.size(); s += g) {
+    for (size_t s = 0; s < v.size(); s += kSmallPerCta) {
       WorkItem w;
       w.inst = (int32_t)order->size();
       w.prog = (int16_t)kv.first;
-      w.count = (int16_t)std::min<size_t>(g, v.size() - s);
-      w.r0 = kSmallPerCta / g;  // warps per instance
+      w.count = (int16_t)std::min<size_t>(kSmallPerCta, v.size() - s);
+      w.r0 = 0;
       w.c0 = 0;
       for (int i = 0; i < w.count; ++i) order->push_back((int32_t)v[s + i]);
       items->push_back(w);
@@ -358,6 +385,16 @@ void build_items(const std::vector<int64_t>& ids, const std::vector<std::array<i
   std::vector<WorkItem> sorted(items->size());
   for (size_t i = 0; i < perm.size(); ++i) sorted[i] = (*items)[perm[i]];
   items->swap(sorted);
+  if (full > 0.5 * work) return 1;
+  bool little = true;  // tiles of few outputs only
+  for (const WorkItem& w : *items) {
+    int tm, tn;
+    if (prog_is_small(w.prog) || w.count < 2) little = false;
+    else tile_extent_of(w.count, 0, &tm, &tn);
+    if (!little) break;
+    little = tm * tn <= (w.prog == PROG_C128_TILE ? 2 : 4) * kFp64Threads;
+  }
+  return little ? 3 : 2;
 }
 
 // ---- autotune cache (JSON, one entry per line) --------------------------------------------
@@ -472,7 +509,7 @@ bg_status time_class_fp64(bg_plan* p, int cls, int prog, cudaStream_t st, double
   }
   std::vector<WorkItem> items;
   std::vector<int32_t> order;
-  build_items(sids, smnk, sprog, &items, &order, false, p->grid);
+  const int ctas = build_items(sids, smnk, sprog, &items, &order, false, p->grid);
   void *A = nullptr, *B = nullptr, *C = nullptr;
   int64_t* dt = nullptr;
   int32_t* dord = nullptr;
@@ -503,7 +540,7 @@ bg_status time_class_fp64(bg_plan* p, int cls, int prog, cudaStream_t st, double
     for (int r = 0; r < 4; ++r) {
       cudaEventRecord(e0, st);
       cudaError_t e = launch_fp64_table(p->dtype, dt, dord, dit, (int64_t)items.size(), A, B, C,
-                                        s, p->grid, st);
+                                        s, ctas, st);
       cudaEventRecord(e1, st);
       if (e != cudaSuccess) {
         rs = cuda_fail(e, "autotune launch");
@@ -730,7 +767,8 @@ bg_status build_fp64_schedule(bg_plan* p, const char* cache_path, cudaStream_t s
     if (p->table[i].m > 0 && p->table[i].n > 0 && !is_split_route(prog_of[i])) live.push_back(i);
   std::vector<WorkItem> items;
   std::vector<int32_t> order;
-  build_items(live, mnk, prog_of, &items, &order, (p->flags & BG_PLAN_HERK) != 0, p->grid);
+  p->ctas = build_items(live, mnk, prog_of, &items, &order, (p->flags & BG_PLAN_HERK) != 0,
+                        p->grid);
   p->n_items = (int64_t)items.size();
   bg_status s;
   if ((s = upload(&p->d_order, order, &p->workspace_bytes)) != BG_OK) return s;
@@ -822,9 +860,9 @@ bg_status batched_gemm_fixed(bg_dtype dtype, int64_t m, int64_t n, int64_t k, co
   if ((s = get_ctx(&ctx)) != BG_OK) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (pr.mode == BG_MODE_FP64) {
-    const int prog = default_prog(dtype, m, n, k);
+    const int prog = default_prog(dtype, m, n, batch, ctx->sms);
     cudaError_t e = launch_fp64_fixed(dtype, prog, m, n, k, sc, A, lda, strideA, B, ldb, strideB,
-                                      C, ldc, strideC, batch, 0, st);
+                                      C, ldc, strideC, batch, st);
     if (e != cudaSuccess) return cuda_fail(e, "FP64 batched kernel launch");
     return BG_OK;
   }
@@ -896,7 +934,7 @@ bg_status batched_gemm_plan(bg_plan** out, bg_dtype dtype, int64_t count,
   p->flags = flags;
   p->count = count;
   p->table.assign(host_table, host_table + count);
-  p->grid = ctx->sms * fp64_blocks_per_sm(dtype);
+  p->grid = 2 * ctx->sms;
   assign_classes(p);
   std::vector<int64_t> flat(count * 9);
   for (int64_t i = 0; i < count; ++i) memcpy(&flat[9 * i], &p->table[i], 9 * sizeof(int64_t));
@@ -955,7 +993,7 @@ static bg_status run_grouped_direct(bg_plan* p, const void* A, const void* B, vo
   }
   if (p->prec.mode == BG_MODE_FP64) {
     cudaError_t e = launch_fp64_table(p->dtype, p->d_table, p->d_order, p->d_items, p->n_items, A,
-                                      B, C, sc, p->grid, st, (p->flags & BG_PLAN_HERK) != 0);
+                                      B, C, sc, p->ctas, st, (p->flags & BG_PLAN_HERK) != 0);
     if (e != cudaSuccess) return cuda_fail(e, "grouped FP64 launch");
     if (ev)
       for (int i = 1; i < 4; ++i) BG_CUDA(cudaEventRecord(ev[i], st), "profiling event record");
@@ -974,7 +1012,7 @@ static bg_status run_grouped_direct(bg_plan* p, const void* A, const void* B, vo
   if (p->n_items > 0) {
     // classes the autotuner gave to the FP64 path (timed with the GEMM slot)
     cudaError_t e = launch_fp64_table(p->dtype, p->d_table, p->d_order, p->d_items, p->n_items, A,
-                                      B, C, sc, p->grid, st, (p->flags & BG_PLAN_HERK) != 0);
+                                      B, C, sc, p->ctas, st, (p->flags & BG_PLAN_HERK) != 0);
     if (e != cudaSuccess) return cuda_fail(e, "grouped FP64 launch");
     if (ev) BG_CUDA(cudaEventRecord(ev[3], st), "profiling event record");
   }
@@ -1092,7 +1130,7 @@ bg_status chain_plan(bg_plan** out, bg_dtype dtype, int32_t walkers, const int64
   p->pool_n.assign(pool_n, pool_n + pool_count);
   p->pool_off.assign(pool_off, pool_off + pool_count);
   p->count = walkers;
-  p->grid = ctx->sms * fp64_blocks_per_sm(dtype);
+  p->grid = 2 * ctx->sms;
   // walkers as instances n x n x n (offsets unused by the FP64 chain source)
   for (int32_t w = 0; w < walkers; ++w) {
     const int64_t n = walker_n[w];
@@ -1144,7 +1182,7 @@ static bg_status run_chain_direct(bg_plan* p, const void* U, const int32_t* idx,
     if (p->prec.mode == BG_MODE_FP64) {
       cudaError_t e = launch_fp64_chain(p->dtype, p->d_wn, p->d_woff, p->d_pool_off, p->d_pool_n,
                                         p->pool_count, p->d_order,
-                                        row, p->d_items, p->n_items, U, cin, cout, p->grid, st);
+                                        row, p->d_items, p->n_items, U, cin, cout, p->ctas, st);
       if (e != cudaSuccess) return cuda_fail(e, "chain step launch");
     } else {
       s = split_chain_step(p->split, U, row, cin, cout, ctx->d_err, st, &g_last_error);

@@ -16,7 +16,7 @@ namespace bg {
 // Tile programs of the FP64 path. A work item names one program and the part
 // of the batch it covers.
 enum Prog : int16_t {
-  PROG_R64_SMALL = 0,   // a warp per instance (8 per CTA), or 8 warps on one instance
+  PROG_R64_SMALL = 0,   // a warp per instance, 8 per CTA
   PROG_R64_TILE = 1,    // 64x64 output tile, DFMA, 4x4 outputs per thread
   PROG_R64_DMMA = 2,    // 64x64 output tile, FP64 tensor-core mma.sync m8n8k4
   PROG_C128_SMALL = 3,  // one warp per complex instance
@@ -25,7 +25,8 @@ enum Prog : int16_t {
 };
 
 // One unit of work of the persistent FP64 kernel (16 bytes).
-//  - tile programs: `inst` = instance id, (r0, c0) = first row/col of the tile
+//  - tile programs: `inst` = instance id, (r0, c0) = first row/col of the tile,
+//    `count` = its rows and columns (tile_extent)
 //  - small programs: `inst` = first position in the class-ordered instance
 //    list, `count` = number of consecutive instances (<= 8), r0 = c0 = 0
 struct WorkItem {
@@ -37,13 +38,21 @@ struct WorkItem {
 };
 static_assert(sizeof(WorkItem) == 16, "WorkItem must stay 16 bytes");
 
+// Rows and columns (1..64 each) of a tile in WorkItem.count; 0 and 1 mean the
+// program's full tile.
+__host__ __device__ inline int16_t tile_extent(int tm, int tn) { return (int16_t)(2 + (tm - 1) * 64 + (tn - 1)); }
+__host__ __device__ inline void tile_extent_of(int count, int full, int* tm, int* tn) {
+  *tm = *tn = full;
+  if (count >= 2) {
+    *tm = (count - 2) / 64 + 1;
+    *tn = (count - 2) % 64 + 1;
+  }
+}
+
 constexpr int kSmallPerCta = 8;   // warps (instances) per CTA in the small programs
-// Real small-program work items hold g instances that the CTA's 8 warps
-// share: g = 8 (a warp each), or g = 1 (all 8 warps on one instance) for
-// batches too small to give every resident CTA an item of 8; WorkItem.r0
-// carries the warps per instance (0 reads as 1).
-inline int small_group(int64_t instances, int64_t grid) {
-  return (instances + kSmallPerCta - 1) / kSmallPerCta >= grid ? kSmallPerCta : 1;
+// Whether the small programs' groups of 8 fill `grid` CTAs.
+inline bool small_fills(int64_t instances, int64_t grid) {
+  return (instances + kSmallPerCta - 1) / kSmallPerCta >= grid;
 }
 constexpr int kFp64Threads = 256;
 
@@ -52,11 +61,19 @@ struct Scalars {
   int alpha_zero, beta_zero;
 };
 
-// Program picked for a size (FP64 path) when no tuned choice exists.
-int default_prog(bg_dtype dt, int64_t m, int64_t n, int64_t k);
+// Program of a fixed-size batch (FP64 path).
+int default_prog(bg_dtype dt, int64_t m, int64_t n, int64_t batch, int sms);
 // Output-tile extent of a tile program (rows, cols); small programs return 0.
 void prog_tile(int prog, int* tm, int* tn);
 bool prog_is_small(int prog);
+// Whether a tile of tm x tn outputs can run: the full tile, or at most as many
+// outputs as the threads hold in linear order.
+bool fp64_tile_ok(bg_dtype dt, int64_t tm, int64_t tn);
+// Rows and columns of the tiles that `batch` instances of one shape are cut
+// into (at most 64 x 64 real, 32 x 32 complex, evenly split), so that a batch
+// smaller than the chip still spreads over its SMs.
+void fp64_tile_split(bg_dtype dt, int64_t m, int64_t n, int64_t k, int64_t batch, int sms, int* tm,
+                     int* tn);
 bool prog_fits(int prog, bg_dtype dt, int64_t m, int64_t n);
 
 // ---- FP64 launchers (fp64.cu) ---------------------------------------------------
@@ -64,24 +81,23 @@ bool prog_fits(int prog, bg_dtype dt, int64_t m, int64_t n);
 cudaError_t launch_fp64_fixed(bg_dtype dt, int prog, int64_t m, int64_t n, int64_t k,
                               const Scalars& s, const void* A, int64_t lda, int64_t sA,
                               const void* B, int64_t ldb, int64_t sB, void* C, int64_t ldc,
-                              int64_t sC, int64_t batch, int grid_cap, cudaStream_t st);
+                              int64_t sC, int64_t batch, cudaStream_t st);
 
+// ctas: CTAs per SM: 1 (most work in full tiles), 2, or 3 (no small programs,
+// tiles of at most 1024 real or 512 complex outputs).
 // herm: the plan's instances are Hermitian rank-k updates (B = A^H, lower
 // triangle stored).
 cudaError_t launch_fp64_table(bg_dtype dt, const int64_t* d_table, const int32_t* d_order,
                               const WorkItem* d_items, int64_t n_items, const void* A,
-                              const void* B, void* C, const Scalars& s, int grid,
+                              const void* B, void* C, const Scalars& s, int ctas,
                               cudaStream_t st, bool herm = false);
 
 cudaError_t launch_fp64_chain(bg_dtype dt, const int64_t* d_wn, const int64_t* d_woff,
                               const int64_t* d_pool_off, const int64_t* d_pool_n,
                               int32_t pool_count, const int32_t* d_order,
                               const int32_t* d_idx_row, const WorkItem* d_items, int64_t n_items,
-                              const void* U, const void* Cin, void* Cout, int grid,
+                              const void* U, const void* Cin, void* Cout, int ctas,
                               cudaStream_t st);
-
-// Resident CTAs per SM of the persistent FP64 kernel (for grid sizing).
-int fp64_blocks_per_sm(bg_dtype dt);
 
 // ---- split-BF16 path (split.cu) ---------------------------------------------------
 

@@ -5,7 +5,10 @@
 //  * small programs: one warp per instance, several instances per CTA (the
 //    tiny-matrix idea the paper cites in Sec. 2: several small C per block);
 //  * tile programs: a 2-D output tile per CTA (the tiling of Sec. 2), operands
-//    staged through shared memory in double-buffered k-slices.
+//    staged through shared memory in double-buffered k-slices. A tile of fewer
+//    outputs than the full one deals them to the threads in linear order, so
+//    that the FP64 instructions grow with the outputs and not with the tile,
+//    and ends at the instance's k.
 // On GB300 the FP64 pipe issues 2 DFMA per clock per SM (measured 1.19
 // TFLOP/s chip-wide, DMMA 1.05), i.e. one warp-wide DFMA per 64 clocks per
 // SM sub-partition, so every program here is FP64-issue-bound long before
@@ -129,17 +132,16 @@ struct ChainSrc {
 
 struct FixedSched {
   int prog;
-  int tm, tn;
-  int g;  // small programs: instances per item
+  int tm, tn;  // 0: small program
   int64_t tiles_m, tiles_n, batch;
   __device__ WorkItem get(int64_t it) const {
     WorkItem w;
     w.prog = (int16_t)prog;
     if (tm == 0) {
-      w.inst = (int32_t)(it * g);
-      const int64_t left = batch - it * g;
-      w.count = (int16_t)(left < g ? left : g);
-      w.r0 = kSmallPerCta / g;  // warps per instance
+      w.inst = (int32_t)(it * kSmallPerCta);
+      const int64_t left = batch - it * kSmallPerCta;
+      w.count = (int16_t)(left < kSmallPerCta ? left : kSmallPerCta);
+      w.r0 = 0;
       w.c0 = 0;
     } else {
       const int64_t per = tiles_m * tiles_n;
@@ -147,7 +149,7 @@ struct FixedSched {
       const int64_t t = it - (it / per) * per;
       w.r0 = (int32_t)((t % tiles_m) * tm);
       w.c0 = (int32_t)((t / tiles_m) * tn);
-      w.count = 1;
+      w.count = tile_extent(tm, tn);
     }
     return w;
   }
@@ -167,16 +169,38 @@ struct SmemR64 {
   double b[2][BKR][TR];  // b[s][kk][col]
 };
 
-__device__ __forceinline__ void tile_r64(const Desc& d, int r0, int c0, const Scalars& s,
-                                         SmemR64& sm) {
+// Rows r0 .. r0 + tm - 1 and columns c0 .. c0 + tn - 1 (tm, tn <= 64) of one
+// instance; FULL: a 64 x 64 tile that the instance fills, 4 x 4 outputs per
+// thread. Otherwise output o of the tile's mb x nb (column-major) goes to
+// thread o mod 256, NJ outputs to a thread: a DFMA takes its 16 clocks per SM
+// whether 1 or 32 of the warp's lanes are active (measured), so padding a
+// ragged tile to 64 x 64 costs in full, while the two extra shared-memory
+// reads per DFMA of this order are hidden behind it.
+template <bool FULL, int NJ>
+__device__ __forceinline__ void tile_r64(const Desc& d, int r0, int c0, int mb, int nb,
+                                         const Scalars& s, SmemR64& sm) {
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
   const int K = s.alpha_zero ? 0 : d.k;
-  double acc[4][4];
+  double acc[FULL ? 4 : 1][4];
+  double lin[FULL ? 1 : NJ];
+  int rc[FULL ? 1 : NJ];  // row and column of each output in the tile, row | column << 16
+  if constexpr (FULL) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+      for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+  } else {
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const int o = tid + kFp64Threads * j;
+      lin[j] = 0.0;
+      const int col = o / mb;
+      rc[j] = col < nb ? (o - col * mb) | col << 16 : 0;  // beyond the tile: computed, not stored
+    }
+  }
+  // outputs of this warp's lanes: a warp past the tile's end issues nothing
+  const int nj = (mb * nb - (tid & ~31) + kFp64Threads - 1) / kFp64Threads;
 
   // global -> register staging: A 64 rows x 16 k, B 16 k x 64 cols
   const int ar = tid & 63, ak = tid >> 6;  // row, k (+4j)
@@ -186,9 +210,9 @@ __device__ __forceinline__ void tile_r64(const Desc& d, int r0, int c0, const Sc
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int r = r0 + ar, kk = k0 + ak + 4 * j;
-      ra[j] = (r < d.m && kk < K) ? __ldg(d.A + r + (int64_t)kk * d.lda) : 0.0;
+      ra[j] = (ar < mb && kk < K) ? __ldg(d.A + r + (int64_t)kk * d.lda) : 0.0;
       const int kb = k0 + bk, c = c0 + bc + 16 * j;
-      rb[j] = (kb < K && c < d.n) ? ld_b(d, kb, c) : 0.0;
+      rb[j] = (kb < K && bc + 16 * j < nb) ? ld_b(d, kb, c) : 0.0;
     }
   };
   auto sstore = [&](int st) {
@@ -208,6 +232,14 @@ __device__ __forceinline__ void tile_r64(const Desc& d, int r0, int c0, const Sc
   for (int k0 = 0; k0 < K; k0 += BKR) {
     const bool more = k0 + BKR < K;
     if (more) gload(k0 + BKR);
+    if constexpr (!FULL) {
+      const int kend = min(BKR, K - k0);
+#pragma unroll 2
+      for (int kk = 0; kk < kend; ++kk)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+          if (j < nj) lin[j] = fma(sm.a[st][kk][rc[j] & 0xFFFF], sm.b[st][kk][rc[j] >> 16], lin[j]);
+    } else
 #pragma unroll
     for (int kk = 0; kk < BKR; ++kk) {
       const double2 a01 = *reinterpret_cast<const double2*>(&sm.a[st][kk][ty * 4]);
@@ -226,6 +258,18 @@ __device__ __forceinline__ void tile_r64(const Desc& d, int r0, int c0, const Sc
     st ^= 1;
   }
 
+  if constexpr (!FULL) {
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const int r = r0 + (rc[j] & 0xFFFF), c = c0 + (rc[j] >> 16);
+      if (tid + kFp64Threads * j >= mb * nb || !keep_out(d, r, c)) continue;
+      double* cp = d.C + r + (int64_t)c * d.ldc;
+      double v = s.alpha_re * lin[j];
+      if (!s.beta_zero) v = fma(s.beta_re, *cp, v);
+      *cp = v;
+    }
+    return;
+  } else
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int c = c0 + tx * 4 + j;
@@ -356,17 +400,34 @@ __device__ __forceinline__ double2 c_epilogue(double2 acc, const double2* cp, co
   return v;
 }
 
-__device__ __forceinline__ void tile_c128(const Desc& d, int r0, int c0, const Scalars& s,
-                                          SmemC128& sm) {
+// As tile_r64: FULL is a whole 32 x 32 tile (2 x 2 outputs per thread), NJ the
+// outputs per thread in linear order otherwise.
+template <bool FULL, int NJ>
+__device__ __forceinline__ void tile_c128(const Desc& d, int r0, int c0, int mb, int nb,
+                                          const Scalars& s, SmemC128& sm) {
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
   const int K = s.alpha_zero ? 0 : d.k;
   const double2* A = reinterpret_cast<const double2*>(d.A);
-  double2 acc[2][2];
+  double2 acc[FULL ? 2 : 1][2];
+  double2 lin[FULL ? 1 : NJ];
+  int rc[FULL ? 1 : NJ];
+  if constexpr (FULL) {
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 2; ++j) acc[i][j] = make_double2(0.0, 0.0);
+      for (int j = 0; j < 2; ++j) acc[i][j] = make_double2(0.0, 0.0);
+  } else {
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const int o = tid + kFp64Threads * j;
+      lin[j] = make_double2(0.0, 0.0);
+      const int col = o / mb;
+      rc[j] = col < nb ? (o - col * mb) | col << 16 : 0;
+    }
+  }
+  // outputs of this warp's lanes: a warp past the tile's end issues nothing
+  const int nj = (mb * nb - (tid & ~31) + kFp64Threads - 1) / kFp64Threads;
 
   const int ar = tid & 31, ak = tid >> 5;  // row, k (+8j)
   const int bk = tid & 15, bc = tid >> 4;  // k, col (+16j)
@@ -376,9 +437,9 @@ __device__ __forceinline__ void tile_c128(const Desc& d, int r0, int c0, const S
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int r = r0 + ar, kk = k0 + ak + 8 * j;
-      ra[j] = (r < d.m && kk < K) ? __ldg(A + r + (int64_t)kk * d.lda) : z;
+      ra[j] = (ar < mb && kk < K) ? __ldg(A + r + (int64_t)kk * d.lda) : z;
       const int kb = k0 + bk, c = c0 + bc + 16 * j;
-      rb[j] = (kb < K && c < d.n) ? ld_bc(d, kb, c) : z;
+      rb[j] = (kb < K && bc + 16 * j < nb) ? ld_bc(d, kb, c) : z;
     }
   };
   auto sstore = [&](int st) {
@@ -397,6 +458,14 @@ __device__ __forceinline__ void tile_c128(const Desc& d, int r0, int c0, const S
   for (int k0 = 0; k0 < K; k0 += BKC) {
     const bool more = k0 + BKC < K;
     if (more) gload(k0 + BKC);
+    if constexpr (!FULL) {
+      const int kend = min(BKC, K - k0);
+#pragma unroll 2
+      for (int kk = 0; kk < kend; ++kk)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+          if (j < nj) cmac(lin[j], sm.a[st][kk][rc[j] & 0xFFFF], sm.b[st][kk][rc[j] >> 16]);
+    } else
 #pragma unroll
     for (int kk = 0; kk < BKC; ++kk) {
       const double2 a0 = sm.a[st][kk][ty * 2], a1 = sm.a[st][kk][ty * 2 + 1];
@@ -411,6 +480,18 @@ __device__ __forceinline__ void tile_c128(const Desc& d, int r0, int c0, const S
     st ^= 1;
   }
   double2* C = reinterpret_cast<double2*>(d.C);
+  if constexpr (!FULL) {
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const int r = r0 + (rc[j] & 0xFFFF), c = c0 + (rc[j] >> 16);
+      if (tid + kFp64Threads * j >= mb * nb || !keep_out(d, r, c)) continue;
+      double2* cp = C + r + (int64_t)c * d.ldc;
+      double2 v = c_epilogue(lin[j], cp, s);
+      if (d.herm && r == c) v.y = 0.0;
+      *cp = v;
+    }
+    return;
+  } else
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     const int c = c0 + tx * 2 + j;
@@ -427,17 +508,16 @@ __device__ __forceinline__ void tile_c128(const Desc& d, int r0, int c0, const S
   }
 }
 
-// ---- small programs: W warps per instance (real), one warp (complex) ----------
-// Thread t (0 <= t < 32 W) of an instance owns outputs o = t + 32 W j
-// (j < MAXOUT) of the m*n outputs in column-major order, i.e. (r, c) =
-// (o mod m, o div m). When m divides 32 the row is the same for every j and
-// the column steps by 32 W / m, so one A load feeds MAXOUT DFMAs; otherwise
-// every output loads its own A element.
+// ---- small programs: a warp per instance --------------------------------------
+// Lane t owns outputs o = t + 32 j (j < MAXOUT) of the m*n outputs in
+// column-major order, i.e. (r, c) = (o mod m, o div m). When m divides 32 the
+// row is the same for every j and the column steps by 32 / m, so one A load
+// feeds MAXOUT DFMAs; otherwise every output loads its own A element.
 
-template <int MAXOUT, int W>
-__device__ __forceinline__ void small_r64(const Desc& d, const Scalars& s, int t) {
-  const int lane = t;  // thread of the instance
-  constexpr int stride = 32 * W;
+template <int MAXOUT>
+__device__ __forceinline__ void small_r64(const Desc& d, const Scalars& s) {
+  const int lane = threadIdx.x & 31;
+  constexpr int stride = 32;
   const int m = d.m, n = d.n, mn = m * n;
   const int K = s.alpha_zero ? 0 : d.k;
   double acc[MAXOUT];
@@ -448,6 +528,7 @@ __device__ __forceinline__ void small_r64(const Desc& d, const Scalars& s, int t
     const double* ap = d.A + r;
     const double* bp = d.B + (int64_t)c0 * d.ldb;
     const int64_t bstep = (int64_t)cstep * d.ldb;
+#pragma unroll 1
     for (int p = 0; p < K; ++p) {
       const double a = __ldg(ap + (int64_t)p * d.lda);
 #pragma unroll
@@ -466,6 +547,7 @@ __device__ __forceinline__ void small_r64(const Desc& d, const Scalars& s, int t
       }
     }
   } else {
+#pragma unroll 1
     for (int p = 0; p < K; ++p) {
 #pragma unroll
       for (int j = 0; j < MAXOUT; ++j) {
@@ -506,6 +588,7 @@ __device__ __forceinline__ void small_c128(const Desc& d, const Scalars& s) {
     const int r = lane % m, c0 = lane / m, cstep = 32 / m;
     const int64_t bstep = (int64_t)cstep * d.ldb;
     const double2* bp = B + (int64_t)c0 * d.ldb;
+#pragma unroll 1
     for (int p = 0; p < K; ++p) {
       const double2 a = __ldg(A + r + (int64_t)p * d.lda);
 #pragma unroll
@@ -524,6 +607,7 @@ __device__ __forceinline__ void small_c128(const Desc& d, const Scalars& s) {
       }
     }
   } else {
+#pragma unroll 1
     for (int p = 0; p < K; ++p) {
 #pragma unroll
       for (int j = 0; j < MAXOUT; ++j) {
@@ -549,9 +633,8 @@ __device__ __forceinline__ void small_c128(const Desc& d, const Scalars& s) {
   }
 }
 
-// Small-program limits (outputs per warp).
-constexpr int kSmallR64Fast = 1024, kSmallR64Gen = 512;   // MAXOUT 32 / 16
-constexpr int kSmallC128Fast = 512, kSmallC128Gen = 256;  // MAXOUT 16 / 8
+// Small-program limits (outputs per warp): MAXOUT 8 real, 4 complex.
+constexpr int kSmallR64 = 256, kSmallC128 = 128;
 
 // ---- the persistent kernel ---------------------------------------------------------
 
@@ -560,41 +643,77 @@ union SmemFp64 {
   SmemC128 c;
 };
 
-template <class Src, class Sched>
-__global__ void __launch_bounds__(kFp64Threads, 1)
+// CTAS: CTAs per SM. Several hide each other's start (work item, first operand
+// loads): two where tiles are ragged (33^3 x 1000: 150 -> 102 us), three where
+// all are small, in the registers that the small tiles leave (32^3 x 20000:
+// 2710, 1540 and 1257 us with one, two and three). Full tiles run 2-5% faster
+// alone (128^3 x 100: 430 -> 411 us).
+template <int CTAS, class Src, class Sched>
+__global__ void __launch_bounds__(kFp64Threads, CTAS)
     fp64_persistent(Src src, Sched sched, int64_t n_items, Scalars s) {
   __shared__ __align__(16) SmemFp64 sm;
   const int warp = threadIdx.x >> 5;
+  if constexpr (CTAS == 3) {  // small tiles only
+    for (int64_t it = blockIdx.x; it < n_items; it += gridDim.x) {
+      const WorkItem w = sched.get(it);
+      const Desc d = src.desc(w.inst);
+      int tm, tn;
+      tile_extent_of(w.count, TR, &tm, &tn);
+      const int mb = min(tm, d.m - w.r0), nb = min(tn, d.n - w.c0);
+      if (mb <= 0 || nb <= 0) continue;
+      if (w.prog == PROG_R64_TILE) {
+        if (mb * nb > 2 * kFp64Threads) tile_r64<false, 4>(d, w.r0, w.c0, mb, nb, s, sm.r);
+        else tile_r64<false, 2>(d, w.r0, w.c0, mb, nb, s, sm.r);
+      } else if (mb * nb > kFp64Threads) {
+        tile_c128<false, 2>(d, w.r0, w.c0, mb, nb, s, sm.c);
+      } else {
+        tile_c128<false, 1>(d, w.r0, w.c0, mb, nb, s, sm.c);
+      }
+    }
+    return;
+  }
   for (int64_t it = blockIdx.x; it < n_items; it += gridDim.x) {
     const WorkItem w = sched.get(it);
     switch (w.prog) {
-      case PROG_R64_TILE:
-        tile_r64(src.desc(w.inst), w.r0, w.c0, s, sm.r);
+      case PROG_R64_TILE: {
+        const Desc d = src.desc(w.inst);
+        int tm, tn;
+        tile_extent_of(w.count, TR, &tm, &tn);
+        const int mb = min(tm, d.m - w.r0), nb = min(tn, d.n - w.c0);
+        if (mb <= 0 || nb <= 0) break;  // (a chain index that names no matrix)
+        const int out = mb * nb;
+        if (out == TR * TR) tile_r64<true, 1>(d, w.r0, w.c0, mb, nb, s, sm.r);
+        else if (out > 4 * kFp64Threads) tile_r64<false, 8>(d, w.r0, w.c0, mb, nb, s, sm.r);
+        else if (out > 2 * kFp64Threads) tile_r64<false, 4>(d, w.r0, w.c0, mb, nb, s, sm.r);
+        else tile_r64<false, 2>(d, w.r0, w.c0, mb, nb, s, sm.r);
         break;
+      }
       case PROG_R64_DMMA:
         tile_r64_dmma(src.desc(w.inst), w.r0, w.c0, s, sm.r);
         break;
-      case PROG_C128_TILE:
-        tile_c128(src.desc(w.inst), w.r0, w.c0, s, sm.c);
-        break;
-      case PROG_R64_SMALL: {
-        const int W = w.r0 > 0 ? w.r0 : 1;  // warps per instance
-        const int slot = warp / W;
-        if (slot < w.count) {
-          const Desc d = src.desc(src.small_inst((int64_t)w.inst + slot));
-          const int t = (warp - slot * W) * 32 + (threadIdx.x & 31);
-          const bool fast = d.m > 0 && (32 % d.m) == 0;
-          // outputs per thread: at most 1024 (fast) or 512 (other shapes) per instance
-          if (W == 1) fast ? small_r64<32, 1>(d, s, t) : small_r64<16, 1>(d, s, t);
-          else fast ? small_r64<4, 8>(d, s, t) : small_r64<2, 8>(d, s, t);
-        }
+      case PROG_C128_TILE: {
+        const Desc d = src.desc(w.inst);
+        int tm, tn;
+        tile_extent_of(w.count, TC, &tm, &tn);
+        const int mb = min(tm, d.m - w.r0), nb = min(tn, d.n - w.c0);
+        if (mb <= 0 || nb <= 0) break;
+        const int out = mb * nb;
+        if (out == TC * TC) tile_c128<true, 1>(d, w.r0, w.c0, mb, nb, s, sm.c);
+        else if (out > 2 * kFp64Threads) tile_c128<false, 4>(d, w.r0, w.c0, mb, nb, s, sm.c);
+        else if (out > kFp64Threads) tile_c128<false, 2>(d, w.r0, w.c0, mb, nb, s, sm.c);
+        else tile_c128<false, 1>(d, w.r0, w.c0, mb, nb, s, sm.c);
         break;
       }
+      case PROG_R64_SMALL:
+        if (warp < w.count) {
+          const Desc d = src.desc(src.small_inst((int64_t)w.inst + warp));
+          small_r64<kSmallR64 / 32>(d, s);
+        }
+        break;
       case PROG_C128_SMALL:
         if (warp < w.count) {
           const Desc d = src.desc(src.small_inst((int64_t)w.inst + warp));
-          if (d.m > 0 && (32 % d.m) == 0) small_c128<16>(d, s);
-          else small_c128<8>(d, s);
+          small_c128<kSmallC128 / 32>(d, s);
         }
         break;
       default:
@@ -618,10 +737,9 @@ void prog_tile(int prog, int* tm, int* tn) {
 
 bool prog_fits(int prog, bg_dtype dt, int64_t m, int64_t n) {
   const int64_t mn = m * n;
-  const bool div32 = m > 0 && (32 % m) == 0;
   switch (prog) {
-    case PROG_R64_SMALL: return dt == BG_R64 && (div32 ? mn <= kSmallR64Fast : mn <= kSmallR64Gen);
-    case PROG_C128_SMALL: return dt == BG_C128 && (div32 ? mn <= kSmallC128Fast : mn <= kSmallC128Gen);
+    case PROG_R64_SMALL: return dt == BG_R64 && mn <= kSmallR64;
+    case PROG_C128_SMALL: return dt == BG_C128 && mn <= kSmallC128;
     case PROG_R64_TILE:
     case PROG_R64_DMMA: return dt == BG_R64;
     case PROG_C128_TILE: return dt == BG_C128;
@@ -629,23 +747,45 @@ bool prog_fits(int prog, bg_dtype dt, int64_t m, int64_t n) {
   }
 }
 
-int default_prog(bg_dtype dt, int64_t m, int64_t n, int64_t k) {
-  (void)k;
-  if (dt == BG_R64) return prog_fits(PROG_R64_SMALL, dt, m, n) ? PROG_R64_SMALL : PROG_R64_TILE;
-  return prog_fits(PROG_C128_SMALL, dt, m, n) ? PROG_C128_SMALL : PROG_C128_TILE;
+bool fp64_tile_ok(bg_dtype dt, int64_t tm, int64_t tn) {
+  const int64_t T = dt == BG_C128 ? TC : TR;
+  if (tm > T || tn > T) return false;
+  return (tm == T && tn == T) || tm * tn <= (dt == BG_C128 ? 4 : 8) * kFp64Threads;
 }
 
-static int g_bps[2] = {0, 0};
+void fp64_tile_split(bg_dtype dt, int64_t m, int64_t n, int64_t k, int64_t batch, int sms, int* tm,
+                     int* tn) {
+  const int64_t T = dt == BG_C128 ? TC : TR;
+  *tm = (int)T;
+  *tn = dt == BG_C128 ? (int)T : (int)T / 2;
+  if (m < 1 || n < 1) return;
+  // time in clocks: the tiles' DFMAs (16 clocks of an SM per warp and k), in
+  // whole rounds over the SMs, plus what starting a tile costs where the two
+  // CTAs of an SM cannot hide it
+  const double dfma = (dt == BG_C128 ? 4.0 : 1.0) * 16.0 * (double)std::max<int64_t>(k, 1);
+  double best = 1e300;
+  const int64_t pm0 = (m + T - 1) / T, pn0 = (n + T - 1) / T;
+  for (int64_t pm = pm0; pm <= pm0 + 3 && pm <= m; ++pm)
+    for (int64_t pn = pn0; pn <= pn0 + 15 && pn <= n; ++pn) {
+      const int64_t a = (m + pm - 1) / pm, b = (n + pn - 1) / pn;
+      if (!fp64_tile_ok(dt, a, b)) continue;
+      // (outputs in linear order measured 10% slower than a full tile)
+      const double rate = a == T && b == T ? 1.0 : 1.12;
+      const int64_t items = batch * ((m + a - 1) / a) * ((n + b - 1) / b);
+      const double rounds = (double)((items + sms - 1) / sms);
+      const double cost = rounds * ((double)((a * b + 31) / 32) * dfma * rate + 1500.0);
+      if (cost < 0.97 * best) {
+        best = cost;
+        *tm = (int)a;
+        *tn = (int)b;
+      }
+    }
+}
 
-int fp64_blocks_per_sm(bg_dtype dt) {
-  int& v = g_bps[dt == BG_C128 ? 1 : 0];
-  if (v == 0) {
-    int b = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &b, fp64_persistent<TableSrc, TableSched>, kFp64Threads, 0);
-    v = (e == cudaSuccess && b > 0) ? b : 1;
-  }
-  return v;
+int default_prog(bg_dtype dt, int64_t m, int64_t n, int64_t batch, int sms) {
+  const int small = dt == BG_R64 ? PROG_R64_SMALL : PROG_C128_SMALL;
+  if (prog_fits(small, dt, m, n) && small_fills(batch, 2 * (int64_t)sms)) return small;
+  return dt == BG_R64 ? PROG_R64_TILE : PROG_C128_TILE;
 }
 
 static int sm_count() {
@@ -655,10 +795,21 @@ static int sm_count() {
   return sms > 0 ? sms : 1;
 }
 
+template <class Src, class Sched>
+static void launch_persistent(int ctas, int grid, cudaStream_t st, const Src& src,
+                              const Sched& sched, int64_t n_items, const Scalars& s) {
+  if (ctas == 1)
+    fp64_persistent<1, Src, Sched><<<grid, kFp64Threads, 0, st>>>(src, sched, n_items, s);
+  else if (ctas == 3)
+    fp64_persistent<3, Src, Sched><<<grid, kFp64Threads, 0, st>>>(src, sched, n_items, s);
+  else
+    fp64_persistent<2, Src, Sched><<<grid, kFp64Threads, 0, st>>>(src, sched, n_items, s);
+}
+
 cudaError_t launch_fp64_fixed(bg_dtype dt, int prog, int64_t m, int64_t n, int64_t k,
                               const Scalars& s, const void* A, int64_t lda, int64_t sA,
                               const void* B, int64_t ldb, int64_t sB, void* C, int64_t ldc,
-                              int64_t sC, int64_t batch, int grid_cap, cudaStream_t st) {
+                              int64_t sC, int64_t batch, cudaStream_t st) {
   FixedSrc src;
   src.A = static_cast<const double*>(A);
   src.B = static_cast<const double*>(B);
@@ -672,30 +823,32 @@ cudaError_t launch_fp64_fixed(bg_dtype dt, int prog, int64_t m, int64_t n, int64
   prog_tile(prog, &sched.tm, &sched.tn);
   sched.batch = batch;
   int64_t n_items;
-  int64_t grid = (int64_t)sm_count() * fp64_blocks_per_sm(dt);
-  if (grid_cap > 0 && grid > grid_cap) grid = grid_cap;
-  sched.g = kSmallPerCta;
+  const int sms = sm_count();
   if (sched.tm == 0) {
-    // the real small program spreads small batches over more CTAs
-    if (prog == PROG_R64_SMALL) sched.g = small_group(batch, grid);
     sched.tiles_m = sched.tiles_n = 1;
-    n_items = (batch + sched.g - 1) / sched.g;
+    n_items = (batch + kSmallPerCta - 1) / kSmallPerCta;
   } else {
+    if (prog != PROG_R64_DMMA)
+      fp64_tile_split(dt, m, n, k, batch, sms, &sched.tm, &sched.tn);
     sched.tiles_m = (m + sched.tm - 1) / sched.tm;
     sched.tiles_n = (n + sched.tn - 1) / sched.tn;
     n_items = batch * sched.tiles_m * sched.tiles_n;
   }
   if (n_items <= 0) return cudaSuccess;
-  if (grid > n_items) grid = n_items;
-  fp64_persistent<FixedSrc, FixedSched><<<(unsigned)grid, kFp64Threads, 0, st>>>(src, sched,
-                                                                                 n_items, s);
+  const int T = dt == BG_C128 ? TC : TR;
+  const int ctas = sched.tm == T && sched.tn == T ? 1
+                   : sched.tm > 0 && sched.tm * sched.tn <= (dt == BG_C128 ? 2 : 4) * kFp64Threads
+                       ? 3
+                       : 2;
+  launch_persistent(ctas, (int)std::min<int64_t>(n_items, (int64_t)sms * ctas), st, src, sched,
+                    n_items, s);
   count_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_fp64_table(bg_dtype dt, const int64_t* d_table, const int32_t* d_order,
                               const WorkItem* d_items, int64_t n_items, const void* A,
-                              const void* B, void* C, const Scalars& s, int grid,
+                              const void* B, void* C, const Scalars& s, int ctas,
                               cudaStream_t st, bool herm) {
   if (n_items <= 0) return cudaSuccess;
   TableSrc src;
@@ -707,9 +860,8 @@ cudaError_t launch_fp64_table(bg_dtype dt, const int64_t* d_table, const int32_t
   src.C = static_cast<double*>(C);
   src.esz = dt == BG_C128 ? 2 : 1;
   TableSched sched{d_items};
-  if (grid <= 0) grid = sm_count() * fp64_blocks_per_sm(dt);
-  if (grid > n_items) grid = (int)n_items;
-  fp64_persistent<TableSrc, TableSched><<<grid, kFp64Threads, 0, st>>>(src, sched, n_items, s);
+  launch_persistent(ctas, (int)std::min<int64_t>(n_items, (int64_t)sm_count() * ctas), st, src,
+                    sched, n_items, s);
   count_launch();
   return cudaGetLastError();
 }
@@ -718,7 +870,7 @@ cudaError_t launch_fp64_chain(bg_dtype dt, const int64_t* d_wn, const int64_t* d
                               const int64_t* d_pool_off, const int64_t* d_pool_n,
                               int32_t pool_count, const int32_t* d_order,
                               const int32_t* d_idx_row, const WorkItem* d_items, int64_t n_items,
-                              const void* U, const void* Cin, void* Cout, int grid,
+                              const void* U, const void* Cin, void* Cout, int ctas,
                               cudaStream_t st) {
   if (n_items <= 0) return cudaSuccess;
   ChainSrc src;
@@ -737,9 +889,8 @@ cudaError_t launch_fp64_chain(bg_dtype dt, const int64_t* d_wn, const int64_t* d
   s.alpha_re = 1.0; s.alpha_im = 0.0; s.beta_re = 0.0; s.beta_im = 0.0;
   s.alpha_zero = 0; s.beta_zero = 1;
   TableSched sched{d_items};
-  if (grid <= 0) grid = sm_count() * fp64_blocks_per_sm(dt);
-  if (grid > n_items) grid = (int)n_items;
-  fp64_persistent<ChainSrc, TableSched><<<grid, kFp64Threads, 0, st>>>(src, sched, n_items, s);
+  launch_persistent(ctas, (int)std::min<int64_t>(n_items, (int64_t)sm_count() * ctas), st, src,
+                    sched, n_items, s);
   count_launch();
   return cudaGetLastError();
 }
