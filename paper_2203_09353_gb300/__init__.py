@@ -124,6 +124,8 @@ def _bind(lib: ctypes.CDLL) -> ctypes.CDLL:
 def load_library(path: str | None = None) -> ctypes.CDLL:
     """Load libbgemm.so (built by ``paper_2203_09353_gb300.build``); raises if it is missing."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             p = path or LIB_PATH
@@ -145,20 +147,25 @@ def _check(status: int) -> None:
 
 
 def _ptr(x) -> int | None:
-    if x is None:
-        return None
-    if isinstance(x, int):
+    if x is None or type(x) is int:
         return x
-    if hasattr(x, "data_ptr"):
-        if hasattr(x, "is_cuda") and not x.is_cuda:
-            raise ValueError("the library takes CUDA device tensors")
-        return x.data_ptr()
-    raise TypeError(f"expected a torch CUDA tensor or an int pointer, got {type(x)}")
+    get = getattr(x, "data_ptr", None)
+    if get is None:
+        if isinstance(x, int):
+            return x
+        raise TypeError(f"expected a torch CUDA tensor or an int pointer, got {type(x)}")
+    if not getattr(x, "is_cuda", True):
+        raise ValueError("the library takes CUDA device tensors")
+    return get()
 
 
 def _stream(stream) -> int | None:
     if stream is None:
         import torch
+        if torch.cuda.is_initialized():
+            # the current stream's handle without the Stream object that
+            # torch.cuda.current_stream() makes (half of a small call's time)
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
@@ -185,12 +192,16 @@ def precision(mode: str = "fp64", slices: int = 0, beta_bits: int = 0) -> Precis
     return Precision(m, int(slices), int(beta_bits), 0)
 
 
+_Pair = ctypes.c_double * 2
+
+
 def _scalar(dt: int, v):
+    if type(v) is float:
+        return _Pair(v, 0.0)
     c = complex(v)
-    arr = (ctypes.c_double * 2)(c.real, c.imag)
     if dt == BG_R64 and c.imag != 0:
         raise ValueError("complex scalar for a real problem")
-    return arr
+    return _Pair(c.real, c.imag)
 
 
 def batched_gemm_fixed(dtype, m, n, k, alpha, A, lda, strideA, B, ldb, strideB, beta, C, ldc,

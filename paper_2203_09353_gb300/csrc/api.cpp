@@ -540,7 +540,7 @@ bg_status time_class_fp64(bg_plan* p, int cls, int prog, cudaStream_t st, double
     for (int r = 0; r < 4; ++r) {
       cudaEventRecord(e0, st);
       cudaError_t e = launch_fp64_table(p->dtype, dt, dord, dit, (int64_t)items.size(), A, B, C,
-                                        s, ctas, st);
+                                        s, ctas, p->grid / 2, st);
       cudaEventRecord(e1, st);
       if (e != cudaSuccess) {
         rs = cuda_fail(e, "autotune launch");
@@ -862,7 +862,7 @@ bg_status batched_gemm_fixed(bg_dtype dtype, int64_t m, int64_t n, int64_t k, co
   if (pr.mode == BG_MODE_FP64) {
     const int prog = default_prog(dtype, m, n, batch, ctx->sms);
     cudaError_t e = launch_fp64_fixed(dtype, prog, m, n, k, sc, A, lda, strideA, B, ldb, strideB,
-                                      C, ldc, strideC, batch, st);
+                                      C, ldc, strideC, batch, ctx->sms, st);
     if (e != cudaSuccess) return cuda_fail(e, "FP64 batched kernel launch");
     return BG_OK;
   }
@@ -993,7 +993,7 @@ static bg_status run_grouped_direct(bg_plan* p, const void* A, const void* B, vo
   }
   if (p->prec.mode == BG_MODE_FP64) {
     cudaError_t e = launch_fp64_table(p->dtype, p->d_table, p->d_order, p->d_items, p->n_items, A,
-                                      B, C, sc, p->ctas, st, (p->flags & BG_PLAN_HERK) != 0);
+                                      B, C, sc, p->ctas, p->grid / 2, st, (p->flags & BG_PLAN_HERK) != 0);
     if (e != cudaSuccess) return cuda_fail(e, "grouped FP64 launch");
     if (ev)
       for (int i = 1; i < 4; ++i) BG_CUDA(cudaEventRecord(ev[i], st), "profiling event record");
@@ -1012,7 +1012,7 @@ static bg_status run_grouped_direct(bg_plan* p, const void* A, const void* B, vo
   if (p->n_items > 0) {
     // classes the autotuner gave to the FP64 path (timed with the GEMM slot)
     cudaError_t e = launch_fp64_table(p->dtype, p->d_table, p->d_order, p->d_items, p->n_items, A,
-                                      B, C, sc, p->ctas, st, (p->flags & BG_PLAN_HERK) != 0);
+                                      B, C, sc, p->ctas, p->grid / 2, st, (p->flags & BG_PLAN_HERK) != 0);
     if (e != cudaSuccess) return cuda_fail(e, "grouped FP64 launch");
     if (ev) BG_CUDA(cudaEventRecord(ev[3], st), "profiling event record");
   }
@@ -1182,7 +1182,7 @@ static bg_status run_chain_direct(bg_plan* p, const void* U, const int32_t* idx,
     if (p->prec.mode == BG_MODE_FP64) {
       cudaError_t e = launch_fp64_chain(p->dtype, p->d_wn, p->d_woff, p->d_pool_off, p->d_pool_n,
                                         p->pool_count, p->d_order,
-                                        row, p->d_items, p->n_items, U, cin, cout, p->ctas, st);
+                                        row, p->d_items, p->n_items, U, cin, cout, p->ctas, p->grid / 2, st);
       if (e != cudaSuccess) return cuda_fail(e, "chain step launch");
     } else {
       s = split_chain_step(p->split, U, row, cin, cout, ctx->d_err, st, &g_last_error);

@@ -81,7 +81,7 @@ bool prog_fits(int prog, bg_dtype dt, int64_t m, int64_t n);
 cudaError_t launch_fp64_fixed(bg_dtype dt, int prog, int64_t m, int64_t n, int64_t k,
                               const Scalars& s, const void* A, int64_t lda, int64_t sA,
                               const void* B, int64_t ldb, int64_t sB, void* C, int64_t ldc,
-                              int64_t sC, int64_t batch, cudaStream_t st);
+                              int64_t sC, int64_t batch, int sms, cudaStream_t st);
 
 // ctas: CTAs per SM: 1 (most work in full tiles), 2, or 3 (no small programs,
 // tiles of at most 1024 real or 512 complex outputs).
@@ -89,14 +89,14 @@ cudaError_t launch_fp64_fixed(bg_dtype dt, int prog, int64_t m, int64_t n, int64
 // triangle stored).
 cudaError_t launch_fp64_table(bg_dtype dt, const int64_t* d_table, const int32_t* d_order,
                               const WorkItem* d_items, int64_t n_items, const void* A,
-                              const void* B, void* C, const Scalars& s, int ctas,
+                              const void* B, void* C, const Scalars& s, int ctas, int sms,
                               cudaStream_t st, bool herm = false);
 
 cudaError_t launch_fp64_chain(bg_dtype dt, const int64_t* d_wn, const int64_t* d_woff,
                               const int64_t* d_pool_off, const int64_t* d_pool_n,
                               int32_t pool_count, const int32_t* d_order,
                               const int32_t* d_idx_row, const WorkItem* d_items, int64_t n_items,
-                              const void* U, const void* Cin, void* Cout, int ctas,
+                              const void* U, const void* Cin, void* Cout, int ctas, int sms,
                               cudaStream_t st);
 
 // ---- split-BF16 path (split.cu) ---------------------------------------------------

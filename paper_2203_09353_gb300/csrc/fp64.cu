@@ -759,6 +759,19 @@ void fp64_tile_split(bg_dtype dt, int64_t m, int64_t n, int64_t k, int64_t batch
   *tm = (int)T;
   *tn = dt == BG_C128 ? (int)T : (int)T / 2;
   if (m < 1 || n < 1) return;
+  // (the search takes a good part of a microsecond: a caller's next call most
+  // often has the same shape)
+  struct Last {
+    int64_t key[6];
+    int tm, tn;
+  };
+  static thread_local Last last = {{-1, 0, 0, 0, 0, 0}, 0, 0};
+  const int64_t key[6] = {(int64_t)dt, m, n, k, batch, sms};
+  if (std::equal(key, key + 6, last.key)) {
+    *tm = last.tm;
+    *tn = last.tn;
+    return;
+  }
   // time in clocks: the tiles' DFMAs (16 clocks of an SM per warp and k), in
   // whole rounds over the SMs, plus what starting a tile costs where the two
   // CTAs of an SM cannot hide it
@@ -780,19 +793,15 @@ void fp64_tile_split(bg_dtype dt, int64_t m, int64_t n, int64_t k, int64_t batch
         *tn = (int)b;
       }
     }
+  std::copy(key, key + 6, last.key);
+  last.tm = *tm;
+  last.tn = *tn;
 }
 
 int default_prog(bg_dtype dt, int64_t m, int64_t n, int64_t batch, int sms) {
   const int small = dt == BG_R64 ? PROG_R64_SMALL : PROG_C128_SMALL;
   if (prog_fits(small, dt, m, n) && small_fills(batch, 2 * (int64_t)sms)) return small;
   return dt == BG_R64 ? PROG_R64_TILE : PROG_C128_TILE;
-}
-
-static int sm_count() {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms > 0 ? sms : 1;
 }
 
 template <class Src, class Sched>
@@ -809,7 +818,7 @@ static void launch_persistent(int ctas, int grid, cudaStream_t st, const Src& sr
 cudaError_t launch_fp64_fixed(bg_dtype dt, int prog, int64_t m, int64_t n, int64_t k,
                               const Scalars& s, const void* A, int64_t lda, int64_t sA,
                               const void* B, int64_t ldb, int64_t sB, void* C, int64_t ldc,
-                              int64_t sC, int64_t batch, cudaStream_t st) {
+                              int64_t sC, int64_t batch, int sms, cudaStream_t st) {
   FixedSrc src;
   src.A = static_cast<const double*>(A);
   src.B = static_cast<const double*>(B);
@@ -823,7 +832,6 @@ cudaError_t launch_fp64_fixed(bg_dtype dt, int prog, int64_t m, int64_t n, int64
   prog_tile(prog, &sched.tm, &sched.tn);
   sched.batch = batch;
   int64_t n_items;
-  const int sms = sm_count();
   if (sched.tm == 0) {
     sched.tiles_m = sched.tiles_n = 1;
     n_items = (batch + kSmallPerCta - 1) / kSmallPerCta;
@@ -848,7 +856,7 @@ cudaError_t launch_fp64_fixed(bg_dtype dt, int prog, int64_t m, int64_t n, int64
 
 cudaError_t launch_fp64_table(bg_dtype dt, const int64_t* d_table, const int32_t* d_order,
                               const WorkItem* d_items, int64_t n_items, const void* A,
-                              const void* B, void* C, const Scalars& s, int ctas,
+                              const void* B, void* C, const Scalars& s, int ctas, int sms,
                               cudaStream_t st, bool herm) {
   if (n_items <= 0) return cudaSuccess;
   TableSrc src;
@@ -860,7 +868,7 @@ cudaError_t launch_fp64_table(bg_dtype dt, const int64_t* d_table, const int32_t
   src.C = static_cast<double*>(C);
   src.esz = dt == BG_C128 ? 2 : 1;
   TableSched sched{d_items};
-  launch_persistent(ctas, (int)std::min<int64_t>(n_items, (int64_t)sm_count() * ctas), st, src,
+  launch_persistent(ctas, (int)std::min<int64_t>(n_items, (int64_t)sms * ctas), st, src,
                     sched, n_items, s);
   count_launch();
   return cudaGetLastError();
@@ -870,7 +878,7 @@ cudaError_t launch_fp64_chain(bg_dtype dt, const int64_t* d_wn, const int64_t* d
                               const int64_t* d_pool_off, const int64_t* d_pool_n,
                               int32_t pool_count, const int32_t* d_order,
                               const int32_t* d_idx_row, const WorkItem* d_items, int64_t n_items,
-                              const void* U, const void* Cin, void* Cout, int ctas,
+                              const void* U, const void* Cin, void* Cout, int ctas, int sms,
                               cudaStream_t st) {
   if (n_items <= 0) return cudaSuccess;
   ChainSrc src;
@@ -889,7 +897,7 @@ cudaError_t launch_fp64_chain(bg_dtype dt, const int64_t* d_wn, const int64_t* d
   s.alpha_re = 1.0; s.alpha_im = 0.0; s.beta_re = 0.0; s.beta_im = 0.0;
   s.alpha_zero = 0; s.beta_zero = 1;
   TableSched sched{d_items};
-  launch_persistent(ctas, (int)std::min<int64_t>(n_items, (int64_t)sm_count() * ctas), st, src,
+  launch_persistent(ctas, (int)std::min<int64_t>(n_items, (int64_t)sms * ctas), st, src,
                     sched, n_items, s);
   count_launch();
   return cudaGetLastError();
