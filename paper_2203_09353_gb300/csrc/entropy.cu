@@ -13,7 +13,7 @@
 // (3 instructions a step at 2 per clock per SM), so most of the bisection
 // runs in FP32 and in pairs of floats; few eigenvalues per SM are bound by
 // the counts' latency and get several lanes each. Measured: 128 matrices of
-// order 256 3.05 -> 1.5 ms, 16 of order 1024 47.8 -> 3.7 ms.
+// order 256 3.05 -> 1.3 ms, 16 of order 1024 47.8 -> 3.7 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -213,19 +213,15 @@ __device__ __forceinline__ int sturm_count3ff(const float4* de, int n, float xh,
   return cnt;
 }
 
-// One narrowing of the bracket [a, b] of eigenvalue k by P lanes, one point
-// each: `below` says whether this lane's point j (at a + w (j + 1) / (P + 1))
-// has at most k eigenvalues below it. Returns how many points, from the
-// first on, do.
+// One narrowing of the bracket [a, b] of eigenvalue k by P >= 2 lanes, one
+// point each: `below` says whether this lane's point j (at a + w (j + 1) /
+// (P + 1)) has at most k eigenvalues below it. Returns how many points, from
+// the first on, do.
 template <int P>
 __device__ __forceinline__ int points_below(bool below) {
-  if constexpr (P == 1) {
-    return below ? 1 : 0;
-  } else {
-    const uint32_t all = __ballot_sync(0xFFFFFFFFu, below);
-    const uint32_t mask = P == 32 ? all : (all >> (threadIdx.x & 31 & ~(P - 1))) & ((1u << (P & 31)) - 1u);
-    return P == 32 && mask == 0xFFFFFFFFu ? 32 : __ffs(~mask) - 1;
-  }
+  const uint32_t all = __ballot_sync(0xFFFFFFFFu, below);
+  const uint32_t mask = P == 32 ? all : (all >> (threadIdx.x & 31 & ~(P - 1))) & ((1u << (P & 31)) - 1u);
+  return P == 32 && mask == 0xFFFFFFFFu ? 32 : __ffs(~mask) - 1;
 }
 
 // Eigenvalues of each walker's tridiagonal matrix (blockIdx.y) by bisection,
@@ -239,9 +235,8 @@ __device__ __forceinline__ int points_below(bool below) {
 // point proving the result; otherwise (a cluster, or a secant that missed)
 // the bisection goes on. That leaves about 5 FP64 counts per eigenvalue of
 // the 35 that bisecting from the FP32 bracket took.
-// P: batches with few eigenvalues per SM give each one several lanes, which
-// cut the bracket into P + 1 parts per count, so that fewer counts follow
-// one another.
+// P: the lanes cut the bracket into P + 1 parts per count, so that fewer counts
+// follow one another.
 // Dynamic shared memory: d and e^2 (2 n doubles), the same as float pairs
 // (n float4).
 constexpr int kBisThreads = 128;
@@ -338,21 +333,16 @@ __global__ void __launch_bounds__(kBisThreads) bisect_kernel(const double* d, co
   }
   a -= delff;
   b += delff;
-  // two points at once: by two lanes, or one after the other
+  // two points at once, by the even and the odd lanes
   auto two = [&](double x0, double x1, SturmValue& v0, SturmValue& v1) {
-    if constexpr (P == 1) {
-      v0 = sturm_count3(sd, se2, n, x0);
-      v1 = sturm_count3(sd, se2, n, x1);
-    } else {
-      const SturmValue v = sturm_count3(sd, se2, n, (j & 1) ? x1 : x0);
-      const int l0 = t & 31 & ~(P - 1);
-      v0.cnt = __shfl_sync(0xFFFFFFFFu, v.cnt, l0);
-      v0.shifts = __shfl_sync(0xFFFFFFFFu, v.shifts, l0);
-      v0.value = __shfl_sync(0xFFFFFFFFu, v.value, l0);
-      v1.cnt = __shfl_sync(0xFFFFFFFFu, v.cnt, l0 + 1);
-      v1.shifts = __shfl_sync(0xFFFFFFFFu, v.shifts, l0 + 1);
-      v1.value = __shfl_sync(0xFFFFFFFFu, v.value, l0 + 1);
-    }
+    const SturmValue v = sturm_count3(sd, se2, n, (j & 1) ? x1 : x0);
+    const int l0 = t & 31 & ~(P - 1);
+    v0.cnt = __shfl_sync(0xFFFFFFFFu, v.cnt, l0);
+    v0.shifts = __shfl_sync(0xFFFFFFFFu, v.shifts, l0);
+    v0.value = __shfl_sync(0xFFFFFFFFu, v.value, l0);
+    v1.cnt = __shfl_sync(0xFFFFFFFFu, v.cnt, l0 + 1);
+    v1.shifts = __shfl_sync(0xFFFFFFFFu, v.shifts, l0 + 1);
+    v1.value = __shfl_sync(0xFFFFFFFFu, v.value, l0 + 1);
   };
   SturmValue va, vb;
   two(a, b, va, vb);
@@ -448,18 +438,28 @@ cudaError_t bisect_launch(const double* d, const double* e, int64_t walkers, int
 
 }  // namespace
 
-// Lanes per eigenvalue: as many as keep the eigenvalues' lanes within 256 per
-// SM (8 warps of dependent FP32 and FP64 chains fill the pipes; more lanes
-// than that cost more counts than the shorter chain saves).
+// Lanes per eigenvalue, by the eigenvalues per SM: more lanes shorten the chain
+// of dependent counts but add counts, so each line lies where the pipes fill.
+// Measured (us, with 1 / 2 / 4 / 8 / 16 / 32 lanes; eigenvalues per SM first):
+//   1.7 (4 of order 64)    211   145  113   99   86   82
+//   6.7 (1 of 1024)       5200  3280 2450 1900 1720 1990
+//   13  (8 of 256)        1310   516  621  351  442  712
+//   27  (32 of 128)        403   268  206  256  381  582
+//   54  (128 of 64)        210   145  150  217  318  573
+//   108 (16 of 1024)      5200  3900 4110 4910 8240
+//   216 (128 of 256)      1610  1280 1490 2050 3770
+//   1700 (4096 of 64)     2025  1300 2300
+// One lane was the fastest nowhere and is not built.
 cudaError_t launch_entropy_bisect(const double* d, const double* e, int64_t walkers, int n,
                                   double* lam, double* entropy, double* eigs, int sms,
                                   cudaStream_t st) {
   if (walkers <= 0) return cudaSuccess;
-  const int64_t lanes = (int64_t)sms * 256 / (walkers * n);
-  cudaError_t err = lanes >= 32  ? bisect_launch<32>(d, e, walkers, n, lam, st)
-                    : lanes >= 8 ? bisect_launch<8>(d, e, walkers, n, lam, st)
-                    : lanes >= 2 ? bisect_launch<2>(d, e, walkers, n, lam, st)
-                                 : bisect_launch<1>(d, e, walkers, n, lam, st);
+  const int64_t per_sm = (walkers * n + sms - 1) / sms;
+  cudaError_t err = per_sm <= 4    ? bisect_launch<32>(d, e, walkers, n, lam, st)
+                    : per_sm <= 10 ? bisect_launch<16>(d, e, walkers, n, lam, st)
+                    : per_sm <= 20 ? bisect_launch<8>(d, e, walkers, n, lam, st)
+                    : per_sm <= 40 ? bisect_launch<4>(d, e, walkers, n, lam, st)
+                                   : bisect_launch<2>(d, e, walkers, n, lam, st);
   if (err != cudaSuccess) return err;
   entropy_sum_kernel<<<(unsigned)walkers, kEntThreads, 0, st>>>(lam, n, entropy, eigs);
   count_launch();
