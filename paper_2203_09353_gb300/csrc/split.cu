@@ -32,25 +32,29 @@
 // real and imaginary parts of a row of A / a column of B.
 //
 // Kernels:
-//  * split_slice_kernel: one CTA per line block (128 rows of A, or BN columns
-//    of B), or per part of one: exponents, digit planes written as
+//  * split_slice_kernel: one CTA per line block (128 rows of A, or a tile's
+//    columns of B), or per part of one: exponents, digit planes written as
 //    pre-swizzled BF16 tiles of 64 k (the exact SWIZZLE_128B K-major
 //    shared-memory image), the s planes of one k-block stored next to each
 //    other, per-line norm exponents. Integer arithmetic, plus exact
 //    conversions of small integers to FP32 and BF16.
 //  * split_gemm_kernel<BN>: persistent, one CTA per SM, warp-specialised.
-//    Output tile 128 x BN with BN = the largest multiple of 16 with
-//    s BN <= 512, so that the s level accumulators (one per t) all live in
-//    TMEM at once. Per k-block, warp 0 copies the s B planes with one 1-D TMA
-//    bulk copy (cp.async.bulk) and streams the s A planes through a ring of
-//    16 KiB slots; warp 1 issues, for each A plane p, one tcgen05.mma over the
-//    N-concatenation of B planes 1..s+1-p, which lands every product of the
-//    plane pair (p, q) in the accumulator of its level p + q -- one A tile
-//    and one B tile read per plane instead of per plane pair. Warps 2-9 drain
-//    each level as soon as its last MMA completes, do the integer
-//    recombination, free TMEM and then convert and store while the next tile
-//    is already being multiplied.
-//    Small instances are packed along the diagonal of a 128 x BN tile.
+//    Output tile 128 x w, w <= BN and s BN <= 512, so that the s level
+//    accumulators (one per t) all live in TMEM at once. Per k-block, the last
+//    warp copies the s B planes with one 1-D TMA bulk copy (cp.async.bulk) and
+//    warp 0 streams the s A planes through a ring of 16 KiB slots; warp 1
+//    issues, for each A plane p, one tcgen05.mma over the N-concatenation of B
+//    planes 1..s+1-p, which lands every product of the plane pair (p, q) in
+//    the accumulator of its level p + q -- one A tile and one B tile read per
+//    plane instead of per plane pair. The warps between drain each level as
+//    soon as its last MMA completes, do the integer recombination, free TMEM
+//    (taking the last plane group's levels as they are, before their sums) and
+//    then convert and store while the next tile is already being multiplied.
+//    It is bound by the MMAs and, for few k-blocks, by the epilogue between
+//    them (152 complex instances of order 256, 9 slices: 59% of the tensor
+//    cycles before, the whole call 940 -> 900 us; 4096 of order 64 1186 ->
+//    1006 us; 32 of order 512 1205 -> 1159 us).
+//    Small instances are packed along the diagonal of a tile.
 #include <algorithm>
 #include <array>
 #include <cmath>
@@ -70,7 +74,7 @@ namespace {
 // ---- slicer ----------------------------------------------------------------------------------
 
 // Tile layout (A and B alike): the tile of plane p (0-based) and k-block kb
-// of a block is tile number tile0 + kb * S + p; tiles are `lines` rows of 128
+// of a block is number kb * S + p from the block's first; tiles are w rows of 128
 // bytes (64 BF16 values of k), chunk c of row r stored at chunk c ^ (r & 7).
 //
 // Work distribution: the (group of 4 lines) x (k-block) items of a block are
@@ -282,11 +286,10 @@ __global__ void __launch_bounds__(kSliceThreads, BETA > 0 ? 6 : 4)
     const bool isA = J.side == 0;
     const bool rows = isA || a.herk;
     const int kv = J.kv;
-    const int lines = isA ? BM : a.bn;
     const int groups = J.nl / 4;  // the job's lines [l0, l0 + nl) in groups of 4
     if (groups <= 0) continue;    // (the planner makes none; same for every thread)
-    const int tile_bytes = lines * kLineBytes;
-    uint8_t* tiles = isA ? a.tilesA : a.tilesB;
+    const int tile_bytes = J.w * kLineBytes;
+    uint8_t* tiles = isA ? a.tilesA + J.tile0 * kATileBytes : a.tilesB + J.tile0 * kBPiece;
     if (t < 128) {
       s_max[t] = 0;
       s_n2[t] = 0;
@@ -325,7 +328,7 @@ __global__ void __launch_bounds__(kSliceThreads, BETA > 0 ? 6 : 4)
           const int l = J.l0 + r;
           double x[8];
           load8(a, rows, src, kb * BK + 8 * cc, kv, x);
-          uint8_t* dst = tiles + (J.tile0 + (int64_t)kb * S) * tile_bytes + l * kLineBytes +
+          uint8_t* dst = tiles + (int64_t)kb * S * tile_bytes + l * kLineBytes +
                          ((cc ^ (l & 7)) << 4);
           cut_item<S, BETA>(x, s_e[l], dc, dst, tile_bytes, cc, &s_n2[l]);
         }
@@ -564,11 +567,11 @@ static int kmma_last_of(int kv) {
 // fewer lines (halving while the count stays a multiple of 4). The slicer
 // reads a job's values twice (line maxima, then digits); smaller jobs keep
 // what all resident CTAs read between the two passes within L2.
-static void split_jobs(std::vector<SliceJob>* jobs, int bn) {
+static void split_jobs(std::vector<SliceJob>* jobs) {
   std::vector<SliceJob> out;
   out.reserve(jobs->size() * 2);
   for (const SliceJob& j : *jobs) {
-    const int lines = j.side == 0 ? BM : bn;
+    const int lines = j.w;
     const int64_t line_bytes = (int64_t)j.nkb * BK * 8;
     int nl = lines;
     while (nl * line_bytes > kSliceJobBytes && nl % 2 == 0 && (nl / 2) % 4 == 0) nl /= 2;
@@ -581,6 +584,21 @@ static void split_jobs(std::vector<SliceJob>* jobs, int bn) {
   }
   jobs->swap(out);
 }
+
+// The column tiles of an instance: cbs of them, tile cb from column
+// start(cb), the widths (multiples of tile_granule) as even as they go.
+struct ColTiles {
+  int64_t cbs, pieces;
+  int gran;
+  ColTiles(int64_t n, int s)
+      : cbs((n + bn_for(s) - 1) / bn_for(s)),
+        pieces((n + tile_granule(s) - 1) / tile_granule(s)),
+        gran(tile_granule(s)) {}
+  int64_t start(int64_t cb) const {
+    return gran * (cb * (pieces / cbs) + std::min(cb, pieces % cbs));
+  }
+  int width(int64_t cb) const { return (int)(start(cb + 1) - start(cb)); }
+};
 
 // Host-side schedule of a (non-chain) split plan: instances, order list,
 // slice jobs, GEMM units and the sizes of the tile and meta stores.
@@ -598,7 +616,7 @@ struct HostTables {
 static void make_tables(const SplitPlan* p, const std::vector<bg_instance>& table,
                         HostTables* out) {
   const bool cplx = p->dt == BG_C128;
-  const int s = p->s, BN = p->bn;
+  const int s = p->s, BN = p->bn, gran = tile_granule(p->s);
   std::vector<SInst> inst(table.size());
   for (size_t i = 0; i < table.size(); ++i) {
     const bg_instance& t = table[i];
@@ -657,11 +675,12 @@ static void make_tables(const SplitPlan* p, const std::vector<bg_instance>& tabl
         const int gc = (int)std::min<size_t>(gmax, ids.size() - s0);
         const int32_t pos = (int32_t)order.size();
         for (int i = 0; i < gc; ++i) order.push_back(ids[s0 + i]);
+        const int w = (int)((gc * n + gran - 1) / gran * gran);
         if (nkb > 0) {
           jobsA.push_back(SliceJob{tileA, blkA, pos, 0, (int16_t)gc, (int16_t)mv, (int16_t)nkb, 0,
-                                   (int32_t)kvv});
+                                   (int32_t)kvv, 0, 0, (int16_t)BM});
           jobsB.push_back(SliceJob{tileB, blkB, pos, 1, (int16_t)gc, (int16_t)n, (int16_t)nkb, 0,
-                                   (int32_t)kvv});
+                                   (int32_t)kvv, 0, 0, (int16_t)w});
         }
         SplitUnit U{};
         U.a_tile0 = tileA;
@@ -674,9 +693,10 @@ static void make_tables(const SplitPlan* p, const std::vector<bg_instance>& tabl
         U.kmma_last = (int16_t)kmma_last_of((int)kvv);
         U.mrow = (int16_t)mv;
         U.ncol = (int16_t)n;
+        U.w = (int16_t)w;
         units.push_back(U);
         tileA += (int64_t)s * nkb;
-        tileB += (int64_t)s * nkb;
+        tileB += (int64_t)s * nkb * (w / 16);
         ++blkA;
         ++blkB;
       }
@@ -684,33 +704,36 @@ static void make_tables(const SplitPlan* p, const std::vector<bg_instance>& tabl
       for (int32_t id : ids) {
         const int32_t pos = (int32_t)order.size();
         order.push_back(id);
-        const int64_t rbs = (mv + BM - 1) / BM, cbs = (n + BN - 1) / BN;
+        const int64_t rbs = (mv + BM - 1) / BM;
+        const ColTiles ct(n, s);
         const int64_t tA0 = tileA, tB0 = tileB;
         const int32_t bA0 = blkA, bB0 = blkB;
         for (int64_t rb = 0; rb < rbs; ++rb) {
           if (nkb > 0)
             jobsA.push_back(SliceJob{tileA, blkA, pos, 0, 1, (int16_t)BM, (int16_t)nkb,
-                                     (int32_t)(rb * BM), (int32_t)kvv});
+                                     (int32_t)(rb * BM), (int32_t)kvv, 0, 0, (int16_t)BM});
           tileA += (int64_t)s * nkb;
           ++blkA;
         }
-        for (int64_t cb = 0; cb < cbs; ++cb) {
+        for (int64_t cb = 0; cb < ct.cbs; ++cb) {
+          const int16_t w = (int16_t)ct.width(cb);
           if (nkb > 0)
-            jobsB.push_back(SliceJob{tileB, blkB, pos, 1, 1, (int16_t)BN, (int16_t)nkb,
-                                     (int32_t)(cb * BN), (int32_t)kvv});
-          tileB += (int64_t)s * nkb;
+            jobsB.push_back(SliceJob{tileB, blkB, pos, 1, 1, w, (int16_t)nkb,
+                                     (int32_t)ct.start(cb), (int32_t)kvv, 0, 0, w});
+          tileB += (int64_t)s * nkb * (w / 16);
           ++blkB;
         }
         // row blocks inner: the units sharing a B block run side by side (L2 reuse)
-        for (int64_t cb = 0; cb < cbs; ++cb)
+        for (int64_t cb = 0; cb < ct.cbs; ++cb)
           for (int64_t rb = 0; rb < rbs; ++rb) {
             // Hermitian update: a tile wholly above the diagonal (its last row,
             // counted in complex rows, before its first column) is not needed
-            if (p->herk && ((std::min<int64_t>(mv, (rb + 1) * BM) - 1) >> (cplx ? 1 : 0)) < cb * BN)
+            if (p->herk && ((std::min<int64_t>(mv, (rb + 1) * BM) - 1) >> (cplx ? 1 : 0)) <
+                               ct.start(cb))
               continue;
             SplitUnit U{};
             U.a_tile0 = tA0 + rb * s * nkb;
-            U.b_tile0 = tB0 + cb * s * nkb;
+            U.b_tile0 = tB0 + s * nkb * (ct.start(cb) / 16);
             U.a_blk = bA0 + (int32_t)rb;
             U.b_blk = bB0 + (int32_t)cb;
             U.pos = pos;
@@ -720,7 +743,8 @@ static void make_tables(const SplitPlan* p, const std::vector<bg_instance>& tabl
             U.mrow = (int16_t)std::min<int64_t>(mv, 32767);
             U.ncol = (int16_t)std::min<int64_t>(n, 32767);
             U.r0 = (int32_t)(rb * BM);
-            U.c0 = (int32_t)(cb * BN);
+            U.c0 = (int32_t)ct.start(cb);
+            U.w = (int16_t)ct.width(cb);
             units.push_back(U);
           }
       }
@@ -739,7 +763,7 @@ static void make_tables(const SplitPlan* p, const std::vector<bg_instance>& tabl
     if (ia < jobsA.size()) jobs.push_back(jobsA[ia++]);
     if (ib < jobsB.size()) jobs.push_back(jobsB[ib++]);
   }
-  split_jobs(&jobs, BN);
+  split_jobs(&jobs);
   out->inst = std::move(inst);
   out->order = std::move(order);
   out->jobs = std::move(jobs);
@@ -772,7 +796,6 @@ static bg_status build_instances(SplitPlan* p, const std::vector<bg_instance>& t
     p->small_ab += (double)x.m * x.k + (double)x.k * x.n;
   }
   p->count = (int64_t)table.size();
-  const size_t btile = (size_t)p->bn * kLineBytes;
   cudaError_t e;
   if ((e = dput(&p->d_jobs, t.jobs, &p->bytes)) != cudaSuccess ||
       (e = dput(&p->d_units, t.units, &p->bytes)) != cudaSuccess ||
@@ -782,7 +805,7 @@ static bg_status build_instances(SplitPlan* p, const std::vector<bg_instance>& t
       (e = dput(&p->d_small_items, t.small_items, &p->bytes)) != cudaSuccess ||
       (e = dalloc(reinterpret_cast<void**>(&p->tilesA), (size_t)tileA * kATileBytes, &p->bytes)) !=
           cudaSuccess ||
-      (e = dalloc(reinterpret_cast<void**>(&p->tilesB), (size_t)tileB * btile, &p->bytes)) !=
+      (e = dalloc(reinterpret_cast<void**>(&p->tilesB), (size_t)tileB * kBPiece, &p->bytes)) !=
           cudaSuccess ||
       (e = dalloc(reinterpret_cast<void**>(&p->metaA), (size_t)std::max(blkA, 1) * kMetaStride * 4,
                   &p->bytes)) != cudaSuccess ||
@@ -795,7 +818,7 @@ static bg_status build_instances(SplitPlan* p, const std::vector<bg_instance>& t
   if ((e = cudaMemset(p->metaA, 0, (size_t)std::max(blkA, 1) * kMetaStride * 4)) != cudaSuccess ||
       (e = cudaMemset(p->metaB, 0, (size_t)std::max(blkB, 1) * kMetaStride * 4)) != cudaSuccess ||
       (e = cudaMemset(p->tilesA, 0, (size_t)tileA * kATileBytes)) != cudaSuccess ||
-      (e = cudaMemset(p->tilesB, 0, (size_t)tileB * btile)) != cudaSuccess)
+      (e = cudaMemset(p->tilesB, 0, (size_t)tileB * kBPiece)) != cudaSuccess)
     return cuda_err(err, e, "split plan workspace clear");
   return BG_OK;
 }
@@ -881,7 +904,6 @@ static cudaError_t launch_slicer(SplitPlan* p, const SliceJob* jobs, int64_t njo
   a.cplx = p->dt == BG_C128;
   a.s = p->s;
   a.beta = p->beta;
-  a.bn = p->bn;
   a.herk = p->herk ? 1 : 0;
   const int grid = (int)std::min<int64_t>(p->grid_slice, njobs);
   // compile-time (slices, digit width) versions for the documented modes
@@ -1044,7 +1066,7 @@ bg_status split_fixed_in_scratch(bg_dtype dt, const bg_precision& pr, int64_t m,
   const size_t o_small = off;  off += up(t.small.size() * sizeof(int32_t) + 1);
   const size_t o_items = off;  off += up(t.small_items.size() * sizeof(SmallItem) + 1);
   const size_t o_ta = off;     off += up((size_t)t.tileA * kATileBytes);
-  const size_t o_tb = off;     off += up((size_t)t.tileB * p.bn * kLineBytes);
+  const size_t o_tb = off;     off += up((size_t)t.tileB * kBPiece);
   if (off > scratch_bytes) {
     char buf[256];
     snprintf(buf, sizeof buf,
@@ -1106,7 +1128,7 @@ bg_status split_chain_create(SplitPlan** out, bg_dtype dt, const bg_precision& p
   }
   p->chain = true;
   const bool cplx = dt == BG_C128;
-  const int s = p->s, BN = p->bn;
+  const int s = p->s;
   // pool entries: A blocks (row blocks), sliced once per chain_step call
   std::vector<SInst> pool(pool_n.size());
   std::vector<int32_t> pool_order(pool_n.size());
@@ -1127,7 +1149,7 @@ bg_status split_chain_create(SplitPlan** out, bg_dtype dt, const bg_precision& p
     for (int64_t rb = 0; rb < (mv + BM - 1) / BM; ++rb) {
       if (nkb > 0)
         jobsA.push_back(SliceJob{tileA, blkA, (int32_t)j, 0, 1, (int16_t)BM, (int16_t)nkb,
-                                 (int32_t)(rb * BM), (int32_t)kvv});
+                                 (int32_t)(rb * BM), (int32_t)kvv, 0, 0, (int16_t)BM});
       tileA += (int64_t)s * nkb;
       ++blkA;
     }
@@ -1147,20 +1169,22 @@ bg_status split_chain_create(SplitPlan** out, bg_dtype dt, const bg_precision& p
     if (n == 0) continue;
     const int64_t mv = cplx ? 2 * n : n, kvv = mv;
     const int nkb = (int)((kvv + BK - 1) / BK);
-    const int64_t rbs = (mv + BM - 1) / BM, cbs = (n + BN - 1) / BN;
+    const int64_t rbs = (mv + BM - 1) / BM;
+    const ColTiles ct(n, s);
     const int64_t tB0 = tileB;
     const int32_t bB0 = blkB;
-    for (int64_t cb = 0; cb < cbs; ++cb) {
-      jobsB.push_back(SliceJob{tileB, blkB, (int32_t)w, 1, 1, (int16_t)BN, (int16_t)nkb,
-                               (int32_t)(cb * BN), (int32_t)kvv});
-      tileB += (int64_t)s * nkb;
+    for (int64_t cb = 0; cb < ct.cbs; ++cb) {
+      const int16_t cw = (int16_t)ct.width(cb);
+      jobsB.push_back(SliceJob{tileB, blkB, (int32_t)w, 1, 1, cw, (int16_t)nkb,
+                               (int32_t)ct.start(cb), (int32_t)kvv, 0, 0, cw});
+      tileB += (int64_t)s * nkb * (cw / 16);
       ++blkB;
     }
-    for (int64_t cb = 0; cb < cbs; ++cb)
+    for (int64_t cb = 0; cb < ct.cbs; ++cb)
       for (int64_t rb = 0; rb < rbs; ++rb) {
         SplitUnit U{};
         U.a_tile0 = rb * s * nkb;  // relative to the pool entry's first tile
-        U.b_tile0 = tB0 + cb * s * nkb;
+        U.b_tile0 = tB0 + s * nkb * (ct.start(cb) / 16);
         U.a_blk = (int32_t)rb;     // relative to the pool entry's first block
         U.b_blk = bB0 + (int32_t)cb;
         U.pos = (int32_t)w;
@@ -1170,15 +1194,16 @@ bg_status split_chain_create(SplitPlan** out, bg_dtype dt, const bg_precision& p
         U.mrow = (int16_t)std::min<int64_t>(mv, 32767);
         U.ncol = (int16_t)std::min<int64_t>(n, 32767);
         U.r0 = (int32_t)(rb * BM);
-        U.c0 = (int32_t)(cb * BN);
+        U.c0 = (int32_t)ct.start(cb);
+        U.w = (int16_t)ct.width(cb);
         units.push_back(U);
       }
   }
   std::stable_sort(units.begin(), units.end(),
                    [](const SplitUnit& a, const SplitUnit& b) { return a.nkb > b.nkb; });
   // pool jobs first, then walker jobs (the chain step slices the two parts separately)
-  split_jobs(&jobsA, BN);
-  split_jobs(&jobsB, BN);
+  split_jobs(&jobsA);
+  split_jobs(&jobsB);
   std::vector<SliceJob> jobs = jobsA;
   jobs.insert(jobs.end(), jobsB.begin(), jobsB.end());
   p->n_jobs = (int64_t)jobs.size();
@@ -1186,7 +1211,6 @@ bg_status split_chain_create(SplitPlan** out, bg_dtype dt, const bg_precision& p
   p->n_units = (int64_t)units.size();
   p->count = (int64_t)wn.size();
   p->n_pool = (int32_t)pool_n.size();
-  const size_t btile = (size_t)BN * kLineBytes;
   cudaError_t e;
   if ((e = dput(&p->d_jobs, jobs, &p->bytes)) != cudaSuccess ||
       (e = dput(&p->d_units, units, &p->bytes)) != cudaSuccess ||
@@ -1198,7 +1222,7 @@ bg_status split_chain_create(SplitPlan** out, bg_dtype dt, const bg_precision& p
       (e = dput(&p->d_pool_blk0, pool_blk0, &p->bytes)) != cudaSuccess ||
       (e = dalloc(reinterpret_cast<void**>(&p->tilesA), (size_t)tileA * kATileBytes, &p->bytes)) !=
           cudaSuccess ||
-      (e = dalloc(reinterpret_cast<void**>(&p->tilesB), (size_t)tileB * btile, &p->bytes)) !=
+      (e = dalloc(reinterpret_cast<void**>(&p->tilesB), (size_t)tileB * kBPiece, &p->bytes)) !=
           cudaSuccess ||
       (e = dalloc(reinterpret_cast<void**>(&p->metaA), (size_t)std::max(blkA, 1) * kMetaStride * 4,
                   &p->bytes)) != cudaSuccess ||
@@ -1211,7 +1235,7 @@ bg_status split_chain_create(SplitPlan** out, bg_dtype dt, const bg_precision& p
   cudaMemset(p->metaA, 0, (size_t)std::max(blkA, 1) * kMetaStride * 4);
   cudaMemset(p->metaB, 0, (size_t)std::max(blkB, 1) * kMetaStride * 4);
   cudaMemset(p->tilesA, 0, (size_t)tileA * kATileBytes);
-  cudaMemset(p->tilesB, 0, (size_t)tileB * btile);
+  cudaMemset(p->tilesB, 0, (size_t)tileB * kBPiece);
   grids(p);
   finish_desc(p);
   *out = p;

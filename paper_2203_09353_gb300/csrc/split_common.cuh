@@ -22,8 +22,8 @@ constexpr int kLineBytes = BK * 2;        // 128 bytes: one row of a tile
 // per plane held a 9-slice k-block about 40% above its MMA time.
 constexpr int kAGroup = 3;
 constexpr int kMaxAGroups = 4;
-// Split GEMM CTA: producer warp, MMA warp, then 4 H epilogue warps.
-__host__ __device__ constexpr int gemm_threads(int h) { return 64 + 128 * h; }
+// Split GEMM CTA: A producer warp, MMA warp, 4 H epilogue warps, B producer warp.
+__host__ __device__ constexpr int gemm_threads(int h) { return 96 + 128 * h; }
 constexpr int kMetaStride = 264;  // int32 per block: e[128], R[128] (then padding)
 constexpr int kTmemCols = 512;
 constexpr int kSliceThreads = 256;
@@ -43,6 +43,17 @@ __host__ __device__ constexpr int bn_for(int s) {
   return s <= 2 ? 128 : s <= 4 ? 64 : s == 5 ? 48 : s == 6 ? 48 : s <= 8 ? 64 : s <= 10 ? 48 : 32;
 }
 __host__ __device__ constexpr bool double_buffered(int s) { return s <= 5; }
+// Epilogue warps per TMEM lane quadrant (split_gemm_kernel's H).
+__host__ __device__ constexpr int epi_groups(int s) { return s == 3 ? 4 : s == 6 || s == 9 ? 3 : 2; }
+// A tile may be narrower than bn_for(s): its width w is a multiple of the
+// columns of one epilogue warp (where those are whole MMA steps of 16), and an
+// instance's n columns are dealt evenly over ceil(n / bn_for(s)) tiles, so that
+// the last one is not mostly padding (n = 64 in tiles of 48: 32 + 32 columns
+// instead of 48 + 48; 256: 256 columns multiplied instead of 288).
+__host__ __device__ constexpr int tile_granule(int s) {
+  return bn_for(s) / epi_groups(s) % 16 == 0 ? bn_for(s) / epi_groups(s) : bn_for(s);
+}
+constexpr int kBPiece = 16 * kLineBytes;  // B tiles are addressed in pieces of 16 lines
 
 struct SInst {
   int64_t a_off, b_off, c_off;  // user element offsets
@@ -52,7 +63,7 @@ struct SInst {
 };
 
 struct SliceJob {
-  int64_t tile0;  // first tile of the block (k-block 0, plane 1)
+  int64_t tile0;  // first tile of the block (k-block 0, plane 1); B: in pieces of 16 lines
   int32_t blk;    // block id = meta index
   int32_t pos;    // first position in the order list
   int16_t side;   // 0: A block (rows), 1: B block (columns)
@@ -63,10 +74,13 @@ struct SliceJob {
   int32_t kv;     // virtual k' of the instances
   int16_t l0;     // first line of the block this job cuts
   int16_t nl;     // lines this job cuts (a multiple of 4)
+  int16_t w;      // lines of the block's tiles (A: 128, B: the tile width)
+  int16_t pad[3];
 };
 
 struct SplitUnit {
-  int64_t a_tile0, b_tile0;  // first tiles (chain mode: a_tile0 is relative to the pool entry)
+  int64_t a_tile0, b_tile0;  // first tiles (chain mode: a_tile0 is relative to the pool entry;
+                             // b_tile0 in pieces of 16 lines)
   int32_t a_blk, b_blk;      // meta blocks (chain mode: a_blk is the row block index)
   int32_t pos;               // order position of the (first) instance
   int16_t g;                 // packed instances (1 = a tile of one instance)
@@ -74,7 +88,7 @@ struct SplitUnit {
   int16_t kmma_last;         // MMA K-steps (16 each) in the last k-block
   int16_t mrow;              // virtual rows per packed instance
   int16_t ncol;              // columns per packed instance
-  int16_t pad;
+  int16_t w;                 // tile width (columns, a multiple of tile_granule)
   int32_t r0, c0;            // tile origin in the instance (virtual rows, columns)
 };
 
@@ -91,7 +105,7 @@ struct SliceArgs {
   uint8_t* tilesB;
   int32_t* metaA;
   int32_t* metaB;
-  int cplx, s, beta, bn;
+  int cplx, s, beta;
   int herk;  // Hermitian update: B lines are rows of A (conjugated), read through the A side
 };
 
@@ -242,6 +256,18 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
 __host__ __device__ constexpr uint32_t make_idesc(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
          ((uint32_t)(M >> 4) << 24);
+}
+
+// True in one lane of the (converged) warp. The compiler keeps what a branch on
+// it uses warp-uniform, in the uniform registers that tcgen05 instructions take.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "elect.sync _|q, 0xFFFFFFFF;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(p));
+  return p != 0;
 }
 
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
@@ -488,9 +514,18 @@ __device__ __forceinline__ double valB(const double* B, const SInst& in, int cpl
 
 // ---- GEMM --------------------------------------------------------------------------------------
 
+// One k-block as the B producer announces it to the MMA issuer (w == 0: no more).
+struct KBlock {
+  int32_t w;     // tile width
+  int16_t nk;    // MMA K-steps
+  int8_t first, last;  // of its pass
+  int32_t unit;
+  int32_t pad;
+};
+
 struct GemmBars {
-  uint64_t b_full[2];
-  uint64_t b_empty[2];
+  uint64_t b_full[2];             // B buffer b holds its planes, kb[b] what to do with them
+  uint64_t b_empty[2];            // the MMAs are done with B buffer b (and kb[b] is read)
   uint64_t a_full[kMaxAGroups];   // A ring group g holds its planes
   uint64_t a_empty[kMaxAGroups];  // the MMAs are done with A ring group g
   uint64_t lvl_full[kMaxSlices];  // entry i: the levels of plane group i are complete
@@ -498,6 +533,7 @@ struct GemmBars {
   uint64_t acc_empty[2];  // double-buffered TMEM: the epilogue has emptied copy b
   uint64_t tmem_free;
   uint64_t mma_done;
+  KBlock kb[2];
   uint32_t tmem_base;
   int abort_flag;
 };

@@ -2,6 +2,8 @@
 // included by the per-type instantiation units.
 #pragma once
 
+#include <type_traits>
+
 #include "split_common.cuh"
 
 namespace bg {
@@ -98,6 +100,22 @@ __device__ __forceinline__ void epi_store8_for(const GemmArgs& g, const long lon
 #undef BG_EPI
 }
 
+// The order in which the A planes of a k-block go through the ring, kAGroup to
+// a group. Plane p's MMAs are (s - p) w columns wide, and each wait and commit
+// at a group's end takes the issuing thread about 100 clocks, which only the
+// MMAs still queued hide: in the mixed order every group ends with its widest
+// (planes 6 3 0, 7 4 1, 8 5 2 of nine: 4920 -> 4770 clocks per k-block of
+// 48 columns, 3800 -> 3380 of 32). The first k-block of a pass starts with plane
+// 0, which initialises every level, and the last one keeps the plain order,
+// in which the levels complete one after the other for the epilogue.
+__host__ __device__ constexpr int ring_plane(bool mixed, int group, int j, int ngroups) {
+  return mixed ? (kAGroup - 1 - j) * ngroups + group : group * kAGroup + j;
+}
+template <int SF>
+__device__ __forceinline__ bool mixed_order(bool first, bool last) {
+  return SF > 0 && SF % kAGroup == 0 && !first && !last;
+}
+
 // SF > 0: the slice count is the compile-time constant SF (the MMA issue loop
 // unrolls completely); SF == 0: any slice count g.s with this tile width.
 // CPLX: complex instances (compile-time, so that each version carries only
@@ -126,7 +144,7 @@ __global__ void __launch_bounds__(gemm_threads(H), 1) split_gemm_kernel(const Ge
   uint8_t* aring = smem + 2 * bplanes_bytes;     // a_groups x kAGroup x 16 KiB
   GemmBars& S = *reinterpret_cast<GemmBars*>(aring + g.a_groups * kAGroup * kATileBytes);
   volatile int* abort_flag = &S.abort_flag;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int NG = g.a_groups;
   const int ngroups = (s + kAGroup - 1) / kAGroup;  // plane groups per k-block
 
@@ -160,154 +178,198 @@ __global__ void __launch_bounds__(gemm_threads(H), 1) split_gemm_kernel(const Ge
   tc_fence_after();
   const uint32_t tmem_base = S.tmem_base;
 
-  if (warp == 0) {
-    // ---------------- producer: one TMA bulk copy of the s B planes per k-block, and
-    // the s A planes of the k-block through the A ring, kAGroup planes per group
+  if (warp == 0 || warp == kEpi + 2) {
+    // ---------------- producers: warp 0 the s A planes of each k-block, through the
+    // ring, kAGroup planes per group; the last warp its s B planes with one TMA bulk
+    // copy into one of two buffers. Two warps, so that B runs up to two k-blocks
+    // ahead: behind A's turn in one warp it arrived late.
     if (lane == 0) {
+      const bool isA = warp == 0;
       uint32_t kbc = 0, gfill = 0;
+      int grp = 0;
+      uint32_t gphase = 1;  // (the first round of the ring waits for nothing)
+      auto wait = [&](uint64_t* bar, uint32_t parity, int64_t u) {
+        if (mbar_wait(bar, parity, abort_flag)) return true;
+        record_error(g.err, BG_ERR_TIMEOUT, ERRLOC_SPLIT_EMPTY_BARRIER, (int)u);
+        *abort_flag = 1;
+        return false;
+      };
       bool ok = true;
+      SplitUnit next{};
+      if (blockIdx.x < g.nunits) next = g.units[blockIdx.x];
       for (int64_t u = blockIdx.x; u < g.nunits && ok; u += gridDim.x) {
-        const SplitUnit U = g.units[u];
+        const SplitUnit U = next;
+        if (u + gridDim.x < g.nunits) next = g.units[u + gridDim.x];
         int64_t at, bt;
         int ablk;
         if (!unit_tiles(g, U, &at, &bt, &ablk)) continue;
         const int npass = unit_passes(g, U);
+        const uint32_t bbytes = (uint32_t)(s * U.w * kLineBytes);
+        const uint8_t* src = isA ? g.tilesA + at * kATileBytes : g.tilesB + bt * kBPiece;
         for (int c = 0; c < npass && ok; ++c) {
           const int kb_lo = c * g.kpass, kb_hi = min((int)U.nkb, kb_lo + g.kpass);
           for (int kb = kb_lo; kb < kb_hi && ok; ++kb, ++kbc) {
-            const int buf = kbc & 1;
-            const uint32_t use = kbc >> 1;
-            if (use > 0 && !mbar_wait(&S.b_empty[buf], (use - 1) & 1, abort_flag)) {
-              record_error(g.err, BG_ERR_TIMEOUT, ERRLOC_SPLIT_EMPTY_BARRIER, (int)u);
-              *abort_flag = 1;
-              ok = false;
-              break;
+            const bool first = kb == kb_lo, last = kb == kb_hi - 1;
+            if (!isA) {
+              const int buf = kbc & 1;
+              if (kbc > 1 && !(ok = wait(&S.b_empty[buf], ((kbc >> 1) - 1) & 1, u))) break;
+              S.kb[buf] = KBlock{U.w, (int16_t)(kb == U.nkb - 1 ? U.kmma_last : 4), first, last,
+                                 (int32_t)u, 0};
+              mbar_arrive_expect_tx(&S.b_full[buf], bbytes);
+              bulk_g2s(bbuf + buf * bplanes_bytes, src + (int64_t)kb * bbytes, bbytes,
+                       &S.b_full[buf]);
+              continue;
             }
-            mbar_arrive_expect_tx(&S.b_full[buf], (uint32_t)bplanes_bytes);
-            bulk_g2s(bbuf + buf * bplanes_bytes, g.tilesB + (bt + (int64_t)kb * s) * BTILE,
-                     (uint32_t)bplanes_bytes, &S.b_full[buf]);
+            const bool mixed = mixed_order<SF>(first, last);
             for (int gi = 0; gi < ngroups; ++gi, ++gfill) {
-              const int grp = gfill % NG;
-              const uint32_t guse = gfill / NG;
-              const int p0 = gi * kAGroup, gs = min(kAGroup, s - p0);
-              if (guse > 0 && !mbar_wait(&S.a_empty[grp], (guse - 1) & 1, abort_flag)) {
-                record_error(g.err, BG_ERR_TIMEOUT, ERRLOC_SPLIT_EMPTY_BARRIER, (int)u);
-                *abort_flag = 1;
-                ok = false;
-                break;
-              }
+              if (!(ok = wait(&S.a_empty[grp], gphase, u))) break;
+              const int gs = min(kAGroup, s - gi * kAGroup);
               mbar_arrive_expect_tx(&S.a_full[grp], (uint32_t)(gs * kATileBytes));
               for (int j = 0; j < gs; ++j)
                 bulk_g2s(aring + (grp * kAGroup + j) * kATileBytes,
-                         g.tilesA + (at + (int64_t)kb * s + p0 + j) * kATileBytes, kATileBytes,
-                         &S.a_full[grp]);
+                         src + ((int64_t)kb * s + ring_plane(mixed, gi, j, ngroups)) * kATileBytes,
+                         kATileBytes, &S.a_full[grp]);
+              if (++grp == NG) {
+                grp = 0;
+                gphase ^= 1;
+              }
             }
           }
         }
       }
+      // B: the end, in the place of one more k-block
+      if (!isA && ok && (kbc <= 1 || wait(&S.b_empty[kbc & 1], ((kbc >> 1) - 1) & 1, g.nunits))) {
+        S.kb[kbc & 1].w = 0;
+        mbar_arrive(&S.b_full[kbc & 1]);
+        ++kbc;
+      }
       // let every copy this thread started land before the CTA can exit
-      for (uint32_t j = kbc > 2 ? kbc - 2 : 0; j < kbc; ++j)
-        mbar_wait_time(&S.b_full[j & 1], (j >> 1) & 1);
+      if (!isA)
+        for (uint32_t j = kbc > 2 ? kbc - 2 : 0; j < kbc; ++j)
+          mbar_wait_time(&S.b_full[j & 1], (j >> 1) & 1);
       for (uint32_t j = gfill > (uint32_t)NG ? gfill - NG : 0; j < gfill; ++j)
         mbar_wait_time(&S.a_full[j % NG], (j / NG) & 1);
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer: one N-concatenated MMA per A plane and K-step
-    if (lane == 0) {
-      uint32_t kbc = 0, passc = 0;
-      int grp = 0;
-      uint32_t gphase = 0;
-      bool ok = true;
-      const uint32_t bbase = smem_u32(bbuf);
-      const uint32_t abase = smem_u32(aring);
-      for (int64_t u = blockIdx.x; u < g.nunits && ok; u += gridDim.x) {
-        const SplitUnit U = g.units[u];
-        int64_t at_, bt_;
-        int ablk_;
-        if (!unit_tiles(g, U, &at_, &bt_, &ablk_)) continue;
-        const int npass = unit_passes(g, U);
-        for (int c = 0; c < npass && ok; ++c, ++passc) {
-          // accumulator copy of this pass (always 0 without double buffering)
-          const uint32_t buf_off = DB ? (passc & 1) * (uint32_t)(s * BN) : 0u;
-          bool free_ok = true;
-          if constexpr (DB) {
-            if (passc >= 2)
-              free_ok = mbar_wait(&S.acc_empty[passc & 1], ((passc >> 1) - 1) & 1, abort_flag);
-          } else {
-            if (passc > 0) free_ok = mbar_wait(&S.tmem_free, (passc - 1) & 1, abort_flag);
-          }
-          if (!free_ok) {
-            record_error(g.err, BG_ERR_TIMEOUT, ERRLOC_SPLIT_ACC_EMPTY, (int)u);
-            *abort_flag = 1;
-            ok = false;
-            break;
-          }
+    // ---------------- MMA issuer: one N-concatenated MMA per A plane and K-step.
+    // All lanes run the loop on warp-uniform values and one elected lane issues.
+    // With a loop in one lane the operands went through vector registers, and
+    // beside the epilogue's warps on the same scheduler an MMA took about 80
+    // clocks to issue (9 slices, tile of 32 columns: 4320 -> 3270 clocks per
+    // k-block; 48 columns: 5030 -> 4610; the MMAs alone 2880 and 4320).
+    uint32_t passc = 0;
+    int grp = 0;
+    uint32_t gphase = 0;
+    const uint32_t bbase = smem_u32(bbuf);
+    const uint32_t abase = smem_u32(aring);
+    auto wait = [&](uint64_t* bar, uint32_t parity, int loc, int u) {
+      if (__all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag))) return true;
+      if (lane == 0) {
+        record_error(g.err, BG_ERR_TIMEOUT, loc, u);
+        *abort_flag = 1;
+      }
+      return false;
+    };
+    // One k-block of a tile of width W (0: the runtime width), planes in the
+    // plain or the mixed order (-1: as `mixed` says).
+    auto kblock = [&](auto width, auto order, int wr, bool mixed, int nk, bool first, bool last,
+                      int unit, uint64_t bdesc, uint32_t dbase) {
+      constexpr int W = decltype(width)::value, kOrder = decltype(order)::value;
+      const int w = W > 0 ? W : wr;
+      const bool mix = kOrder < 0 ? mixed : kOrder == 1;
+#pragma unroll
+      for (int q = 0; q < (SF > 0 ? SF : kMaxSlices); ++q) {
+        if (SF == 0 && q >= s) break;
+        const int j = q % kAGroup;  // plane within its ring group
+        const int p = ring_plane(mix, q / kAGroup, j, SF / kAGroup);
+        if (j == 0) {
+          if (!wait(&S.a_full[grp], gphase, ERRLOC_SPLIT_FULL_BARRIER, unit)) return false;
           tc_fence_after();
-          const int kb_lo = c * g.kpass, kb_hi = min((int)U.nkb, kb_lo + g.kpass);
-          for (int kb = kb_lo; kb < kb_hi && ok; ++kb, ++kbc) {
-            const int buf = kbc & 1;
-            if (!mbar_wait(&S.b_full[buf], (kbc >> 1) & 1, abort_flag)) {
-              record_error(g.err, BG_ERR_TIMEOUT, ERRLOC_SPLIT_FULL_BARRIER, (int)u);
-              *abort_flag = 1;
-              ok = false;
-              break;
-            }
-            const uint64_t bdesc = sw128_desc(bbase + buf * bplanes_bytes);
-            const int nk = (kb == U.nkb - 1) ? U.kmma_last : 4;
-            const bool last_kb = kb == kb_hi - 1;
-            uint32_t acc0 = kb == kb_lo ? 0u : 1u;  // the first MMA of a pass initialises TMEM
+        }
+        const uint64_t adesc = sw128_desc(abase + (grp * kAGroup + j) * kATileBytes);
+        // B planes 1..s-p (levels p+2 .. s+1) as one N range, cut in pieces of <= 256
+        const int ncat = (s - p) * w;
+        const int n1 = ncat > 256 ? ncat - 256 : 0;
+        const uint32_t id0 = make_idesc(BM, ncat > 256 ? 256 : ncat);
+        const uint32_t id1 = make_idesc(BM, n1 > 0 ? n1 : 16);
+        const uint32_t d0 = dbase + p * w;
+        constexpr uint64_t kB256 = (256 * kLineBytes) >> 4;
+        if (elect_one()) {
 #pragma unroll
-            for (int p = 0; p < (SF > 0 ? SF : kMaxSlices); ++p) {
-              if (SF == 0 && p >= s) break;
-              const int j = p % kAGroup;  // plane within its ring group
-              if (j == 0) {
-                if (!mbar_wait(&S.a_full[grp], gphase, abort_flag)) {
-                  record_error(g.err, BG_ERR_TIMEOUT, ERRLOC_SPLIT_FULL_BARRIER, (int)u);
-                  *abort_flag = 1;
-                  ok = false;
-                  break;
-                }
-                tc_fence_after();
-              }
-              const uint64_t adesc = sw128_desc(abase + (grp * kAGroup + j) * kATileBytes);
-              // B planes 1..s-p (levels p+2 .. s+1) as one N range, cut in pieces of <= 256
-              const int ncat = (s - p) * BN;
-              const int n1 = ncat > 256 ? ncat - 256 : 0;
-              const uint32_t id0 = make_idesc(BM, ncat > 256 ? 256 : ncat);
-              const uint32_t id1 = make_idesc(BM, n1 > 0 ? n1 : 16);
-              const uint32_t d0 = tmem_base + buf_off + p * BN;
-              constexpr uint64_t kB256 = (256 * kLineBytes) >> 4;
-#pragma unroll
-              for (int kk = 0; kk < 4; ++kk) {
-                if (kk < nk) {
-                  const uint32_t acc = kk == 0 ? acc0 : 1u;
-                  umma_bf16(d0, adesc + 2 * kk, bdesc + 2 * kk, id0, acc);
-                  if (n1 > 0) umma_bf16(d0 + 256, adesc + 2 * kk, bdesc + kB256 + 2 * kk, id1, acc);
-                }
-              }
-              acc0 = 1u;
-              if (j == kAGroup - 1 || p == s - 1) {
-                // the group's planes are done: release its slots; in the last k-block of
-                // the pass every level up to p is complete
-                umma_commit(&S.a_empty[grp]);
-                if (!DB && last_kb) umma_commit(&S.lvl_full[p / kAGroup]);
-                if (++grp == NG) {
-                  grp = 0;
-                  gphase ^= 1;
-                }
-              }
+          for (int kk = 0; kk < 4; ++kk) {
+            if (kk < nk) {
+              // the first MMA of a pass (plane 0, in the plain order) initialises TMEM
+              const uint32_t acc = kOrder != 1 && q == 0 && kk == 0 ? (mix || !first) : 1u;
+              umma_bf16(d0, adesc + 2 * kk, bdesc + 2 * kk, id0, acc);
+              if (n1 > 0) umma_bf16(d0 + 256, adesc + 2 * kk, bdesc + kB256 + 2 * kk, id1, acc);
             }
-            if (!ok) break;
-            umma_commit(&S.b_empty[buf]);
-            if (DB && last_kb) umma_commit(&S.acc_full[passc & 1]);  // the whole tile is done
+          }
+          if (j == kAGroup - 1 || q == s - 1) {
+            // the group's planes are done: release its slots; in the last k-block of
+            // the pass every level up to p is complete
+            umma_commit(&S.a_empty[grp]);
+            if (!DB && last) umma_commit(&S.lvl_full[q / kAGroup]);
           }
         }
+        if ((j == kAGroup - 1 || q == s - 1) && ++grp == NG) {
+          grp = 0;
+          gphase ^= 1;
+        }
       }
-      // all MMAs issued by this thread are complete once mma_done fires
-      umma_commit(&S.mma_done);
-      mbar_wait_time(&S.mma_done, 0);
+      return true;
+    };
+    for (uint32_t kbc = 0;; ++kbc) {
+      const int buf = kbc & 1;
+      if (!wait(&S.b_full[buf], (kbc >> 1) & 1, ERRLOC_SPLIT_FULL_BARRIER, (int)blockIdx.x)) break;
+      // (the shuffles tell the compiler that the values are warp-uniform)
+      const KBlock* kb = &S.kb[buf];
+      const int w = __shfl_sync(0xFFFFFFFFu, kb->w, 0);
+      const int nk = __shfl_sync(0xFFFFFFFFu, (int)kb->nk, 0);
+      const int ends = __shfl_sync(0xFFFFFFFFu, kb->first | kb->last << 1, 0);
+      const int unit = __shfl_sync(0xFFFFFFFFu, kb->unit, 0);
+      const bool first = ends & 1, last = ends & 2;
+      if (w == 0) break;
+      if (first) {
+        // this pass's accumulators (one copy, or copy passc & 1) are free
+        bool ok = true;
+        if constexpr (DB) {
+          if (passc >= 2)
+            ok = wait(&S.acc_empty[passc & 1], ((passc >> 1) - 1) & 1, ERRLOC_SPLIT_ACC_EMPTY, unit);
+        } else {
+          if (passc > 0) ok = wait(&S.tmem_free, (passc - 1) & 1, ERRLOC_SPLIT_ACC_EMPTY, unit);
+        }
+        if (!ok) break;
+      }
+      const uint32_t dbase = tmem_base + (DB ? (passc & 1) * (uint32_t)(s * BN) : 0u);
+      const uint64_t bdesc = sw128_desc(bbase + buf * bplanes_bytes);
+      const bool mixed = mixed_order<SF>(first, last);
+      using std::integral_constant;
+      const integral_constant<int, 0> plain{};
+      const integral_constant<int, 1> mix{};
+      const integral_constant<int, -1> either{};
+      const integral_constant<int, BN> full{};
+      const integral_constant<int, BN - COLS> narrow{};
+      const integral_constant<int, 0> other{};
+      bool ok;
+      if (SF > 0 && w == BN)
+        ok = mixed ? kblock(full, mix, w, mixed, nk, first, last, unit, bdesc, dbase)
+                   : kblock(full, plain, w, mixed, nk, first, last, unit, bdesc, dbase);
+      else if (SF > 0 && w == BN - COLS)
+        ok = mixed ? kblock(narrow, mix, w, mixed, nk, first, last, unit, bdesc, dbase)
+                   : kblock(narrow, plain, w, mixed, nk, first, last, unit, bdesc, dbase);
+      else
+        ok = kblock(other, either, w, mixed, nk, first, last, unit, bdesc, dbase);
+      if (!ok) break;
+      if (elect_one()) {
+        umma_commit(&S.b_empty[buf]);
+        if (DB && last) umma_commit(&S.acc_full[passc & 1]);  // the whole tile is done
+      }
+      if (last) ++passc;
     }
-  } else {
+    // all MMAs issued by this warp are complete once mma_done fires
+    if (elect_one()) umma_commit(&S.mma_done);
+    mbar_wait_time(&S.mma_done, 0);
+  } else if (warp < kEpi + 2) {
     // ---------------- epilogue: drain levels, recombine, free TMEM, store
     const int quad = warp & 3;
     const int half = (warp - 2) >> 2;  // column group of this warp within its quadrant
@@ -330,8 +392,10 @@ __global__ void __launch_bounds__(gemm_threads(H), 1) split_gemm_kernel(const Ge
       const int32_t* mb = g.metaB + (int64_t)U.b_blk * kMetaStride;
       const int e_i = ma[row];
       // frame: the row's norm exponent plus the largest one of the B block
+      const int w = U.w;
+      const bool mine = col0 < w;  // this warp has columns of the tile
       int rbmax = -126;
-      for (int c = lane; c < BN; c += 32) rbmax = max(rbmax, mb[128 + c]);
+      for (int c = lane; c < w; c += 32) rbmax = max(rbmax, mb[128 + c]);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) rbmax = max(rbmax, __shfl_xor_sync(0xFFFFFFFFu, rbmax, o));
       const int F = ma[128 + row] + rbmax + 1;
@@ -351,7 +415,7 @@ __global__ void __launch_bounds__(gemm_threads(H), 1) split_gemm_kernel(const Ge
         inst_pos = U.pos;
         rvalid = true;
         cmin = 0;
-        cmax = BN;
+        cmax = w;
         coff = U.c0;
       }
       const SInst in = g.inst[g.order[inst_pos]];
@@ -391,7 +455,7 @@ __global__ void __launch_bounds__(gemm_threads(H), 1) split_gemm_kernel(const Ge
           }
           const uint32_t tb = tq + b * (uint32_t)(s * BN);
 #pragma unroll 1
-          for (int j0 = 0; j0 < COLS; j0 += 8) {
+          for (int j0 = mine ? 0 : COLS; j0 < COLS; j0 += 8) {
             long long acc[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) acc[j] = 0;
@@ -402,7 +466,7 @@ __global__ void __launch_bounds__(gemm_threads(H), 1) split_gemm_kernel(const Ge
               uint32_t v[NV][8];
               if constexpr (SF > 0) {
 #pragma unroll
-                for (int lv = 0; lv < SF; ++lv) tmem_ld8(tb + lv * BN + j0, v[lv]);
+                for (int lv = 0; lv < SF; ++lv) tmem_ld8(tb + lv * w + j0, v[lv]);
                 tmem_ld_wait();
               }
 #pragma unroll
@@ -410,7 +474,7 @@ __global__ void __launch_bounds__(gemm_threads(H), 1) split_gemm_kernel(const Ge
                 if (SF == 0 && lv >= s) break;
                 uint32_t(&vl)[8] = v[SF > 0 ? lv : 0];
                 if constexpr (SF == 0) {
-                  tmem_ld8(tb + lv * BN + j0, vl);
+                  tmem_ld8(tb + lv * w + j0, vl);
                   tmem_ld_wait();
                 }
                 int sh = 62 - F - g.beta * lv;
@@ -444,51 +508,104 @@ __global__ void __launch_bounds__(gemm_threads(H), 1) split_gemm_kernel(const Ge
             // levels first combine exactly in 32 bits (|L_t 2^beta + L_t+1| <
             // 2^30 + 2^24), which halves the 64-bit shifts and adds.
             const bool pairs = kMayPair && g.beta <= 6;
-#pragma unroll 1
-            for (int lv = 0; lv < s;) {
-              const int nlv = (pairs && lv + 1 < s) ? 2 : 1;
+            // level t is complete once its plane group (t / kAGroup) is
+            auto level_wait = [&](int lv) {
               bool got = true;
-              // level t is complete once its plane group (t / kAGroup) is
-              if (lane == 0)
-                got = mbar_wait(&S.lvl_full[(lv + nlv - 1) / kAGroup], passc & 1, abort_flag);
+              if (lane == 0) got = mbar_wait(&S.lvl_full[lv / kAGroup], passc & 1, abort_flag);
               got = __shfl_sync(0xFFFFFFFFu, got ? 1 : 0, 0) != 0;
-              if (!got) {
-                if (lane == 0) {
-                  record_error(g.err, BG_ERR_TIMEOUT, ERRLOC_SPLIT_ACC_FULL, (int)u);
-                  *abort_flag = 1;
-                }
-                ok = false;
-                break;
+              if (!got && lane == 0) {
+                record_error(g.err, BG_ERR_TIMEOUT, ERRLOC_SPLIT_ACC_FULL, (int)u);
+                *abort_flag = 1;
               }
               tc_fence_after();
-              const int lvl = lv + nlv - 1;  // the combined value sits at this level's weight
+              return got;
+            };
+            // 8 columns of whole numbers at the weight of level lvl
+            auto add8 = [&](int j0, int lvl, const uint32_t(&v)[8]) {
               int sh = 62 - F - g.beta * lvl;
               sh = max(-63, min(62, sh));
               const int lsh = sh > 0 ? sh : 0, rsh = sh < 0 ? -sh : 0;
               const long long rnd = rsh > 0 ? (1ll << (rsh - 1)) : 0ll;
 #pragma unroll
+              for (int j = 0; j < 8; ++j)
+                acc[j0 + j] += (((long long)(int)v[j] << lsh) + rnd) >> rsh;
+            };
+            auto level_int = [](uint32_t(&v)[8]) -> uint32_t(&)[8] {
+#pragma unroll
+              for (int j = 0; j < 8; ++j) v[j] = (uint32_t)__float2int_rn(__uint_as_float(v[j]));
+              return v;
+            };
+            // The levels of the last plane group are taken as they are and TMEM
+            // given back before their sums: the next tile's MMAs wait for this.
+            const int kLast = SF > 0 && SF % kAGroup == 0 && (!kMayPair || pairs) ? kAGroup : 0;
+#pragma unroll 1
+            for (int lv = 0; lv < s - kLast;) {
+              // (a warp without columns waits for the last level alone)
+              const int nlv = !mine ? s - lv : (pairs && lv + 1 < s - kLast) ? 2 : 1;
+              if (!(ok = level_wait(lv + nlv - 1)) || !mine) break;
+#pragma unroll
               for (int j0 = 0; j0 < COLS; j0 += 8) {
                 uint32_t v0[8], v1[8];
-                tmem_ld8(tq + lv * BN + j0, v0);
-                if (nlv == 2) tmem_ld8(tq + (lv + 1) * BN + j0, v1);
+                tmem_ld8(tq + lv * w + j0, v0);
+                if (nlv == 2) tmem_ld8(tq + (lv + 1) * w + j0, v1);
                 tmem_ld_wait();
+                level_int(v0);
+                if (nlv == 2) {
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  int L = __float2int_rn(__uint_as_float(v0[j]));
-                  if (nlv == 2) L = (L << g.beta) + __float2int_rn(__uint_as_float(v1[j]));
-                  acc[j0 + j] += (((long long)L << lsh) + rnd) >> rsh;
+                  for (int j = 0; j < 8; ++j)
+                    v0[j] = (uint32_t)(((int)v0[j] << g.beta) +
+                                       __float2int_rn(__uint_as_float(v1[j])));
                 }
+                add8(j0, lv + nlv - 1, v0);
               }
               lv += nlv;
             }
+            if constexpr (SF > 0 && SF % kAGroup == 0) {
+              if (ok && kLast > 0) ok = level_wait(s - 1);
+              if (ok && mine && kLast > 0) {
+                uint32_t v[kAGroup][COLS / 8][8];
+#pragma unroll
+                for (int i = 0; i < kAGroup; ++i) {
+#pragma unroll
+                  for (int j0 = 0; j0 < COLS; j0 += 8)
+                    tmem_ld8(tq + (s - kAGroup + i) * w + j0, v[i][j0 / 8]);
+                  if (kMayPair && i == 1) {  // (two levels become one: fewer registers)
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int j = 0; j < COLS; ++j)
+                      v[0][j / 8][j % 8] =
+                          (uint32_t)((__float2int_rn(__uint_as_float(v[0][j / 8][j % 8]))
+                                      << g.beta) +
+                                     __float2int_rn(__uint_as_float(v[1][j / 8][j % 8])));
+                  }
+                }
+                tmem_ld_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&S.tmem_free);
+#pragma unroll
+                for (int j0 = 0; j0 < COLS; j0 += 8) {
+                  const int c8 = j0 / 8;
+                  if (kMayPair) {
+                    add8(j0, s - 2, v[0][c8]);
+                  } else {
+                    add8(j0, s - 3, level_int(v[0][c8]));
+                    add8(j0, s - 2, level_int(v[1][c8]));
+                  }
+                  add8(j0, s - 1, level_int(v[2][c8]));
+                }
+              }
+            }
             if (!ok) break;
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&S.tmem_free);
+            if (kLast == 0 || !mine) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&S.tmem_free);
+            }
             ++passc;
           }
           // ---- exact conversion, alpha/beta, store (TMEM already free: overlaps the next MMAs).
-          for (int j0 = 0; j0 < COLS; j0 += 8) {
+          for (int j0 = mine ? 0 : COLS; j0 < COLS; j0 += 8) {
             epi_store8_for<CPLX, kFastConv>(g, *reinterpret_cast<const long long(*)[8]>(acc), mb, col0 + j0,
                              rvalid, cmin, cmax, coff, cbase, ldcv, Ebase, c == 0, alpha_one, rr, dcol);
             // rotate the next 8 accumulators into place (keeps the loop body small)
@@ -514,15 +631,15 @@ __global__ void __launch_bounds__(gemm_threads(H), 1) split_gemm_kernel(const Ge
 // and the compile-time slice count (3, 6 and 9 have unrolled versions).
 #define BG_DISPATCH_GEMM(s, ...)                                                    \
   switch (s) {                                                                      \
-    case 3: { constexpr int BNV = bn_for(3), SFV = 3, HV = 4; constexpr bool DBV = true; __VA_ARGS__; } \
-    case 6: { constexpr int BNV = bn_for(6), SFV = 6, HV = 3; constexpr bool DBV = false; __VA_ARGS__; } \
-    case 9: { constexpr int BNV = bn_for(9), SFV = 9, HV = 3; constexpr bool DBV = false; __VA_ARGS__; } \
-    case 1: case 2: { constexpr int BNV = 128, SFV = 0, HV = 2; constexpr bool DBV = true; __VA_ARGS__; } \
-    case 4: { constexpr int BNV = 64, SFV = 0, HV = 2; constexpr bool DBV = true; __VA_ARGS__; }   \
-    case 5: { constexpr int BNV = 48, SFV = 0, HV = 2; constexpr bool DBV = true; __VA_ARGS__; }   \
-    case 7: case 8: { constexpr int BNV = 64, SFV = 0, HV = 2; constexpr bool DBV = false; __VA_ARGS__; } \
-    case 10: { constexpr int BNV = 48, SFV = 0, HV = 2; constexpr bool DBV = false; __VA_ARGS__; } \
-    case 11: case 12: { constexpr int BNV = 32, SFV = 0, HV = 2; constexpr bool DBV = false; __VA_ARGS__; } \
+    case 3: { constexpr int BNV = bn_for(3), SFV = 3, HV = epi_groups(3); constexpr bool DBV = true; __VA_ARGS__; } \
+    case 6: { constexpr int BNV = bn_for(6), SFV = 6, HV = epi_groups(6); constexpr bool DBV = false; __VA_ARGS__; } \
+    case 9: { constexpr int BNV = bn_for(9), SFV = 9, HV = epi_groups(9); constexpr bool DBV = false; __VA_ARGS__; } \
+    case 1: case 2: { constexpr int BNV = bn_for(2), SFV = 0, HV = epi_groups(2); constexpr bool DBV = true; __VA_ARGS__; } \
+    case 4: { constexpr int BNV = bn_for(4), SFV = 0, HV = epi_groups(4); constexpr bool DBV = true; __VA_ARGS__; }   \
+    case 5: { constexpr int BNV = bn_for(5), SFV = 0, HV = epi_groups(5); constexpr bool DBV = true; __VA_ARGS__; }   \
+    case 7: case 8: { constexpr int BNV = bn_for(8), SFV = 0, HV = epi_groups(8); constexpr bool DBV = false; __VA_ARGS__; } \
+    case 10: { constexpr int BNV = bn_for(10), SFV = 0, HV = epi_groups(10); constexpr bool DBV = false; __VA_ARGS__; } \
+    case 11: case 12: { constexpr int BNV = bn_for(12), SFV = 0, HV = epi_groups(12); constexpr bool DBV = false; __VA_ARGS__; } \
     default: return cudaErrorInvalidValue;                                          \
   }
 
