@@ -57,6 +57,7 @@
 //    Small instances are packed along the diagonal of a tile.
 #include <algorithm>
 #include <array>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -118,6 +119,7 @@ __device__ __forceinline__ LineSrc line_src(const SliceArgs& a, const SliceJob& 
 
 // The 8 values x[u] = (line, k' = q0 + u) of the block's operand, 0 beyond
 // k' or for a line beyond its instance; rows: the lines are rows of A.
+template <bool CPLX>
 __device__ __forceinline__ void load8(const SliceArgs& a, bool rows, LineSrc src, int q0, int kv,
                                       double (&x)[8]) {
   if (src.off < 0) {
@@ -127,7 +129,7 @@ __device__ __forceinline__ void load8(const SliceArgs& a, bool rows, LineSrc src
   }
   const int64_t ld = src.ldx >> 1;
   if (rows) {
-    if (!a.cplx) {
+    if (!CPLX) {
       const double* p = a.A + src.off + (int64_t)q0 * ld;
       if (q0 + 8 <= kv) {
 #pragma unroll
@@ -200,9 +202,10 @@ __device__ __forceinline__ void merge_max(const double (&x)[8], int cc, unsigned
 // Digit planes of the 8 values of a lane (chunk cc of a line with exponent e),
 // stored at dst (plane p at dst + p tile_bytes); the line's sum of squared
 // absolute digit weights is merged into s_n2.
+// All lanes of the warp take part; `on`: this lane's line and chunk exist.
 template <int S, int BETA>
 __device__ __forceinline__ void cut_item(const double (&x)[8], int e, const DigitCtx& dc,
-                                         uint8_t* dst, int tile_bytes, int cc,
+                                         uint8_t* dst, int tile_bytes, int cc, bool on,
                                          unsigned long long* s_n2_l) {
   float n2f = 0.f;
   if constexpr (BETA > 0) {
@@ -221,10 +224,10 @@ __device__ __forceinline__ void cut_item(const double (&x)[8], int e, const Digi
       n2f = fmaf(al0, al0, n2f);
       n2f = fmaf(al1, al1, n2f);
     }
-    *reinterpret_cast<uint4*>(dst) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
+    if (on) *reinterpret_cast<uint4*>(dst) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
 #pragma unroll
     for (int p = 1; p < S; ++p)
-      *reinterpret_cast<uint4*>(dst + (int64_t)p * tile_bytes) =
+      if (on) *reinterpret_cast<uint4*>(dst + (int64_t)p * tile_bytes) =
           make_uint4(lower_digit_pair<S, BETA>(p, lo[0], hi[0], lo[1], hi[1]),
                      lower_digit_pair<S, BETA>(p, lo[2], hi[2], lo[3], hi[3]),
                      lower_digit_pair<S, BETA>(p, lo[4], hi[4], lo[5], hi[5]),
@@ -243,14 +246,14 @@ __device__ __forceinline__ void cut_item(const double (&x)[8], int e, const Digi
     }
 #pragma unroll
     for (int p = 0; p < S; ++p)
-      *reinterpret_cast<uint4*>(dst + (int64_t)p * tile_bytes) =
+      if (on) *reinterpret_cast<uint4*>(dst + (int64_t)p * tile_bytes) =
           make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
   }
   // 8 values of at most 257.51^2 each, in units of 2^-8: < 2^28 per lane; 8 lanes < 2^31
   uint32_t n2 = __float2uint_ru(n2f * 256.0f * 1.0001f);
 #pragma unroll
   for (int o = 1; o < 8; o <<= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, o);
-  if (cc == 0 && n2) atomicAdd(s_n2_l, (unsigned long long)n2);
+  if (on && cc == 0 && n2) atomicAdd(s_n2_l, (unsigned long long)n2);
 }
 
 // Advances a warp's item (group g of 4 lines, k-block kb) by `step` items in
@@ -263,20 +266,76 @@ __device__ __forceinline__ void next_item(int& g, int& kb, int step, int groups)
   }
 }
 
+// Where element k of complex row er of a stage of E rows lies: rows side by side,
+// as they are loaded, and swizzled by the chunk of 4 so that the lanes of the
+// cut, one chunk each, read distinct banks.
+__device__ __forceinline__ int stage_pos(int k, int er, int E) {
+  const int mask = min(E & -E, 8) - 1;  // (E is a multiple of mask + 1)
+  return k * E + (er ^ (k >> 2 & mask));
+}
+
+// First pass over complex rows: consecutive threads take consecutive rows
+// (contiguous in memory), several k at a time; values go to the stage, the
+// exponents to s_e (`lines` of them per row).
+__device__ __forceinline__ void stage_rows(const SliceArgs& a, const LineSrc* s_src, int lines,
+                                           int E, int KE, int KEp, double2* stage, int* s_e) {
+  constexpr int U = 4;
+  const int t = threadIdx.x, per = kSliceThreads / E, er = t % E, k0 = t / E;
+  if (k0 >= per) return;
+  const LineSrc src = s_src[er * lines];
+  const int64_t ld = src.ldx >> 1;
+  const double2* p = reinterpret_cast<const double2*>(a.A) + src.off;
+  uint32_t mh = 0, ml = 0;
+  for (int k = k0; k < KEp; k += per * U) {
+    double2 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int kk = k + u * per;
+      v[u] = make_double2(0.0, 0.0);
+      if (src.off >= 0 && kk < KE) v[u] = __ldg(p + (int64_t)kk * ld);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int kk = k + u * per;
+      if (kk < KEp) stage[stage_pos(kk, er, E)] = v[u];
+      mh = max(mh, max((uint32_t)__double2hiint(v[u].x) & 0x7FFFFFFFu,
+                       (uint32_t)__double2hiint(v[u].y) & 0x7FFFFFFFu));
+      ml = max(ml, max((uint32_t)__double2loint(v[u].x), (uint32_t)__double2loint(v[u].y)));
+    }
+  }
+  if (mh | ml) {
+    const int e = line_exponent((unsigned long long)mh << 32 | ml);
+    for (int i = 0; i < lines; ++i) atomicMax(&s_e[er * lines + i], e);
+  }
+}
+
 // BETA > 0: compile-time digit width (S * BETA <= 60); BETA == 0: any width a.beta.
-// The compile-time cuts run six CTAs per SM (at most 40 registers a thread):
-// the kernel is bound by memory latency, and 48 warps per SM hide it better
-// than 40 (measured 3.41 -> 3.35 ms for 9 slices on the 20000-instance size
-// mix; seven or eight CTAs, with fewer registers, are slower). The generic cut keeps four,
-// where five would spill.
-template <int S, int BETA>
-__global__ void __launch_bounds__(kSliceThreads, BETA > 0 ? 6 : 4)
+//
+// Complex rows of A are staged: read once, side by side, and kept in shared
+// memory while the line maxima are found; each is cut from there into both its
+// lines. Their values lie a leading dimension apart along k, so that a lane's
+// chunk of k took an L1 access per 32 bytes, in both passes and for both lines:
+// the L1 pipe was 78-91% busy (4096 instances of order 64, 9 slices: slicer
+// 566 -> 404 us, 4.4 TB/s of loads and plane stores; Hermitian updates, 6
+// slices: 246 -> 197 us). Real rows and columns of B, staged the same way, were
+// slower by 0-7%: one line per value leaves too little to save, and the stage
+// costs occupancy.
+//
+// The compile-time cuts of real data run six CTAs per SM (at most 40 registers
+// a thread), bound by memory latency: 48 warps per SM hide it better than 40
+// (3.41 -> 3.35 ms for 9 slices on the 20000-instance size mix; seven or eight
+// CTAs, with fewer registers, are slower). Complex ones run four CTAs (64
+// registers; five, with 48, spill: 32 instances of order 512 1136 against 1167 us,
+// Hermitian updates 545 against 559 us), and so do the generic cuts.
+template <int S, int BETA, bool CPLX>
+__global__ void __launch_bounds__(kSliceThreads, BETA == 0 || CPLX ? 4 : 6)
     split_slice_kernel(const SliceArgs a) {
+  extern __shared__ double2 stage[];
   const DigitCtx dc = digit_ctx<S>(BETA > 0 ? BETA : a.beta);
   __shared__ unsigned long long s_max[128];
   __shared__ unsigned long long s_n2[128];  // sum of alpha^2 in units of 2^-8 (rounded up)
   __shared__ int s_e[128];
-  __shared__ LineSrc s_src[128];            // the job's lines, job-relative
+  __shared__ LineSrc s_src[128];            // the job's lines; all four arrays job-relative
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int cc = lane & 7;        // chunk of 8 k values inside a 64-wide k-block
   const int lsub = lane >> 3;     // line within the warp's group of 4
@@ -285,22 +344,58 @@ __global__ void __launch_bounds__(kSliceThreads, BETA > 0 ? 6 : 4)
     const SliceJob J = a.jobs[jb];
     const bool isA = J.side == 0;
     const bool rows = isA || a.herk;
-    const int kv = J.kv;
-    const int groups = J.nl / 4;  // the job's lines [l0, l0 + nl) in groups of 4
-    if (groups <= 0) continue;    // (the planner makes none; same for every thread)
+    const int kv = J.kv, nl = J.nl;
     const int tile_bytes = J.w * kLineBytes;
     uint8_t* tiles = isA ? a.tilesA + J.tile0 * kATileBytes : a.tilesB + J.tile0 * kBPiece;
-    if (t < 128) {
+    if (t < nl) {
       s_max[t] = 0;
       s_n2[t] = 0;
+      s_e[t] = INT_MIN;
+      s_src[t] = line_src(a, J, isA, J.l0 + t);
     }
-    if (t < J.nl) s_src[t] = line_src(a, J, isA, J.l0 + t);
     __syncthreads();
-    // ---- phase 1: line maxima (exponents). Lines beyond their instance only
-    // meet discarded outputs: a group of 4 such lines is skipped here and in
-    // phase 2 (its tile rows keep whatever finite digits they hold; the
-    // planner zeroes them once).
-    {
+    // this lane's chunk of line r of the job and k-block kb in the tiles
+    auto place = [&](int r, int kb) {
+      const int l = J.l0 + r;
+      return tiles + (int64_t)kb * S * tile_bytes + l * kLineBytes + ((cc ^ (l & 7)) << 4);
+    };
+    // Lines beyond their instance only meet discarded outputs: their tile rows
+    // keep the zeros that the planner wrote once.
+    if (CPLX && J.staged) {
+      const int lines = isA ? 2 : 1;  // per complex row (B = A^H: the real lines alone)
+      const int E = nl / lines;
+      stage_rows(a, s_src, lines, E, kv / 2, J.nkb * (BK / 2), stage, s_e);
+      __syncthreads();
+      if (t < nl && s_e[t] == INT_MIN) s_e[t] = 0;
+      __syncthreads();
+      // digit planes and the norm of the absolute digit weights: 8 lanes to a
+      // complex row and k-block
+      const int first = warp * 4 + lsub;
+      int kb = first / E, er = first - kb * E;
+      while (__any_sync(0xFFFFFFFFu, kb < J.nkb)) {
+        const int r = er * lines, kbc = min(kb, J.nkb - 1);
+        const bool on = kb < J.nkb && s_src[r].off >= 0;
+        if (__any_sync(0xFFFFFFFFu, on)) {
+          double2 z[4];
+#pragma unroll
+          for (int v = 0; v < 4; ++v) z[v] = stage[stage_pos(kbc * (BK / 2) + 4 * cc + v, er, E)];
+          const double x[8] = {z[0].x, -z[0].y, z[1].x, -z[1].y, z[2].x, -z[2].y, z[3].x, -z[3].y};
+          cut_item<S, BETA>(x, s_e[r], dc, place(r, kbc), tile_bytes, cc, on, &s_n2[r]);
+          if (isA) {
+            const double y[8] = {z[0].y, z[0].x, z[1].y, z[1].x, z[2].y, z[2].x, z[3].y, z[3].x};
+            cut_item<S, BETA>(y, s_e[r], dc, place(r + 1, kbc), tile_bytes, cc, on, &s_n2[r + 1]);
+          }
+        }
+        er += kWarps * 4;
+        while (er >= E) {
+          er -= E;
+          ++kb;
+        }
+      }
+    } else {
+      // ---- phase 1: line maxima (exponents); a group of 4 lines beyond their
+      // instance is skipped here and in phase 2
+      const int groups = nl / 4;
       int g = 0, kb = 0;
       next_item(g, kb, warp, groups);
       while (kb < J.nkb) {
@@ -308,37 +403,32 @@ __global__ void __launch_bounds__(kSliceThreads, BETA > 0 ? 6 : 4)
         const LineSrc src = s_src[r];
         if (__any_sync(0xFFFFFFFFu, src.off >= 0)) {
           double x[8];
-          load8(a, rows, src, kb * BK + 8 * cc, kv, x);
-          merge_max(x, cc, &s_max[J.l0 + r]);
+          load8<CPLX>(a, rows, src, kb * BK + 8 * cc, kv, x);
+          merge_max(x, cc, &s_max[r]);
         }
         next_item(g, kb, kWarps, groups);
       }
-    }
-    __syncthreads();
-    if (t < 128) s_e[t] = line_exponent(s_max[t]);
-    __syncthreads();
-    // ---- phase 2: digit planes and the norm of the absolute digit weights
-    {
-      int g = 0, kb = 0;
+      __syncthreads();
+      if (t < nl) s_e[t] = line_exponent(s_max[t]);
+      __syncthreads();
+      // ---- phase 2: digit planes and the norm of the absolute digit weights
+      g = kb = 0;
       next_item(g, kb, warp, groups);
       while (kb < J.nkb) {
         const int r = g * 4 + lsub;
         const LineSrc src = s_src[r];
         if (__any_sync(0xFFFFFFFFu, src.off >= 0)) {
-          const int l = J.l0 + r;
           double x[8];
-          load8(a, rows, src, kb * BK + 8 * cc, kv, x);
-          uint8_t* dst = tiles + (int64_t)kb * S * tile_bytes + l * kLineBytes +
-                         ((cc ^ (l & 7)) << 4);
-          cut_item<S, BETA>(x, s_e[l], dc, dst, tile_bytes, cc, &s_n2[l]);
+          load8<CPLX>(a, rows, src, kb * BK + 8 * cc, kv, x);
+          cut_item<S, BETA>(x, s_e[r], dc, place(r, kb), tile_bytes, cc, true, &s_n2[r]);
         }
         next_item(g, kb, kWarps, groups);
       }
     }
     __syncthreads();
     // ---- phase 3: meta of the job's lines (exponent, norm exponent)
-    int32_t* meta = (isA ? a.metaA : a.metaB) + (int64_t)J.blk * kMetaStride;
-    if (t >= J.l0 && t < J.l0 + J.nl) {
+    int32_t* meta = (isA ? a.metaA : a.metaB) + (int64_t)J.blk * kMetaStride + J.l0;
+    if (t < nl) {
       meta[t] = s_e[t];
       meta[128 + t] = norm_exponent((float)s_n2[t] * (1.0f / 256.0f));
     }
@@ -474,6 +564,7 @@ struct SplitPlan {
   int32_t* metaB = nullptr;
   int64_t bytes = 0;
   int grid_slice = 0, grid_gemm = 0, grid_small = 0;
+  int slice_stage = 0;     // dynamic shared memory of the slicer
   std::vector<int64_t> key;  // fixed-size plan cache key
   std::string desc;
 };
@@ -563,26 +654,36 @@ static int kmma_last_of(int kv) {
   return (rem + 15) / 16;
 }
 
-// Cuts a block job whose FP64 values exceed kSliceJobBytes into jobs of
-// fewer lines (halving while the count stays a multiple of 4). The slicer
-// reads a job's values twice (line maxima, then digits); smaller jobs keep
-// what all resident CTAs read between the two passes within L2.
-static void split_jobs(std::vector<SliceJob>* jobs) {
+// Cuts block jobs into jobs of fewer lines (halving while the count stays a
+// multiple of 4): complex rows to what fits the slicer's shared-memory stage,
+// the rest to kSliceJobBytes. Returns the stage that the longest rows need.
+static int split_jobs(std::vector<SliceJob>* jobs, bool cplx, bool herk) {
   std::vector<SliceJob> out;
   out.reserve(jobs->size() * 2);
+  int64_t stage = 0;
   for (const SliceJob& j : *jobs) {
-    const int lines = j.w;
     const int64_t line_bytes = (int64_t)j.nkb * BK * 8;
-    int nl = lines;
-    while (nl * line_bytes > kSliceJobBytes && nl % 2 == 0 && (nl / 2) % 4 == 0) nl /= 2;
-    for (int l0 = 0; l0 < lines; l0 += nl) {
+    auto lines = [&](int64_t per_line, int64_t bytes) {
+      int nl = j.w;
+      while (nl * per_line > bytes && nl % 2 == 0 && (nl / 2) % 4 == 0) nl /= 2;
+      return nl;
+    };
+    // (a complex value of A serves two values of each of two lines)
+    const int64_t staged_line = j.side == 0 ? line_bytes / 2 : line_bytes;
+    int nl = lines(staged_line, kSliceStage);
+    const bool staged = cplx && (j.side == 0 || herk) && nl * staged_line <= kSliceStageMax;
+    if (staged) stage = std::max({stage, nl * staged_line, kSliceStage});
+    else nl = lines(line_bytes, kSliceJobBytes);
+    for (int l0 = 0; l0 < j.w; l0 += nl) {
       SliceJob sj = j;
       sj.l0 = (int16_t)l0;
       sj.nl = (int16_t)nl;
+      sj.staged = staged;
       out.push_back(sj);
     }
   }
   jobs->swap(out);
+  return (int)stage;
 }
 
 // The column tiles of an instance: cbs of them, tile cb from column
@@ -611,6 +712,7 @@ struct HostTables {
   std::vector<SmallItem> small_items;
   int64_t tileA = 0, tileB = 0, n_jobs_A = 0;
   int32_t blkA = 0, blkB = 0;
+  int stage = 0;
 };
 
 static void make_tables(const SplitPlan* p, const std::vector<bg_instance>& table,
@@ -763,7 +865,7 @@ static void make_tables(const SplitPlan* p, const std::vector<bg_instance>& tabl
     if (ia < jobsA.size()) jobs.push_back(jobsA[ia++]);
     if (ib < jobsB.size()) jobs.push_back(jobsB[ib++]);
   }
-  split_jobs(&jobs);
+  out->stage = split_jobs(&jobs, cplx, p->herk);
   out->inst = std::move(inst);
   out->order = std::move(order);
   out->jobs = std::move(jobs);
@@ -785,6 +887,7 @@ static bg_status build_instances(SplitPlan* p, const std::vector<bg_instance>& t
   make_tables(p, table, &t);
   const int64_t tileA = t.tileA, tileB = t.tileB;
   const int32_t blkA = t.blkA, blkB = t.blkB;
+  p->slice_stage = t.stage;
   p->n_jobs = (int64_t)t.jobs.size();
   p->n_jobs_A = t.n_jobs_A;
   p->n_units = (int64_t)t.units.size();
@@ -846,12 +949,36 @@ static cudaError_t set_gemm_attr(bg_dtype dt, int s) {
   return e;
 }
 
+// Runs f on the plan's slicer kernel: compile-time (slices, digit width)
+// versions for the documented modes.
+template <bool CPLX, class F>
+static cudaError_t with_slicer_of(const SplitPlan* p, const F& f) {
+  if (p->s == 3 && p->beta == 7) return f(split_slice_kernel<3, 7, CPLX>);
+  if (p->s == 6 && p->beta == 7) return f(split_slice_kernel<6, 7, CPLX>);
+  if (p->s == 9 && p->beta == 6) return f(split_slice_kernel<9, 6, CPLX>);
+  BG_DISPATCH_SLICES(p->s, { return f(split_slice_kernel<S, 0, CPLX>); });
+}
+template <class F>
+static cudaError_t with_slicer(const SplitPlan* p, const F& f) {
+  return p->dt == BG_C128 ? with_slicer_of<true>(p, f) : with_slicer_of<false>(p, f);
+}
+
+// CTAs of the slicer per SM, its shared-memory limit set on the way.
+static int slicer_ctas(const SplitPlan* p) {
+  int bps = 0;
+  with_slicer(p, [&](auto kernel) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)kSliceStageMax);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, kSliceThreads,
+                                                         p->slice_stage);
+  });
+  return std::max(bps, 1);
+}
+
 static void grids(SplitPlan* p) {
   set_gemm_attr(p->dt, p->s);
   p->grid_gemm = (int)std::max<int64_t>(1, std::min<int64_t>(p->sms, p->n_units));
-  int bps = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, split_slice_kernel<9, 6>, kSliceThreads, 0);
-  if (bps < 1) bps = 1;
+  const int bps = slicer_ctas(p);
   p->grid_slice = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)p->sms * bps, p->n_jobs));
   if (p->n_small_items > 0)
     p->grid_small = (int)std::max<int64_t>(1, std::min<int64_t>(p->sms, p->n_small_items));
@@ -883,10 +1010,11 @@ bg_status split_plan_create(SplitPlan** out, bg_dtype dt, const bg_precision& pr
   return BG_OK;
 }
 
+// columns: the jobs are all columns of B, which complex data reads like real.
 static cudaError_t launch_slicer(SplitPlan* p, const SliceJob* jobs, int64_t njobs,
                                  const SInst* instA, const SInst* instB, const int32_t* orderA,
                                  const int32_t* orderB, const void* A, const void* B,
-                                 cudaStream_t st) {
+                                 bool columns, cudaStream_t st) {
   if (njobs <= 0) return cudaSuccess;
   SliceArgs a;
   a.jobs = jobs;
@@ -905,23 +1033,13 @@ static cudaError_t launch_slicer(SplitPlan* p, const SliceJob* jobs, int64_t njo
   a.s = p->s;
   a.beta = p->beta;
   a.herk = p->herk ? 1 : 0;
-  const int grid = (int)std::min<int64_t>(p->grid_slice, njobs);
-  // compile-time (slices, digit width) versions for the documented modes
-  if (p->s == 3 && p->beta == 7) {
-    split_slice_kernel<3, 7><<<grid, kSliceThreads, 0, st>>>(a);
-  } else if (p->s == 6 && p->beta == 7) {
-    split_slice_kernel<6, 7><<<grid, kSliceThreads, 0, st>>>(a);
-  } else if (p->s == 9 && p->beta == 6) {
-    split_slice_kernel<9, 6><<<grid, kSliceThreads, 0, st>>>(a);
-  } else {
-    BG_DISPATCH_SLICES(p->s, {
-      split_slice_kernel<S, 0><<<grid, kSliceThreads, 0, st>>>(a);
-      count_launch();
-      return cudaGetLastError();
-    });
-  }
-  count_launch();
-  return cudaGetLastError();
+  const int grid = (int)std::min<int64_t>(columns ? 6ll * p->sms : p->grid_slice, njobs);
+  auto launch = [&](auto kernel) {
+    kernel<<<grid, kSliceThreads, columns ? 0 : p->slice_stage, st>>>(a);
+    count_launch();
+    return cudaGetLastError();
+  };
+  return columns ? with_slicer_of<false>(p, launch) : with_slicer(p, launch);
 }
 
 // The small-instance kernel reads A and B itself (no slicer pass).
@@ -981,7 +1099,7 @@ bg_status split_plan_run(SplitPlan* p, const void* A, const void* B, void* C, co
   cudaError_t e;
   if (!s.alpha_zero) {
     e = launch_slicer(p, p->d_jobs, p->n_jobs, p->d_inst, p->d_inst, p->d_order, p->d_order, A, B,
-                      st);
+                      false, st);
     if (e != cudaSuccess) return cuda_err(err, e, "split slicer launch");
   }
   if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return cuda_err(err, e, "event");
@@ -1086,6 +1204,7 @@ bg_status split_fixed_in_scratch(bg_dtype dt, const bg_precision& pr, int64_t m,
   p.d_small_items = reinterpret_cast<SmallItem*>(base + o_items);
   p.tilesA = base + o_ta;
   p.tilesB = base + o_tb;
+  p.slice_stage = t.stage;
   p.n_jobs = (int64_t)t.jobs.size();
   p.n_jobs_A = t.n_jobs_A;
   p.n_units = (int64_t)t.units.size();
@@ -1202,8 +1321,7 @@ bg_status split_chain_create(SplitPlan** out, bg_dtype dt, const bg_precision& p
   std::stable_sort(units.begin(), units.end(),
                    [](const SplitUnit& a, const SplitUnit& b) { return a.nkb > b.nkb; });
   // pool jobs first, then walker jobs (the chain step slices the two parts separately)
-  split_jobs(&jobsA);
-  split_jobs(&jobsB);
+  p->slice_stage = std::max(split_jobs(&jobsA, cplx, false), split_jobs(&jobsB, cplx, false));
   std::vector<SliceJob> jobs = jobsA;
   jobs.insert(jobs.end(), jobsB.begin(), jobsB.end());
   p->n_jobs = (int64_t)jobs.size();
@@ -1246,7 +1364,7 @@ bg_status split_chain_prepare_pool(SplitPlan* p, const void* U, int* d_err, cuda
                                    std::string* err) {
   (void)d_err;
   cudaError_t e = launch_slicer(p, p->d_jobs, p->n_jobs_A, p->d_pool, p->d_inst, p->d_pool_order,
-                                p->d_order, U, nullptr, st);
+                                p->d_order, U, nullptr, false, st);
   if (e != cudaSuccess) return cuda_err(err, e, "split pool slicer launch");
   return BG_OK;
 }
@@ -1255,7 +1373,8 @@ bg_status split_chain_step(SplitPlan* p, const void* U, const int32_t* idx_row, 
                            void* Cout, int* d_err, cudaStream_t st, std::string* err) {
   (void)U;
   cudaError_t e = launch_slicer(p, p->d_jobs + p->n_jobs_A, p->n_jobs - p->n_jobs_A, p->d_pool,
-                                p->d_inst, p->d_pool_order, p->d_order, nullptr, Cin, st);
+                                p->d_inst, p->d_pool_order, p->d_order, nullptr, Cin, true,
+                                st);
   if (e != cudaSuccess) return cuda_err(err, e, "split state slicer launch");
   Scalars sc;
   sc.alpha_re = 1.0;

@@ -27,8 +27,11 @@ __host__ __device__ constexpr int gemm_threads(int h) { return 96 + 128 * h; }
 constexpr int kMetaStride = 264;  // int32 per block: e[128], R[128] (then padding)
 constexpr int kTmemCols = 512;
 constexpr int kSliceThreads = 256;
-// Largest FP64 footprint of one slicer job (see split_jobs).
-constexpr int64_t kSliceJobBytes = 65536;
+// A slicer job of complex rows holds its values in shared memory between its two
+// passes (see split_jobs): kSliceStage bytes, or up to kSliceStageMax where the
+// shortest job of long rows needs it. Others read the values twice: at most
+// kSliceJobBytes of them, so that what all CTAs hold between the passes stays in L2.
+constexpr int64_t kSliceStage = 32768, kSliceStageMax = 65536, kSliceJobBytes = 65536;
 constexpr int kMaxDynSmem = 232448;
 constexpr unsigned long long kWaitNs = 2000000000ull;  // 2 s bound on any single wait
 
@@ -75,7 +78,8 @@ struct SliceJob {
   int16_t l0;     // first line of the block this job cuts
   int16_t nl;     // lines this job cuts (a multiple of 4)
   int16_t w;      // lines of the block's tiles (A: 128, B: the tile width)
-  int16_t pad[3];
+  int16_t staged;  // the job's values fit the shared-memory stage
+  int16_t pad[2];
 };
 
 struct SplitUnit {
