@@ -78,10 +78,9 @@ namespace {
 // of a block is number kb * S + p from the block's first; tiles are w rows of 128
 // bytes (64 BF16 values of k), chunk c of row r stored at chunk c ^ (r & 7).
 //
-// Work distribution: the (group of 4 lines) x (k-block) items of a block are
-// dealt to the CTA's warps; a warp covers 4 lines x 8 chunks of 8 k values,
-// so each plane store writes 4 whole 128-byte rows (512 contiguous bytes)
-// and every lane keeps 8 values in flight. Line maxima and norm sums meet in
+// Work distribution: items of 4 lines x 8 chunks of 8 k values (or 8 x 4) are
+// dealt to the CTA's warps, a chunk to a lane, so that each plane store writes
+// whole or half 128-byte rows and every lane keeps 8 values in flight. Line maxima and norm sums meet in
 // shared memory through integer atomics (max, and sums of fixed-point
 // squares), so the result does not depend on the order of the items.
 
@@ -176,14 +175,15 @@ __device__ __forceinline__ void load8(const SliceArgs& a, bool rows, LineSrc src
   }
 }
 
-// Line maximum of the 8 values of a lane, merged over the 8 lanes of the line
+// Line maximum of the 8 values of a lane, merged over the W lanes of the line
 // and into s_max. Only line_exponent of the largest |x| is used, and it sees
 // the same value in the pair of separate maxima of the 32-bit halves (sign
 // cleared): the exponent field sits in the high half, and where every
 // exponent is zero, the largest high half, or when those are all zero the
 // largest low half, holds the highest fraction bit. Merging such pairs as
 // 64-bit values keeps this.
-__device__ __forceinline__ void merge_max(const double (&x)[8], int cc, unsigned long long* s_max_l) {
+template <int W>
+__device__ __forceinline__ void merge_max(const double (&x)[8], unsigned long long* s_max_l) {
   uint32_t mh = 0, ml = 0;
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
@@ -191,21 +191,21 @@ __device__ __forceinline__ void merge_max(const double (&x)[8], int cc, unsigned
     ml = max(ml, (uint32_t)__double2loint(x[u]));
   }
 #pragma unroll
-  for (int o = 1; o < 8; o <<= 1) {
+  for (int o = 1; o < W; o <<= 1) {
     mh = max(mh, __shfl_xor_sync(0xFFFFFFFFu, mh, o));
     ml = max(ml, __shfl_xor_sync(0xFFFFFFFFu, ml, o));
   }
   const unsigned long long mx = (unsigned long long)mh << 32 | ml;
-  if (cc == 0 && mx) atomicMax(s_max_l, mx);
+  if (threadIdx.x % W == 0 && mx) atomicMax(s_max_l, mx);
 }
 
 // Digit planes of the 8 values of a lane (chunk cc of a line with exponent e),
 // stored at dst (plane p at dst + p tile_bytes); the line's sum of squared
 // absolute digit weights is merged into s_n2.
 // All lanes of the warp take part; `on`: this lane's line and chunk exist.
-template <int S, int BETA>
+template <int S, int BETA, int W>
 __device__ __forceinline__ void cut_item(const double (&x)[8], int e, const DigitCtx& dc,
-                                         uint8_t* dst, int tile_bytes, int cc, bool on,
+                                         uint8_t* dst, int tile_bytes, bool on,
                                          unsigned long long* s_n2_l) {
   float n2f = 0.f;
   if constexpr (BETA > 0) {
@@ -252,11 +252,11 @@ __device__ __forceinline__ void cut_item(const double (&x)[8], int e, const Digi
   // 8 values of at most 257.51^2 each, in units of 2^-8: < 2^28 per lane; 8 lanes < 2^31
   uint32_t n2 = __float2uint_ru(n2f * 256.0f * 1.0001f);
 #pragma unroll
-  for (int o = 1; o < 8; o <<= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, o);
-  if (on && cc == 0 && n2) atomicAdd(s_n2_l, (unsigned long long)n2);
+  for (int o = 1; o < W; o <<= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, o);
+  if (on && threadIdx.x % W == 0 && n2) atomicAdd(s_n2_l, (unsigned long long)n2);
 }
 
-// Advances a warp's item (group g of 4 lines, k-block kb) by `step` items in
+// Advances a warp's item (line group g, k-block or part of one kb) by `step` items in
 // the group-fastest order, without a division.
 __device__ __forceinline__ void next_item(int& g, int& kb, int step, int groups) {
   g += step;
@@ -337,8 +337,6 @@ __global__ void __launch_bounds__(kSliceThreads, BETA == 0 || CPLX ? 4 : 6)
   __shared__ int s_e[128];
   __shared__ LineSrc s_src[128];            // the job's lines; all four arrays job-relative
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int cc = lane & 7;        // chunk of 8 k values inside a 64-wide k-block
-  const int lsub = lane >> 3;     // line within the warp's group of 4
   constexpr int kWarps = kSliceThreads / 32;
   for (int64_t jb = blockIdx.x; jb < a.njobs; jb += gridDim.x) {
     const SliceJob J = a.jobs[jb];
@@ -354,8 +352,8 @@ __global__ void __launch_bounds__(kSliceThreads, BETA == 0 || CPLX ? 4 : 6)
       s_src[t] = line_src(a, J, isA, J.l0 + t);
     }
     __syncthreads();
-    // this lane's chunk of line r of the job and k-block kb in the tiles
-    auto place = [&](int r, int kb) {
+    // chunk cc (8 values of k) of line r of the job and k-block kb in the tiles
+    auto place = [&](int r, int kb, int cc) {
       const int l = J.l0 + r;
       return tiles + (int64_t)kb * S * tile_bytes + l * kLineBytes + ((cc ^ (l & 7)) << 4);
     };
@@ -370,7 +368,7 @@ __global__ void __launch_bounds__(kSliceThreads, BETA == 0 || CPLX ? 4 : 6)
       __syncthreads();
       // digit planes and the norm of the absolute digit weights: 8 lanes to a
       // complex row and k-block
-      const int first = warp * 4 + lsub;
+      const int cc = lane & 7, first = warp * 4 + (lane >> 3);
       int kb = first / E, er = first - kb * E;
       while (__any_sync(0xFFFFFFFFu, kb < J.nkb)) {
         const int r = er * lines, kbc = min(kb, J.nkb - 1);
@@ -380,10 +378,11 @@ __global__ void __launch_bounds__(kSliceThreads, BETA == 0 || CPLX ? 4 : 6)
 #pragma unroll
           for (int v = 0; v < 4; ++v) z[v] = stage[stage_pos(kbc * (BK / 2) + 4 * cc + v, er, E)];
           const double x[8] = {z[0].x, -z[0].y, z[1].x, -z[1].y, z[2].x, -z[2].y, z[3].x, -z[3].y};
-          cut_item<S, BETA>(x, s_e[r], dc, place(r, kbc), tile_bytes, cc, on, &s_n2[r]);
+          cut_item<S, BETA, 8>(x, s_e[r], dc, place(r, kbc, cc), tile_bytes, on, &s_n2[r]);
           if (isA) {
             const double y[8] = {z[0].y, z[0].x, z[1].y, z[1].x, z[2].y, z[2].x, z[3].y, z[3].x};
-            cut_item<S, BETA>(y, s_e[r], dc, place(r + 1, kbc), tile_bytes, cc, on, &s_n2[r + 1]);
+            cut_item<S, BETA, 8>(y, s_e[r], dc, place(r + 1, kbc, cc), tile_bytes, on,
+                                 &s_n2[r + 1]);
           }
         }
         er += kWarps * 4;
@@ -393,36 +392,43 @@ __global__ void __launch_bounds__(kSliceThreads, BETA == 0 || CPLX ? 4 : 6)
         }
       }
     } else {
-      // ---- phase 1: line maxima (exponents); a group of 4 lines beyond their
+      // ---- phase 1: line maxima (exponents); a group of lines beyond their
       // instance is skipped here and in phase 2
-      const int groups = nl / 4;
-      int g = 0, kb = 0;
-      next_item(g, kb, warp, groups);
-      while (kb < J.nkb) {
-        const int r = g * 4 + lsub;
+      // W lanes to a line and 8 W values of k: up to 6 planes 8 lines by half a
+      // k-block, as 8 rows of A are 64 bytes side by side and a load takes half the
+      // L1 accesses of one of 4 lines by a k-block (3 slices, 1500 real instances
+      // of order 128: 362 -> 324 us); with more planes their stores, of half lines
+      // then, take back what the loads save (9 slices, order 512: 664 -> 677 us).
+      constexpr int W = S <= 6 ? 4 : 8, kLines = 32 / W, kParts = 8 / W;
+      const int groups = nl / kLines, lsub = lane / W, cw = lane % W;
+      int g = 0, h = 0;  // part h of the k-blocks
+      next_item(g, h, warp, groups);
+      while (h < kParts * J.nkb) {
+        const int r = g * kLines + lsub;
         const LineSrc src = s_src[r];
         if (__any_sync(0xFFFFFFFFu, src.off >= 0)) {
           double x[8];
-          load8<CPLX>(a, rows, src, kb * BK + 8 * cc, kv, x);
-          merge_max(x, cc, &s_max[r]);
+          load8<CPLX>(a, rows, src, (h * W + cw) * 8, kv, x);
+          merge_max<W>(x, &s_max[r]);
         }
-        next_item(g, kb, kWarps, groups);
+        next_item(g, h, kWarps, groups);
       }
       __syncthreads();
       if (t < nl) s_e[t] = line_exponent(s_max[t]);
       __syncthreads();
       // ---- phase 2: digit planes and the norm of the absolute digit weights
-      g = kb = 0;
-      next_item(g, kb, warp, groups);
-      while (kb < J.nkb) {
-        const int r = g * 4 + lsub;
+      g = h = 0;
+      next_item(g, h, warp, groups);
+      while (h < kParts * J.nkb) {
+        const int r = g * kLines + lsub;
         const LineSrc src = s_src[r];
         if (__any_sync(0xFFFFFFFFu, src.off >= 0)) {
           double x[8];
-          load8<CPLX>(a, rows, src, kb * BK + 8 * cc, kv, x);
-          cut_item<S, BETA>(x, s_e[r], dc, place(r, kb), tile_bytes, cc, true, &s_n2[r]);
+          load8<CPLX>(a, rows, src, (h * W + cw) * 8, kv, x);
+          cut_item<S, BETA, W>(x, s_e[r], dc, place(r, h / kParts, h % kParts * W + cw), tile_bytes, true,
+                               &s_n2[r]);
         }
-        next_item(g, kb, kWarps, groups);
+        next_item(g, h, kWarps, groups);
       }
     }
     __syncthreads();
@@ -655,7 +661,7 @@ static int kmma_last_of(int kv) {
 }
 
 // Cuts block jobs into jobs of fewer lines (halving while the count stays a
-// multiple of 4): complex rows to what fits the slicer's shared-memory stage,
+// multiple of 4, or 8 unstaged): complex rows to what fits the slicer's shared-memory stage,
 // the rest to kSliceJobBytes. Returns the stage that the longest rows need.
 static int split_jobs(std::vector<SliceJob>* jobs, bool cplx, bool herk) {
   std::vector<SliceJob> out;
@@ -663,17 +669,17 @@ static int split_jobs(std::vector<SliceJob>* jobs, bool cplx, bool herk) {
   int64_t stage = 0;
   for (const SliceJob& j : *jobs) {
     const int64_t line_bytes = (int64_t)j.nkb * BK * 8;
-    auto lines = [&](int64_t per_line, int64_t bytes) {
+    auto lines = [&](int64_t per_line, int64_t bytes, int unit) {
       int nl = j.w;
-      while (nl * per_line > bytes && nl % 2 == 0 && (nl / 2) % 4 == 0) nl /= 2;
+      while (nl * per_line > bytes && nl % (2 * unit) == 0) nl /= 2;
       return nl;
     };
     // (a complex value of A serves two values of each of two lines)
     const int64_t staged_line = j.side == 0 ? line_bytes / 2 : line_bytes;
-    int nl = lines(staged_line, kSliceStage);
+    int nl = lines(staged_line, kSliceStage, 4);
     const bool staged = cplx && (j.side == 0 || herk) && nl * staged_line <= kSliceStageMax;
     if (staged) stage = std::max({stage, nl * staged_line, kSliceStage});
-    else nl = lines(line_bytes, kSliceJobBytes);
+    else nl = lines(line_bytes, kSliceJobBytes, 8);
     for (int l0 = 0; l0 < j.w; l0 += nl) {
       SliceJob sj = j;
       sj.l0 = (int16_t)l0;

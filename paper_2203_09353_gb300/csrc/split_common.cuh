@@ -35,19 +35,21 @@ constexpr int64_t kSliceStage = 32768, kSliceStageMax = 65536, kSliceJobBytes = 
 constexpr int kMaxDynSmem = 232448;
 constexpr unsigned long long kWaitNs = 2000000000ull;  // 2 s bound on any single wait
 
-// Tile width (columns of the output tile, rows of a B tile) for s planes:
-// the largest multiple of 16 (at most 128) with s * BN <= 512 TMEM columns.
-// Output tile width of the split GEMM for s slices. Up to 5 slices the tile's
-// s level accumulators fit TMEM twice (2 s BN <= 512 columns): the MMAs of the
-// next tile then run while the epilogue empties the other copy. From 6
-// slices on one copy fills TMEM and the epilogue empties it level by level
-// (a double-buffered 6-slice tile would be 32 wide, which measured slower).
+// Tile width (columns of the output tile, rows of a B tile) of the split GEMM
+// for s slices: a multiple of 16 (at most 128) with s * BN <= 512 TMEM columns.
+// Up to 5 slices the tile's s level accumulators fit TMEM twice (2 s BN <= 512
+// columns): the MMAs of the next tile then run while the epilogue empties the
+// other copy. From 6 slices on one copy is filled and the epilogue empties it
+// level by level (6 slices: 64 columns with 16 epilogue warps instead of 48 with
+// 12, which read A's planes a third less often: Hermitian updates 547 -> 496 us,
+// 152 complex instances of order 256 602 -> 563 us; double-buffered, 32 wide,
+// was slower than 48).
 __host__ __device__ constexpr int bn_for(int s) {
-  return s <= 2 ? 128 : s <= 4 ? 64 : s == 5 ? 48 : s == 6 ? 48 : s <= 8 ? 64 : s <= 10 ? 48 : 32;
+  return s <= 2 ? 128 : s <= 4 ? 64 : s == 5 ? 48 : s == 6 ? 64 : s <= 8 ? 64 : s <= 10 ? 48 : 32;
 }
 __host__ __device__ constexpr bool double_buffered(int s) { return s <= 5; }
 // Epilogue warps per TMEM lane quadrant (split_gemm_kernel's H).
-__host__ __device__ constexpr int epi_groups(int s) { return s == 3 ? 4 : s == 6 || s == 9 ? 3 : 2; }
+__host__ __device__ constexpr int epi_groups(int s) { return s == 3 || s == 6 ? 4 : s == 9 ? 3 : 2; }
 // A tile may be narrower than bn_for(s): its width w is a multiple of the
 // columns of one epilogue warp (where those are whole MMA steps of 16), and an
 // instance's n columns are dealt evenly over ceil(n / bn_for(s)) tiles, so that

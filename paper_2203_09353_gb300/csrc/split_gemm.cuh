@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(gemm_threads(H), 1) split_gemm_kernel(const Ge
   static_assert(BN % (8 * H) == 0, "epilogue column groups of 8");
   constexpr int COLS = BN / H;  // output columns per epilogue thread
   constexpr int kEpi = 4 * H;   // epilogue warps
-  // The 6-slice tile (40 accumulators per thread) is register-bound: it keeps
+  // The 6-slice tile (96 registers a thread) is register-bound: it keeps
   // the compact conversion and drains one level at a time.
   constexpr bool kFastConv = SF != 6;
   constexpr bool kMayPair = SF != 6;
@@ -563,36 +563,43 @@ __global__ void __launch_bounds__(gemm_threads(H), 1) split_gemm_kernel(const Ge
             if constexpr (SF > 0 && SF % kAGroup == 0) {
               if (ok && kLast > 0) ok = level_wait(s - 1);
               if (ok && mine && kLast > 0) {
-                uint32_t v[kAGroup][COLS / 8][8];
+                // 6 slices: 8 columns at a time, for want of registers
+                constexpr int CH = kMayPair ? COLS : 8;
 #pragma unroll
-                for (int i = 0; i < kAGroup; ++i) {
+                for (int c0 = 0; c0 < COLS; c0 += CH) {
+                  uint32_t v[kAGroup][CH / 8][8];
 #pragma unroll
-                  for (int j0 = 0; j0 < COLS; j0 += 8)
-                    tmem_ld8(tq + (s - kAGroup + i) * w + j0, v[i][j0 / 8]);
-                  if (kMayPair && i == 1) {  // (two levels become one: fewer registers)
-                    tmem_ld_wait();
+                  for (int i = 0; i < kAGroup; ++i) {
 #pragma unroll
-                    for (int j = 0; j < COLS; ++j)
-                      v[0][j / 8][j % 8] =
-                          (uint32_t)((__float2int_rn(__uint_as_float(v[0][j / 8][j % 8]))
-                                      << g.beta) +
-                                     __float2int_rn(__uint_as_float(v[1][j / 8][j % 8])));
+                    for (int j0 = 0; j0 < CH; j0 += 8)
+                      tmem_ld8(tq + (s - kAGroup + i) * w + c0 + j0, v[i][j0 / 8]);
+                    if (kMayPair && i == 1) {  // (two levels become one: fewer registers)
+                      tmem_ld_wait();
+#pragma unroll
+                      for (int j = 0; j < CH; ++j)
+                        v[0][j / 8][j % 8] =
+                            (uint32_t)((__float2int_rn(__uint_as_float(v[0][j / 8][j % 8]))
+                                        << g.beta) +
+                                       __float2int_rn(__uint_as_float(v[1][j / 8][j % 8])));
+                    }
                   }
-                }
-                tmem_ld_wait();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&S.tmem_free);
-#pragma unroll
-                for (int j0 = 0; j0 < COLS; j0 += 8) {
-                  const int c8 = j0 / 8;
-                  if (kMayPair) {
-                    add8(j0, s - 2, v[0][c8]);
-                  } else {
-                    add8(j0, s - 3, level_int(v[0][c8]));
-                    add8(j0, s - 2, level_int(v[1][c8]));
+                  tmem_ld_wait();
+                  if (c0 + CH == COLS) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&S.tmem_free);
                   }
-                  add8(j0, s - 1, level_int(v[2][c8]));
+#pragma unroll
+                  for (int j0 = 0; j0 < CH; j0 += 8) {
+                    const int c8 = j0 / 8;
+                    if (kMayPair) {
+                      add8(c0 + j0, s - 2, v[0][c8]);
+                    } else {
+                      add8(c0 + j0, s - 3, level_int(v[0][c8]));
+                      add8(c0 + j0, s - 2, level_int(v[1][c8]));
+                    }
+                    add8(c0 + j0, s - 1, level_int(v[2][c8]));
+                  }
                 }
               }
             }
