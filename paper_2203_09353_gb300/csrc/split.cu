@@ -987,7 +987,8 @@ static void grids(SplitPlan* p) {
   const int bps = slicer_ctas(p);
   p->grid_slice = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)p->sms * bps, p->n_jobs));
   if (p->n_small_items > 0)
-    p->grid_small = (int)std::max<int64_t>(1, std::min<int64_t>(p->sms, p->n_small_items));
+    p->grid_small = (int)std::max<int64_t>(1, std::min<int64_t>(
+        (int64_t)p->sms * split_small_ctas(p->s), p->n_small_items));
 }
 
 bg_status split_plan_create(SplitPlan** out, bg_dtype dt, const bg_precision& pr,

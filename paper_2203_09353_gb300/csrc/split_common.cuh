@@ -636,6 +636,7 @@ bool split_small_supported(int s, int beta);
 bool split_small_route(int s, int64_t m, int64_t n, int64_t k);  // instance to this kernel?
 int split_small_groups(int s, int t);  // instances per item for padded edge t
 size_t split_small_smem(int s);
+int split_small_ctas(int s);  // CTAs per SM
 cudaError_t launch_split_small(int s, int grid, cudaStream_t st, const SmallArgs& g);
 
 // GEMM launchers, one per element type (split_gemm_r64.cu, split_gemm_c128.cu).

@@ -395,8 +395,14 @@ __device__ __forceinline__ void small_item(const SmallArgs& g, const SmallItem& 
   small_instance<S, BETA, T>(g, in, sm + gid * SH::GROUP_BYTES, gid, tg, dc, next);
 }
 
+// 3 slices: two CTAs per SM (78 KB of shared memory, 64 registers a thread). A
+// CTA runs one instance of edge 64 at a time, a chain of dependent steps.
+template <int S>
+constexpr int small_ctas() {
+  return S <= 3 ? 2 : 1;
+}
 template <int S, int BETA>
-__global__ void __launch_bounds__(kSmallThreads, 1) split_small_kernel(const SmallArgs g) {
+__global__ void __launch_bounds__(kSmallThreads, small_ctas<S>()) split_small_kernel(const SmallArgs g) {
   extern __shared__ __align__(16) uint8_t sm[];
   const DigitCtx dc = digit_ctx<S>(BETA);
   for (int64_t it = blockIdx.x; it < g.nitems; it += gridDim.x) {
@@ -452,6 +458,8 @@ int split_small_groups(int s, int t) {
       return 0;
   }
 }
+
+int split_small_ctas(int s) { return s == 3 ? small_ctas<3>() : 1; }
 
 size_t split_small_smem(int s) {
   return s == 3 ? small_smem_of<3>() : s == 6 ? small_smem_of<6>() : s == 9 ? small_smem_of<9>() : 0;
