@@ -1062,6 +1062,7 @@ static cudaError_t launch_small(SplitPlan* p, const void* A, const void* B, void
   g.B = static_cast<const double*>(B);
   g.C = static_cast<double*>(C);
   g.sc = sc;
+  g.ap = take_alpha_pow2(&g.sc);
   g.skip_product = sc.alpha_zero;
   const cudaError_t e = launch_split_small(p->s, p->grid_small, st, g);
   count_launch();
@@ -1087,6 +1088,7 @@ static cudaError_t launch_gemm(SplitPlan* p, void* C, const Scalars& sc, const i
   g.pool = p->d_pool;
   g.pool_count = p->n_pool;
   g.sc = sc;
+  g.ap = take_alpha_pow2(&g.sc);
   g.cplx = p->dt == BG_C128;
   g.s = p->s;
   g.beta = p->beta;

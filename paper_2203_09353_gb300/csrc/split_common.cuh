@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 #include "split.h"
 
 namespace bg {
@@ -115,6 +117,29 @@ struct SliceArgs {
   int herk;  // Hermitian update: B lines are rows of A (conjugated), read through the A side
 };
 
+// A real alpha that is plus or minus a power of two needs no FP64 multiply (16
+// clocks of the SM for a warp's 32 outputs, as long as one beta C): the product
+// is the exponent of the conversion and the sign bit. alpha is then passed as 1.
+struct AlphaPow2 {
+  int exp = 0;         // added to the exponent
+  uint32_t flip = 0;   // sign bit of the high word
+};
+inline AlphaPow2 take_alpha_pow2(Scalars* sc) {
+  AlphaPow2 r;
+  int e = 0;
+  const double f = std::frexp(std::fabs(sc->alpha_re), &e);
+  if (sc->alpha_im == 0.0 && f == 0.5) {  // (not zero, infinite or NaN)
+    r.exp = e - 1;
+    r.flip = std::signbit(sc->alpha_re) ? 0x80000000u : 0u;
+    sc->alpha_re = 1.0;
+    sc->alpha_im = 0.0;
+  }
+  return r;
+}
+__device__ __forceinline__ double flip_sign(double x, uint32_t flip) {
+  return __hiloint2double(__double2hiint(x) ^ (int)flip, __double2loint(x));
+}
+
 struct GemmArgs {
   const SplitUnit* units;
   int64_t nunits;
@@ -135,6 +160,7 @@ struct GemmArgs {
   int kpass;                  // k-blocks per exact pass
   int a_groups;               // groups of kAGroup slots in the A ring
   int herk;                   // Hermitian update: store only the lower triangle
+  AlphaPow2 ap;
   int* err;
 };
 
@@ -158,6 +184,7 @@ struct SmallArgs {
   const double* B;
   double* C;
   Scalars sc;
+  AlphaPow2 ap;
   int skip_product;  // alpha == 0: C = beta C
 };
 

@@ -50,7 +50,7 @@ __device__ __forceinline__ void epi_store8(const GemmArgs& g, const long long (&
   for (int j = 0; j < 8; ++j) {
     const int col = colb + j;
     const bool valid = rvalid && col >= cmin && col < cmax;
-    const double x = valid ? xs[j] : 0.0;
+    const double x = valid ? flip_sign(xs[j], g.ap.flip) : 0.0;
     double* cp = g.C + cbase + (int64_t)(col + coff) * ldcv;
     if constexpr (!CPLX) {
       if (valid) {
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(gemm_threads(H), 1) split_gemm_kernel(const Ge
       }
       const int64_t cbase = (CPLX ? 2 * in.c_off : in.c_off) + rr;
       const int64_t ldcv = CPLX ? 2 * in.ldc : in.ldc;
-      const int Ebase = F - 62 + e_i - 2 * g.beta;
+      const int Ebase = F - 62 + e_i - 2 * g.beta + g.ap.exp;
       const int npass = unit_passes(g, U);
       if constexpr (DB) {
         // ---- double-buffered TMEM: take the finished tile whole, 8 columns at a time

@@ -360,7 +360,7 @@ __device__ __forceinline__ void small_instance(const SmallArgs& g, const SInst& 
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int i = min(rows[h], T - 1);
-    const int Ebase = F[h] - 62 + line_e(eA[i]) - 2 * BETA;
+    const int Ebase = F[h] - 62 + line_e(eA[i]) - 2 * BETA + g.ap.exp;
 #pragma unroll
     for (int nh = 0; nh < 2; ++nh)
 #pragma unroll
@@ -372,6 +372,7 @@ __device__ __forceinline__ void small_instance(const SmallArgs& g, const SInst& 
           bool bad = false;
           xs[h][nh][c] = fixed_to_double_fast(accI[h][nh][c], E, bad);
           if (bad) xs[h][nh][c] = fixed_to_double(accI[h][nh][c], E);
+          xs[h][nh][c] = flip_sign(xs[h][nh][c], g.ap.flip);
         }
       }
   }
