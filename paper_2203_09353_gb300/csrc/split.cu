@@ -256,6 +256,9 @@ __device__ __forceinline__ void cut_item(const double (&x)[8], int e, const Digi
   if (on && threadIdx.x % W == 0 && n2) atomicAdd(s_n2_l, (unsigned long long)n2);
 }
 
+// Lines of a warp's item of an unstaged job.
+__host__ __device__ constexpr int item_lines(int s) { return s <= 6 ? 8 : 4; }
+
 // Advances a warp's item (line group g, k-block or part of one kb) by `step` items in
 // the group-fastest order, without a division.
 __device__ __forceinline__ void next_item(int& g, int& kb, int step, int groups) {
@@ -399,7 +402,7 @@ __global__ void __launch_bounds__(kSliceThreads, BETA == 0 || CPLX ? 4 : 6)
       // L1 accesses of one of 4 lines by a k-block (3 slices, 1500 real instances
       // of order 128: 362 -> 324 us); with more planes their stores, of half lines
       // then, take back what the loads save (9 slices, order 512: 664 -> 677 us).
-      constexpr int W = S <= 6 ? 4 : 8, kLines = 32 / W, kParts = 8 / W;
+      constexpr int kLines = item_lines(S), W = 32 / kLines, kParts = 8 / W;
       const int groups = nl / kLines, lsub = lane / W, cw = lane % W;
       int g = 0, h = 0;  // part h of the k-blocks
       next_item(g, h, warp, groups);
@@ -661,9 +664,9 @@ static int kmma_last_of(int kv) {
 }
 
 // Cuts block jobs into jobs of fewer lines (halving while the count stays a
-// multiple of 4, or 8 unstaged): complex rows to what fits the slicer's shared-memory stage,
+// multiple of the lines of a warp's item): complex rows to what fits the slicer's shared-memory stage,
 // the rest to kSliceJobBytes. Returns the stage that the longest rows need.
-static int split_jobs(std::vector<SliceJob>* jobs, bool cplx, bool herk) {
+static int split_jobs(std::vector<SliceJob>* jobs, int s, bool cplx, bool herk) {
   std::vector<SliceJob> out;
   out.reserve(jobs->size() * 2);
   int64_t stage = 0;
@@ -679,7 +682,7 @@ static int split_jobs(std::vector<SliceJob>* jobs, bool cplx, bool herk) {
     int nl = lines(staged_line, kSliceStage, 4);
     const bool staged = cplx && (j.side == 0 || herk) && nl * staged_line <= kSliceStageMax;
     if (staged) stage = std::max({stage, nl * staged_line, kSliceStage});
-    else nl = lines(line_bytes, kSliceJobBytes, 8);
+    else nl = lines(line_bytes, kSliceJobBytes, item_lines(s));
     for (int l0 = 0; l0 < j.w; l0 += nl) {
       SliceJob sj = j;
       sj.l0 = (int16_t)l0;
@@ -871,7 +874,7 @@ static void make_tables(const SplitPlan* p, const std::vector<bg_instance>& tabl
     if (ia < jobsA.size()) jobs.push_back(jobsA[ia++]);
     if (ib < jobsB.size()) jobs.push_back(jobsB[ib++]);
   }
-  out->stage = split_jobs(&jobs, cplx, p->herk);
+  out->stage = split_jobs(&jobs, s, cplx, p->herk);
   out->inst = std::move(inst);
   out->order = std::move(order);
   out->jobs = std::move(jobs);
@@ -973,8 +976,9 @@ static cudaError_t with_slicer(const SplitPlan* p, const F& f) {
 static int slicer_ctas(const SplitPlan* p) {
   int bps = 0;
   with_slicer(p, [&](auto kernel) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)kSliceStageMax);
+    if (p->slice_stage > kSliceStage)
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kSliceStageMax);
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, kSliceThreads,
                                                          p->slice_stage);
   });
@@ -1330,7 +1334,7 @@ bg_status split_chain_create(SplitPlan** out, bg_dtype dt, const bg_precision& p
   std::stable_sort(units.begin(), units.end(),
                    [](const SplitUnit& a, const SplitUnit& b) { return a.nkb > b.nkb; });
   // pool jobs first, then walker jobs (the chain step slices the two parts separately)
-  p->slice_stage = std::max(split_jobs(&jobsA, cplx, false), split_jobs(&jobsB, cplx, false));
+  p->slice_stage = std::max(split_jobs(&jobsA, s, cplx, false), split_jobs(&jobsB, s, cplx, false));
   std::vector<SliceJob> jobs = jobsA;
   jobs.insert(jobs.end(), jobsB.begin(), jobsB.end());
   p->n_jobs = (int64_t)jobs.size();
