@@ -493,9 +493,9 @@ def gate_line(bg, fp64_peak, hbm_peak, hbm_src, steps: int = 20, S: int = 17,
                         f"and step on a random neighbouring pair",
             "steps": steps, "ms_per_step": ms, "value": amps / (ms * 1e-3) / 1e9,
             "unit": "G amplitudes/s", "fp64_tflops": tflops, "hbm_gbs": gbs,
-            "roofline": {"bound": "alu", "achieved": tflops, "peak": fp64_peak, "unit": "TFLOP/s",
-                         "frac": tflops / fp64_peak if fp64_peak else None,
-                         "peak_source": "DFMA probe measured live (bg_probe_fp64_peak)"},
+            "roofline": {"bound": "hbm", "achieved": gbs, "peak": hbm_peak, "unit": "GB/s",
+                         "frac": gbs / hbm_peak, "peak_source": hbm_src},
+            "fp64_probe_tflops": fp64_peak,
             "hbm_frac_of_copy_peak": gbs / hbm_peak,
             "hbm_peak": {"value": hbm_peak, "unit": "GB/s", "source": hbm_src},
             "gpu_launches": launches,
@@ -666,8 +666,7 @@ def entropy_line(bg, fp64_peak, steps: int = 5, warmup: int = 2, S: int = 17,
     """The entanglement entropy of Alg. 1 ("Calculate Entropy") for `walkers`
     random complex states of S spins (cut after floor(S/2) spins: K = 256,
     M = 512 at S = 17): the Gram matrices through the Hermitian update (FP64 or
-    9 slices), then tridiagonalisation and bisection; with 9 slices the
-    reduction is blocked, its trailing updates running as 9-slice GEMMs.
+    9 slices), then tridiagonalisation in 60-bit fixed point and bisection.
     Roofline of the eigenvalue step: the flops of the reduction, (16/3) K^3
     per walker (the LAPACK count of zhetrd), against the live DFMA probe."""
     import torch
@@ -696,11 +695,8 @@ def entropy_line(bg, fp64_peak, steps: int = 5, warmup: int = 2, S: int = 17,
         got = ent.cpu().numpy()[sample]
         eig_ms = kt[1] / max(calls, 1)
         ach = tri_flops / (eig_ms * 1e-3) / 1e12
-        # 9 slices, K > 64: the blocked reduction, whose rank-32 trailing updates
-        # (about half the flops) run on the tensor cores
-        kernels = ("tridiag_kernel + bisect_kernel" if mode == "fp64" or K <= 64 else
-                   "tri_mirror_kernel + (tri_panel_kernel + tri_pack_kernel + split "
-                   "GEMM) per 16-column panel + tridiag_kernel (last 64) + bisect_kernel")
+        # (fixed point on the integer pipe: above the DFMA probe's rate is possible)
+        kernels = "tri_reduce_kernel + bisect_kernel + entropy_sum_kernel"
         res[mode] = {"ms_per_call": ms, "gram_ms": kt[0] / max(calls, 1), "eig_ms": eig_ms,
                      "value": walkers / (ms * 1e-3), "unit": "walkers/s",
                      "max_abs_err_vs_oracle": float(np.max(np.abs(got - want))),
@@ -715,7 +711,7 @@ def entropy_line(bg, fp64_peak, steps: int = 5, warmup: int = 2, S: int = 17,
 def anneal_line(bg, steps: int = 10, warmup: int = 2, S: int = 17, walkers: int = 128):
     """Whole annealing steps of Alg. 1 for `walkers` states of S spins: per step
     and walker a Haar gate on a random neighbouring pair, the proposal's
-    entropy (Gram and trailing updates with 9 slices) and the Metropolis decision
+    entropy (Gram with 9 slices) and the Metropolis decision
     at a geometric temperature schedule T_t = 0.05 x 0.9^t, minimising the
     entropy. The CPU oracle's step is timed on two walkers for context."""
     import torch

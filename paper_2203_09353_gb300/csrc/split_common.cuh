@@ -83,8 +83,8 @@ struct SliceJob {
   int16_t nl;     // lines this job cuts (a multiple of 4)
   int16_t w;      // lines of the block's tiles (A: 128, B: the tile width)
   int16_t staged;  // the job's values fit the shared-memory stage
-  int16_t pad[2];
 };
+static_assert(sizeof(SliceJob) == 40, "the static scratch of a call holds the job table");
 
 struct SplitUnit {
   int64_t a_tile0, b_tile0;  // first tiles (chain mode: a_tile0 is relative to the pool entry;
