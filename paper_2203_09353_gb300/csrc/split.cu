@@ -319,8 +319,8 @@ __device__ __forceinline__ void stage_rows(const SliceArgs& a, const LineSrc* s_
 // lines. Their values lie a leading dimension apart along k, so that a lane's
 // chunk of k took an L1 access per 32 bytes, in both passes and for both lines:
 // the L1 pipe was 78-91% busy (4096 instances of order 64, 9 slices: slicer
-// 566 -> 404 us, 4.4 TB/s of loads and plane stores; Hermitian updates, 6
-// slices: 246 -> 197 us). Real rows and columns of B, staged the same way, were
+// 566 -> 404 us, 4.2 -> 5.7 TB/s of DRAM traffic; Hermitian updates, 6 slices:
+// 246 -> 190 us). Real rows and columns of B, staged the same way, were
 // slower by 0-7%: one line per value leaves too little to save, and the stage
 // costs occupancy.
 //
