@@ -56,6 +56,17 @@ inline bool small_fills(int64_t instances, int64_t grid) {
 }
 constexpr int kFp64Threads = 256;
 
+// Outputs per thread of the program that runs a tile with `out` outputs inside
+// its instance: the smallest that holds them all. The largest is the
+// register-blocked one of the full tile; it guards its edges, so it also runs
+// what an instance leaves of a full tile (127 rows are 64 + 63).
+__host__ __device__ constexpr int tile_program_r64(int out) {
+  return out > 8 * kFp64Threads ? 16 : out > 4 * kFp64Threads ? 8 : out > 2 * kFp64Threads ? 4 : 2;
+}
+__host__ __device__ constexpr int tile_program_c128(int out) {
+  return out > 2 * kFp64Threads ? 4 : out > kFp64Threads ? 2 : 1;
+}
+
 struct Scalars {
   double alpha_re, alpha_im, beta_re, beta_im;
   int alpha_zero, beta_zero;

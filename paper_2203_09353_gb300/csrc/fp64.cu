@@ -170,8 +170,8 @@ struct SmemR64 {
 };
 
 // Rows r0 .. r0 + tm - 1 and columns c0 .. c0 + tn - 1 (tm, tn <= 64) of one
-// instance; FULL: a 64 x 64 tile that the instance fills, 4 x 4 outputs per
-// thread. Otherwise output o of the tile's mb x nb (column-major) goes to
+// instance; FULL: 64 x 64, or what the instance leaves of it, 4 x 4 outputs per
+// thread (for more outputs than NJ = 8 holds). Otherwise output o of the tile's mb x nb (column-major) goes to
 // thread o mod 256, NJ outputs to a thread: a DFMA takes its 16 clocks per SM
 // whether 1 or 32 of the warp's lanes are active (measured), so padding a
 // ragged tile to 64 x 64 costs in full, while the two extra shared-memory
@@ -662,9 +662,9 @@ __global__ void __launch_bounds__(kFp64Threads, CTAS)
       const int mb = min(tm, d.m - w.r0), nb = min(tn, d.n - w.c0);
       if (mb <= 0 || nb <= 0) continue;
       if (w.prog == PROG_R64_TILE) {
-        if (mb * nb > 2 * kFp64Threads) tile_r64<false, 4>(d, w.r0, w.c0, mb, nb, s, sm.r);
+        if (tile_program_r64(mb * nb) > 2) tile_r64<false, 4>(d, w.r0, w.c0, mb, nb, s, sm.r);
         else tile_r64<false, 2>(d, w.r0, w.c0, mb, nb, s, sm.r);
-      } else if (mb * nb > kFp64Threads) {
+      } else if (tile_program_c128(mb * nb) > 1) {
         tile_c128<false, 2>(d, w.r0, w.c0, mb, nb, s, sm.c);
       } else {
         tile_c128<false, 1>(d, w.r0, w.c0, mb, nb, s, sm.c);
@@ -681,10 +681,10 @@ __global__ void __launch_bounds__(kFp64Threads, CTAS)
         tile_extent_of(w.count, TR, &tm, &tn);
         const int mb = min(tm, d.m - w.r0), nb = min(tn, d.n - w.c0);
         if (mb <= 0 || nb <= 0) break;  // (a chain index that names no matrix)
-        const int out = mb * nb;
-        if (out == TR * TR) tile_r64<true, 1>(d, w.r0, w.c0, mb, nb, s, sm.r);
-        else if (out > 4 * kFp64Threads) tile_r64<false, 8>(d, w.r0, w.c0, mb, nb, s, sm.r);
-        else if (out > 2 * kFp64Threads) tile_r64<false, 4>(d, w.r0, w.c0, mb, nb, s, sm.r);
+        const int per = tile_program_r64(mb * nb);
+        if (per == 16) tile_r64<true, 1>(d, w.r0, w.c0, mb, nb, s, sm.r);
+        else if (per == 8) tile_r64<false, 8>(d, w.r0, w.c0, mb, nb, s, sm.r);
+        else if (per == 4) tile_r64<false, 4>(d, w.r0, w.c0, mb, nb, s, sm.r);
         else tile_r64<false, 2>(d, w.r0, w.c0, mb, nb, s, sm.r);
         break;
       }
@@ -697,10 +697,10 @@ __global__ void __launch_bounds__(kFp64Threads, CTAS)
         tile_extent_of(w.count, TC, &tm, &tn);
         const int mb = min(tm, d.m - w.r0), nb = min(tn, d.n - w.c0);
         if (mb <= 0 || nb <= 0) break;
-        const int out = mb * nb;
-        if (out == TC * TC) tile_c128<true, 1>(d, w.r0, w.c0, mb, nb, s, sm.c);
-        else if (out > 2 * kFp64Threads) tile_c128<false, 4>(d, w.r0, w.c0, mb, nb, s, sm.c);
-        else if (out > kFp64Threads) tile_c128<false, 2>(d, w.r0, w.c0, mb, nb, s, sm.c);
+        const int per = tile_program_c128(mb * nb);
+        if (mb == TC && nb == TC) tile_c128<true, 1>(d, w.r0, w.c0, mb, nb, s, sm.c);
+        else if (per == 4) tile_c128<false, 4>(d, w.r0, w.c0, mb, nb, s, sm.c);
+        else if (per == 2) tile_c128<false, 2>(d, w.r0, w.c0, mb, nb, s, sm.c);
         else tile_c128<false, 1>(d, w.r0, w.c0, mb, nb, s, sm.c);
         break;
       }
