@@ -236,7 +236,8 @@ struct bg_plan {
   double* d_tri_d = nullptr;
   double* d_tri_e = nullptr;
   int ent_n = 0;
-  void* d_tri_p = nullptr;  // the reduction's panel vectors, where it needs them in device memory
+  TriShape tri;             // how the reduction runs, and
+  void* d_tri_p = nullptr;  // its panel vectors, where it needs them in device memory
   // annealing-step plans (Alg. 1): the entropy plan over the proposals, the
   // proposal buffer (walkers x 2^spins, contiguous) and the new energies
   bool is_anneal = false;
@@ -1481,7 +1482,8 @@ bg_status entropy_plan(bg_plan** out, int64_t walkers, int32_t spins, int32_t sp
     }
     p->workspace_bytes = p->gram->workspace_bytes + (int64_t)(gb + 2 * tb);
     p->launches_per_call = p->gram->launches_per_call + 3;
-    const size_t pb = tri_workspace(walkers, (int)K);
+    p->tri = tri_shape(walkers, (int)K);
+    const size_t pb = (size_t)walkers * p->tri.panel;
     if (pb > 0) {
       if ((e = cudaMalloc(&p->d_tri_p, pb)) != cudaSuccess) {
         destroy_plan(p);
@@ -1525,8 +1527,8 @@ bg_status batched_entropy(const bg_plan* plan, const void* states, double* entro
   DeviceCtx* ctx;
   if ((s = get_ctx(&ctx)) != BG_OK) return s;
   // (the eigenvalues go over the Gram matrices, which the reduction has used up)
-  cudaError_t e = launch_tridiag(p->d_gram, p->count, p->ent_n, p->d_tri_p, p->d_tri_d,
-                                 p->d_tri_e, st);
+  cudaError_t e = launch_tridiag(p->d_gram, p->count, p->ent_n, p->tri, p->d_tri_p,
+                                 p->d_tri_d, p->d_tri_e, st);
   if (e == cudaSuccess)
     e = launch_entropy_bisect(p->d_tri_d, p->d_tri_e, p->count, p->ent_n,
                               reinterpret_cast<double*>(p->d_gram), entropy, eigenvalues, ctx->sms,

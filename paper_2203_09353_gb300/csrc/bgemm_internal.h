@@ -154,11 +154,20 @@ bg_status static_scratch(void** out, size_t* bytes, std::string* err);
 
 // Householder reduction of each walker's Hermitian positive semidefinite
 // n x n Gram matrix (lower triangle, overwritten) to a real tridiagonal matrix
-// (tridiag.cu). panel: tri_workspace bytes of device memory, or null where
-// that is 0.
-size_t tri_workspace(int64_t walkers, int n);
-cudaError_t launch_tridiag(double2* gram, int64_t walkers, int n, void* panel, double* d,
-                           double* e, cudaStream_t st);
+// (tridiag.cu). The shape is chosen once, for the current device, and kept with
+// the panel memory that it needs: the device's answer to how many clusters fit
+// may differ from one query to the next. panel: walkers x TriShape::panel bytes
+// of device memory, or null where that is 0.
+struct TriShape {
+  int cl = 1;        // CTAs per walker
+  int own = 0;       // rows a CTA owns at most
+  bool vws = true;   // the panel's own rows are in shared memory
+  size_t smem = 0;   // dynamic shared memory of a CTA
+  size_t panel = 0;  // bytes of panel vectors per walker in device memory
+};
+TriShape tri_shape(int64_t walkers, int n);
+cudaError_t launch_tridiag(double2* gram, int64_t walkers, int n, const TriShape& shape,
+                           void* panel, double* d, double* e, cudaStream_t st);
 
 // Eigenvalues of the tridiagonal matrices and the entropies (entropy.cu).
 // lam: workspace of walkers x n doubles; eigs: optional device [walkers][n],

@@ -958,14 +958,13 @@ constexpr size_t tail_smem() {
   return ((size_t)3 * kTail + (size_t)kWarps * 32 + (size_t)kTail * kTailLd) * 16;
 }
 
-struct TriShape {
-  int cl = 1, own = 0;
-  bool vws = false;
-  size_t smem = 0;
-};
-
+// What an order-n reduction on clusters of cl CTAs asks for.
 TriShape shape_for(int n, int cl) {
   TriShape s;
+  if (n <= kTail) {
+    s.smem = tail_smem();
+    return s;
+  }
   s.cl = cl;
   const int groups = (n + 31) / 32;
   s.own = (groups + cl - 1) / cl * 32;
@@ -975,6 +974,7 @@ TriShape shape_for(int n, int cl) {
   const size_t budget = kSmemMax - sizeof(Shared) - 512;
   s.vws = fixed + vw + (cl > 1 ? stage : 0) <= budget;
   s.smem = std::max(tail_smem(), fixed + (s.vws ? vw : 0) + (cl > 1 || !s.vws ? stage : 0));
+  s.panel = cl > 1 || !s.vws ? (size_t)2 * kNb * n * sizeof(int4) : 0;
   return s;
 }
 
@@ -1006,8 +1006,6 @@ cudaError_t launch_reduce(const TriArgs& a, int64_t walkers, const TriShape& s, 
   count_launch();
   return cudaGetLastError();
 }
-
-}  // namespace
 
 // CTAs per walker: the most (up to 8, and a group of 32 rows each before the
 // tail) for which the device holds every walker's cluster at once. Clusters
@@ -1047,23 +1045,15 @@ int tri_cluster(int64_t walkers, int n) {
   return 1;
 }
 
-size_t tri_workspace(int64_t walkers, int n) {
-  if (n <= kTail) return 0;
-  const TriShape s = shape_for(n, tri_cluster(walkers, n));
-  return s.cl > 1 || !s.vws ? (size_t)walkers * 2 * kNb * n * sizeof(int4) : 0;
-}
+}  // namespace
 
-cudaError_t launch_tridiag(double2* gram, int64_t walkers, int n, void* panel, double* d,
-                           double* e, cudaStream_t st) {
+TriShape tri_shape(int64_t walkers, int n) { return shape_for(n, tri_cluster(walkers, n)); }
+
+cudaError_t launch_tridiag(double2* gram, int64_t walkers, int n, const TriShape& s, void* panel,
+                           double* d, double* e, cudaStream_t st) {
   if (walkers <= 0) return cudaSuccess;
-  TriArgs a{gram, static_cast<int4*>(panel), d, e, n, 0};
-  if (n <= kTail) {
-    TriShape s;
-    s.smem = tail_smem();
-    return launch_reduce<false, true, true>(a, walkers, s, st);
-  }
-  const TriShape s = shape_for(n, tri_cluster(walkers, n));
-  a.own = s.own;
+  const TriArgs a{gram, static_cast<int4*>(panel), d, e, n, s.own};
+  if (n <= kTail) return launch_reduce<false, true, true>(a, walkers, s, st);
   if (s.cl > 1)
     return s.vws ? launch_reduce<true, true, false>(a, walkers, s, st)
                  : launch_reduce<true, false, false>(a, walkers, s, st);
