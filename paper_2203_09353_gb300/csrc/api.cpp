@@ -1482,7 +1482,10 @@ bg_status entropy_plan(bg_plan** out, int64_t walkers, int32_t spins, int32_t sp
     }
     p->workspace_bytes = p->gram->workspace_bytes + (int64_t)(gb + 2 * tb);
     p->launches_per_call = p->gram->launches_per_call + 3;
-    p->tri = tri_shape(walkers, (int)K);
+    if ((e = tri_shape(walkers, (int)K, &p->tri)) != cudaSuccess) {
+      destroy_plan(p);
+      return cuda_fail(e, "entropy plan");
+    }
     const size_t pb = (size_t)walkers * p->tri.panel;
     if (pb > 0) {
       if ((e = cudaMalloc(&p->d_tri_p, pb)) != cudaSuccess) {

@@ -165,7 +165,8 @@ struct TriShape {
   size_t smem = 0;   // dynamic shared memory of a CTA
   size_t panel = 0;  // bytes of panel vectors per walker in device memory
 };
-TriShape tri_shape(int64_t walkers, int n);
+// (also sets the kernels' shared-memory limits on the current device)
+cudaError_t tri_shape(int64_t walkers, int n, TriShape* out);
 cudaError_t launch_tridiag(double2* gram, int64_t walkers, int n, const TriShape& shape,
                            void* panel, double* d, double* e, cudaStream_t st);
 

@@ -27,21 +27,6 @@ namespace {
 
 constexpr int kEntThreads = 256;  // the entropy sums
 
-// A kernel's dynamic shared-memory limit is a property of the device: set it
-// once per device (at every call for ordinals beyond the table).
-constexpr int kAttrDevices = 64;
-template <typename Kernel>
-cudaError_t smem_limit(Kernel kernel, int bytes, bool (&done)[kAttrDevices]) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const bool tracked = dev >= 0 && dev < kAttrDevices;
-  if (tracked && done[dev]) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess && tracked) done[dev] = true;
-  return e;
-}
-
 // Sum of v over the block (all threads call it; the result reaches every thread).
 // red: one double per warp.
 __device__ double block_sum(double v, double* red) {
@@ -426,9 +411,7 @@ __global__ void __launch_bounds__(kEntThreads) entropy_sum_kernel(const double* 
 template <int P>
 cudaError_t bisect_launch(const double* d, const double* e, int64_t walkers, int n, double* lam,
                           cudaStream_t st) {
-  static bool attr[kAttrDevices] = {};
-  const cudaError_t err = smem_limit(bisect_kernel<P>, 96 * 1024, attr);
-  if (err != cudaSuccess) return err;
+  // (n <= 1024: at most 32 KB, which needs no raised limit)
   constexpr int per = kBisThreads / P;
   bisect_kernel<P><<<dim3((unsigned)((n + per - 1) / per), (unsigned)walkers), kBisThreads,
                      (size_t)n * 32, st>>>(d, e, n, lam);

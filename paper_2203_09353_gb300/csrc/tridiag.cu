@@ -958,6 +958,11 @@ constexpr size_t tail_smem() {
   return ((size_t)3 * kTail + (size_t)kWarps * 32 + (size_t)kTail * kTailLd) * 16;
 }
 
+// The largest shared-memory request of any order. The limit is a property of
+// the kernel on a device, shared by all threads that launch it: it is set to
+// this one value, so that no plan's launch depends on another's order.
+constexpr size_t kSmemLimit = kSmemMax - sizeof(Shared) - 512;
+
 // What an order-n reduction on clusters of cl CTAs asks for.
 TriShape shape_for(int n, int cl) {
   TriShape s;
@@ -971,8 +976,7 @@ TriShape shape_for(int n, int cl) {
   const size_t fixed = (size_t)n * 16 + (size_t)std::max(kWarps, s.own / 32) * 32 * 16;
   const size_t vw = (size_t)2 * kNb * s.own * 16;
   const size_t stage = (size_t)kWarps * 2 * kNb * kStrip * 16;
-  const size_t budget = kSmemMax - sizeof(Shared) - 512;
-  s.vws = fixed + vw + (cl > 1 ? stage : 0) <= budget;
+  s.vws = fixed + vw + (cl > 1 ? stage : 0) <= kSmemLimit;
   s.smem = std::max(tail_smem(), fixed + (s.vws ? vw : 0) + (cl > 1 || !s.vws ? stage : 0));
   s.panel = cl > 1 || !s.vws ? (size_t)2 * kNb * n * sizeof(int4) : 0;
   return s;
@@ -994,24 +998,34 @@ void launch_config(const TriShape& s, int64_t walkers, cudaStream_t st, cudaLaun
 
 template <bool MULTI, bool VWS, bool SMALL>
 cudaError_t launch_reduce(const TriArgs& a, int64_t walkers, const TriShape& s, cudaStream_t st) {
-  auto kernel = tri_reduce_kernel<MULTI, VWS, SMALL>;
-  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)s.smem);
-  if (err != cudaSuccess) return err;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
   launch_config(s, walkers, st, &cfg, at);
-  err = cudaLaunchKernelEx(&cfg, kernel, a);
+  const cudaError_t err = cudaLaunchKernelEx(&cfg, tri_reduce_kernel<MULTI, VWS, SMALL>, a);
   if (err != cudaSuccess) return err;
   count_launch();
   return cudaGetLastError();
+}
+
+cudaError_t set_smem_limits() {
+  const void* kernels[] = {(const void*)tri_reduce_kernel<false, true, true>,
+                           (const void*)tri_reduce_kernel<true, true, false>,
+                           (const void*)tri_reduce_kernel<true, false, false>,
+                           (const void*)tri_reduce_kernel<false, true, false>,
+                           (const void*)tri_reduce_kernel<false, false, false>};
+  for (const void* k : kernels) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // CTAs per walker: the most (up to 8, and a group of 32 rows each before the
 // tail) for which the device holds every walker's cluster at once. Clusters
 // of 8 fit 15 times on a GB300 (GPCs of 18 to 20 SMs, one CTA per SM), of 4
 // 36 times, so 16 walkers run on clusters of 7 at most; a second wave would
-// double the time.
+// double the time. The shared-memory limits must be set.
 int tri_cluster(int64_t walkers, int n) {
   if (n <= kTail || walkers <= 0) return 1;
   static std::mutex mu;
@@ -1023,18 +1037,15 @@ int tri_cluster(int64_t walkers, int n) {
     int& a = active[dev][cl];
     if (a == 0) {
       // the largest request any order makes: one CTA per SM
-      auto kernel = tri_reduce_kernel<true, true, false>;
       cudaLaunchConfig_t cfg = {};
       cudaLaunchAttribute at[1];
       TriShape s;
       s.cl = cl;
-      s.smem = kSmemMax - sizeof(Shared) - 512;
+      s.smem = kSmemLimit;
       int c = 0;
-      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)s.smem) != cudaSuccess)
-        return 1;
       launch_config(s, 1, nullptr, &cfg, at);
-      if (cudaOccupancyMaxActiveClusters(&c, kernel, &cfg) != cudaSuccess) {
+      if (cudaOccupancyMaxActiveClusters(&c, tri_reduce_kernel<true, true, false>, &cfg) !=
+          cudaSuccess) {
         cudaGetLastError();
         return 1;
       }
@@ -1047,7 +1058,11 @@ int tri_cluster(int64_t walkers, int n) {
 
 }  // namespace
 
-TriShape tri_shape(int64_t walkers, int n) { return shape_for(n, tri_cluster(walkers, n)); }
+cudaError_t tri_shape(int64_t walkers, int n, TriShape* out) {
+  const cudaError_t e = set_smem_limits();
+  *out = shape_for(n, e == cudaSuccess ? tri_cluster(walkers, n) : 1);
+  return e;
+}
 
 cudaError_t launch_tridiag(double2* gram, int64_t walkers, int n, const TriShape& s, void* panel,
                            double* d, double* e, cudaStream_t st) {

@@ -14,7 +14,8 @@ int main() {
   int bad = 0;
   for (int n = 2; n <= 1024; n *= 2)
     for (long walkers : {0L, 1L, 4L, 16L, 76L, 65535L}) {
-      const bg::TriShape s = bg::tri_shape(walkers, n);
+      bg::TriShape s;
+      bg::tri_shape(walkers, n, &s);
       const bool device_panel = n > 96 && (s.cl > 1 || !s.vws);
       bad += (s.panel > 0) != device_panel || s.panel % 16 != 0;
       bad += s.smem == 0 || s.smem > 227 * 1024 || s.cl < 1 || s.cl > 8;
