@@ -125,7 +125,7 @@ __device__ __forceinline__ long long warp_sum(long long v) {
   return v;
 }
 
-// Unsigned 128-bit sums of squares.
+// Unsigned 128-bit sums of squares (a difference below zero wraps).
 struct U128 {
   unsigned long long hi = 0, lo = 0;
   __device__ __forceinline__ void add(unsigned long long h, unsigned long long l) {
@@ -135,8 +135,16 @@ struct U128 {
     const unsigned long long u = x < 0 ? 0ull - (unsigned long long)x : (unsigned long long)x;
     add(__umul64hi(u, u), u * u);
   }
-  __device__ __forceinline__ double value() const {
-    return fma((double)hi, 0x1p64, (double)lo);
+  __device__ __forceinline__ void subtract(const U128& v) {
+    asm("sub.cc.u64 %0, %0, %2;\n\tsubc.u64 %1, %1, %3;"
+        : "+l"(lo), "+l"(hi)
+        : "l"(v.lo), "l"(v.hi));
+  }
+  __device__ __forceinline__ U128 shifted_right(int s) const {  // 0 < s < 64
+    return {hi >> s, lo >> s | hi << (64 - s)};
+  }
+  __device__ __forceinline__ U128 shifted_left(int s) const {  // 0 <= s < 64
+    return {hi << s | (lo >> 1) >> (63 - s), lo << s};
   }
 };
 __device__ __forceinline__ U128 warp_sum(U128 v) {

@@ -77,12 +77,14 @@ struct ColumnScalars {  // a column's scalars, written by one thread
   int z;           // u = column 2^z
   int skip;
   long long u0r, u0i, nint;
+  longlong2 sum;   // squares below the diagonal (uA^2; hi, lo)
 };
 
 struct Shared {
   longlong2 alpha[2];
   long long diag[2];                   // the column's diagonal entry
   long long trace;                     // of the rows not reduced yet (2^kTraceUnit uA)
+  longlong2 fro;                       // their squared Frobenius norm (2^kFroUnit uA^2; hi, lo)
   int tail_z[2], unit[2];              // the tail's shift after a column, the column's unit
   longlong2 norm[2][kMaxCl * kWarps];  // sums of squares (hi, lo) of every warp
   longlong2 spart[2 * kNb][kMaxCl];    // V^H u and W^H u, a partial per CTA
@@ -153,18 +155,53 @@ __device__ __forceinline__ void walker_sync() {
   }
 }
 
-// How far the trailing matrix may be scaled up once its trace (which bounds its
-// norm) has fallen: a low-entropy state leaves most of its weight in the first
-// columns, and the rest then keeps its precision. At most kMaxShift bits in all,
-// so that the rounding noise of the first columns, which is not positive
-// semidefinite, stays far below full scale.
-// The trace is kept in units of 2^kTraceUnit uA (n full-scale entries fit).
+// How far the trailing matrix may be scaled up once it has become small: a
+// low-entropy state leaves most of its weight in the first columns, and the rest
+// then keeps its precision. At most kMaxShift bits in all, so that the rounding
+// noise of the first columns stays far below full scale.
+// Two bounds on its norm, both followed exactly from column to column, the
+// smaller shift taken. The trace bounds the norm of a positive semidefinite
+// matrix and resolves it to the last bit. A Gram matrix of few digit planes is not
+// one: its truncation error, 2^-14 of the norm with 2 slices, can leave a
+// trailing trace near zero or below under a matrix that is not (with the trace
+// alone, 2 slices and K = 64, the entries for Schmidt weights 2^-i left the
+// 60-bit range and its eigenvalues were off by 1e-5 of the largest). The
+// Frobenius norm bounds any Hermitian matrix. A reflector does not change it, so
+// each column takes d^2 + 2 |e|^2 from its square, which resolves the norm to
+// about 2^-27: below the noise that kMaxShift allows for.
+// Units: n full-scale entries fit the trace, n of their squares the other.
 constexpr int kMaxShift = 24;
 constexpr int kTraceUnit = 10;
-__device__ __forceinline__ int rescale(long long trace, int shifted) {
-  // trace 2^z < 2^60 uA
-  const int z = trace > 0 ? __clzll(trace) - (64 - fx::kFull) - kTraceUnit : kMaxShift;
-  return max(0, min(z, kMaxShift - shifted));
+constexpr int kFroUnit = 12;
+__device__ __forceinline__ int rescale(long long trace, const fx::U128& fro, int shifted) {
+  // trace 2^z < 2^60 uA, and the same for the square root of fro
+  const int zt = trace > 0 ? __clzll(trace) - (64 - fx::kFull) - kTraceUnit : kMaxShift;
+  const int lz = fro.hi ? __clzll((long long)fro.hi) : 64 + __clzll((long long)fro.lo);
+  const int zf = lz > 0 ? (2 * fx::kFull - kFroUnit - 128 + lz) >> 1 : kMaxShift;  // (0: negative)
+  return max(0, min(min(zt, zf), kMaxShift - shifted));
+}
+
+__device__ __forceinline__ fx::U128 unpack(const longlong2& v) {
+  return {(unsigned long long)v.x, (unsigned long long)v.y};
+}
+__device__ __forceinline__ longlong2 pack(const fx::U128& v) {
+  return make_longlong2((long long)v.hi, (long long)v.lo);
+}
+
+// |x|^2 of the lower triangle's entry x, twice off the diagonal, and what a column with
+// diagonal d and the squares `below` under it takes from the trailing matrix.
+__device__ __forceinline__ fx::U128 fro_entry(long long re, long long im, bool diagonal) {
+  fx::U128 v;
+  v.add_square(re);
+  v.add_square(im);
+  return v.shifted_right(diagonal ? kFroUnit : kFroUnit - 1);
+}
+__device__ __forceinline__ fx::U128 fro_column(long long d, const longlong2& below) {
+  fx::U128 v;
+  v.add_square(d);
+  v.add((unsigned long long)below.x, (unsigned long long)below.y);
+  v.add((unsigned long long)below.x, (unsigned long long)below.y);
+  return v.shifted_right(kFroUnit);
 }
 
 // The reflector of a column (alpha, x...) with |x|^2 = sum: beta = -+N, N the
@@ -172,14 +209,14 @@ __device__ __forceinline__ int rescale(long long trace, int shifted) {
 // [2^58, 2^59).
 __device__ __forceinline__ ColumnScalars reflector(const fx::U128& sum, long long alr,
                                                    long long ali) {
-  ColumnScalars sc{0, 0, 0, 0, 0};
+  fx::U128 all = sum;
+  all.add_square(alr);
+  all.add_square(ali);
+  ColumnScalars sc{0, 0, 0, 0, 0, pack(all)};
   if (sum.hi == 0 && sum.lo == 0 && ali == 0) {
     sc.skip = 1;  // already reduced: H = I
     return sc;
   }
-  fx::U128 all = sum;
-  all.add_square(alr);
-  all.add_square(ali);
   sc.nint = fx::sqrt_scaled(all, &sc.z);
   const long long xr = fx::shift(alr, sc.z);
   sc.u0r = alr < 0 ? xr - sc.nint : xr + sc.nint;
@@ -336,9 +373,14 @@ __device__ __forceinline__ void reduce(Red& R, int cend) {
       }
       __syncthreads();
       const ColumnScalars sc = S.sc;
-      if (rank == 0 && t == kThreads - 32) {
-        R.d[c] = fx::to_double(S.diag[par], eunit);
-        R.e[c] = column_beta(sc, S.alpha[par].x, eunit);
+      if (t == kThreads - 32) {
+        fx::U128 fro = unpack(S.fro);
+        fro.subtract(fro_column(S.diag[par], sc.sum));
+        S.fro = pack(fro);
+        if (rank == 0) {
+          R.d[c] = fx::to_double(S.diag[par], eunit);
+          R.e[c] = column_beta(sc, S.alpha[par].x, eunit);
+        }
       }
       // u to every CTA; V's column i
       for (int k = warp; k < kmax; k += kWarps) {
@@ -510,7 +552,7 @@ __device__ __forceinline__ void reduce(Red& R, int cend) {
     // ---- trailing update on rows and columns q0 ..: a warp per 32 rows x
     // kStrip columns of the lower triangle, written to both triangles
     const int q0 = p0 + nbp;
-    const int z = rescale(S.trace, R.shifted);
+    const int z = rescale(S.trace, unpack(S.fro), R.shifted);
     R.shifted += z;
     eunit -= z;
     {
@@ -587,7 +629,10 @@ __device__ __forceinline__ void reduce(Red& R, int cend) {
       }
     }
     walker_sync<MULTI>();
-    if (t == 0) S.trace <<= z;
+    if (t == 0) {
+      S.trace <<= z;
+      S.fro = pack(unpack(S.fro).shifted_left(2 * z));
+    }
   }
   R.eunit = eunit;
 }
@@ -608,6 +653,7 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
   constexpr int kRows = kTail / 32;  // rows per lane of warp 0
   constexpr int ld = kTailLd;
   long long trace = S.trace;  // (warp 0's)
+  fx::U128 fro = unpack(S.fro);
   for (int c = 0; c < n; ++c) {
     const int z = c > 0 ? S.tail_z[(c - 1) & 1] : 0;  // the previous column's update is scaled up by 2^z
     int4* u = us + (c & 1) * kTail;
@@ -643,6 +689,7 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
         }
       }
       trace <<= z;
+      fro = fro.shifted_left(2 * z);
       eunit -= z;
       if (c < n - 1) {
         sq = fx::warp_sum(sq);
@@ -672,7 +719,8 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
             u[r] = v;
           }
         }
-        const int zn = rescale(trace, shifted);
+        fro.subtract(fro_column(dr, sc.sum));
+        const int zn = rescale(trace, fro, shifted);
         shifted += zn;
         if (lane == 0) {
           S.sc = sc;
@@ -886,6 +934,7 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
   int4* tail_ws = tail_us + 2 * kTail;                          // kTail
   longlong2* tail_part = reinterpret_cast<longlong2*>(tail_ws + kTail);
   int4* tail_A = reinterpret_cast<int4*>(tail_part + kWarps * 32);  // kTail x kTailLd
+  fx::U128 fro;
   {
     int4* A = SMALL ? tail_A : reinterpret_cast<int4*>(G);
     const int ld = SMALL ? kTailLd : n;
@@ -910,14 +959,25 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
           if (r >= n || cc > r) continue;
           const long long re = fx::from_double(z[x].x, -eunit);
           const long long im = r == cc ? 0 : fx::from_double(z[x].y, -eunit);
+          const fx::U128 sq = fro_entry(re, im, r == cc);
+          fro.add(sq.hi, sq.lo);
           A[r + (size_t)cc * ld] = fx::pack(re, im);
           if (r != cc) A[cc + (size_t)r * ld] = fx::pack(re, -im);
         }
       }
     }
   }
+  fro = fx::warp_sum(fro);
+  if (lane == 0)  // (norm[1]: column 0 uses norm[0])
+    publish<MULTI>(&S.norm[1][rank * kWarps + warp], (long long)fro.hi, (long long)fro.lo, cl);
   walker_sync<MULTI>();
   if (warp == 0) {
+    fro = fx::U128();
+    for (int x = lane; x < cl * kWarps; x += 32) {
+      const longlong2 v = S.norm[1][x];
+      fro.add((unsigned long long)v.x, (unsigned long long)v.y);
+    }
+    fro = fx::warp_sum(fro);
     const int4* A = SMALL ? tail_A : reinterpret_cast<int4*>(G);
     const int ld = SMALL ? kTailLd : n;
     long long tr0 = 0;
@@ -926,7 +986,10 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
       tr0 += fx::join(v.x, v.y) >> kTraceUnit;
     }
     tr0 = fx::warp_sum(tr0);
-    if (lane == 0) S.trace = tr0;
+    if (lane == 0) {
+      S.trace = tr0;
+      S.fro = pack(fro);
+    }
     __syncwarp();
   }
   R.shifted = 0;
