@@ -1482,7 +1482,7 @@ bg_status entropy_plan(bg_plan** out, int64_t walkers, int32_t spins, int32_t sp
     }
     p->workspace_bytes = p->gram->workspace_bytes + (int64_t)(gb + 2 * tb);
     p->launches_per_call = p->gram->launches_per_call + 3;
-    if ((e = tri_shape(walkers, (int)K, &p->tri)) != cudaSuccess) {
+    if ((e = tri_shape(walkers, (int)K, ctx->sms, &p->tri)) != cudaSuccess) {
       destroy_plan(p);
       return cuda_fail(e, "entropy plan");
     }

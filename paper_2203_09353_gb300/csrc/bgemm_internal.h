@@ -160,13 +160,14 @@ bg_status static_scratch(void** out, size_t* bytes, std::string* err);
 // of device memory, or null where that is 0.
 struct TriShape {
   int cl = 1;        // CTAs per walker
+  int warps = 0;     // warps per CTA
   int own = 0;       // rows a CTA owns at most
   bool vws = true;   // the panel's own rows are in shared memory
   size_t smem = 0;   // dynamic shared memory of a CTA
   size_t panel = 0;  // bytes of panel vectors per walker in device memory
 };
 // (also sets the kernels' shared-memory limits on the current device)
-cudaError_t tri_shape(int64_t walkers, int n, TriShape* out);
+cudaError_t tri_shape(int64_t walkers, int n, int sms, TriShape* out);
 cudaError_t launch_tridiag(double2* gram, int64_t walkers, int n, const TriShape& shape,
                            void* panel, double* d, double* e, cudaStream_t st);
 

@@ -369,42 +369,63 @@ __global__ void __launch_bounds__(kBisThreads) bisect_kernel(const double* d, co
   if (store) lam[at] = scalbn(0.5 * (a + b), ex);
 }
 
-// S = -sum p ln p over p = lambda / sum(lambda) > 0, a CTA per walker; eigs
+// S = -sum p ln p over p = lambda / sum(lambda) > 0, T threads per walker: a CTA,
+// or a warp where n <= 32 (16000 walkers of order 2: 254 us with a CTA each); eigs
 // (optional) receives the eigenvalues in ascending order: two that lie within
 // the bisection's tolerance of each other may come in either order, so each
 // takes the largest value up to it.
-__global__ void __launch_bounds__(kEntThreads) entropy_sum_kernel(const double* lam, int n,
-                                                                  double* entropy, double* eigs) {
+template <int T>
+__global__ void __launch_bounds__(kEntThreads)
+    entropy_sum_kernel(const double* lam, int64_t walkers, int n, double* entropy, double* eigs) {
+  static_assert(T == 32 || T == kEntThreads, "a warp or the CTA per walker");
+  constexpr bool kWarp = T == 32;
   __shared__ double red[kEntThreads / 32];
   __shared__ double top[2][kEntThreads];
-  const int t = threadIdx.x, T = kEntThreads;
-  const double* l = lam + (size_t)blockIdx.x * n;
+  const int t = threadIdx.x % T;
+  const int64_t w = blockIdx.x * (int64_t)(kEntThreads / T) + threadIdx.x / T;
+  if (w >= walkers) return;
+  auto sum = [&](double v) {
+    if constexpr (!kWarp) return block_sum(v, red);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+  };
+  const double* l = lam + (size_t)w * n;
   double tot = 0.0;
   for (int k = t; k < n; k += T) tot += l[k];
-  tot = block_sum(tot, red);
+  tot = sum(tot);
   double s = tot != tot ? tot : 0.0;
   for (int k = t; k < n; k += T) {
     const double p = tot > 0.0 ? l[k] / tot : 0.0;
     if (p > 0.0) s -= p * log(p);
   }
-  s = block_sum(s, red);
-  if (t == 0) entropy[blockIdx.x] = s;
+  s = sum(s);
+  if (t == 0) entropy[w] = s;
   if (!eigs) return;
   const int per = (n + T - 1) / T, k0 = t * per, k1 = min(n, k0 + per);
   double m = -DBL_MAX;
   for (int k = k0; k < k1; ++k) m = fmax(m, l[k]);
-  top[0][t] = m;
-  __syncthreads();
-  int cur = 0;
-  for (int o = 1; o < T; o <<= 1, cur ^= 1) {  // inclusive running maximum over the threads
-    top[cur ^ 1][t] = t >= o ? fmax(top[cur][t], top[cur][t - o]) : top[cur][t];
+  // running maximum over the threads before this one
+  if constexpr (kWarp) {
+    for (int o = 1; o < 32; o <<= 1) {
+      const double v = __shfl_up_sync(0xFFFFFFFFu, m, o);
+      if (t >= o) m = fmax(m, v);
+    }
+    m = __shfl_up_sync(0xFFFFFFFFu, m, 1);
+  } else {
+    top[0][t] = m;
     __syncthreads();
+    int cur = 0;
+    for (int o = 1; o < T; o <<= 1, cur ^= 1) {
+      top[cur ^ 1][t] = t >= o ? fmax(top[cur][t], top[cur][t - o]) : top[cur][t];
+      __syncthreads();
+    }
+    m = t > 0 ? top[cur][t - 1] : 0.0;
   }
-  m = t > 0 ? top[cur][t - 1] : -DBL_MAX;
+  if (t == 0) m = -DBL_MAX;
   for (int k = k0; k < k1; ++k) {
     const double v = l[k];
     m = fmax(m, v);
-    eigs[(size_t)blockIdx.x * n + k] = v != v ? v : m;
+    eigs[(size_t)w * n + k] = v != v ? v : m;
   }
 }
 
@@ -444,7 +465,12 @@ cudaError_t launch_entropy_bisect(const double* d, const double* e, int64_t walk
                     : per_sm <= 40 ? bisect_launch<4>(d, e, walkers, n, lam, st)
                                    : bisect_launch<2>(d, e, walkers, n, lam, st);
   if (err != cudaSuccess) return err;
-  entropy_sum_kernel<<<(unsigned)walkers, kEntThreads, 0, st>>>(lam, n, entropy, eigs);
+  if (n <= 32)
+    entropy_sum_kernel<32><<<(unsigned)((walkers + kEntThreads / 32 - 1) / (kEntThreads / 32)),
+                             kEntThreads, 0, st>>>(lam, walkers, n, entropy, eigs);
+  else
+    entropy_sum_kernel<kEntThreads><<<(unsigned)walkers, kEntThreads, 0, st>>>(lam, walkers, n,
+                                                                             entropy, eigs);
   count_launch();
   return cudaGetLastError();
 }

@@ -57,7 +57,14 @@ constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kNb = 16;       // panel width
 constexpr int kTail = 96;     // columns reduced with the matrix in shared memory
-constexpr int kTailLd = kTail + 1;
+// Orders up to kPacked of more walkers than SMs: several CTAs of fewer warps per
+// SM. With the shared memory and threads of order 96 an SM held one walker at a
+// time, whatever its order: 16000 matrices of order 2 took 0.90 ms where the FP64
+// kernel before it took 0.45. Whole calls, with one CTA and with five per SM:
+// 16000 of order 2 2290 -> 1340 us (FP64 kernel: 1730), of 8 4400 -> 2160 us, of 32
+// 17.5 -> 10.1 ms, 153 of order 32 350 -> 256 us. Up to one walker per SM the 16
+// warps are no slower and are kept.
+constexpr int kPacked = 32, kPackedWarps = 4, kPackedCtas = 5;
 constexpr int kStrip = 4;     // columns per update work item
 constexpr int kMaxCl = 8;
 constexpr float kScaleRoom = 1.4f;
@@ -373,15 +380,17 @@ __device__ __forceinline__ void reduce(Red& R, int cend) {
       }
       __syncthreads();
       const ColumnScalars sc = S.sc;
-      if (t == kThreads - 32) {
+      // the column's results, beside step 4 (by a warp with few rows there or none)
+      auto finish_column = [&]() {
+        if (t != kThreads - 32) return;
         fx::U128 fro = unpack(S.fro);
-        fro.subtract(fro_column(S.diag[par], sc.sum));
+        fro.subtract(fro_column(S.diag[par], S.sc.sum));
         S.fro = pack(fro);
         if (rank == 0) {
           R.d[c] = fx::to_double(S.diag[par], eunit);
-          R.e[c] = column_beta(sc, S.alpha[par].x, eunit);
+          R.e[c] = column_beta(S.sc, S.alpha[par].x, eunit);
         }
-      }
+      };
       // u to every CTA; V's column i
       for (int k = warp; k < kmax; k += kWarps) {
         const int r = 32 * (rank + cl * k) + lane, lr = 32 * k + lane;
@@ -417,6 +426,7 @@ __device__ __forceinline__ void reduce(Red& R, int cend) {
       };
       if (sc.skip) {
         publish_row();
+        finish_column();
         if (t == 0) S.rowV[i] = S.rowW[i] = make_int4(0, 0, 0, 0);
         walker_sync<MULTI>();
         continue;
@@ -526,6 +536,7 @@ __device__ __forceinline__ void reduce(Red& R, int cend) {
       rho = fx::warp_sum(rho);
       if (lane == 0) publish<MULTI>(&S.rho[rank * kWarps + warp], rho, cl);
       publish_row();
+      finish_column();
       walker_sync<MULTI>();
       // ---- 5. w = p - (|tau|^2 rho / 2) u
       rho = 0;
@@ -637,27 +648,29 @@ __device__ __forceinline__ void reduce(Red& R, int cend) {
   R.eunit = eunit;
 }
 
-// The reduction of a matrix of order n <= kTail held in shared memory (both
-// triangles, leading dimension kTailLd), column by column: at this order the
-// columns are bound by latency, not by the products, so warp 0 takes the
-// chain from one column to the next alone (its 3 rows per lane need no
-// barrier) and three barriers part it from what the other warps do: the
+// The reduction of a matrix of order n <= 32 ROWS held in shared memory (both
+// triangles, leading dimension 32 ROWS + 1) by W warps, column by column: at
+// this order the columns are bound by latency, not by the products, so warp 0
+// takes the chain from one column to the next alone (its ROWS rows per lane
+// need no barrier) and three barriers part it from what the other warps do: the
 // rank-2 update of the previous column beside the norm, square root and u of
 // this one, then the product A u beside tau, then w. (As panels of 16 columns
 // in the general routine, the last 96 columns took 16 k clocks each; here
 // 8 k.) us: u of this column and the last, ws: w.
+template <int ROWS, int W>
 __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, longlong2* part,
                                             double* d, double* e, int eunit, int shifted,
-                                           Shared& S) {
+                                            Shared& S) {
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  constexpr int kRows = kTail / 32;  // rows per lane of warp 0
-  constexpr int ld = kTailLd;
-  long long trace = S.trace;  // (warp 0's)
-  fx::U128 fro = unpack(S.fro);
+  constexpr int kRows = ROWS;  // rows per lane of warp 0
+  constexpr int N = 32 * ROWS, ld = N + 1;
+  long long trace = 0;  // (these two in the thread that chooses the next shift)
+  fx::U128 fro;
   for (int c = 0; c < n; ++c) {
-    const int z = c > 0 ? S.tail_z[(c - 1) & 1] : 0;  // the previous column's update is scaled up by 2^z
-    int4* u = us + (c & 1) * kTail;
-    const int4* up = us + ((c & 1) ^ 1) * kTail;
+    // (the previous column's update is scaled up by 2^z)
+    const int z = c > 0 ? S.tail_z[(c - 1) & 1] : 0;
+    int4* u = us + (c & 1) * N;
+    const int4* up = us + ((c & 1) ^ 1) * N;
     if (warp == 0) {
       // ---- column c, with the previous column's update
       fx::U128 sq;
@@ -688,8 +701,6 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
           }
         }
       }
-      trace <<= z;
-      fro = fro.shifted_left(2 * z);
       eunit -= z;
       if (c < n - 1) {
         sq = fx::warp_sum(sq);
@@ -704,7 +715,6 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
           }
         }
         dr = __shfl_sync(0xFFFFFFFFu, dr, c & 31);
-        trace -= dr >> kTraceUnit;
         ar = __shfl_sync(0xFFFFFFFFu, ar, (c + 1) & 31);
         ai = __shfl_sync(0xFFFFFFFFu, ai, (c + 1) & 31);
         const ColumnScalars sc = reflector(sq, ar, ai);
@@ -719,12 +729,8 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
             u[r] = v;
           }
         }
-        fro.subtract(fro_column(dr, sc.sum));
-        const int zn = rescale(trace, fro, shifted);
-        shifted += zn;
         if (lane == 0) {
           S.sc = sc;
-          S.tail_z[c & 1] = zn;
           S.alpha[c & 1] = make_longlong2(ar, dr);
           S.unit[c & 1] = eunit;
         }
@@ -743,7 +749,7 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
       // above c: a warp per pair of columns j, m - 1 - j (m + 1 elements
       // below and on the diagonal together)
       const int b0 = c + 1, m = n - b0;
-      for (int j = warp - 1; 2 * j < m; j += kWarps - 1) {
+      for (int j = warp - 1; 2 * j < m; j += W - 1) {
         const int first = m - j, len = 2 * j == m - 1 ? first : m + 1;
         for (int x = lane; x < len; x += 32) {
           const int cc = b0 + (x < first ? j : m - 1 - j);
@@ -764,18 +770,28 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
     const ColumnScalars sc = S.sc;
     const int m = n - c - 1;
     const int g0 = (c + 1) >> 5, cnt = ((n + 31) >> 5) - g0;  // groups of 32 rows with one > c
-    const int nch = (kWarps - 1) / cnt;
-    if (t == kThreads - 64) {  // (a warp that seldom has a share of the product)
-      d[c] = fx::to_double(S.alpha[c & 1].y, S.unit[c & 1]);
+    const int nch = (W - 1) / cnt;
+    // the column's results and the next shift, by a warp that has no part in w
+    auto finish_column = [&]() {
+      if (t != 32 * W - 64) return;
+      const long long dr = S.alpha[c & 1].y;
+      trace = (c > 0 ? trace << z : S.trace) - (dr >> kTraceUnit);
+      fro = c > 0 ? fro.shifted_left(2 * z) : unpack(S.fro);
+      fro.subtract(fro_column(dr, sc.sum));
+      const int zn = rescale(trace, fro, shifted);
+      shifted += zn;
+      S.tail_z[c & 1] = zn;
+      d[c] = fx::to_double(dr, S.unit[c & 1]);
       e[c] = column_beta(sc, S.alpha[c & 1].x, S.unit[c & 1]);
-    }
+    };
     if (sc.skip) {  // H = I: w = 0 like u
       if (warp == 0)
         for (int r = c + 1 + lane; r < n; r += 32) ws[r] = make_int4(0, 0, 0, 0);
+      finish_column();
       __syncthreads();
       continue;
     }
-    if (warp == kWarps - 1) {
+    if (warp == W - 1) {
       if (lane == 0) reflector_tau(sc, &S.tau, &S.t2);
     } else if (warp < cnt * nch) {
       // ---- y = A u: one group of rows x a run of columns
@@ -791,6 +807,7 @@ __device__ __forceinline__ void reduce_tail(int4* A, int n, int4* us, int4* ws, 
       part[warp * 32 + lane] = make_longlong2(s.re(), s.im());
     }
     __syncthreads();
+    finish_column();
     if (warp == 0) {
       // ---- p = tau y, rho, w
       const int4 tau = S.tau;
@@ -837,16 +854,18 @@ __device__ __forceinline__ float scaled_abs(double x, int e) {
   return __int_as_float((ef << 23) | (int)((h & 0xFFFFFu) << 3));
 }
 
-// The whole reduction of walker blockIdx.x / cl. SMALL: n <= kTail, the
-// matrix goes straight to shared memory. Bound by the multiply pipe (76-80%
+// The whole reduction of walker blockIdx.x / cl by W warps. ROWS: n <= 32 ROWS,
+// the matrix goes straight to shared memory (0: any order above kTail). Bound by the multiply pipe (76-80%
 // busy at n = 256, with 1.6 times the products' own instructions) and, in the
 // last columns and for few walkers, by the latency of a column. Measured
 // against panels with an FP64 product, split GEMMs between them and an FP64
 // kernel for the last 64 columns: 128 matrices of order 256 12.6 -> 5.3 ms, 16
 // of 1024 382 -> 52.8 ms (6 CTAs each), 4 of 64 0.89 -> 0.25 ms; against the
 // FP64 kernel alone 32 of 128 4.5 -> 1.0 ms.
-template <bool MULTI, bool VWS, bool SMALL>
-__global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g) {
+template <bool MULTI, bool VWS, int ROWS, int W>
+__global__ void __launch_bounds__(32 * W, W < kWarps ? kPackedCtas : 1) tri_reduce_kernel(const TriArgs g) {
+  static_assert(W == kWarps || (ROWS > 0 && !MULTI), "reduce() takes kWarps warps");
+  constexpr bool SMALL = ROWS > 0;
   extern __shared__ __align__(16) int4 sm4[];
   __shared__ Shared S;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -863,16 +882,16 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
   // ---- the scale: with t the mean eigenvalue (trace / n), the largest one is
   // at most t + sqrt((n - 1) (||G||_F^2 / n - t^2))
   double dm = 0.0;
-  for (int i = t; i < n; i += kThreads) dm = fmax(dm, fabs(__ldcg(&G[i + (size_t)i * n].x)));
+  for (int i = t; i < n; i += 32 * W) dm = fmax(dm, fabs(__ldcg(&G[i + (size_t)i * n].x)));
   for (int o = 16; o > 0; o >>= 1) dm = fmax(dm, __shfl_xor_sync(0xFFFFFFFFu, dm, o));
   if (lane == 0) S.dred[warp] = dm;
   walker_sync<MULTI>();  // also: every CTA of the cluster runs before its memory is written
   dm = 0.0;
-  for (int i = 0; i < kWarps; ++i) dm = fmax(dm, S.dred[i]);
+  for (int i = 0; i < W; ++i) dm = fmax(dm, S.dred[i]);
   const int e0 = dm > 0.0 ? (int)((__double2hiint(dm) >> 20) & 0x7FF) - 1022 : 0;
   const int ngroups = (n + 31) >> 5;
   float f2 = 0.0f, tr = 0.0f;
-  for (int idx = rank * kWarps + warp; idx < n; idx += cl * kWarps) {
+  for (int idx = rank * W + warp; idx < n; idx += cl * W) {
     // a warp per column, its lower part
     for (int r = idx + lane; r < n; r += 32) {
       const double2 z = __ldcg(&G[r + (size_t)idx * n]);
@@ -890,7 +909,7 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
     if constexpr (MULTI) {
       for (int x = 0; x < cl; ++x)
         asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(
-                         mapa(smem_addr(&S.fsum[rank * kWarps + warp]), x)),
+                         mapa(smem_addr(&S.fsum[rank * W + warp]), x)),
                      "f"(f2), "f"(tr)
                      : "memory");
     } else {
@@ -899,7 +918,7 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
   }
   walker_sync<MULTI>();
   float F2 = 0.0f, mean = 0.0f;
-  for (int x = 0; x < cl * kWarps; ++x) {
+  for (int x = 0; x < cl * W; ++x) {
     F2 += S.fsum[x].x;
     mean += S.fsum[x].y;
   }
@@ -907,7 +926,7 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
   if (!(F2 < __int_as_float(0x7F800000))) {  // a NaN or infinity in G
     const double nan = __longlong_as_double(0x7FF8000000000000ll);
     if (rank == 0)
-      for (int i = t; i < n; i += kThreads) {
+      for (int i = t; i < n; i += 32 * W) {
         dw[i] = nan;
         ew[i] = i + 1 < n ? nan : 0.0;
       }
@@ -928,17 +947,18 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
   R.d = dw;
   R.e = ew;
   int4* sm = sm4;
+  constexpr int kOrder = SMALL ? 32 * ROWS : kTail, kLd = kOrder + 1;
   const int nt = SMALL ? n : kTail;
   // ---- fixed point, both triangles (in place, or into shared memory)
-  int4* tail_us = sm;                                           // 2 kTail
-  int4* tail_ws = tail_us + 2 * kTail;                          // kTail
-  longlong2* tail_part = reinterpret_cast<longlong2*>(tail_ws + kTail);
-  int4* tail_A = reinterpret_cast<int4*>(tail_part + kWarps * 32);  // kTail x kTailLd
+  int4* tail_us = sm;                                        // 2 kOrder
+  int4* tail_ws = tail_us + 2 * kOrder;                      // kOrder
+  longlong2* tail_part = reinterpret_cast<longlong2*>(tail_ws + kOrder);
+  int4* tail_A = reinterpret_cast<int4*>(tail_part + W * 32);  // kOrder x kLd
   fx::U128 fro;
   {
     int4* A = SMALL ? tail_A : reinterpret_cast<int4*>(G);
-    const int ld = SMALL ? kTailLd : n;
-    const int nw = cl * kWarps, gw = rank * kWarps + warp;
+    const int ld = SMALL ? kLd : n;
+    const int nw = cl * W, gw = rank * W + warp;
     int base = 0;
     for (int I = 0; I < ngroups; ++I) {
       const int cntI = (min(32 * I + 32, n) + kStrip - 1) / kStrip;
@@ -969,17 +989,17 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
   }
   fro = fx::warp_sum(fro);
   if (lane == 0)  // (norm[1]: column 0 uses norm[0])
-    publish<MULTI>(&S.norm[1][rank * kWarps + warp], (long long)fro.hi, (long long)fro.lo, cl);
+    publish<MULTI>(&S.norm[1][rank * W + warp], (long long)fro.hi, (long long)fro.lo, cl);
   walker_sync<MULTI>();
   if (warp == 0) {
     fro = fx::U128();
-    for (int x = lane; x < cl * kWarps; x += 32) {
+    for (int x = lane; x < cl * W; x += 32) {
       const longlong2 v = S.norm[1][x];
       fro.add((unsigned long long)v.x, (unsigned long long)v.y);
     }
     fro = fx::warp_sum(fro);
     const int4* A = SMALL ? tail_A : reinterpret_cast<int4*>(G);
-    const int ld = SMALL ? kTailLd : n;
+    const int ld = SMALL ? kLd : n;
     long long tr0 = 0;
     for (int i = lane; i < n; i += 32) {
       const int4 v = SMALL ? A[i + i * ld] : __ldcg(A + i + (size_t)i * ld);
@@ -1007,18 +1027,18 @@ __global__ void __launch_bounds__(kThreads, 1) tri_reduce_kernel(const TriArgs g
     reduce<MULTI, VWS>(R, n - kTail);  // ends with a barrier of the walker
     if (rank != 0) return;
     const int4* A0 = R.A + (n - kTail) + (size_t)(n - kTail) * n;
-    for (int x = t; x < kTail * kTail; x += kThreads) {
+    for (int x = t; x < kTail * kTail; x += 32 * W) {
       const int r = x % kTail, c = x / kTail;
-      tail_A[r + c * kTailLd] = __ldcg(A0 + r + (size_t)c * n);
+      tail_A[r + c * kLd] = __ldcg(A0 + r + (size_t)c * n);
     }
     __syncthreads();
   }
-  reduce_tail(tail_A, nt, tail_us, tail_ws, tail_part, dw + (n - nt), ew + (n - nt), R.eunit,
+  reduce_tail<kOrder / 32, W>(tail_A, nt, tail_us, tail_ws, tail_part, dw + (n - nt), ew + (n - nt), R.eunit,
               R.shifted, S);
 }
 
-constexpr size_t tail_smem() {
-  return ((size_t)3 * kTail + (size_t)kWarps * 32 + (size_t)kTail * kTailLd) * 16;
+constexpr size_t tail_smem(int order, int warps) {
+  return ((size_t)3 * order + (size_t)warps * 32 + (size_t)order * (order + 1)) * 16;
 }
 
 // The largest shared-memory request of any order. The limit is a property of
@@ -1027,10 +1047,11 @@ constexpr size_t tail_smem() {
 constexpr size_t kSmemLimit = kSmemMax - sizeof(Shared) - 512;
 
 // What an order-n reduction on clusters of cl CTAs asks for.
-TriShape shape_for(int n, int cl) {
+TriShape shape_for(int n, int cl, bool packed) {
   TriShape s;
+  s.warps = packed ? kPackedWarps : kWarps;
   if (n <= kTail) {
-    s.smem = tail_smem();
+    s.smem = packed ? tail_smem(kPacked, kPackedWarps) : tail_smem(kTail, kWarps);
     return s;
   }
   s.cl = cl;
@@ -1040,7 +1061,7 @@ TriShape shape_for(int n, int cl) {
   const size_t vw = (size_t)2 * kNb * s.own * 16;
   const size_t stage = (size_t)kWarps * 2 * kNb * kStrip * 16;
   s.vws = fixed + vw + (cl > 1 ? stage : 0) <= kSmemLimit;
-  s.smem = std::max(tail_smem(), fixed + (s.vws ? vw : 0) + (cl > 1 || !s.vws ? stage : 0));
+  s.smem = std::max(tail_smem(kTail, kWarps), fixed + (s.vws ? vw : 0) + (cl > 1 || !s.vws ? stage : 0));
   s.panel = cl > 1 || !s.vws ? (size_t)2 * kNb * n * sizeof(int4) : 0;
   return s;
 }
@@ -1048,7 +1069,7 @@ TriShape shape_for(int n, int cl) {
 void launch_config(const TriShape& s, int64_t walkers, cudaStream_t st, cudaLaunchConfig_t* cfg,
                    cudaLaunchAttribute* at) {
   cfg->gridDim = dim3((unsigned)(walkers * s.cl));
-  cfg->blockDim = dim3(kThreads);
+  cfg->blockDim = dim3((unsigned)s.warps * 32);
   cfg->dynamicSmemBytes = s.smem;
   cfg->stream = st;
   at->id = cudaLaunchAttributeClusterDimension;
@@ -1059,23 +1080,25 @@ void launch_config(const TriShape& s, int64_t walkers, cudaStream_t st, cudaLaun
   cfg->numAttrs = s.cl > 1 ? 1 : 0;
 }
 
-template <bool MULTI, bool VWS, bool SMALL>
+template <bool MULTI, bool VWS, int ROWS, int W = kWarps>
 cudaError_t launch_reduce(const TriArgs& a, int64_t walkers, const TriShape& s, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
   launch_config(s, walkers, st, &cfg, at);
-  const cudaError_t err = cudaLaunchKernelEx(&cfg, tri_reduce_kernel<MULTI, VWS, SMALL>, a);
+  const cudaError_t err = cudaLaunchKernelEx(&cfg, tri_reduce_kernel<MULTI, VWS, ROWS, W>, a);
   if (err != cudaSuccess) return err;
   count_launch();
   return cudaGetLastError();
 }
 
 cudaError_t set_smem_limits() {
-  const void* kernels[] = {(const void*)tri_reduce_kernel<false, true, true>,
-                           (const void*)tri_reduce_kernel<true, true, false>,
-                           (const void*)tri_reduce_kernel<true, false, false>,
-                           (const void*)tri_reduce_kernel<false, true, false>,
-                           (const void*)tri_reduce_kernel<false, false, false>};
+  // (the packed kernel's request needs no raised limit)
+  static_assert(tail_smem(kPacked, kPackedWarps) + sizeof(Shared) <= 48 * 1024, "packed CTA");
+  const void* kernels[] = {(const void*)tri_reduce_kernel<false, true, kTail / 32, kWarps>,
+                           (const void*)tri_reduce_kernel<true, true, 0, kWarps>,
+                           (const void*)tri_reduce_kernel<true, false, 0, kWarps>,
+                           (const void*)tri_reduce_kernel<false, true, 0, kWarps>,
+                           (const void*)tri_reduce_kernel<false, false, 0, kWarps>};
   for (const void* k : kernels) {
     const cudaError_t e =
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
@@ -1104,10 +1127,11 @@ int tri_cluster(int64_t walkers, int n) {
       cudaLaunchAttribute at[1];
       TriShape s;
       s.cl = cl;
+      s.warps = kWarps;
       s.smem = kSmemLimit;
       int c = 0;
       launch_config(s, 1, nullptr, &cfg, at);
-      if (cudaOccupancyMaxActiveClusters(&c, tri_reduce_kernel<true, true, false>, &cfg) !=
+      if (cudaOccupancyMaxActiveClusters(&c, tri_reduce_kernel<true, true, 0, kWarps>, &cfg) !=
           cudaSuccess) {
         cudaGetLastError();
         return 1;
@@ -1121,9 +1145,10 @@ int tri_cluster(int64_t walkers, int n) {
 
 }  // namespace
 
-cudaError_t tri_shape(int64_t walkers, int n, TriShape* out) {
+cudaError_t tri_shape(int64_t walkers, int n, int sms, TriShape* out) {
   const cudaError_t e = set_smem_limits();
-  *out = shape_for(n, e == cudaSuccess ? tri_cluster(walkers, n) : 1);
+  *out = shape_for(n, e == cudaSuccess ? tri_cluster(walkers, n) : 1,
+                   n <= kPacked && walkers > sms);
   return e;
 }
 
@@ -1131,12 +1156,14 @@ cudaError_t launch_tridiag(double2* gram, int64_t walkers, int n, const TriShape
                            double* d, double* e, cudaStream_t st) {
   if (walkers <= 0) return cudaSuccess;
   const TriArgs a{gram, static_cast<int4*>(panel), d, e, n, s.own};
-  if (n <= kTail) return launch_reduce<false, true, true>(a, walkers, s, st);
+  if (s.warps < kWarps)
+    return launch_reduce<false, true, kPacked / 32, kPackedWarps>(a, walkers, s, st);
+  if (n <= kTail) return launch_reduce<false, true, kTail / 32>(a, walkers, s, st);
   if (s.cl > 1)
-    return s.vws ? launch_reduce<true, true, false>(a, walkers, s, st)
-                 : launch_reduce<true, false, false>(a, walkers, s, st);
-  return s.vws ? launch_reduce<false, true, false>(a, walkers, s, st)
-               : launch_reduce<false, false, false>(a, walkers, s, st);
+    return s.vws ? launch_reduce<true, true, 0>(a, walkers, s, st)
+                 : launch_reduce<true, false, 0>(a, walkers, s, st);
+  return s.vws ? launch_reduce<false, true, 0>(a, walkers, s, st)
+               : launch_reduce<false, false, 0>(a, walkers, s, st);
 }
 
 }  // namespace bg

@@ -15,10 +15,10 @@ int main() {
   for (int n = 2; n <= 1024; n *= 2)
     for (long walkers : {0L, 1L, 4L, 16L, 76L, 65535L}) {
       bg::TriShape s;
-      bg::tri_shape(walkers, n, &s);
+      bg::tri_shape(walkers, n, 152, &s);
       const bool device_panel = n > 96 && (s.cl > 1 || !s.vws);
       bad += (s.panel > 0) != device_panel || s.panel % 16 != 0;
-      bad += s.smem == 0 || s.smem > 227 * 1024 || s.cl < 1 || s.cl > 8;
+      bad += s.warps < 4 || s.smem == 0 || s.smem > 227 * 1024 || s.cl < 1 || s.cl > 8;
       bad += n > 96 && (long)s.own * s.cl < n;
     }
   printf("%d\n", bad);
