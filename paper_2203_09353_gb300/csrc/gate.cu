@@ -19,18 +19,23 @@
 // copy bandwidth. In fixed point (fixed60.cuh), with three real products per
 // complex one (Gauss's form), it is 36 integer multiply-adds, 1.1 clocks,
 // where the copy bandwidth allows 1.4; with the conversions around them it
-// measured 0.98 ms, 65% of the copy bandwidth (four real products: 1.04 ms).
+// measured 0.97 ms, 65% of the copy bandwidth (four real products: 1.04 ms).
 // A group's four amplitudes get one exponent, 59 bits below the largest
-// component, the gate another; the sums are cut at 2^-59 of full scale and
-// rounded once to FP64.
+// component (2^E above it), the gate's entries another (2^EU); the sums are in
+// units of 2^(E + EU - 58), rounded to nearest and then once more to FP64.
 //
-// That error is absolute: about 2^-60 of the group's largest component. The
-// FP64 chain's is about 2^-54 of the sum of |U| |psi| over a row, so the fixed
-// form is no less exact as long as no entry of U is below 2^-6 of the
-// largest: a gate with smaller or zero entries (a permutation, a controlled
-// gate, 1% of random ones) keeps the FP64 chain for its walker, exact where
-// its entries are. So do groups with an infinity, a NaN or magnitudes within
-// a factor 2^300 of the ends of the range.
+// The error before that last rounding comes from the cut of the operands to 59
+// bits, the dropped products of two low limbs and the rounding of the cross
+// sums: 0.4 units rms (0.5 for one large amplitude), 13 at most. With the last
+// rounding, Haar gates on random amplitudes are off by 31 x 2^-60 of the
+// group's largest component rms, the FP64 chain by 65; one large amplitude in
+// a group: 22 against 59. The chain's error goes with the sum of |U| |psi| over
+// a row, the fixed form's with the largest of each: an output that only small
+// entries of U meet can be the less exact one (4% of them with one large
+// amplitude), by a few units. A gate with an entry below 2^-6 of its largest (a
+// permutation, a controlled gate, 1% of random ones) keeps the FP64 chain for
+// its walker, exact where its entries are. So do groups with an infinity, a NaN
+// or magnitudes within a factor 2^300 of the ends of the range.
 #include <algorithm>
 
 #include "bgemm_internal.h"
@@ -186,6 +191,7 @@ __global__ void __launch_bounds__(kGateThreads, 3)
       }
       // psi = f 2^(E - 59), U = u 2^(EU - 59): the sums are in 2^(E + EU - 58).
       // The cross sums stay below 2^61 (x1, x2) and 4 (2^30 2^30 + 2^30 2^29) < 2^63 (x3).
+      // They are rounded to nearest (cut, every result was half a unit low on average).
       const int k = (top - 1022) + (utop - 1022) - 58;
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
@@ -204,10 +210,11 @@ __global__ void __launch_bounds__(kGateThreads, 3)
           fx::mac(x3, sc.x, fs[c].y);
           fx::mac(x3, sc.y, fs[c].x);
         }
-        o[a] = make_double2(scaled_double(h1 - h2 + ((x1 - x2) >> fx::kLow), k),
-                            scaled_double(h3 - h1 - h2 + (((x3 >> 1) - ((x1 + x2) >> 1)) >>
-                                                          (fx::kLow - 1)),
-                                          k));
+        o[a] = make_double2(
+            scaled_double(h1 - h2 + ((x1 - x2 + (1 << (fx::kLow - 1))) >> fx::kLow), k),
+            scaled_double(h3 - h1 - h2 + (((x3 >> 1) - ((x1 + x2) >> 1) + (1 << (fx::kLow - 2))) >>
+                                          (fx::kLow - 1)),
+                          k));
       }
     } else if (m == 0) {  // (the FP64 chain gives +0 as well)
 #pragma unroll
