@@ -330,6 +330,11 @@ __device__ __forceinline__ void stage_rows(const SliceArgs& a, const LineSrc* s_
 // CTAs, with fewer registers, are slower). Complex ones run four CTAs (64
 // registers; five, with 48, spill: 32 instances of order 512 1136 against 1167 us,
 // Hermitian updates 545 against 559 us), and so do the generic cuts.
+//
+// A CTA per job, so that the SMs even out what the jobs' sizes and the cuts' CTAs
+// per SM leave: with as many CTAs as fit at once, taking jobs in turn, 2000 real
+// instances of 64 x 17 x 64 took 118 us with 7 slices (CTA per job: 89; 10 slices
+// 132 and 99), 4096 complex ones of order 64 with 9 slices 408 (383).
 template <int S, int BETA, bool CPLX>
 __global__ void __launch_bounds__(kSliceThreads, BETA == 0 || CPLX ? 4 : 6)
     split_slice_kernel(const SliceArgs a) {
@@ -341,107 +346,104 @@ __global__ void __launch_bounds__(kSliceThreads, BETA == 0 || CPLX ? 4 : 6)
   __shared__ LineSrc s_src[128];            // the job's lines; all four arrays job-relative
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   constexpr int kWarps = kSliceThreads / 32;
-  for (int64_t jb = blockIdx.x; jb < a.njobs; jb += gridDim.x) {
-    const SliceJob J = a.jobs[jb];
-    const bool isA = J.side == 0;
-    const bool rows = isA || a.herk;
-    const int kv = J.kv, nl = J.nl;
-    const int tile_bytes = J.w * kLineBytes;
-    uint8_t* tiles = isA ? a.tilesA + J.tile0 * kATileBytes : a.tilesB + J.tile0 * kBPiece;
-    if (t < nl) {
-      s_max[t] = 0;
-      s_n2[t] = 0;
-      s_e[t] = INT_MIN;
-      s_src[t] = line_src(a, J, isA, J.l0 + t);
-    }
+  const SliceJob J = a.jobs[blockIdx.x];
+  const bool isA = J.side == 0;
+  const bool rows = isA || a.herk;
+  const int kv = J.kv, nl = J.nl;
+  const int tile_bytes = J.w * kLineBytes;
+  uint8_t* tiles = isA ? a.tilesA + J.tile0 * kATileBytes : a.tilesB + J.tile0 * kBPiece;
+  if (t < nl) {
+    s_max[t] = 0;
+    s_n2[t] = 0;
+    s_e[t] = INT_MIN;
+    s_src[t] = line_src(a, J, isA, J.l0 + t);
+  }
+  __syncthreads();
+  // chunk cc (8 values of k) of line r of the job and k-block kb in the tiles
+  auto place = [&](int r, int kb, int cc) {
+    const int l = J.l0 + r;
+    return tiles + (int64_t)kb * S * tile_bytes + l * kLineBytes + ((cc ^ (l & 7)) << 4);
+  };
+  // Lines beyond their instance only meet discarded outputs: their tile rows
+  // keep the zeros that the planner wrote once.
+  if (CPLX && J.staged) {
+    const int lines = isA ? 2 : 1;  // per complex row (B = A^H: the real lines alone)
+    const int E = nl / lines;
+    stage_rows(a, s_src, lines, E, kv / 2, J.nkb * (BK / 2), stage, s_e);
     __syncthreads();
-    // chunk cc (8 values of k) of line r of the job and k-block kb in the tiles
-    auto place = [&](int r, int kb, int cc) {
-      const int l = J.l0 + r;
-      return tiles + (int64_t)kb * S * tile_bytes + l * kLineBytes + ((cc ^ (l & 7)) << 4);
-    };
-    // Lines beyond their instance only meet discarded outputs: their tile rows
-    // keep the zeros that the planner wrote once.
-    if (CPLX && J.staged) {
-      const int lines = isA ? 2 : 1;  // per complex row (B = A^H: the real lines alone)
-      const int E = nl / lines;
-      stage_rows(a, s_src, lines, E, kv / 2, J.nkb * (BK / 2), stage, s_e);
-      __syncthreads();
-      if (t < nl && s_e[t] == INT_MIN) s_e[t] = 0;
-      __syncthreads();
-      // digit planes and the norm of the absolute digit weights: 8 lanes to a
-      // complex row and k-block
-      const int cc = lane & 7, first = warp * 4 + (lane >> 3);
-      int kb = first / E, er = first - kb * E;
-      while (__any_sync(0xFFFFFFFFu, kb < J.nkb)) {
-        const int r = er * lines, kbc = min(kb, J.nkb - 1);
-        const bool on = kb < J.nkb && s_src[r].off >= 0;
-        if (__any_sync(0xFFFFFFFFu, on)) {
-          double2 z[4];
+    if (t < nl && s_e[t] == INT_MIN) s_e[t] = 0;
+    __syncthreads();
+    // digit planes and the norm of the absolute digit weights: 8 lanes to a
+    // complex row and k-block
+    const int cc = lane & 7, first = warp * 4 + (lane >> 3);
+    int kb = first / E, er = first - kb * E;
+    while (__any_sync(0xFFFFFFFFu, kb < J.nkb)) {
+      const int r = er * lines, kbc = min(kb, J.nkb - 1);
+      const bool on = kb < J.nkb && s_src[r].off >= 0;
+      if (__any_sync(0xFFFFFFFFu, on)) {
+        double2 z[4];
 #pragma unroll
-          for (int v = 0; v < 4; ++v) z[v] = stage[stage_pos(kbc * (BK / 2) + 4 * cc + v, er, E)];
-          const double x[8] = {z[0].x, -z[0].y, z[1].x, -z[1].y, z[2].x, -z[2].y, z[3].x, -z[3].y};
-          cut_item<S, BETA, 8>(x, s_e[r], dc, place(r, kbc, cc), tile_bytes, on, &s_n2[r]);
-          if (isA) {
-            const double y[8] = {z[0].y, z[0].x, z[1].y, z[1].x, z[2].y, z[2].x, z[3].y, z[3].x};
-            cut_item<S, BETA, 8>(y, s_e[r], dc, place(r + 1, kbc, cc), tile_bytes, on,
-                                 &s_n2[r + 1]);
-          }
-        }
-        er += kWarps * 4;
-        while (er >= E) {
-          er -= E;
-          ++kb;
+        for (int v = 0; v < 4; ++v) z[v] = stage[stage_pos(kbc * (BK / 2) + 4 * cc + v, er, E)];
+        const double x[8] = {z[0].x, -z[0].y, z[1].x, -z[1].y, z[2].x, -z[2].y, z[3].x, -z[3].y};
+        cut_item<S, BETA, 8>(x, s_e[r], dc, place(r, kbc, cc), tile_bytes, on, &s_n2[r]);
+        if (isA) {
+          const double y[8] = {z[0].y, z[0].x, z[1].y, z[1].x, z[2].y, z[2].x, z[3].y, z[3].x};
+          cut_item<S, BETA, 8>(y, s_e[r], dc, place(r + 1, kbc, cc), tile_bytes, on,
+                               &s_n2[r + 1]);
         }
       }
-    } else {
-      // ---- phase 1: line maxima (exponents); a group of lines beyond their
-      // instance is skipped here and in phase 2
-      // W lanes to a line and 8 W values of k: up to 6 planes 8 lines by half a
-      // k-block, as 8 rows of A are 64 bytes side by side and a load takes half the
-      // L1 accesses of one of 4 lines by a k-block (3 slices, 1500 real instances
-      // of order 128: 362 -> 324 us); with more planes their stores, of half lines
-      // then, take back what the loads save (9 slices, order 512: 664 -> 677 us).
-      constexpr int kLines = item_lines(S), W = 32 / kLines, kParts = 8 / W;
-      const int groups = nl / kLines, lsub = lane / W, cw = lane % W;
-      int g = 0, h = 0;  // part h of the k-blocks
-      next_item(g, h, warp, groups);
-      while (h < kParts * J.nkb) {
-        const int r = g * kLines + lsub;
-        const LineSrc src = s_src[r];
-        if (__any_sync(0xFFFFFFFFu, src.off >= 0)) {
-          double x[8];
-          load8<CPLX>(a, rows, src, (h * W + cw) * 8, kv, x);
-          merge_max<W>(x, &s_max[r]);
-        }
-        next_item(g, h, kWarps, groups);
-      }
-      __syncthreads();
-      if (t < nl) s_e[t] = line_exponent(s_max[t]);
-      __syncthreads();
-      // ---- phase 2: digit planes and the norm of the absolute digit weights
-      g = h = 0;
-      next_item(g, h, warp, groups);
-      while (h < kParts * J.nkb) {
-        const int r = g * kLines + lsub;
-        const LineSrc src = s_src[r];
-        if (__any_sync(0xFFFFFFFFu, src.off >= 0)) {
-          double x[8];
-          load8<CPLX>(a, rows, src, (h * W + cw) * 8, kv, x);
-          cut_item<S, BETA, W>(x, s_e[r], dc, place(r, h / kParts, h % kParts * W + cw), tile_bytes, true,
-                               &s_n2[r]);
-        }
-        next_item(g, h, kWarps, groups);
+      er += kWarps * 4;
+      while (er >= E) {
+        er -= E;
+        ++kb;
       }
     }
-    __syncthreads();
-    // ---- phase 3: meta of the job's lines (exponent, norm exponent)
-    int32_t* meta = (isA ? a.metaA : a.metaB) + (int64_t)J.blk * kMetaStride + J.l0;
-    if (t < nl) {
-      meta[t] = s_e[t];
-      meta[128 + t] = norm_exponent((float)s_n2[t] * (1.0f / 256.0f));
+  } else {
+    // ---- phase 1: line maxima (exponents); a group of lines beyond their
+    // instance is skipped here and in phase 2
+    // W lanes to a line and 8 W values of k: up to 6 planes 8 lines by half a
+    // k-block, as 8 rows of A are 64 bytes side by side and a load takes half the
+    // L1 accesses of one of 4 lines by a k-block (3 slices, 1500 real instances
+    // of order 128: 362 -> 324 us); with more planes their stores, of half lines
+    // then, take back what the loads save (9 slices, order 512: 664 -> 677 us).
+    constexpr int kLines = item_lines(S), W = 32 / kLines, kParts = 8 / W;
+    const int groups = nl / kLines, lsub = lane / W, cw = lane % W;
+    int g = 0, h = 0;  // part h of the k-blocks
+    next_item(g, h, warp, groups);
+    while (h < kParts * J.nkb) {
+      const int r = g * kLines + lsub;
+      const LineSrc src = s_src[r];
+      if (__any_sync(0xFFFFFFFFu, src.off >= 0)) {
+        double x[8];
+        load8<CPLX>(a, rows, src, (h * W + cw) * 8, kv, x);
+        merge_max<W>(x, &s_max[r]);
+      }
+      next_item(g, h, kWarps, groups);
     }
     __syncthreads();
+    if (t < nl) s_e[t] = line_exponent(s_max[t]);
+    __syncthreads();
+    // ---- phase 2: digit planes and the norm of the absolute digit weights
+    g = h = 0;
+    next_item(g, h, warp, groups);
+    while (h < kParts * J.nkb) {
+      const int r = g * kLines + lsub;
+      const LineSrc src = s_src[r];
+      if (__any_sync(0xFFFFFFFFu, src.off >= 0)) {
+        double x[8];
+        load8<CPLX>(a, rows, src, (h * W + cw) * 8, kv, x);
+        cut_item<S, BETA, W>(x, s_e[r], dc, place(r, h / kParts, h % kParts * W + cw), tile_bytes, true,
+                             &s_n2[r]);
+      }
+      next_item(g, h, kWarps, groups);
+    }
+  }
+  __syncthreads();
+  // ---- phase 3: meta of the job's lines (exponent, norm exponent)
+  int32_t* meta = (isA ? a.metaA : a.metaB) + (int64_t)J.blk * kMetaStride + J.l0;
+  if (t < nl) {
+    meta[t] = s_e[t];
+    meta[128 + t] = norm_exponent((float)s_n2[t] * (1.0f / 256.0f));
   }
 }
 
@@ -572,7 +574,7 @@ struct SplitPlan {
   int32_t* metaA = nullptr;
   int32_t* metaB = nullptr;
   int64_t bytes = 0;
-  int grid_slice = 0, grid_gemm = 0, grid_small = 0;
+  int grid_gemm = 0, grid_small = 0;
   int slice_stage = 0;     // dynamic shared memory of the slicer
   std::vector<int64_t> key;  // fixed-size plan cache key
   std::string desc;
@@ -972,24 +974,19 @@ static cudaError_t with_slicer(const SplitPlan* p, const F& f) {
   return p->dt == BG_C128 ? with_slicer_of<true>(p, f) : with_slicer_of<false>(p, f);
 }
 
-// CTAs of the slicer per SM, its shared-memory limit set on the way.
-static int slicer_ctas(const SplitPlan* p) {
-  int bps = 0;
-  with_slicer(p, [&](auto kernel) {
-    if (p->slice_stage > kSliceStage)
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kSliceStageMax);
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, kSliceThreads,
-                                                         p->slice_stage);
+// The slicer's shared-memory limit, where the stage needs a raised one.
+static void set_slicer_limit(const SplitPlan* p) {
+  if (p->slice_stage <= kSliceStage) return;
+  with_slicer(p, [](auto kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kSliceStageMax);
   });
-  return std::max(bps, 1);
 }
 
 static void grids(SplitPlan* p) {
   set_gemm_attr(p->dt, p->s);
   p->grid_gemm = (int)std::max<int64_t>(1, std::min<int64_t>(p->sms, p->n_units));
-  const int bps = slicer_ctas(p);
-  p->grid_slice = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)p->sms * bps, p->n_jobs));
+  set_slicer_limit(p);
   if (p->n_small_items > 0)
     p->grid_small = (int)std::max<int64_t>(1, std::min<int64_t>(
         (int64_t)p->sms * split_small_ctas(p->s), p->n_small_items));
@@ -1029,7 +1026,6 @@ static cudaError_t launch_slicer(SplitPlan* p, const SliceJob* jobs, int64_t njo
   if (njobs <= 0) return cudaSuccess;
   SliceArgs a;
   a.jobs = jobs;
-  a.njobs = njobs;
   a.instA = instA;
   a.instB = instB;
   a.orderA = orderA;
@@ -1044,9 +1040,8 @@ static cudaError_t launch_slicer(SplitPlan* p, const SliceJob* jobs, int64_t njo
   a.s = p->s;
   a.beta = p->beta;
   a.herk = p->herk ? 1 : 0;
-  const int grid = (int)std::min<int64_t>(columns ? 6ll * p->sms : p->grid_slice, njobs);
   auto launch = [&](auto kernel) {
-    kernel<<<grid, kSliceThreads, columns ? 0 : p->slice_stage, st>>>(a);
+    kernel<<<(unsigned)njobs, kSliceThreads, columns ? 0 : p->slice_stage, st>>>(a);
     count_launch();
     return cudaGetLastError();
   };

@@ -102,7 +102,6 @@ struct SplitUnit {
 
 struct SliceArgs {
   const SliceJob* jobs;
-  int64_t njobs;
   const SInst* instA;
   const SInst* instB;
   const int32_t* orderA;
