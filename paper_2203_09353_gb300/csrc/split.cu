@@ -259,6 +259,14 @@ __device__ __forceinline__ void cut_item(const double (&x)[8], int e, const Digi
 // Lines of a warp's item of an unstaged job.
 __host__ __device__ constexpr int item_lines(int s) { return s <= 6 ? 8 : 4; }
 
+// Whether a cut takes complex rows from the shared-memory stage: the generic ones
+// keep s digits of both lines beside the row's values, and from 6 slices on
+// that leaves the registers (12 slices, 2000 instances of order 48: slicer 673 us
+// unstaged, 1154 staged; 10: 16^3 63 and 79; 4: 64^3 293 and 233).
+__host__ __device__ constexpr bool staged_cut(int s, bool compile_time) {
+  return compile_time || s <= 5;
+}
+
 // Advances a warp's item (line group g, k-block or part of one kb) by `step` items in
 // the group-fastest order, without a division.
 __device__ __forceinline__ void next_item(int& g, int& kb, int step, int groups) {
@@ -366,7 +374,7 @@ __global__ void __launch_bounds__(kSliceThreads, BETA == 0 || CPLX ? 4 : 6)
   };
   // Lines beyond their instance only meet discarded outputs: their tile rows
   // keep the zeros that the planner wrote once.
-  if (CPLX && J.staged) {
+  if (CPLX && staged_cut(S, BETA > 0) && J.staged) {
     const int lines = isA ? 2 : 1;  // per complex row (B = A^H: the real lines alone)
     const int E = nl / lines;
     stage_rows(a, s_src, lines, E, kv / 2, J.nkb * (BK / 2), stage, s_e);
@@ -665,10 +673,16 @@ static int kmma_last_of(int kv) {
   return (rem + 15) / 16;
 }
 
+// The documented modes have a slicer of their own (split_slice_kernel).
+static bool compile_time_cut(int s, int beta) {
+  return (s == 3 && beta == 7) || (s == 6 && beta == 7) || (s == 9 && beta == 6);
+}
+
 // Cuts block jobs into jobs of fewer lines (halving while the count stays a
 // multiple of the lines of a warp's item): complex rows to what fits the slicer's shared-memory stage,
 // the rest to kSliceJobBytes. Returns the stage that the longest rows need.
-static int split_jobs(std::vector<SliceJob>* jobs, int s, bool cplx, bool herk) {
+static int split_jobs(std::vector<SliceJob>* jobs, const SplitPlan* p) {
+  const bool rows = p->dt == BG_C128 && staged_cut(p->s, compile_time_cut(p->s, p->beta));
   std::vector<SliceJob> out;
   out.reserve(jobs->size() * 2);
   int64_t stage = 0;
@@ -682,9 +696,9 @@ static int split_jobs(std::vector<SliceJob>* jobs, int s, bool cplx, bool herk) 
     // (a complex value of A serves two values of each of two lines)
     const int64_t staged_line = j.side == 0 ? line_bytes / 2 : line_bytes;
     int nl = lines(staged_line, kSliceStage, 4);
-    const bool staged = cplx && (j.side == 0 || herk) && nl * staged_line <= kSliceStageMax;
+    const bool staged = rows && (j.side == 0 || p->herk) && nl * staged_line <= kSliceStageMax;
     if (staged) stage = std::max({stage, nl * staged_line, kSliceStage});
-    else nl = lines(line_bytes, kSliceJobBytes, item_lines(s));
+    else nl = lines(line_bytes, kSliceJobBytes, item_lines(p->s));
     for (int l0 = 0; l0 < j.w; l0 += nl) {
       SliceJob sj = j;
       sj.l0 = (int16_t)l0;
@@ -876,7 +890,7 @@ static void make_tables(const SplitPlan* p, const std::vector<bg_instance>& tabl
     if (ia < jobsA.size()) jobs.push_back(jobsA[ia++]);
     if (ib < jobsB.size()) jobs.push_back(jobsB[ib++]);
   }
-  out->stage = split_jobs(&jobs, s, cplx, p->herk);
+  out->stage = split_jobs(&jobs, p);
   out->inst = std::move(inst);
   out->order = std::move(order);
   out->jobs = std::move(jobs);
@@ -964,9 +978,10 @@ static cudaError_t set_gemm_attr(bg_dtype dt, int s) {
 // versions for the documented modes.
 template <bool CPLX, class F>
 static cudaError_t with_slicer_of(const SplitPlan* p, const F& f) {
-  if (p->s == 3 && p->beta == 7) return f(split_slice_kernel<3, 7, CPLX>);
-  if (p->s == 6 && p->beta == 7) return f(split_slice_kernel<6, 7, CPLX>);
-  if (p->s == 9 && p->beta == 6) return f(split_slice_kernel<9, 6, CPLX>);
+  if (compile_time_cut(p->s, p->beta))
+    return p->s == 3   ? f(split_slice_kernel<3, 7, CPLX>)
+           : p->s == 6 ? f(split_slice_kernel<6, 7, CPLX>)
+                       : f(split_slice_kernel<9, 6, CPLX>);
   BG_DISPATCH_SLICES(p->s, { return f(split_slice_kernel<S, 0, CPLX>); });
 }
 template <class F>
@@ -1329,7 +1344,7 @@ bg_status split_chain_create(SplitPlan** out, bg_dtype dt, const bg_precision& p
   std::stable_sort(units.begin(), units.end(),
                    [](const SplitUnit& a, const SplitUnit& b) { return a.nkb > b.nkb; });
   // pool jobs first, then walker jobs (the chain step slices the two parts separately)
-  p->slice_stage = std::max(split_jobs(&jobsA, s, cplx, false), split_jobs(&jobsB, s, cplx, false));
+  p->slice_stage = std::max(split_jobs(&jobsA, p), split_jobs(&jobsB, p));
   std::vector<SliceJob> jobs = jobsA;
   jobs.insert(jobs.end(), jobsB.begin(), jobsB.end());
   p->n_jobs = (int64_t)jobs.size();
