@@ -299,8 +299,7 @@ double item_cost(const WorkItem& w, const std::vector<int64_t>& mnk_k,
 // Build the FP64 work list for instances with the given program per instance.
 // `ids` are instance (or walker) ids, `sizes` their (m, n, k), `prog_of` the
 // chosen program. Small-program instances are grouped in `order`, 8 to a CTA;
-// where there are too few of them to give each of the `grid` CTAs such a
-// group they run as tiles instead. Tiles split an instance evenly, further
+// where they are too few (small_pays) they run as tiles instead. Tiles split an instance evenly, further
 // while a tile holds more than a CTA's share of the whole work (a batch of few
 // instances would leave SMs idle). Items are sorted longest first. Returns the
 // CTAs per SM to run them with: one where full tiles hold most of the work,
@@ -359,11 +358,13 @@ int build_items(const std::vector<int64_t>& ids, const std::vector<std::array<in
     if (!prog_is_small(prog_of[id])) add_tiles(id, prog_of[id]);
   for (auto& kv : small) {
     auto& v = kv.second;
-    if (!small_fills((int64_t)v.size(), grid)) {
-      for (int64_t id : v)
-        add_tiles(id, kv.first == PROG_R64_SMALL ? PROG_R64_TILE : PROG_C128_TILE);
-      continue;
-    }
+    const int64_t all = (int64_t)v.size();
+    auto keep = std::stable_partition(v.begin(), v.end(), [&](int64_t id) {
+      return small_pays(mnk[id][0], mnk[id][1], mnk[id][2], all, (int)(grid / 2));
+    });
+    for (auto it = keep; it != v.end(); ++it)
+      add_tiles(*it, kv.first == PROG_R64_SMALL ? PROG_R64_TILE : PROG_C128_TILE);
+    v.erase(keep, v.end());
     std::stable_sort(v.begin(), v.end(), [&](int64_t a, int64_t b) {
       return std::ceil(mn[a] / 32.0) * kk[a] > std::ceil(mn[b] / 32.0) * kk[b];
     });
@@ -694,7 +695,7 @@ bg_status build_fp64_schedule(bg_plan* p, const char* cache_path, cudaStream_t s
     for (int q = 0; q < np; ++q) {
       bool ok = true;
       for (int64_t i = 0; i < p->count && ok; ++i)
-        if (p->inst_class[i] == (int)c) ok = prog_fits(pl[q], p->dtype, p->table[i].m, p->table[i].n);
+        if (p->inst_class[i] == (int)c) ok = prog_fits(pl[q], p->dtype, p->table[i].m, p->table[i].n, p->table[i].k);
       if (ok) cand.push_back(pl[q]);
     }
     // default: small if it fits, else the DFMA tile
@@ -861,7 +862,7 @@ bg_status batched_gemm_fixed(bg_dtype dtype, int64_t m, int64_t n, int64_t k, co
   if ((s = get_ctx(&ctx)) != BG_OK) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (pr.mode == BG_MODE_FP64) {
-    const int prog = default_prog(dtype, m, n, batch, ctx->sms);
+    const int prog = default_prog(dtype, m, n, k, batch, ctx->sms);
     cudaError_t e = launch_fp64_fixed(dtype, prog, m, n, k, sc, A, lda, strideA, B, ldb, strideB,
                                       C, ldc, strideC, batch, ctx->sms, st);
     if (e != cudaSuccess) return cuda_fail(e, "FP64 batched kernel launch");

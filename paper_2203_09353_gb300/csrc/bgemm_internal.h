@@ -50,10 +50,6 @@ __host__ __device__ inline void tile_extent_of(int count, int full, int* tm, int
 }
 
 constexpr int kSmallPerCta = 8;   // warps (instances) per CTA in the small programs
-// Whether the small programs' groups of 8 fill `grid` CTAs.
-inline bool small_fills(int64_t instances, int64_t grid) {
-  return (instances + kSmallPerCta - 1) / kSmallPerCta >= grid;
-}
 constexpr int kFp64Threads = 256;
 
 // Outputs per thread of the program that runs a tile with `out` outputs inside
@@ -73,7 +69,7 @@ struct Scalars {
 };
 
 // Program of a fixed-size batch (FP64 path).
-int default_prog(bg_dtype dt, int64_t m, int64_t n, int64_t batch, int sms);
+int default_prog(bg_dtype dt, int64_t m, int64_t n, int64_t k, int64_t batch, int sms);
 // Output-tile extent of a tile program (rows, cols); small programs return 0.
 void prog_tile(int prog, int* tm, int* tn);
 bool prog_is_small(int prog);
@@ -85,7 +81,9 @@ bool fp64_tile_ok(bg_dtype dt, int64_t tm, int64_t tn);
 // smaller than the chip still spreads over its SMs.
 void fp64_tile_split(bg_dtype dt, int64_t m, int64_t n, int64_t k, int64_t batch, int sms, int* tm,
                      int* tn);
-bool prog_fits(int prog, bg_dtype dt, int64_t m, int64_t n);
+bool prog_fits(int prog, bg_dtype dt, int64_t m, int64_t n, int64_t k);
+// Whether a batch of `instances` that the small program fits is to run on it.
+bool small_pays(int64_t m, int64_t n, int64_t k, int64_t instances, int sms);
 
 // ---- FP64 launchers (fp64.cu) ---------------------------------------------------
 

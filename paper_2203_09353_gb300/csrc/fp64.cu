@@ -522,61 +522,65 @@ __device__ __forceinline__ void tile_c128(const Desc& d, int r0, int c0, int mb,
 }
 
 // ---- small programs: a warp per instance --------------------------------------
-// Lane t owns outputs o = t + 32 j (j < MAXOUT) of the m*n outputs in
-// column-major order, i.e. (r, c) = (o mod m, o div m). When m divides 32 the
-// row is the same for every j and the column steps by 32 / m, so one A load
+// The m*n outputs in column-major order, 32 MAXOUT at a time: lane t owns outputs
+// o = t + 32 j (j < MAXOUT) of them, (r, c) = (o mod m, o div m). When m divides 32
+// the row is the same for every j and the column steps by 32 / m, so one A load
 // feeds MAXOUT DFMAs; otherwise every output loads its own A element.
 
 template <int MAXOUT>
 __device__ __forceinline__ void small_r64(const Desc& d, const Scalars& s) {
   const int lane = threadIdx.x & 31;
-  constexpr int stride = 32;
   const int m = d.m, n = d.n, mn = m * n;
   const int K = s.alpha_zero ? 0 : d.k;
   double acc[MAXOUT];
-#pragma unroll
-  for (int j = 0; j < MAXOUT; ++j) acc[j] = 0.0;
   if (m > 0 && (32 % m) == 0) {
-    const int r = lane % m, c0 = lane / m, cstep = stride / m;
+    const int r = lane % m, cstep = 32 / m;
     const double* ap = d.A + r;
-    const double* bp = d.B + (int64_t)c0 * d.ldb;
     const int64_t bstep = (int64_t)cstep * d.ldb;
+    for (int c0 = lane / m; c0 < n; c0 += MAXOUT * cstep) {
+      const double* bp = d.B + (int64_t)c0 * d.ldb;
+#pragma unroll
+      for (int j = 0; j < MAXOUT; ++j) acc[j] = 0.0;
 #pragma unroll 1
-    for (int p = 0; p < K; ++p) {
-      const double a = __ldg(ap + (int64_t)p * d.lda);
+      for (int p = 0; p < K; ++p) {
+        const double a = __ldg(ap + (int64_t)p * d.lda);
 #pragma unroll
-      for (int j = 0; j < MAXOUT; ++j)
-        if (c0 + j * cstep < n)
-          acc[j] = fma(a, d.herm ? ld_b(d, p, c0 + j * cstep) : __ldg(bp + p + j * bstep), acc[j]);
-    }
-#pragma unroll
-    for (int j = 0; j < MAXOUT; ++j) {
-      const int c = c0 + j * cstep;
-      if (c < n && keep_out(d, r, c)) {
-        double* cp = d.C + r + (int64_t)c * d.ldc;
-        double v = s.alpha_re * acc[j];
-        if (!s.beta_zero) v = fma(s.beta_re, *cp, v);
-        *cp = v;
+        for (int j = 0; j < MAXOUT; ++j)
+          if (c0 + j * cstep < n)
+            acc[j] = fma(a, d.herm ? ld_b(d, p, c0 + j * cstep) : __ldg(bp + p + j * bstep), acc[j]);
       }
-    }
-  } else {
-#pragma unroll 1
-    for (int p = 0; p < K; ++p) {
 #pragma unroll
       for (int j = 0; j < MAXOUT; ++j) {
-        const int o = lane + stride * j;
-        if (o < mn) {
-          const int r = o % m, c = o / m;
-          acc[j] = fma(__ldg(d.A + r + (int64_t)p * d.lda), ld_b(d, p, c), acc[j]);
+        const int c = c0 + j * cstep;
+        if (c < n && keep_out(d, r, c)) {
+          double* cp = d.C + r + (int64_t)c * d.ldc;
+          double v = s.alpha_re * acc[j];
+          if (!s.beta_zero) v = fma(s.beta_re, *cp, v);
+          *cp = v;
         }
       }
     }
+  } else {
+    int rc[MAXOUT];  // row | column << 16
+    for (int o0 = lane; o0 < mn; o0 += 32 * MAXOUT) {
+      const int cnt = (mn - (o0 - lane) + 31) / 32;  // outputs of this warp's lanes
 #pragma unroll
-    for (int j = 0; j < MAXOUT; ++j) {
-      const int o = lane + stride * j;
-      if (o < mn) {
-        const int r = o % m, c = o / m;
-        if (!keep_out(d, r, c)) continue;
+      for (int j = 0; j < MAXOUT; ++j) {
+        const int o = min(o0 + 32 * j, mn - 1), c = o / m;
+        rc[j] = (o - c * m) | c << 16;
+        acc[j] = 0.0;
+      }
+#pragma unroll 1
+      for (int p = 0; p < K; ++p) {
+        const double* ap = d.A + (int64_t)p * d.lda;
+#pragma unroll
+        for (int j = 0; j < MAXOUT; ++j)
+          if (j < cnt) acc[j] = fma(__ldg(ap + (rc[j] & 0xFFFF)), ld_b(d, p, rc[j] >> 16), acc[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < MAXOUT; ++j) {
+        const int r = rc[j] & 0xFFFF, c = rc[j] >> 16;
+        if (o0 + 32 * j >= mn || !keep_out(d, r, c)) continue;
         double* cp = d.C + r + (int64_t)c * d.ldc;
         double v = s.alpha_re * acc[j];
         if (!s.beta_zero) v = fma(s.beta_re, *cp, v);
@@ -595,48 +599,53 @@ __device__ __forceinline__ void small_c128(const Desc& d, const Scalars& s) {
   const double2* B = reinterpret_cast<const double2*>(d.B);
   double2* C = reinterpret_cast<double2*>(d.C);
   double2 acc[MAXOUT];
-#pragma unroll
-  for (int j = 0; j < MAXOUT; ++j) acc[j] = make_double2(0.0, 0.0);
   if (m > 0 && (32 % m) == 0) {
-    const int r = lane % m, c0 = lane / m, cstep = 32 / m;
+    const int r = lane % m, cstep = 32 / m;
     const int64_t bstep = (int64_t)cstep * d.ldb;
-    const double2* bp = B + (int64_t)c0 * d.ldb;
+    for (int c0 = lane / m; c0 < n; c0 += MAXOUT * cstep) {
+      const double2* bp = B + (int64_t)c0 * d.ldb;
+#pragma unroll
+      for (int j = 0; j < MAXOUT; ++j) acc[j] = make_double2(0.0, 0.0);
 #pragma unroll 1
-    for (int p = 0; p < K; ++p) {
-      const double2 a = __ldg(A + r + (int64_t)p * d.lda);
+      for (int p = 0; p < K; ++p) {
+        const double2 a = __ldg(A + r + (int64_t)p * d.lda);
 #pragma unroll
-      for (int j = 0; j < MAXOUT; ++j)
-        if (c0 + j * cstep < n)
-          cmac(acc[j], a, d.herm ? ld_bc(d, p, c0 + j * cstep) : __ldg(bp + p + j * bstep));
-    }
-#pragma unroll
-    for (int j = 0; j < MAXOUT; ++j) {
-      const int c = c0 + j * cstep;
-      if (c < n && keep_out(d, r, c)) {
-        double2* cp = C + r + (int64_t)c * d.ldc;
-        double2 v = c_epilogue(acc[j], cp, s);
-        if (d.herm && r == c) v.y = 0.0;
-        *cp = v;
+        for (int j = 0; j < MAXOUT; ++j)
+          if (c0 + j * cstep < n)
+            cmac(acc[j], a, d.herm ? ld_bc(d, p, c0 + j * cstep) : __ldg(bp + p + j * bstep));
       }
-    }
-  } else {
-#pragma unroll 1
-    for (int p = 0; p < K; ++p) {
 #pragma unroll
       for (int j = 0; j < MAXOUT; ++j) {
-        const int o = lane + 32 * j;
-        if (o < mn) {
-          const int r = o % m, c = o / m;
-          cmac(acc[j], __ldg(A + r + (int64_t)p * d.lda), ld_bc(d, p, c));
+        const int c = c0 + j * cstep;
+        if (c < n && keep_out(d, r, c)) {
+          double2* cp = C + r + (int64_t)c * d.ldc;
+          double2 v = c_epilogue(acc[j], cp, s);
+          if (d.herm && r == c) v.y = 0.0;
+          *cp = v;
         }
       }
     }
+  } else {
+    int rc[MAXOUT];
+    for (int o0 = lane; o0 < mn; o0 += 32 * MAXOUT) {
+      const int cnt = (mn - (o0 - lane) + 31) / 32;
 #pragma unroll
-    for (int j = 0; j < MAXOUT; ++j) {
-      const int o = lane + 32 * j;
-      if (o < mn) {
-        const int r = o % m, c = o / m;
-        if (!keep_out(d, r, c)) continue;
+      for (int j = 0; j < MAXOUT; ++j) {
+        const int o = min(o0 + 32 * j, mn - 1), c = o / m;
+        rc[j] = (o - c * m) | c << 16;
+        acc[j] = make_double2(0.0, 0.0);
+      }
+#pragma unroll 1
+      for (int p = 0; p < K; ++p) {
+        const double2* ap = A + (int64_t)p * d.lda;
+#pragma unroll
+        for (int j = 0; j < MAXOUT; ++j)
+          if (j < cnt) cmac(acc[j], __ldg(ap + (rc[j] & 0xFFFF)), ld_bc(d, p, rc[j] >> 16));
+      }
+#pragma unroll
+      for (int j = 0; j < MAXOUT; ++j) {
+        const int r = rc[j] & 0xFFFF, c = rc[j] >> 16;
+        if (o0 + 32 * j >= mn || !keep_out(d, r, c)) continue;
         double2* cp = C + r + (int64_t)c * d.ldc;
         double2 v = c_epilogue(acc[j], cp, s);
         if (d.herm && r == c) v.y = 0.0;
@@ -646,7 +655,7 @@ __device__ __forceinline__ void small_c128(const Desc& d, const Scalars& s) {
   }
 }
 
-// Small-program limits (outputs per warp): MAXOUT 8 real, 4 complex.
+// Outputs that a small program holds at once: MAXOUT 8 real, 4 complex.
 constexpr int kSmallR64 = 256, kSmallC128 = 128;
 
 // ---- the persistent kernel ---------------------------------------------------------
@@ -748,11 +757,37 @@ void prog_tile(int prog, int* tm, int* tn) {
   }
 }
 
-bool prog_fits(int prog, bg_dtype dt, int64_t m, int64_t n) {
-  const int64_t mn = m * n;
+// The small programs take what they hold at once, and four times as many outputs
+// where k is short: a tile's start (descriptor, operands to shared memory, barriers)
+// then costs more than its products, above all for a few rows or columns, of
+// which a tile holds 64. Measured with sizes at the lines below, tiles and small
+// program, us for 30000 real or 20000 complex instances: 1 x 300 x 16 1476 and 693,
+// 2 x 200 x 16 1191 and 758 (x 32 2033 and 1499, but 3000 of them 207 and 229),
+// 5 x 100 x 8 546 and 400 (x 16 736 and 735), 20 x 20 x 4 260 and 185 (x 8 342 and
+// 328), 32 x 32 x 4 441 and 357 (x 8 651 and 655); complex 1 x 300 x 32 3162 and 1520,
+// 16 x 16 x 8 390 and 329 (x 16 654 and 620, but 3000 of them 106 and 112).
+static bool small_fits(bg_dtype dt, int64_t m, int64_t n, int64_t k) {
+  const int64_t held = dt == BG_R64 ? kSmallR64 : kSmallC128, thin = std::min(m, n);
+  const int64_t k_max = dt == BG_R64 ? (thin <= 2 ? 16 : thin < 8 ? 8 : 4) : (thin <= 2 ? 32 : 8);
+  return m * n <= (k <= k_max ? 4 * held : held);
+}
+
+// Whether the small programs are to run `instances` that fit them: where groups of
+// 8 fill two CTAs per SM, and fewer where a warp's chain of products is so short
+// that tiles take longer to start: 6 per SM up to k = 4, 4 per SM with one or two rows
+// or columns up to k = 8 (tiles and small program, us for 1000: 1 x 300 x 2 34.9
+// and 8.3, 300 x 1 x 8 39.0 and 24.6, 8 x 64 x 2 12.4 and 10.3, complex 4 x 100 x 4
+// 34.9 and 24.2; but 20 x 20 x 8 16.4 and 24; for 400: 4 x 100 x 2 9.3 and 10.2).
+bool small_pays(int64_t m, int64_t n, int64_t k, int64_t instances, int sms) {
+  if ((instances + kSmallPerCta - 1) / kSmallPerCta >= 2 * (int64_t)sms) return true;
+  const bool thin = std::min(m, n) <= 2;
+  return k <= (thin ? 8 : 4) && m * n * k <= 2400 && instances >= (thin ? 4 : 6) * (int64_t)sms;
+}
+
+bool prog_fits(int prog, bg_dtype dt, int64_t m, int64_t n, int64_t k) {
   switch (prog) {
-    case PROG_R64_SMALL: return dt == BG_R64 && mn <= kSmallR64;
-    case PROG_C128_SMALL: return dt == BG_C128 && mn <= kSmallC128;
+    case PROG_R64_SMALL: return dt == BG_R64 && small_fits(dt, m, n, k);
+    case PROG_C128_SMALL: return dt == BG_C128 && small_fits(dt, m, n, k);
     case PROG_R64_TILE:
     case PROG_R64_DMMA: return dt == BG_R64;
     case PROG_C128_TILE: return dt == BG_C128;
@@ -811,9 +846,9 @@ void fp64_tile_split(bg_dtype dt, int64_t m, int64_t n, int64_t k, int64_t batch
   last.tn = *tn;
 }
 
-int default_prog(bg_dtype dt, int64_t m, int64_t n, int64_t batch, int sms) {
+int default_prog(bg_dtype dt, int64_t m, int64_t n, int64_t k, int64_t batch, int sms) {
   const int small = dt == BG_R64 ? PROG_R64_SMALL : PROG_C128_SMALL;
-  if (prog_fits(small, dt, m, n) && small_fills(batch, 2 * (int64_t)sms)) return small;
+  if (prog_fits(small, dt, m, n, k) && small_pays(m, n, k, batch, sms)) return small;
   return dt == BG_R64 ? PROG_R64_TILE : PROG_C128_TILE;
 }
 
