@@ -15,6 +15,7 @@
 // memory matters: the design goal is only to keep DFMAs flowing on every SM
 // with few non-FMA instructions.
 #include <algorithm>
+#include <type_traits>
 
 #include "bgemm_internal.h"
 
@@ -169,6 +170,97 @@ struct SmemR64 {
   double b[2][BKR][TR];  // b[s][kk][col]
 };
 
+// f with beta's part of Eq. (1) in or out: a branch outside the loop over the outputs,
+// where the compiler cannot predicate the FP64 instructions that it skips (20000
+// complex instances of 16 x 16 x 1 122 us with the test inside, 82 without).
+template <class F>
+__device__ __forceinline__ void with_beta(const Scalars& s, const F& f) {
+  if (s.beta_zero) f(std::false_type{});
+  else f(std::true_type{});
+}
+
+// alpha acc + beta c (Eq. 1).
+template <bool BETA>
+__device__ __forceinline__ double combine(double acc, double c, const Scalars& s) {
+  double v = s.alpha_re * acc;
+  if constexpr (BETA) v = fma(s.beta_re, c, v);
+  return v;
+}
+template <bool BETA>
+__device__ __forceinline__ double2 combine(double2 acc, double2 c, const Scalars& s) {
+  double2 v;
+  v.x = s.alpha_re * acc.x - s.alpha_im * acc.y;
+  v.y = s.alpha_re * acc.y + s.alpha_im * acc.x;
+  if constexpr (BETA) {
+    v.x = fma(s.beta_re, c.x, fma(-s.beta_im, c.y, v.x));
+    v.y = fma(s.beta_re, c.y, fma(s.beta_im, c.x, v.y));
+  }
+  return v;
+}
+__device__ __forceinline__ void real_diagonal(double&) {}
+__device__ __forceinline__ void real_diagonal(double2& v) { v.y = 0.0; }
+
+// Output (r, c) of an instance (T: double or double2).
+template <bool BETA, class T>
+__device__ __forceinline__ void store_out(const Desc& d, const Scalars& s, int r, int c, T acc) {
+  if (!keep_out(d, r, c)) return;
+  T* cp = reinterpret_cast<T*>(d.C) + r + (int64_t)c * d.ldc;
+  T v = combine<BETA>(acc, BETA ? *cp : T{}, s);
+  if (d.herm && r == c) real_diagonal(v);
+  *cp = v;
+}
+
+// A thread's N x N outputs from (r, c) on; all of C is loaded before the first use.
+template <class T, int N>
+__device__ __forceinline__ void store_block(const Desc& d, const Scalars& s, int r, int c,
+                                            const T (&acc)[N][N]) {
+  with_beta(s, [&](auto beta) {
+    constexpr bool BETA = decltype(beta)::value;
+    T* cp = reinterpret_cast<T*>(d.C) + r + (int64_t)c * d.ldc;
+    T cv[N][N];
+    bool on[N][N];
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        on[i][j] = r + i < d.m && c + j < d.n && keep_out(d, r + i, c + j);
+        if (BETA && on[i][j]) cv[i][j] = cp[i + (int64_t)j * d.ldc];
+      }
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        if (!on[i][j]) continue;
+        T v = combine<BETA>(acc[i][j], BETA ? cv[i][j] : T{}, s);
+        if (d.herm && r + i == c + j) real_diagonal(v);
+        cp[i + (int64_t)j * d.ldc] = v;
+      }
+  });
+}
+
+// The products of a k-slice for a warp's nj <= NJ outputs in linear order (nj is
+// the same in all its lanes). A warp with fewer than NJ takes one output after
+// another, so that a branch on nj lies outside the loop over k: inside it the
+// compiler may predicate instead, and a DFMA that is off in every lane holds the
+// FP64 pipe as long as one that is on (456 complex instances of 32 x 9 x 32 61 us
+// so and 35 with the branch outside, 30000 real ones of 2 x 200 x 64 8010 and 3820).
+template <int NJ, class F>
+__device__ __forceinline__ void linear_products(int nj, int kend, F mul) {
+  if (nj >= NJ) {
+#pragma unroll 2
+    for (int kk = 0; kk < kend; ++kk)
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) mul(j, kk);
+  } else {
+#pragma unroll
+    for (int j = 0; j < NJ - 1; ++j) {
+      if (j >= nj) break;
+#pragma unroll 2
+      for (int kk = 0; kk < kend; ++kk) mul(j, kk);
+    }
+  }
+}
+
 // Rows r0 .. r0 + tm - 1 and columns c0 .. c0 + tn - 1 (tm, tn <= 64) of one
 // instance; FULL: 64 x 64, or what the instance leaves of it, 4 x 4 outputs per
 // thread (for more outputs than NJ = 8 holds). Otherwise output o of the tile's mb x nb (column-major) goes to
@@ -182,7 +274,7 @@ __device__ __forceinline__ void tile_r64(const Desc& d, int r0, int c0, int mb, 
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
   const int K = s.alpha_zero ? 0 : d.k;
-  double acc[FULL ? 4 : 1][4];
+  double acc[FULL ? 4 : 1][FULL ? 4 : 1];
   double lin[FULL ? 1 : NJ];
   int rc[FULL ? 1 : NJ];  // row and column of each output in the tile, row | column << 16
   if constexpr (FULL) {
@@ -234,11 +326,9 @@ __device__ __forceinline__ void tile_r64(const Desc& d, int r0, int c0, int mb, 
     if (more) gload(k0 + BKR);
     if constexpr (!FULL) {
       const int kend = min(BKR, K - k0);
-#pragma unroll 2
-      for (int kk = 0; kk < kend; ++kk)
-#pragma unroll
-        for (int j = 0; j < NJ; ++j)
-          if (j < nj) lin[j] = fma(sm.a[st][kk][rc[j] & 0xFFFF], sm.b[st][kk][rc[j] >> 16], lin[j]);
+      linear_products<NJ>(nj, kend, [&](int j, int kk) {
+        lin[j] = fma(sm.a[st][kk][rc[j] & 0xFFFF], sm.b[st][kk][rc[j] >> 16], lin[j]);
+      });
     } else
 #pragma unroll
     for (int kk = 0; kk < BKR; ++kk) {
@@ -259,31 +349,15 @@ __device__ __forceinline__ void tile_r64(const Desc& d, int r0, int c0, int mb, 
   }
 
   if constexpr (!FULL) {
+    with_beta(s, [&](auto beta) {
 #pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-      const int r = r0 + (rc[j] & 0xFFFF), c = c0 + (rc[j] >> 16);
-      if (tid + kFp64Threads * j >= mb * nb || !keep_out(d, r, c)) continue;
-      double* cp = d.C + r + (int64_t)c * d.ldc;
-      double v = s.alpha_re * lin[j];
-      if (!s.beta_zero) v = fma(s.beta_re, *cp, v);
-      *cp = v;
-    }
+      for (int j = 0; j < NJ; ++j)
+        if (tid + kFp64Threads * j < mb * nb)
+          store_out<decltype(beta)::value>(d, s, r0 + (rc[j] & 0xFFFF), c0 + (rc[j] >> 16), lin[j]);
+    });
     return;
   } else
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int c = c0 + tx * 4 + j;
-    if (c >= d.n) continue;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = r0 + ty * 4 + i;
-      if (r >= d.m || !keep_out(d, r, c)) continue;
-      double* cp = d.C + r + (int64_t)c * d.ldc;
-      double v = s.alpha_re * acc[i][j];
-      if (!s.beta_zero) v = fma(s.beta_re, *cp, v);
-      *cp = v;
-    }
-  }
+  store_block(d, s, r0 + ty * 4, c0 + tx * 4, acc);
 }
 
 // ---- real tile program on the FP64 tensor cores: mma.sync m8n8k4 -----------------
@@ -388,18 +462,6 @@ __device__ __forceinline__ void cmac(double2& acc, double2 a, double2 b) {
   acc.y = fma(a.y, b.x, acc.y);
 }
 
-__device__ __forceinline__ double2 c_epilogue(double2 acc, const double2* cp, const Scalars& s) {
-  double2 v;
-  v.x = s.alpha_re * acc.x - s.alpha_im * acc.y;
-  v.y = s.alpha_re * acc.y + s.alpha_im * acc.x;
-  if (!s.beta_zero) {
-    const double2 c = *cp;
-    v.x = fma(s.beta_re, c.x, fma(-s.beta_im, c.y, v.x));
-    v.y = fma(s.beta_re, c.y, fma(s.beta_im, c.x, v.y));
-  }
-  return v;
-}
-
 // As tile_r64: FULL is a whole 32 x 32 tile (2 x 2 outputs per thread), NJ the
 // outputs per thread in linear order otherwise.
 template <bool FULL, int NJ>
@@ -409,7 +471,7 @@ __device__ __forceinline__ void tile_c128(const Desc& d, int r0, int c0, int mb,
   const int tx = tid & 15, ty = tid >> 4;
   const int K = s.alpha_zero ? 0 : d.k;
   const double2* A = reinterpret_cast<const double2*>(d.A);
-  double2 acc[FULL ? 2 : 1][2];
+  double2 acc[FULL ? 2 : 1][FULL ? 2 : 1];
   double2 lin[FULL ? 1 : NJ];
   int rc[FULL ? 1 : NJ];
   if constexpr (FULL) {
@@ -460,24 +522,9 @@ __device__ __forceinline__ void tile_c128(const Desc& d, int r0, int c0, int mb,
     if (more) gload(k0 + BKC);
     if constexpr (!FULL) {
       const int kend = min(BKC, K - k0);
-      if constexpr (NJ == 2) {
-        // (an output at a time: with the outputs inside, as below, a warp with one of
-        // them took as long as one with both; 500 of order 17 45.1 -> 30.8 us, 200 of
-        // order 32 97 -> 66 us. With four outputs the order below is 2% faster)
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-          if (j >= nj) break;
-          const int r = rc[j] & 0xFFFF, c = rc[j] >> 16;
-#pragma unroll 2
-          for (int kk = 0; kk < kend; ++kk) cmac(lin[j], sm.a[st][kk][r], sm.b[st][kk][c]);
-        }
-      } else {
-#pragma unroll 2
-        for (int kk = 0; kk < kend; ++kk)
-#pragma unroll
-          for (int j = 0; j < NJ; ++j)
-            if (j < nj) cmac(lin[j], sm.a[st][kk][rc[j] & 0xFFFF], sm.b[st][kk][rc[j] >> 16]);
-      }
+      linear_products<NJ>(nj, kend, [&](int j, int kk) {
+        cmac(lin[j], sm.a[st][kk][rc[j] & 0xFFFF], sm.b[st][kk][rc[j] >> 16]);
+      });
     } else
 #pragma unroll
     for (int kk = 0; kk < BKC; ++kk) {
@@ -492,166 +539,105 @@ __device__ __forceinline__ void tile_c128(const Desc& d, int r0, int c0, int mb,
     __syncthreads();
     st ^= 1;
   }
-  double2* C = reinterpret_cast<double2*>(d.C);
   if constexpr (!FULL) {
+    with_beta(s, [&](auto beta) {
 #pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-      const int r = r0 + (rc[j] & 0xFFFF), c = c0 + (rc[j] >> 16);
-      if (tid + kFp64Threads * j >= mb * nb || !keep_out(d, r, c)) continue;
-      double2* cp = C + r + (int64_t)c * d.ldc;
-      double2 v = c_epilogue(lin[j], cp, s);
-      if (d.herm && r == c) v.y = 0.0;
-      *cp = v;
-    }
+      for (int j = 0; j < NJ; ++j)
+        if (tid + kFp64Threads * j < mb * nb)
+          store_out<decltype(beta)::value>(d, s, r0 + (rc[j] & 0xFFFF), c0 + (rc[j] >> 16), lin[j]);
+    });
     return;
   } else
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const int c = c0 + tx * 2 + j;
-    if (c >= d.n) continue;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int r = r0 + ty * 2 + i;
-      if (r >= d.m || !keep_out(d, r, c)) continue;
-      double2* cp = C + r + (int64_t)c * d.ldc;
-      double2 v = c_epilogue(acc[i][j], cp, s);
-      if (d.herm && r == c) v.y = 0.0;
-      *cp = v;
-    }
-  }
+  store_block(d, s, r0 + ty * 2, c0 + tx * 2, acc);
 }
 
 // ---- small programs: a warp per instance --------------------------------------
 // The m*n outputs in column-major order, 32 MAXOUT at a time: lane t owns outputs
 // o = t + 32 j (j < MAXOUT) of them, (r, c) = (o mod m, o div m). When m divides 32
 // the row is the same for every j and the column steps by 32 / m, so one A load
-// feeds MAXOUT DFMAs; otherwise every output loads its own A element.
+// feeds up to MAXOUT DFMAs; otherwise every output loads its own A element.
 
-template <int MAXOUT>
-__device__ __forceinline__ void small_r64(const Desc& d, const Scalars& s) {
-  const int lane = threadIdx.x & 31;
-  const int m = d.m, n = d.n, mn = m * n;
-  const int K = s.alpha_zero ? 0 : d.k;
-  double acc[MAXOUT];
-  if (m > 0 && (32 % m) == 0) {
-    const int r = lane % m, cstep = 32 / m;
-    const double* ap = d.A + r;
-    const int64_t bstep = (int64_t)cstep * d.ldb;
-    for (int c0 = lane / m; c0 < n; c0 += MAXOUT * cstep) {
-      const double* bp = d.B + (int64_t)c0 * d.ldb;
-#pragma unroll
-      for (int j = 0; j < MAXOUT; ++j) acc[j] = 0.0;
-#pragma unroll 1
-      for (int p = 0; p < K; ++p) {
-        const double a = __ldg(ap + (int64_t)p * d.lda);
-#pragma unroll
-        for (int j = 0; j < MAXOUT; ++j)
-          if (c0 + j * cstep < n)
-            acc[j] = fma(a, d.herm ? ld_b(d, p, c0 + j * cstep) : __ldg(bp + p + j * bstep), acc[j]);
-      }
-#pragma unroll
-      for (int j = 0; j < MAXOUT; ++j) {
-        const int c = c0 + j * cstep;
-        if (c < n && keep_out(d, r, c)) {
-          double* cp = d.C + r + (int64_t)c * d.ldc;
-          double v = s.alpha_re * acc[j];
-          if (!s.beta_zero) v = fma(s.beta_re, *cp, v);
-          *cp = v;
-        }
-      }
-    }
-  } else {
-    int rc[MAXOUT];  // row | column << 16
-    for (int o0 = lane; o0 < mn; o0 += 32 * MAXOUT) {
-      const int cnt = (mn - (o0 - lane) + 31) / 32;  // outputs of this warp's lanes
-#pragma unroll
-      for (int j = 0; j < MAXOUT; ++j) {
-        const int o = min(o0 + 32 * j, mn - 1), c = o / m;
-        rc[j] = (o - c * m) | c << 16;
-        acc[j] = 0.0;
-      }
-#pragma unroll 1
-      for (int p = 0; p < K; ++p) {
-        const double* ap = d.A + (int64_t)p * d.lda;
-#pragma unroll
-        for (int j = 0; j < MAXOUT; ++j)
-          if (j < cnt) acc[j] = fma(__ldg(ap + (rc[j] & 0xFFFF)), ld_b(d, p, rc[j] >> 16), acc[j]);
-      }
-#pragma unroll
-      for (int j = 0; j < MAXOUT; ++j) {
-        const int r = rc[j] & 0xFFFF, c = rc[j] >> 16;
-        if (o0 + 32 * j >= mn || !keep_out(d, r, c)) continue;
-        double* cp = d.C + r + (int64_t)c * d.ldc;
-        double v = s.alpha_re * acc[j];
-        if (!s.beta_zero) v = fma(s.beta_re, *cp, v);
-        *cp = v;
-      }
+// Runs f with the smallest of the powers of two up to MAXOUT that is not below cnt
+// (the outputs per lane, the same in all lanes): a DFMA that is off in every
+// lane would take the FP64 pipe as long as one that is on.
+template <int MAXOUT, class F>
+__device__ __forceinline__ void with_outputs(int cnt, const F& f) {
+  if constexpr (MAXOUT > 1) {
+    if (cnt <= MAXOUT / 2) {
+      with_outputs<MAXOUT / 2>(cnt, f);
+      return;
     }
   }
+  f(std::integral_constant<int, MAXOUT>{});
 }
 
-template <int MAXOUT>
-__device__ __forceinline__ void small_c128(const Desc& d, const Scalars& s) {
+__device__ __forceinline__ void small_product(double& acc, double a, double b) {
+  acc = fma(a, b, acc);
+}
+__device__ __forceinline__ void small_product(double2& acc, double2 a, double2 b) {
+  cmac(acc, a, b);
+}
+__device__ __forceinline__ double small_b(const Desc& d, int p, int c, double) {
+  return ld_b(d, p, c);
+}
+__device__ __forceinline__ double2 small_b(const Desc& d, int p, int c, double2) {
+  return ld_bc(d, p, c);
+}
+// T: double or double2.
+template <class T, int MAXOUT>
+__device__ __forceinline__ void small_instance(const Desc& d, const Scalars& s) {
   const int lane = threadIdx.x & 31;
   const int m = d.m, n = d.n, mn = m * n;
   const int K = s.alpha_zero ? 0 : d.k;
-  const double2* A = reinterpret_cast<const double2*>(d.A);
-  const double2* B = reinterpret_cast<const double2*>(d.B);
-  double2* C = reinterpret_cast<double2*>(d.C);
-  double2 acc[MAXOUT];
-  if (m > 0 && (32 % m) == 0) {
-    const int r = lane % m, cstep = 32 / m;
-    const int64_t bstep = (int64_t)cstep * d.ldb;
-    for (int c0 = lane / m; c0 < n; c0 += MAXOUT * cstep) {
-      const double2* bp = B + (int64_t)c0 * d.ldb;
-#pragma unroll
-      for (int j = 0; j < MAXOUT; ++j) acc[j] = make_double2(0.0, 0.0);
+  const T* A = reinterpret_cast<const T*>(d.A);
+  const T* B = reinterpret_cast<const T*>(d.B);
+  const bool divides = m > 0 && (32 % m) == 0;
+  for (int o0 = 0; o0 < mn; o0 += 32 * MAXOUT) {
+    with_outputs<MAXOUT>((mn - o0 + 31) / 32, [&](auto outputs) {
+      constexpr int N = decltype(outputs)::value;
+      T acc[N] = {};
+      if (divides) {
+        const int r = lane % m, cstep = 32 / m, c0 = o0 / m + lane / m;
+        const T* ap = A + r;
+        const T* bp = B + (int64_t)c0 * d.ldb;
+        const int64_t bstep = (int64_t)cstep * d.ldb;
 #pragma unroll 1
-      for (int p = 0; p < K; ++p) {
-        const double2 a = __ldg(A + r + (int64_t)p * d.lda);
+        for (int p = 0; p < K; ++p) {
+          const T a = __ldg(ap + (int64_t)p * d.lda);
 #pragma unroll
-        for (int j = 0; j < MAXOUT; ++j)
-          if (c0 + j * cstep < n)
-            cmac(acc[j], a, d.herm ? ld_bc(d, p, c0 + j * cstep) : __ldg(bp + p + j * bstep));
-      }
-#pragma unroll
-      for (int j = 0; j < MAXOUT; ++j) {
-        const int c = c0 + j * cstep;
-        if (c < n && keep_out(d, r, c)) {
-          double2* cp = C + r + (int64_t)c * d.ldc;
-          double2 v = c_epilogue(acc[j], cp, s);
-          if (d.herm && r == c) v.y = 0.0;
-          *cp = v;
+          for (int j = 0; j < N; ++j)
+            if (c0 + j * cstep < n)
+              small_product(acc[j], a, d.herm ? small_b(d, p, c0 + j * cstep, T{})
+                                              : __ldg(bp + p + j * bstep));
         }
-      }
-    }
-  } else {
-    int rc[MAXOUT];
-    for (int o0 = lane; o0 < mn; o0 += 32 * MAXOUT) {
-      const int cnt = (mn - (o0 - lane) + 31) / 32;
+        with_beta(s, [&](auto beta) {
 #pragma unroll
-      for (int j = 0; j < MAXOUT; ++j) {
-        const int o = min(o0 + 32 * j, mn - 1), c = o / m;
-        rc[j] = (o - c * m) | c << 16;
-        acc[j] = make_double2(0.0, 0.0);
-      }
+          for (int j = 0; j < N; ++j)
+            if (c0 + j * cstep < n)
+              store_out<decltype(beta)::value>(d, s, r, c0 + j * cstep, acc[j]);
+        });
+      } else {
+        int rc[N];  // row | column << 16
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+          const int o = min(o0 + lane + 32 * j, mn - 1), c = o / m;
+          rc[j] = (o - c * m) | c << 16;
+        }
 #pragma unroll 1
-      for (int p = 0; p < K; ++p) {
-        const double2* ap = A + (int64_t)p * d.lda;
+        for (int p = 0; p < K; ++p) {
+          const T* ap = A + (int64_t)p * d.lda;
 #pragma unroll
-        for (int j = 0; j < MAXOUT; ++j)
-          if (j < cnt) cmac(acc[j], __ldg(ap + (rc[j] & 0xFFFF)), ld_bc(d, p, rc[j] >> 16));
-      }
+          for (int j = 0; j < N; ++j)
+            small_product(acc[j], __ldg(ap + (rc[j] & 0xFFFF)), small_b(d, p, rc[j] >> 16, T{}));
+        }
+        with_beta(s, [&](auto beta) {
 #pragma unroll
-      for (int j = 0; j < MAXOUT; ++j) {
-        const int r = rc[j] & 0xFFFF, c = rc[j] >> 16;
-        if (o0 + 32 * j >= mn || !keep_out(d, r, c)) continue;
-        double2* cp = C + r + (int64_t)c * d.ldc;
-        double2 v = c_epilogue(acc[j], cp, s);
-        if (d.herm && r == c) v.y = 0.0;
-        *cp = v;
+          for (int j = 0; j < N; ++j)
+            if (o0 + lane + 32 * j < mn)
+              store_out<decltype(beta)::value>(d, s, rc[j] & 0xFFFF, rc[j] >> 16, acc[j]);
+        });
       }
-    }
+    });
   }
 }
 
@@ -660,86 +646,53 @@ constexpr int kSmallR64 = 256, kSmallC128 = 128;
 
 // ---- the persistent kernel ---------------------------------------------------------
 
-union SmemFp64 {
-  SmemR64 r;
-  SmemC128 c;
-};
-
 // CTAS: CTAs per SM. Several hide each other's start (work item, first operand
 // loads): two where tiles are ragged (33^3 x 1000: 150 -> 102 us), three where
 // all are small, in the registers that the small tiles leave (32^3 x 20000:
 // 2710, 1540 and 1257 us with one, two and three). Full tiles run 2-5% faster
 // alone (128^3 x 100: 430 -> 411 us).
-template <int CTAS, class Src, class Sched>
+// A kernel per element type: with both types' programs in one, either's registers
+// and order of instructions came to depend on the other's.
+template <int CTAS, bool CPLX, class Src, class Sched>
 __global__ void __launch_bounds__(kFp64Threads, CTAS)
     fp64_persistent(Src src, Sched sched, int64_t n_items, Scalars s) {
-  __shared__ __align__(16) SmemFp64 sm;
+  __shared__ __align__(16) std::conditional_t<CPLX, SmemC128, SmemR64> sm;
   const int warp = threadIdx.x >> 5;
-  if constexpr (CTAS == 3) {  // small tiles only
-    for (int64_t it = blockIdx.x; it < n_items; it += gridDim.x) {
-      const WorkItem w = sched.get(it);
-      const Desc d = src.desc(w.inst);
-      int tm, tn;
-      tile_extent_of(w.count, TR, &tm, &tn);
-      const int mb = min(tm, d.m - w.r0), nb = min(tn, d.n - w.c0);
-      if (mb <= 0 || nb <= 0) continue;
-      if (w.prog == PROG_R64_TILE) {
-        if (tile_program_r64(mb * nb) > 2) tile_r64<false, 4>(d, w.r0, w.c0, mb, nb, s, sm.r);
-        else tile_r64<false, 2>(d, w.r0, w.c0, mb, nb, s, sm.r);
-      } else if (tile_program_c128(mb * nb) > 1) {
-        tile_c128<false, 2>(d, w.r0, w.c0, mb, nb, s, sm.c);
-      } else {
-        tile_c128<false, 1>(d, w.r0, w.c0, mb, nb, s, sm.c);
-      }
-    }
-    return;
-  }
   for (int64_t it = blockIdx.x; it < n_items; it += gridDim.x) {
     const WorkItem w = sched.get(it);
-    switch (w.prog) {
-      case PROG_R64_TILE: {
-        const Desc d = src.desc(w.inst);
-        int tm, tn;
-        tile_extent_of(w.count, TR, &tm, &tn);
-        const int mb = min(tm, d.m - w.r0), nb = min(tn, d.n - w.c0);
-        if (mb <= 0 || nb <= 0) break;  // (a chain index that names no matrix)
-        const int per = tile_program_r64(mb * nb);
-        if (per == 16) tile_r64<true, 1>(d, w.r0, w.c0, mb, nb, s, sm.r);
-        else if (per == 8) tile_r64<false, 8>(d, w.r0, w.c0, mb, nb, s, sm.r);
-        else if (per == 4) tile_r64<false, 4>(d, w.r0, w.c0, mb, nb, s, sm.r);
-        else tile_r64<false, 2>(d, w.r0, w.c0, mb, nb, s, sm.r);
-        break;
-      }
-      case PROG_R64_DMMA:
-        tile_r64_dmma(src.desc(w.inst), w.r0, w.c0, s, sm.r);
-        break;
-      case PROG_C128_TILE: {
-        const Desc d = src.desc(w.inst);
-        int tm, tn;
-        tile_extent_of(w.count, TC, &tm, &tn);
-        const int mb = min(tm, d.m - w.r0), nb = min(tn, d.n - w.c0);
-        if (mb <= 0 || nb <= 0) break;
-        const int per = tile_program_c128(mb * nb);
-        if (mb == TC && nb == TC) tile_c128<true, 1>(d, w.r0, w.c0, mb, nb, s, sm.c);
-        else if (per == 4) tile_c128<false, 4>(d, w.r0, w.c0, mb, nb, s, sm.c);
-        else if (per == 2) tile_c128<false, 2>(d, w.r0, w.c0, mb, nb, s, sm.c);
-        else tile_c128<false, 1>(d, w.r0, w.c0, mb, nb, s, sm.c);
-        break;
-      }
-      case PROG_R64_SMALL:
+    if constexpr (CTAS < 3) {  // (three CTAs: small tiles only)
+      if (w.prog == (CPLX ? PROG_C128_SMALL : PROG_R64_SMALL)) {
         if (warp < w.count) {
           const Desc d = src.desc(src.small_inst((int64_t)w.inst + warp));
-          small_r64<kSmallR64 / 32>(d, s);
+          if constexpr (CPLX) small_instance<double2, kSmallC128 / 32>(d, s);
+          else small_instance<double, kSmallR64 / 32>(d, s);
         }
-        break;
-      case PROG_C128_SMALL:
-        if (warp < w.count) {
-          const Desc d = src.desc(src.small_inst((int64_t)w.inst + warp));
-          small_c128<kSmallC128 / 32>(d, s);
+        continue;
+      }
+      if constexpr (!CPLX) {
+        if (w.prog == PROG_R64_DMMA) {
+          tile_r64_dmma(src.desc(w.inst), w.r0, w.c0, s, sm);
+          continue;
         }
-        break;
-      default:
-        break;
+      }
+    }
+    const Desc d = src.desc(w.inst);
+    int tm, tn;
+    tile_extent_of(w.count, CPLX ? TC : TR, &tm, &tn);
+    const int mb = min(tm, d.m - w.r0), nb = min(tn, d.n - w.c0);
+    if (mb <= 0 || nb <= 0) continue;  // (a chain index that names no matrix)
+    if constexpr (CPLX) {
+      const int per = tile_program_c128(mb * nb);
+      if (CTAS < 3 && mb == TC && nb == TC) tile_c128<true, 1>(d, w.r0, w.c0, mb, nb, s, sm);
+      else if (CTAS < 3 && per == 4) tile_c128<false, 4>(d, w.r0, w.c0, mb, nb, s, sm);
+      else if (per > 1) tile_c128<false, 2>(d, w.r0, w.c0, mb, nb, s, sm);
+      else tile_c128<false, 1>(d, w.r0, w.c0, mb, nb, s, sm);
+    } else {
+      const int per = tile_program_r64(mb * nb);
+      if (CTAS < 3 && per == 16) tile_r64<true, 1>(d, w.r0, w.c0, mb, nb, s, sm);
+      else if (CTAS < 3 && per == 8) tile_r64<false, 8>(d, w.r0, w.c0, mb, nb, s, sm);
+      else if (per > 2) tile_r64<false, 4>(d, w.r0, w.c0, mb, nb, s, sm);
+      else tile_r64<false, 2>(d, w.r0, w.c0, mb, nb, s, sm);
     }
   }
 }
@@ -764,11 +717,14 @@ void prog_tile(int prog, int* tm, int* tn) {
 // program, us for 30000 real or 20000 complex instances: 1 x 300 x 16 1476 and 693,
 // 2 x 200 x 16 1191 and 758 (x 32 2033 and 1499, but 3000 of them 207 and 229),
 // 5 x 100 x 8 546 and 400 (x 16 736 and 735), 20 x 20 x 4 260 and 185 (x 8 342 and
-// 328), 32 x 32 x 4 441 and 357 (x 8 651 and 655); complex 1 x 300 x 32 3162 and 1520,
-// 16 x 16 x 8 390 and 329 (x 16 654 and 620, but 3000 of them 106 and 112).
+// 328), 3000 of 32 x 32 x 3 40 and 39 (x 4 43 and 47); complex 1 x 300 x 32 3162 and
+// 1520, 16 x 16 x 8 390 and 329 (x 16 654 and 620, but 3000 of them 106 and 112).
 static bool small_fits(bg_dtype dt, int64_t m, int64_t n, int64_t k) {
   const int64_t held = dt == BG_R64 ? kSmallR64 : kSmallC128, thin = std::min(m, n);
-  const int64_t k_max = dt == BG_R64 ? (thin <= 2 ? 16 : thin < 8 ? 8 : 4) : (thin <= 2 ? 32 : 8);
+  const int64_t k_max = dt == BG_C128       ? (thin <= 2 ? 32 : 8)
+                        : thin < 8          ? (thin <= 2 ? 16 : 8)
+                        : m * n <= 2 * held ? 4
+                                            : 3;
   return m * n <= (k <= k_max ? 4 * held : held);
 }
 
@@ -852,15 +808,23 @@ int default_prog(bg_dtype dt, int64_t m, int64_t n, int64_t k, int64_t batch, in
   return dt == BG_R64 ? PROG_R64_TILE : PROG_C128_TILE;
 }
 
-template <class Src, class Sched>
-static void launch_persistent(int ctas, int grid, cudaStream_t st, const Src& src,
-                              const Sched& sched, int64_t n_items, const Scalars& s) {
+template <bool CPLX, class Src, class Sched>
+static void launch_typed(int ctas, int grid, cudaStream_t st, const Src& src, const Sched& sched,
+                         int64_t n_items, const Scalars& s) {
   if (ctas == 1)
-    fp64_persistent<1, Src, Sched><<<grid, kFp64Threads, 0, st>>>(src, sched, n_items, s);
+    fp64_persistent<1, CPLX, Src, Sched><<<grid, kFp64Threads, 0, st>>>(src, sched, n_items, s);
   else if (ctas == 3)
-    fp64_persistent<3, Src, Sched><<<grid, kFp64Threads, 0, st>>>(src, sched, n_items, s);
+    fp64_persistent<3, CPLX, Src, Sched><<<grid, kFp64Threads, 0, st>>>(src, sched, n_items, s);
   else
-    fp64_persistent<2, Src, Sched><<<grid, kFp64Threads, 0, st>>>(src, sched, n_items, s);
+    fp64_persistent<2, CPLX, Src, Sched><<<grid, kFp64Threads, 0, st>>>(src, sched, n_items, s);
+}
+
+template <class Src, class Sched>
+static void launch_persistent(bg_dtype dt, int ctas, int sms, cudaStream_t st, const Src& src,
+                              const Sched& sched, int64_t n_items, const Scalars& s) {
+  const int grid = (int)std::min<int64_t>(n_items, (int64_t)sms * ctas);
+  if (dt == BG_C128) launch_typed<true>(ctas, grid, st, src, sched, n_items, s);
+  else launch_typed<false>(ctas, grid, st, src, sched, n_items, s);
 }
 
 cudaError_t launch_fp64_fixed(bg_dtype dt, int prog, int64_t m, int64_t n, int64_t k,
@@ -896,8 +860,7 @@ cudaError_t launch_fp64_fixed(bg_dtype dt, int prog, int64_t m, int64_t n, int64
                    : sched.tm > 0 && sched.tm * sched.tn <= (dt == BG_C128 ? 2 : 4) * kFp64Threads
                        ? 3
                        : 2;
-  launch_persistent(ctas, (int)std::min<int64_t>(n_items, (int64_t)sms * ctas), st, src, sched,
-                    n_items, s);
+  launch_persistent(dt, ctas, sms, st, src, sched, n_items, s);
   count_launch();
   return cudaGetLastError();
 }
@@ -916,8 +879,7 @@ cudaError_t launch_fp64_table(bg_dtype dt, const int64_t* d_table, const int32_t
   src.C = static_cast<double*>(C);
   src.esz = dt == BG_C128 ? 2 : 1;
   TableSched sched{d_items};
-  launch_persistent(ctas, (int)std::min<int64_t>(n_items, (int64_t)sms * ctas), st, src,
-                    sched, n_items, s);
+  launch_persistent(dt, ctas, sms, st, src, sched, n_items, s);
   count_launch();
   return cudaGetLastError();
 }
@@ -945,8 +907,7 @@ cudaError_t launch_fp64_chain(bg_dtype dt, const int64_t* d_wn, const int64_t* d
   s.alpha_re = 1.0; s.alpha_im = 0.0; s.beta_re = 0.0; s.beta_im = 0.0;
   s.alpha_zero = 0; s.beta_zero = 1;
   TableSched sched{d_items};
-  launch_persistent(ctas, (int)std::min<int64_t>(n_items, (int64_t)sms * ctas), st, src,
-                    sched, n_items, s);
+  launch_persistent(dt, ctas, sms, st, src, sched, n_items, s);
   count_launch();
   return cudaGetLastError();
 }
