@@ -1091,7 +1091,16 @@ cudaError_t launch_reduce(const TriArgs& a, int64_t walkers, const TriShape& s, 
   return cudaGetLastError();
 }
 
+// Once per device: five calls of the driver, a sixth of a small plan's making.
 cudaError_t set_smem_limits() {
+  static std::mutex mu;
+  static bool done[kAttrDevices];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const bool tracked = dev >= 0 && dev < kAttrDevices;
+  std::lock_guard<std::mutex> lk(mu);
+  if (tracked && done[dev]) return cudaSuccess;
   // (the packed kernel's request needs no raised limit)
   static_assert(tail_smem(kPacked, kPackedWarps) + sizeof(Shared) <= 48 * 1024, "packed CTA");
   const void* kernels[] = {(const void*)tri_reduce_kernel<false, true, kTail / 32, kWarps>,
@@ -1100,10 +1109,10 @@ cudaError_t set_smem_limits() {
                            (const void*)tri_reduce_kernel<false, true, 0, kWarps>,
                            (const void*)tri_reduce_kernel<false, false, 0, kWarps>};
   for (const void* k : kernels) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
     if (e != cudaSuccess) return e;
   }
+  if (tracked) done[dev] = true;
   return cudaSuccess;
 }
 
