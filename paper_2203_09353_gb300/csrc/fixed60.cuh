@@ -71,10 +71,7 @@ __device__ __forceinline__ int4 conj(const int4& a) { return make_int4(a.x, a.y,
 struct Sum {
   long long rh = 0, rx = 0, ih = 0, ix = 0;
   __device__ __forceinline__ void add(const int4& a, const int4& b) {  // += a b
-    add(a, b, make_int2(-b.z, -b.w));
-  }
-  // (nb: -im b, where the caller has it)
-  __device__ __forceinline__ void add(const int4& a, const int4& b, const int2& nb) {
+    const int2 nb = make_int2(-b.z, -b.w);
     mac(rh, a.x, b.x);
     mac(rx, a.x, b.y);
     mac(ih, a.x, b.z);
