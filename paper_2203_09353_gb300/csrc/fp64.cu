@@ -263,8 +263,8 @@ __device__ __forceinline__ void linear_products(int nj, int kend, F mul) {
 
 // Rows r0 .. r0 + tm - 1 and columns c0 .. c0 + tn - 1 (tm, tn <= 64) of one
 // instance; FULL: 64 x 64, or what the instance leaves of it, 4 x 4 outputs per
-// thread (for more outputs than NJ = 8 holds). Otherwise output o of the tile's mb x nb (column-major) goes to
-// thread o mod 256, NJ outputs to a thread: a DFMA takes its 16 clocks per SM
+// thread (for more outputs than NJ = 8 holds). Otherwise output o of the tile's
+// mb x nb (column-major) goes to thread o mod 256, NJ outputs to a thread: a DFMA takes its 16 clocks per SM
 // whether 1 or 32 of the warp's lanes are active (measured), so padding a
 // ragged tile to 64 x 64 costs in full, while the two extra shared-memory
 // reads per DFMA of this order are hidden behind it.

@@ -855,8 +855,8 @@ __device__ __forceinline__ float scaled_abs(double x, int e) {
 }
 
 // The whole reduction of walker blockIdx.x / cl by W warps. ROWS: n <= 32 ROWS,
-// the matrix goes straight to shared memory (0: any order above kTail). Bound by the multiply pipe (76-80%
-// busy at n = 256, with 1.6 times the products' own instructions) and, in the
+// the matrix goes straight to shared memory (0: any order above kTail). Bound by the multiply pipe (77%
+// of a busy SM's cycles at n = 256, 1.7 times what the products need) and, in the
 // last columns and for few walkers, by the latency of a column. Measured
 // against panels with an FP64 product, split GEMMs between them and an FP64
 // kernel for the last 64 columns: 128 matrices of order 256 12.6 -> 5.3 ms, 16
